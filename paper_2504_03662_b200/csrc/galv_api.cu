@@ -99,6 +99,7 @@ int galv_create(galv_ctx** out, int device_ordinal)
     ctx->err[0] = 0;
     ctx->profiling = 0;
     ctx->prof_count = 0;
+    ctx->plan_valid = 0;
     for (auto& ev : ctx->pev) ev = nullptr;
     int cur = -1;
     cudaGetDevice(&cur);
@@ -207,6 +208,7 @@ int galv_dp_search(galv_ctx* ctx, const galv_shape* sh, const int32_t* L, const 
     a.C = C; a.A = A; a.C_last = C_last;
     a.roll = reinterpret_cast<int32_t*>(ws + w.roll);
     a.order = reinterpret_cast<int32_t*>(ws + w.order);
+    a.done = reinterpret_cast<int32_t*>(ws + w.done);
     a.nactive = reinterpret_cast<int32_t*>(ws + w.nactive);
     a.scratch = reinterpret_cast<int32_t*>(ws + w.scratch);
     a.work = reinterpret_cast<unsigned long long*>(a.scratch + 2 * (sh->Lmax + 2));

@@ -1,174 +1,469 @@
-// Small batches: one thread-block cluster per search instance, the table slice kept in shared memory.
+// The whole recurrence of one instance on the SMs of one thread-block cluster, its state kept in shared memory.
 //
-//   C[l][m][s] = time(l,s) + min_{s'} ( C[l-1][m-mem(l,s)][s'] + trans(s',s) )
+//   C[l][m][s] = time(l,s) + G[l][m - mem(l,s)][s],   G[l][m][s] = min_{s'} ( C[l-1][m][s'] + trans(s',s) )
 //
-// (Section 3 of the paper: the selector searches again while the job runs, one model at a time;
-// Section 4: the manager's step.  Such a re-search is a batch of one to a few dozen instances.)
+// (Section 3 of the paper: dynamic-programming search over a performance model; Sections 3-4: it runs again while
+// the job runs.)
 //
-// With fewer work items per layer than the GPU has SMs the tiled kernel's step is a chain of dependent
-// layers, each link paying a trip through L2 and a gpu-scope publish.  Here the chain never leaves the
-// SMs: the budget columns of ONE instance are split over the CTAs of a cluster (CTA r owns columns
-// r*W .. r*W+W-1), each CTA keeps its columns of the previous layer, all S rows, in shared memory,
-// computes G[s][m'] = min_{s'}(Cprev[s'][m'] + T[s'][s]) for its own columns m' (no halo: G does not
-// depend on mem) and PUSHES time + G to where it belongs, column m' + mem(l,s) of the next layer's
-// buffer, which lies in its own shared memory or in that of a CTA further up: a plain store into
-// distributed shared memory.  One hardware cluster barrier per layer (release / acquire) ends the
-// layer.  Cells no column maps to (m < mem(l,s)) are written +inf by the CTA that owns them.
-// The finished slice of a layer goes to the table in HBM by ONE tensor-map bulk store (TMA) straight
-// from the shared-memory buffer, issued by a service warp while the other warps compute the next layer.
+// What a layer hands to the next one is G, and G has one row per DISTINCT COLUMN of the transition matrix: strategies
+// with equal columns have equal G.  Strategies with equal ROWS enter the minimum with the same offset, so only the
+// smallest of them matters.  A matrix that prices a move between layouts (tensor-parallel degree, sequence
+// parallelism) has a handful of distinct rows and columns however many strategies there are (8 among 64, 4 among 24):
+// a cell then costs one addition, one minimum over its class and its store instead of S add-mins, and the state of an
+// instance shrinks from S to 8 rows.  The kernel finds the classes itself, by comparing the matrix's rows and columns
+// word by word (hashes only propose), so nothing is assumed about where a matrix comes from.
+// A matrix without such structure keeps all S rows.  Then a candidate C[l-1][m][s'] that lies more than the largest
+// transition entry above its column's best can neither win nor tie (the best row gives a candidate at most that entry
+// above itself), so a warp relaxes only the rows that are alive in one of its columns.
 //
-// The kernel validates its instance itself, writes the base layer, every layer and C_last: the
-// whole search is one launch.  No spin-waits anywhere: the cluster barrier is a hardware barrier
-// among co-scheduled CTAs, and clusters never wait on one another.  No cluster multicast.
-
-#include <cuda.h>
+// The budget columns are split over the CTAs of the cluster: CTA r owns columns r*W .. r*W+W-1 and keeps their G in two
+// buffers (this layer's, the next one's), with a halo of H columns to their left: C is produced by GATHERING G at
+// m - mem(l,s), from this CTA's own shared memory as long as the shift stays within the halo.  Whoever computes a column
+// writes it to its own buffer and into the halo of the CTAs further up that hold it (distributed shared memory; a store
+// is fired and forgotten, while reading the cells from their owner instead puts a round trip on every gather's chain:
+// 8.4 us a layer on one instance of 24 strategies over 16 CTAs).  A layer ends with one cluster barrier (a block barrier
+// where the cluster is one CTA).  No spin-waits, no cooperative launch, no cluster multicast, no workspace but a word per
+// instance and the path flag; the tables go out as full 128-byte lines and are never read back.
+//
+// Validation is the kernel's own (same rules and status bits as everywhere).  An instance whose state does not fit this
+// launch's shared memory is left alone and marked in done[]; a second launch with larger clusters or the tiled kernels
+// take it.
 
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <type_traits>
 
 #include "galv_internal.h"
-
 
 namespace {
 
 constexpr int kInf = GALV_INF;
 constexpr int kMaxSortedB = 512;          // instances whose lengths fit the ranking scratch below
-constexpr int kRowsPerLane = 4;           // strategies per lane of the service warp: S <= 128
+constexpr int kMaxS = 128;
+constexpr int kMaxWarps = 15;             // compute warps per CTA (with the service warp 512 threads: 128 registers each)
+constexpr int kStaticSmem = 5632;         // the kernel's static shared memory, rounded up
+constexpr int kClassMax = 16;             // classes beyond which the matrix counts as unstructured
 
-struct ClArgs {
+struct RsArgs {
     int B, Lmax, S, M, m_pitch;
     int CL;            // CTAs per cluster
     int W;             // budget columns per CTA (multiple of 32)
-    int G;             // W / 32
-    int NSG;           // ceil(S / 8)
-    int SP8;           // NSG * 8: row pitch of the trans matrix in shared memory
-    int nct;           // column tiles of 32*TM columns per CTA
-    int units;         // nct * NSG work units per CTA and layer
+    int gints;         // words of one state buffer: rows of W columns and their halo
+    int SP;            // row pitch of the full transition matrix in shared memory; 0: no room for unstructured matrices
     int sorted;        // clusters take the instances longest first
+    int second;        // only the instances the first launch left alone
+    int path_value;    // what galv_dp_search_path reports
     const int32_t* L;
     const int32_t* time_q;
     const int32_t* mem_q;
     const int32_t* trans_q;
     long long trans_inst, trans_layer;
     int32_t* C;        // full table or NULL
+    uint8_t* A;        // argmin table or NULL
     int32_t* C_last;
     int32_t* status;
     int32_t* path;     // [4] device flags of the search: error, -, -, kernel that ran
+    int32_t* done;     // [B] 1: this instance needs nothing more
 };
 
-// 3-D view of a table for the tensor-map store: [rows of S strategies per (instance, layer)][m_pitch / 32][32].
-// A CTA's slice [S][G][32] in shared memory is then one box.
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-// address of the same shared-memory location in the CTA of rank `rank` of this cluster
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void st_cluster(uint32_t addr, int v) {
-    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+__device__ __forceinline__ int ld_cluster(uint32_t addr) {
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
 }
-__device__ __forceinline__ void cluster_barrier() {
-    __syncwarp();                                              // the aligned forms want the whole warp together
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+__device__ __forceinline__ int ld_cluster_u8(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return (int)v;
 }
+__device__ __forceinline__ void st_cluster(uint32_t addr, int v) { asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ void st_cluster_u8(uint32_t addr, int v) { asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// One box [S][G][32] from shared memory to element coordinates (0, g0, row0) of the table behind `map`;
-// what lies beyond the tensor's edge (the last CTA's columns past m_pitch) is not written.
-__device__ __forceinline__ void tensor_store_3d(const CUtensorMap* map, const void* src, int g0, int row0) {
-    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
-                 ::"l"(map), "r"(0), "r"(g0), "r"(row0), "r"(smem_addr(src)) : "memory");
+// everyone's shared-memory writes of this layer are visible to the cluster
+__device__ __forceinline__ void layer_barrier(int CL) {
+    __syncwarp();                                              // the aligned forms want the whole warp together
+    if (CL == 1) {
+        asm volatile("bar.sync 0;" ::: "memory");              // the service warp meets it at another place in the code
+    } else {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
 }
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 __device__ __forceinline__ void cp_async_4(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// What the push of one (column tile, strategy) needs, derived once per layer and CTA by the service warp.
-// Column m' of strategy s belongs at column m' + mem(l,s); for the tile that starts at this CTA's column colb:
-//   x = CTA of the cluster that receives the tile's first column (-1: nothing of the tile lands inside the budget),
-//   y = offset of that first column inside the receiving CTA's columns, z = time(l,s),
-//   w = kWholeTile when all nj*32 columns land in CTA x, else the largest offset that still lands inside the
-//       budget (the tile then straddles two CTAs or the budget's edge and every column is checked).
-// mem is clamped to M+1: nothing it shifts by lands inside the budget.  Pad strategies (s >= S) get x = -1.
-constexpr int kWholeTile = 0x7fffffff;
-__device__ __forceinline__ int4 tile_record(bool real, int mem, int time, int M, int W, int rank, int colb, int ncols) {
-    const int mc = mem < M + 1 ? mem : M + 1;
-    const int q = mc / W;
-    int d = rank + q, xb = colb + (mc - q * W);
-    if (xb >= W) { xb -= W; ++d; }
-    const int lim = M - d * W;
-    if (!real || lim < xb) return make_int4(-1, 0, time, 0);
-    const bool whole = xb + ncols <= W && xb + ncols - 1 <= lim;
-    return make_int4(d, xb, time, whole ? kWholeTile : lim);
-}
-// cells of this CTA's own columns that no column maps to (m < mem): written +inf
-__device__ __forceinline__ int fill_count(bool real, int mem, int M, int W, int rank) {
-    const int mc = mem < M + 1 ? mem : M + 1;
-    const int nf = mc - rank * W;
-    return !real ? 0 : (nf < 0 ? 0 : (nf > W ? W : nf));
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ uint32_t mix(uint32_t v, uint32_t k) {
+    v = (v ^ (k * 0x9E3779B1u)) * 0x85EBCA6Bu;
+    v ^= v >> 15;
+    v *= 0xC2B2AE35u;
+    return v ^ (v >> 13);
 }
 
-// One cluster per instance (cluster c takes the c-th longest when `sorted`), CTA `rank` of the cluster owns
-// budget columns rank*W .. rank*W+W-1.  Dynamic shared memory: two buffers [S][W] of table values (previous
-// and next layer, swapping), the transition matrix [S][SP8] (two of them with one matrix per layer), the push
-// records of this layer and the next (one per column tile and strategy), the fill counts, and a dump row for the
-// stores of strategies that land nowhere.  Warps 0..NW-1 compute: warp w takes work units w, w+NW, ...; a unit is
-// 32*TM columns x 8 strategies, one fused add-min per relaxation, accumulators in registers.  The last warp
-// is the service warp: it sends the finished layer to the table (one tensor-map store), prepares the next
-// layer's records and, with one matrix per layer, fetches the next matrix.
-template <int TM>
-__global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, const __grid_constant__ CUtensorMap map_c,
-                                                                const __grid_constant__ CUtensorMap map_last)
+// Everything the layer loop needs; lives in registers (all members are uniform over the CTA).
+struct Ctx {
+    int S, M, W, H, P, G, CL, rank, Li, m_pitch, Kr, Kc, tmax, SP, NW, gints;
+    int32_t* g0;               // [2][gints] state of this layer / the next: rows of P = H + W columns
+    uint8_t* a0;               // [2][gints] its argmin (argmin table only)
+    const int4* rec;           // [3][S] ring of per-layer records, strategies in class order
+    const int* front;          // [3] no column below it holds a finite value in this layer
+    const int* reach;          // [3] the layer's largest shift
+    const int32_t* tsm;        // transition entries: [16][16] by class, or [S][SP] (two of them with one matrix per layer)
+    int tmat;                  // entries of one full matrix when there is one per layer, else 0
+    const int* cs;             // [Kr + 1] first record of each class
+    const int* cdelta;         // [16] cluster-window address of CTA d minus this CTA's own shared address
+    int32_t* C;                // this instance's table
+    uint8_t* A;
+    int32_t* C_last;
+    size_t slice;
+};
+
+// Record of (layer, strategy): x = byte offset, from the start of the state, of the cell column 0 of this CTA reads
+// (the row of the strategy's column class, shifted by mem); y = time (kInf: mem exceeds the budget, the row is +inf);
+// z = mem | strategy << 24; w = byte offset of the strategy's row in the table.
+//
+// G at the columns that column `col` of this CTA (and those 32, 64, ... after it) reads.  FAR: the layer has shifts
+// beyond the halo, whose cells are read from the CTA that owns them.
+template <int TM, bool FAR>
+__device__ __forceinline__ void gather(const Ctx& c, const int32_t* Gp, const int4 r, int col, int (&g)[TM])
+{
+    const int mem = r.z & 0xffffff;
+    if (!FAR || mem <= c.H) {
+        const int32_t* p = reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(Gp + col) + r.x);
+#pragma unroll
+        for (int j = 0; j < TM; ++j) g[j] = p[j * 32];
+    } else {
+        const uint32_t row = smem_addr(Gp) + (uint32_t)r.x + (uint32_t)mem * 4u;
+#pragma unroll
+        for (int j = 0; j < TM; ++j) {
+            const int src = c.rank * c.W + col + 32 * j - mem;
+            const int o = src / c.W;
+            g[j] = kInf;
+            if (src >= 0 && col + 32 * j < c.W) g[j] = ld_cluster(row + (uint32_t)((src - o * c.W) * 4 + c.cdelta[o]));
+        }
+    }
+}
+// ... and their argmin entries
+template <int TM, bool FAR>
+__device__ __forceinline__ void gather_arg(const Ctx& c, const uint8_t* Ap, const int4 r, int col, int (&a)[TM])
+{
+    const int mem = r.z & 0xffffff, off = r.x >> 2;
+    if (!FAR || mem <= c.H) {
+#pragma unroll
+        for (int j = 0; j < TM; ++j) a[j] = Ap[off + col + j * 32];
+    } else {
+        const uint32_t row = smem_addr(Ap) + (uint32_t)(off + mem);
+#pragma unroll
+        for (int j = 0; j < TM; ++j) {
+            const int src = c.rank * c.W + col + 32 * j - mem;
+            const int o = src / c.W;
+            a[j] = 255;
+            if (src >= 0 && col + 32 * j < c.W) a[j] = ld_cluster_u8(row + (uint32_t)(src - o * c.W + c.cdelta[o]));
+        }
+    }
+}
+
+// Values of one state row for the tile: into this CTA's columns, and into the halo of every CTA further up that holds them.
+template <int TM, bool ARG>
+__device__ __forceinline__ void emit(const Ctx& c, int32_t* Gn, uint8_t* An, int k, int colb, int lane, const int (&v)[TM], const int (&a)[TM])
+{
+    const int at = k * c.P + c.H + colb + lane;
+#pragma unroll
+    for (int j = 0; j < TM; ++j)
+        if (colb + 32 * j < c.W) {
+            Gn[at + 32 * j] = v[j];
+            if (ARG) An[at + 32 * j] = (uint8_t)a[j];
+        }
+    for (int d = c.rank + 1, low = c.W - c.H; d < c.CL && colb + 32 * TM > low; ++d, low += c.W) {
+        // CTA d holds the columns from d*W - H on: this CTA's local columns from `low` on
+        const uint32_t ga = smem_addr(Gn) + (uint32_t)(c.cdelta[d] + (at - (d - c.rank) * c.W) * 4);
+        const uint32_t aa = ARG ? smem_addr(An) + (uint32_t)(c.cdelta[d] + at - (d - c.rank) * c.W) : 0u;
+#pragma unroll
+        for (int j = 0; j < TM; ++j)
+            if (colb + 32 * j >= low && colb + 32 * j < c.W) {
+                st_cluster(ga + 128u * j, v[j]);
+                if (ARG) st_cluster_u8(aa + 32u * j, a[j]);
+            }
+    }
+}
+
+// One layer of one tile of TM x 32 columns.  KC: rows of the next state held in accumulators (PRUNE: per block of rows).
+template <int KC, int TM, bool PRUNE, bool STORE, bool ARG, bool FAR>
+__device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
+{
+    const int slot = l % 3;
+    const int4* const rec = c.rec + slot * c.S;
+    const int32_t* const Gp = c.g0 + (l & 1) * c.gints;
+    int32_t* const Gn = c.g0 + ((l + 1) & 1) * c.gints;
+    const uint8_t* const Ap = ARG ? c.a0 + (l & 1) * c.gints : nullptr;
+    uint8_t* const An = ARG ? c.a0 + ((l + 1) & 1) * c.gints : nullptr;
+    const int colg = c.rank * c.W + colb;                      // the tile's first budget column
+    char* const Cl = STORE ? reinterpret_cast<char*>(c.C + (size_t)l * c.slice + colg + lane) : nullptr;
+    uint8_t* const Al = ARG ? c.A + (size_t)l * c.slice + colg + lane : nullptr;
+    const bool whole = colg + 32 * TM - 1 <= c.M && colb + 32 * TM <= c.W;     // every column of the tile is a budget column of this CTA
+    const int last_col = min(c.m_pitch - c.rank * c.W, c.W);   // local columns that exist in the table
+
+    // what goes to the table: +inf in the pad columns beyond the budget
+    auto put = [&](const int4 r, const int (&v)[TM]) {
+        if (STORE) {
+            int32_t* const p = reinterpret_cast<int32_t*>(Cl + (uint32_t)r.w);
+            if (whole) {
+#pragma unroll
+                for (int j = 0; j < TM; ++j) p[32 * j] = v[j];
+            } else {
+#pragma unroll
+                for (int j = 0; j < TM; ++j)
+                    if (colb + 32 * j < last_col) p[32 * j] = colg + lane + 32 * j <= c.M ? v[j] : kInf;
+            }
+        }
+        if (ARG) {
+            int a[TM];
+            gather_arg<TM, FAR>(c, Ap, r, colb + lane, a);
+            uint8_t* const p = Al + ((uint32_t)r.w >> 2);
+#pragma unroll
+            for (int j = 0; j < TM; ++j)
+                if (colb + 32 * j < last_col) p[32 * j] = (uint8_t)(colg + lane + 32 * j <= c.M && v[j] < kInf ? a[j] : 255);
+        }
+    };
+
+    if (colg + 32 * TM - 1 < c.front[slot]) {                  // nothing finite in the tile
+        int inf[TM], none[TM];
+#pragma unroll
+        for (int j = 0; j < TM; ++j) { inf[j] = kInf; none[j] = 255; }
+        if (STORE || ARG)
+#pragma unroll 4
+            for (int e = 0; e < c.S; ++e) {
+                const uint32_t row = (uint32_t)rec[e].w;
+#pragma unroll
+                for (int j = 0; j < TM; ++j)
+                    if (colb + 32 * j < last_col) {
+                        if (STORE) reinterpret_cast<int32_t*>(Cl + row)[32 * j] = kInf;
+                        if (ARG) Al[(row >> 2) + 32 * j] = 255;
+                    }
+            }
+        for (int k = 0; k < c.Kc; ++k) emit<TM, ARG>(c, Gn, An, k, colb, lane, inf, none);
+        return;
+    }
+
+    if (!PRUNE) {
+        int acc[KC][TM], arg[ARG ? KC : 1][TM];
+#pragma unroll
+        for (int k = 0; k < KC; ++k)
+#pragma unroll
+            for (int j = 0; j < TM; ++j) { acc[k][j] = kInf; if (ARG) arg[k][j] = 255; }
+        int e = 0;
+        for (int k = 0; k < c.Kr; ++k) {
+            const int end = c.cs[k + 1];
+            int h[TM], hs[ARG ? TM : 1];
+#pragma unroll
+            for (int j = 0; j < TM; ++j) { h[j] = kInf; if (ARG) hs[j] = 255; }
+#pragma unroll 4
+            for (; e < end; ++e) {
+                const int4 r = rec[e];
+                int g[TM];
+                gather<TM, FAR>(c, Gp, r, colb + lane, g);
+                if (STORE || ARG) {
+                    int v[TM];
+#pragma unroll
+                    for (int j = 0; j < TM; ++j) {
+                        v[j] = __viaddmin_s32(g[j], r.y, kInf);
+                        if (ARG) hs[j] = v[j] < h[j] ? r.z >> 24 : hs[j];  // ascending strategies: the lowest keeps a tie
+                        h[j] = min(h[j], v[j]);
+                    }
+                    put(r, v);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < TM; ++j) h[j] = __viaddmin_s32(g[j], r.y, h[j]);
+                }
+            }
+            const int4* const T4 = reinterpret_cast<const int4*>(c.tsm + k * kClassMax);
+#pragma unroll
+            for (int q = 0; q < KC / 4; ++q) {
+                const int4 t4 = T4[q];
+                const int t[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+                for (int j = 0; j < TM; ++j)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (ARG) {
+                            const int cand = h[j] + t[u], old = acc[4 * q + u][j], oa = arg[4 * q + u][j];
+                            const bool better = cand < old || (cand == old && hs[j] < oa);
+                            if (better && h[j] < kInf) { acc[4 * q + u][j] = cand; arg[4 * q + u][j] = hs[j]; }
+                        } else {
+                            acc[4 * q + u][j] = __viaddmin_s32(h[j], t[u], acc[4 * q + u][j]);
+                        }
+                    }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < KC; ++k)
+            if (k < c.Kc) emit<TM, ARG>(c, Gn, An, k, colb, lane, acc[k], arg[ARG ? k : 0]);
+    } else {
+        int thr[TM];
+#pragma unroll
+        for (int j = 0; j < TM; ++j) thr[j] = kInf;
+#pragma unroll 4
+        for (int s = 0; s < c.S; ++s) {
+            const int4 r = rec[s];
+            int v[TM];
+            gather<TM, FAR>(c, Gp, r, colb + lane, v);
+#pragma unroll
+            for (int j = 0; j < TM; ++j) {
+                v[j] = __viaddmin_s32(v[j], r.y, kInf);
+                thr[j] = min(thr[j], v[j]);
+            }
+            put(r, v);
+        }
+        // a candidate beyond the column's best plus the largest entry cannot win; a column without a finite value
+        // keeps nothing alive
+#pragma unroll
+        for (int j = 0; j < TM; ++j) thr[j] = thr[j] < kInf ? thr[j] + c.tmax : -1;
+        const int32_t* const T = c.tsm + (((l + 1) & 1) ? c.tmat : 0);
+        for (int cb = 0; cb < c.S; cb += KC) {
+            int acc[KC][TM], arg[ARG ? KC : 1][TM];
+#pragma unroll
+            for (int k = 0; k < KC; ++k)
+#pragma unroll
+                for (int j = 0; j < TM; ++j) { acc[k][j] = kInf; if (ARG) arg[k][j] = 255; }
+#pragma unroll 2
+            for (int s = 0; s < c.S; ++s) {
+                const int4 r = rec[s];
+                int v[TM];
+                gather<TM, FAR>(c, Gp, r, colb + lane, v);
+                bool live = false;
+#pragma unroll
+                for (int j = 0; j < TM; ++j) {
+                    v[j] = __viaddmin_s32(v[j], r.y, kInf);
+                    live = live || v[j] <= thr[j];
+                }
+                if (__any_sync(0xffffffffu, live)) {
+                    const int4* const T4 = reinterpret_cast<const int4*>(T + s * c.SP + cb);
+#pragma unroll
+                    for (int q = 0; q < KC / 4; ++q) {
+                        const int4 t4 = T4[q];
+                        const int t[4] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+                        for (int j = 0; j < TM; ++j)
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                if (ARG) {
+                                    const int cand = v[j] + t[u];
+                                    if (v[j] < kInf && cand < acc[4 * q + u][j]) { acc[4 * q + u][j] = cand; arg[4 * q + u][j] = s; }
+                                } else {
+                                    acc[4 * q + u][j] = __viaddmin_s32(v[j], t[u], acc[4 * q + u][j]);
+                                }
+                            }
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < KC; ++k)
+                if (cb + k < c.S) emit<TM, ARG>(c, Gn, An, cb + k, colb, lane, acc[k], arg[ARG ? k : 0]);
+        }
+    }
+}
+
+// The last layer hands nothing on: its values go to the table and to C_last.
+template <bool STORE, bool ARG>
+__device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lane)
+{
+    const int slot = l % 3;
+    const int4* const rec = c.rec + slot * c.S;
+    const int32_t* const Gp = c.g0 + (l & 1) * c.gints;
+    const uint8_t* const Ap = ARG ? c.a0 + (l & 1) * c.gints : nullptr;
+    const int colg = c.rank * c.W + colb, m = colg + lane;
+    if (colg >= c.m_pitch) return;                             // m_pitch is a multiple of 32: a group exists whole or not at all
+    const bool pad = m > c.M;
+    auto step = [&](const int4 r, int g, int a) {
+        const int v = pad ? kInf : __viaddmin_s32(g, r.y, kInf);
+        const size_t row = ((uint32_t)r.w >> 2) + (size_t)m;
+        if (STORE) c.C[(size_t)l * c.slice + row] = v;
+        c.C_last[row] = v;
+        if (ARG) c.A[(size_t)l * c.slice + row] = (uint8_t)(v < kInf ? a : 255);
+    };
+    int g[1], a[1] = {255};
+    if (c.reach[slot] <= c.H) {
+#pragma unroll 4
+        for (int e = 0; e < c.S; ++e) {
+            const int4 r = rec[e];
+            gather<1, false>(c, Gp, r, colb + lane, g);
+            if (ARG) gather_arg<1, false>(c, Ap, r, colb + lane, a);
+            step(r, g[0], a[0]);
+        }
+    } else {
+        for (int e = 0; e < c.S; ++e) {
+            const int4 r = rec[e];
+            gather<1, true>(c, Gp, r, colb + lane, g);
+            if (ARG) gather_arg<1, true>(c, Ap, r, colb + lane, a);
+            step(r, g[0], a[0]);
+        }
+    }
+}
+
+template <int KC, int TM, bool PRUNE, bool STORE, bool ARG>
+__device__ __forceinline__ void run_layers(const Ctx& c, int warp, int lane)
+{
+    for (int l = 0; l + 1 < c.Li; ++l) {
+        if (c.reach[l % 3] <= c.H) {
+            for (int g = warp * TM; g < c.G; g += c.NW * TM) tile<KC, TM, PRUNE, STORE, ARG, false>(c, l, g * 32, lane);
+        } else {
+            for (int g = warp; g < c.G; g += c.NW) tile<KC, 1, PRUNE, STORE, ARG, true>(c, l, g * 32, lane);
+        }
+        layer_barrier(c.CL);
+    }
+    for (int g = warp; g < c.G; g += c.NW) last_tile<STORE, ARG>(c, c.Li - 1, g * 32, lane);
+}
+
+// Cluster c takes instance c (the c-th longest when `sorted`).  Warps 0..NW-1 compute, the last warp fetches the
+// layers' mem / time rows (and with one matrix per layer the matrices) ahead and turns them into records.
+template <bool STORE, bool ARG>
+__global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const RsArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ int s_L[kMaxSortedB];
-    __shared__ int s_inst, s_tmax, s_bad;
-    __shared__ long long s_sum;
+    __shared__ union { int L[kMaxSortedB]; struct { uint32_t rh[kMaxS], ch[kMaxS]; } h; } s_u;
+    __shared__ int s_rrep[kMaxS], s_crep[kMaxS], s_rcls[kMaxS], s_ccls[kMaxS], s_order[kMaxS], s_cs[kMaxS + 1];
+    __shared__ int s_cdelta[16], s_front[3], s_reach[3], s_inst, s_K[2];
+    __shared__ struct { long long sum; int tmax, bad, mmax; } s_part, s_all;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x, NW = (NT >> 5) - 1;
-    const int CL = a.CL, rank = (int)cluster_rank(), cid = blockIdx.x / CL;
-    const int S = a.S, M = a.M, W = a.W, SP8 = a.SP8, Lmax = a.Lmax;
+    const int CL = a.CL, rank = CL > 1 ? (int)cluster_rank() : 0, cid = blockIdx.x / CL;
+    const int S = a.S, M = a.M, W = a.W, Lmax = a.Lmax, gints = a.gints;
 
-    int32_t* const buf0 = reinterpret_cast<int32_t*>(smem_raw);
-    int32_t* const buf1 = buf0 + S * W;
-    int32_t* const tsm = buf1 + S * W;
-    const int tmat = S * SP8;
-    const int nrec = a.nct * SP8;
-    int4* const rows = reinterpret_cast<int4*>(tsm + (a.trans_layer ? 2 : 1) * tmat);     // [2][nct][SP8] push records
-    int* const fillc = reinterpret_cast<int*>(rows + 2 * nrec);                            // [2][SP8] leading cells of each row to fill with +inf
-    int* const fillmax = fillc + 2 * SP8;                                                  // [2] the largest of them (padded to 4 ints)
-    int32_t* const dump = fillmax + 4;                                                     // [32 * TM] where stores of skipped strategies go
-    int* const cdelta = dump + 32 * TM;                                                    // [16] cluster-window address of CTA d minus this CTA's own shared address
+    // ---- shared memory
+    int32_t* const g0 = reinterpret_cast<int32_t*>(smem_raw);                              // [2][gints]
+    const int tfull = S * a.SP;
+    int32_t* const tsm = g0 + 2 * gints;                                                   // [16][16] or [1|2][S][SP]
+    const int tints = max(kClassMax * kClassMax, (a.trans_layer ? 2 : 1) * tfull);
+    int4* const rec = reinterpret_cast<int4*>(tsm + tints);                                // [3][S]
+    int32_t* const raw = reinterpret_cast<int32_t*>(rec + 3 * S);                          // [4][2][S] mem, time rows as they come
+    uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * S);                           // [2][gints] argmin of the state
 
-    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = 2; }      // no error flag to raise; the cluster kernel ran
+    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = a.path_value; }
 
     // ---- which instance: clusters are dispatched in order, so the longest instances go first
     int i = cid;
     if (a.sorted) {
         for (int j = tid; j < a.B; j += NT) {
             const int v = a.L[j];
-            s_L[j] = (v < 1 || v > Lmax) ? 0 : v;
+            s_u.L[j] = (v < 1 || v > Lmax) ? 0 : v;
         }
         __syncthreads();
         for (int j = tid; j < a.B; j += NT) {
-            const int Lj = s_L[j];
+            const int Lj = s_u.L[j];
             int before = 0;
             for (int k = 0; k < a.B; ++k) {
-                const int Lk = s_L[k];
+                const int Lk = s_u.L[k];
                 before += (Lk > Lj) || (Lk == Lj && k < j);
             }
             if (before == cid) s_inst = j;
@@ -176,301 +471,318 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
         __syncthreads();
         i = s_inst;
     }
-
-    // ---- validation (every CTA of the cluster comes to the same result: nobody is left waiting at a barrier)
-    if (tid == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; }
-    __syncthreads();
+    if (a.second && a.done[i]) return;
     const int Li = a.L[i];
     if (Li < 1 || Li > Lmax) {
-        if (rank == 0 && tid == 0) a.status[i] = GALV_STATUS_BAD_INPUT;
+        if (rank == 0 && tid == 0) { a.status[i] = GALV_STATUS_BAD_INPUT; a.done[i] = 1; }
         return;
     }
     const int32_t* const tq = a.time_q + (size_t)i * Lmax * S;
     const int32_t* const mq = a.mem_q + (size_t)i * Lmax * S;
     const int32_t* const T0 = a.trans_q + (size_t)i * a.trans_inst;
+
+    // ---- validation: the CTAs of the cluster share the layers (and matrices); one matrix per instance is staged whole
+    int32_t* const stage = g0;                                 // the state is not in use yet
+    const bool staged = !a.trans_layer && (long long)S * S <= (long long)2 * gints;
+    if (tid == 0) { s_part.sum = 0; s_part.tmax = 0; s_part.bad = 0; s_part.mmax = 0; }
+    for (int x = tid; x < kMaxS; x += NT) { s_u.h.rh[x] = 0; s_u.h.ch[x] = 0; }
+    if (tid < 16) s_cdelta[tid] = CL > 1 ? (int)(map_to_rank(smem_addr(g0), (uint32_t)min(tid, CL - 1)) - smem_addr(g0)) : 0;
+    __syncthreads();
     {
         long long sum = 0;
-        int bad = 0, tmax = 0;
-        for (int l = warp; l < Li; l += NW + 1) {             // a warp per layer: largest time of the layer
+        int bad = 0, tmax = 0, mmax = 0;                        // mmax: the largest shift that stays inside the budget
+        for (int l = rank * (NW + 1) + warp; l < Li; l += CL * (NW + 1)) {      // a warp per layer: largest time of the layer
             int mx = 0;
             for (int s = lane; s < S; s += 32) {
                 const int tv = tq[l * S + s], mv = mq[l * S + s];
                 bad |= (tv < 0) | (mv < 0);
                 mx = max(mx, tv);
+                mmax = max(mmax, mv <= M ? mv : 0);
             }
             mx = __reduce_max_sync(0xffffffffu, mx);
             if (lane == 0) sum += mx;
         }
-        const int xl0 = a.trans_layer ? 1 : 0, xl1 = a.trans_layer ? Li : 1;       // matrices in use
-        const long long nx = (long long)(xl1 - xl0) * S * S;
-        const int32_t* x = T0 + (size_t)xl0 * S * S;
-        for (long long k = tid; k < nx; k += NT) {
-            const int v = x[k];
-            bad |= (v < 0);
-            tmax = max(tmax, v);
+        if (a.trans_layer) {
+            const long long nx = (long long)(Li - 1) * S * S;                     // matrix 0 is unused
+            const int32_t* const x = T0 + (size_t)S * S;
+#pragma unroll 4
+            for (long long k = (long long)rank * NT + tid; k < nx; k += (long long)CL * NT) {
+                const int v = x[k];
+                bad |= v < 0;
+                tmax = max(tmax, v);
+            }
+        } else {
+#pragma unroll 4
+            for (int k = tid; k < S * S; k += NT) {
+                const int v = T0[k];
+                bad |= v < 0;
+                tmax = max(tmax, v);
+                if (staged) stage[k] = v;
+            }
         }
         tmax = __reduce_max_sync(0xffffffffu, tmax);
+        mmax = __reduce_max_sync(0xffffffffu, mmax);
         bad = __any_sync(0xffffffffu, bad != 0);
         if (lane == 0) {
-            if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(&s_sum), static_cast<unsigned long long>(sum));
-            atomicMax(&s_tmax, tmax);
-            if (bad) atomicOr(&s_bad, 1);
+            if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(&s_part.sum), static_cast<unsigned long long>(sum));
+            atomicMax(&s_part.tmax, tmax);
+            atomicMax(&s_part.mmax, mmax);
+            if (bad) atomicOr(&s_part.bad, 1);
         }
     }
-    __syncthreads();
-    {
-        int st = 0;
-        if (s_bad) st = GALV_STATUS_BAD_INPUT;
-        else if (s_sum + (long long)(Li - 1) * s_tmax >= (long long)kInf) st = GALV_STATUS_OVERFLOW_RISK;
-        if (rank == 0 && tid == 0) a.status[i] = st;
-        if (st) return;                                        // flagged: tables left untouched
-    }
-
-    const int col_g0 = rank * W;                               // first budget column of this CTA
-
-    // ---- layer 0, the records of layer 1, the transition matrix
-    // the push records and fill count of strategy s (raw mem / time given) into half `h` of the two arrays
-    auto prepare_one = [&](int h, int s, int mem, int time) -> int {                       // returns the row's fill count
-        const bool real = s < S;
-        const int nf = fill_count(real, mem, M, W, rank);
-        fillc[h * SP8 + s] = nf;
-        for (int ct = 0; ct < a.nct; ++ct) {
-            const int left = a.G - ct * TM;
-            rows[h * nrec + ct * SP8 + s] = tile_record(real, mem, time, M, W, rank, ct * 32 * TM, 32 * (left < TM ? left : TM));
-        }
-        return nf;
-    };
-    // ... of a whole layer by one warp: lane k takes strategies k, k+32, ...
-    auto prepare_layer = [&](int h, const int (&m)[kRowsPerLane], const int (&t)[kRowsPerLane]) {
-        int most = 0;
-#pragma unroll
-        for (int j = 0; j < kRowsPerLane; ++j)
-            if (lane + 32 * j < SP8) most = max(most, prepare_one(h, lane + 32 * j, m[j], t[j]));
-        most = __reduce_max_sync(0xffffffffu, most);
-        if (lane == 0) fillmax[h] = most;
-    };
-    // layers 0 and 1 straight from global memory, a warp each (nothing is being stored yet)
-    if (warp <= 1 && warp < Li) {
-        int m0[kRowsPerLane], t0[kRowsPerLane];
-#pragma unroll
-        for (int j = 0; j < kRowsPerLane; ++j) {
-            const int s = lane + 32 * j;
-            m0[j] = s < S ? mq[warp * S + s] : 0;
-            t0[j] = s < S ? tq[warp * S + s] : 0;
-        }
-        prepare_layer(warp, m0, t0);
-    }
-    for (int x = tid; x < 32 * TM; x += NT) dump[x] = 0;
-    // where the other CTAs' buffers lie in the cluster window: asked once, not once per store (the mapping is an
-    // offset per CTA; asking inside the push puts its latency on every strategy's chain of branches)
-    if (tid < 16) cdelta[tid] = (int)(map_to_rank(smem_addr(buf0), (uint32_t)min(tid, CL - 1)) - smem_addr(buf0));
-    {
-        const int32_t* T = T0 + (a.trans_layer ? a.trans_layer : 0);       // matrix 1 is paid between layers 0 and 1
-        int32_t* dst = tsm + (a.trans_layer ? tmat : 0);                    // per layer: matrix l sits in tsm[l & 1]
-        for (int e = tid; e < tmat; e += NT) {
-            const int k = e / SP8, c = e - k * SP8;
-            dst[e] = (c < S && Li > 1) ? T[k * S + c] : 0;
-            if (a.trans_layer) tsm[e] = 0;                                  // pad columns of the other buffer stay 0
-        }
-    }
-    __syncthreads();
-    for (int s = warp; s < S; s += NW + 1) {
-        const int t0 = rows[s].z;                                           // time(0,s) sits in every record of s
-        const int nf = fillc[s];
-        for (int x = lane; x < W; x += 32) {
-            const bool pad = col_g0 + x > M;
-            buf0[s * W + x] = (pad || x < nf) ? kInf : t0;
-            if (pad) buf1[s * W + x] = kInf;                                // pad columns are never written again
-        }
-    }
-    // Service warp: raw mem / time rows of the layer after next, lane k keeps strategies k, k+32, ... (S <= 128).
-    // They are fetched a whole layer before they are needed and BEFORE that layer's table store is issued: a
-    // global load issued while the SM's bulk stores are in flight comes back after thousands of cycles.
-    int raw_m[kRowsPerLane], raw_t[kRowsPerLane];
-    auto fetch_rows = [&](int lay, int (&m)[kRowsPerLane], int (&t)[kRowsPerLane]) {
-#pragma unroll
-        for (int j = 0; j < kRowsPerLane; ++j) {
-            const int s = lane + 32 * j;
-            m[j] = s < S ? mq[lay * S + s] : 0;
-            t[j] = s < S ? tq[lay * S + s] : 0;
-        }
-    };
-    if (warp == NW && Li > 2) fetch_rows(2, raw_m, raw_t);
-    // every CTA of the cluster has started and holds its layer 0 before anyone writes into a neighbour
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");            // layer 0 goes to the table by a bulk store
-    cluster_barrier();
-
-    for (int l = 1; l < Li; ++l) {
-        const int32_t* const X = (l & 1) ? buf0 : buf1;                     // layer l-1
-        int32_t* const Y = (l & 1) ? buf1 : buf0;                           // layer l
-        const int4* const rl = rows + (l & 1) * nrec;
-        const int32_t* const Tl = tsm + ((a.trans_layer && (l & 1)) ? tmat : 0);
-
-        if (warp == NW) {
-            // ------------------------------------------------------------ service warp
-            // first the loads: rows of layer l+2, and with one matrix per layer the matrix of layer l+1
-            int next_m[kRowsPerLane], next_t[kRowsPerLane];
-            if (l + 2 < Li) fetch_rows(l + 2, next_m, next_t);
-            if (l + 1 < Li && a.trans_layer) {
-                const int32_t* T = T0 + (size_t)(l + 1) * a.trans_layer;
-                int32_t* dst = tsm + (((l + 1) & 1) ? tmat : 0);
-                for (int e = lane; e < S * S; e += 32) {
-                    const int k = e / S, c = e - k * S;
-                    cp_async_4(dst + k * SP8 + c, T + e);
-                }
-            }
-            // layer l-1 is complete in X: to the table while this layer is computed
-            if (a.C && lane == 0) {
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");    // the buffer was written by plain stores
-                tensor_store_3d(&map_c, X, rank * a.G, (i * Lmax + (l - 1)) * S);
-                bulk_commit();
-            }
-            // the records of layer l+1 from the rows fetched a layer ago
-            if (l + 1 < Li) prepare_layer((l + 1) & 1, raw_m, raw_t);
-#pragma unroll
-            for (int j = 0; j < kRowsPerLane; ++j) { raw_m[j] = next_m[j]; raw_t[j] = next_t[j]; }
-            if (l + 1 < Li && a.trans_layer) cp_async_wait_all();
-            if (a.C && lane == 0) bulk_wait_read();                         // X may be overwritten from the next barrier on
+    layer_barrier(CL);
+    if (warp == 0) {
+        long long sum = 0;
+        int tmax = 0, bad = 0, mmax = 0;
+        if (CL == 1) {
+            sum = s_part.sum; tmax = s_part.tmax; bad = s_part.bad; mmax = s_part.mmax;
         } else {
-            // ------------------------------------------------------------ compute warps
-            // cells of this CTA's columns that no column maps to in this layer (m < mem(l,s): the first fillc[s] of
-            // row s): the compute warps share the columns, each takes every strategy in turn (independent predicated
-            // stores; a loop per strategy would be a chain of dependent steps)
-            {
-                const int* const fc = fillc + (l & 1) * SP8;
-                const int most = fillmax[l & 1];
-                for (int x = warp * 32 + lane; x < most; x += NW * 32) {
-#pragma unroll 4
-                    for (int s = 0; s < S; ++s)
-                        if (x < fc[s]) Y[s * W + x] = kInf;
-                }
+            if (lane < CL) {
+                const uint32_t p = map_to_rank(smem_addr(&s_part), (uint32_t)lane);
+                sum = (long long)(((unsigned long long)(uint32_t)ld_cluster(p + 4) << 32) | (uint32_t)ld_cluster(p));
+                tmax = ld_cluster(p + 8);
+                bad = ld_cluster(p + 12);
+                mmax = ld_cluster(p + 16);
             }
-            const uint32_t ybase = smem_addr(Y);
-            for (int unit = warp; unit < a.units; unit += NW) {
-                const int ct = unit / a.NSG, sg = unit - ct * a.NSG;
-                const int colb = ct * (32 * TM);
-                int nj = a.G - ct * TM;                                     // 32-column groups of this tile that exist
-                nj = nj > TM ? TM : nj;
-                int acc[TM][8];
 #pragma unroll
-                for (int j = 0; j < TM; ++j)
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) acc[j][u] = kInf;
-                const int32_t* pc = X + colb + lane;
-                const int32_t* pt = Tl + sg * 8;
-                int k = 0;
-                auto steps = [&](auto ku) {
-                    constexpr int K = decltype(ku)::value;
-                    for (; k + K <= S; k += K) {
-#pragma unroll
-                        for (int kk = 0; kk < K; ++kk) {
-                            int c[TM];
-#pragma unroll
-                            for (int j = 0; j < TM; ++j) c[j] = pc[kk * W + j * 32];
-                            const int4 t0 = *reinterpret_cast<const int4*>(pt + kk * SP8);
-                            const int4 t1 = *reinterpret_cast<const int4*>(pt + kk * SP8 + 4);
-                            const int t[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-#pragma unroll
-                            for (int j = 0; j < TM; ++j)
-#pragma unroll
-                                for (int u = 0; u < 8; ++u) acc[j][u] = __viaddmin_s32(c[j], t[u], acc[j][u]);
-                        }
-                        pc += K * W;
-                        pt += K * SP8;
-                    }
-                };
-                steps(std::integral_constant<int, 8>());
-                steps(std::integral_constant<int, 1>());
-                // push: column m' of strategy s belongs at column m' + mem(l,s): in this CTA's buffer or in one further up.
-                // All eight records first; when every strategy either stays at home in one piece or lands nowhere, the
-                // stores go out in one run without a branch (those that land nowhere go to a dump row).
-                int4 r[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) r[u] = rl[ct * SP8 + sg * 8 + u];
-                bool plain = nj == TM;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) plain = plain && (r[u].x < 0 || (r[u].x == rank && r[u].w == kWholeTile));
-                int32_t* const yl = Y + (sg * 8) * W + lane;
-                if (plain) {
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        int32_t* const y = r[u].x < 0 ? dump + lane : yl + u * W + r[u].y;
-#pragma unroll
-                        for (int j = 0; j < TM; ++j) y[j * 32] = __viaddmin_s32(acc[j][u], r[u].z, kInf);    // +inf stays +inf
-                    }
-                } else {
-                    // Some strategy's tile leaves the CTA or straddles two: the whole unit goes through the cluster window
-                    // (what stays at home too), one predicated store a register and no branch - a chain of branches per
-                    // strategy cost the warps that own such tiles three times the time of the stores themselves.
-                    // A whole tile has w = the largest int: its columns pass the test against w and lie below W.
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const int dx = r[u].x < 0 ? 0 : r[u].x;
-                        const uint32_t row = ybase + (uint32_t)((sg * 8 + u) * W) * 4u;
-                        const uint32_t ra0 = row + (uint32_t)cdelta[dx];
-                        const uint32_t ra1 = row + (uint32_t)cdelta[min(dx + 1, CL - 1)] - (uint32_t)W * 4u;
-                        const bool lands = r[u].x >= 0;
-#pragma unroll
-                        for (int j = 0; j < TM; ++j)
-                            if (j < nj) {
-                                const int x = r[u].y + j * 32 + lane;
-                                const int v = __viaddmin_s32(acc[j][u], r[u].z, kInf);
-                                if (lands && x <= r[u].w) st_cluster((x < W ? ra0 : ra1) + (uint32_t)x * 4u, v);
-                            }
-                    }
-                }
-            }
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            tmax = __reduce_max_sync(0xffffffffu, tmax);
+            mmax = __reduce_max_sync(0xffffffffu, mmax);
+            bad = __any_sync(0xffffffffu, bad != 0);
         }
-        // What this thread stored into shared memory, its own CTA's or a neighbour's, is read next by the bulk store of
-        // the CTA that owns it (async proxy): the writer orders it for that proxy before the barrier that publishes it.
-        asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
-        cluster_barrier();                                                  // layer l is complete everywhere
+        if (lane == 0) { s_all.sum = sum; s_all.tmax = tmax; s_all.bad = bad; s_all.mmax = mmax; }
     }
 
-    // ---- the last layer: to the table and to C_last
-    if (warp == NW && lane == 0) {
-        const int32_t* const F = ((Li - 1) & 1) ? buf1 : buf0;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (a.C) tensor_store_3d(&map_c, F, rank * a.G, (i * Lmax + (Li - 1)) * S);
-        tensor_store_3d(&map_last, F, rank * a.G, i * S);
-        bulk_commit();
-        bulk_wait_all();
+    // ---- classes of equal rows and equal columns
+    int K = S;                                                  // unstructured unless found otherwise
+    if (staged) {
+        // a sum of mixed words per row and per column proposes twins ...
+        for (int r = warp; r < S; r += NW + 1) {
+            uint32_t h = 0;
+            for (int s = lane; s < S; s += 32) h += mix((uint32_t)stage[r * S + s], (uint32_t)s);
+            h = __reduce_add_sync(0xffffffffu, h);
+            if (lane == 0) s_u.h.rh[r] = h;
+        }
+        const int parts = max(1, NT / S);
+        for (int x = tid; x < parts * S; x += NT) {
+            const int s = x % S, p = x / S;
+            uint32_t h = 0;
+            for (int r = p; r < S; r += parts) h += mix((uint32_t)stage[r * S + s], (uint32_t)r);
+            atomicAdd(&s_u.h.ch[s], h);
+        }
+        __syncthreads();
+        for (int x = tid; x < 2 * S; x += NT) {
+            const uint32_t* const hh = x < S ? s_u.h.rh : s_u.h.ch;
+            const int s = x < S ? x : x - S;
+            int o = 0;
+            while (hh[o] != hh[s]) ++o;                         // ends at s itself at the latest
+            (x < S ? s_rrep : s_crep)[s] = o;
+            (x < S ? s_rcls : s_ccls)[s] = 0;                   // for now: words that differ
+        }
+        __syncthreads();
+        // ... and a comparison of all their words decides
+        for (int r = warp; r < S; r += NW + 1) {
+            const int o = s_rrep[r];
+            int diff = 0;
+            for (int s = lane; s < S; s += 32) diff |= stage[r * S + s] != stage[o * S + s];
+            if (__any_sync(0xffffffffu, diff) && lane == 0) s_rcls[r] = 1;
+        }
+        for (int x = tid; x < parts * S; x += NT) {
+            const int s = x % S, p = x / S, o = s_crep[s];
+            int diff = 0;
+            for (int r = p; r < S; r += parts) diff |= stage[r * S + s] != stage[r * S + o];
+            if (diff) s_ccls[s] = 1;
+        }
+        __syncthreads();
+        for (int s = tid; s < S; s += NT) {
+            if (s_rcls[s]) s_rrep[s] = s;
+            if (s_ccls[s]) s_crep[s] = s;
+        }
+        __syncthreads();
+        // class numbers in the order of the classes' first members
+        for (int x = tid; x < 2 * S; x += NT) {
+            const int* const rep = x < S ? s_rrep : s_crep;
+            const int s = x < S ? x : x - S, me = rep[s];
+            int k = 0;
+            for (int o = 0; o < me; ++o) k += rep[o] == o;
+            (x < S ? s_rcls : s_ccls)[s] = k;
+        }
+        if (warp < 2) {                                         // there are at least two warps
+            const int* const rep = warp == 0 ? s_rrep : s_crep;
+            int k = 0;
+            for (int s = lane; s < S; s += 32) k += rep[s] == s;
+            k = __reduce_add_sync(0xffffffffu, k);
+            if (lane == 0) s_K[warp] = k;
+        }
+        __syncthreads();
+        K = max(s_K[0], s_K[1]);
     }
+    const bool classes = staged && K <= kClassMax && s_K[1] * W <= gints;
+    const bool dense = !classes && a.SP > 0 && S * W <= gints;
+    const int Kr = classes ? s_K[0] : S, Kc = classes ? s_K[1] : S;
+    if (classes) {
+        // strategies in class order, ascending inside a class
+        for (int s = tid; s < S; s += NT) {
+            const int me = s_rcls[s];
+            int pos = 0;
+            for (int o = 0; o < S; ++o) pos += s_rcls[o] < me || (s_rcls[o] == me && o < s);
+            s_order[pos] = s;
+        }
+        for (int k = tid; k <= Kr; k += NT) {
+            int n = 0;
+            for (int o = 0; o < S; ++o) n += s_rcls[o] < k;
+            s_cs[k] = n;
+        }
+        for (int x = tid; x < kClassMax * kClassMax; x += NT) tsm[x] = 0;
+        __syncthreads();
+        for (int r = warp; r < S; r += NW + 1)
+            if (s_rrep[r] == r)
+                for (int s = lane; s < S; s += 32)
+                    if (s_crep[s] == s) tsm[s_rcls[r] * kClassMax + s_ccls[s]] = stage[r * S + s];
+    } else if (dense) {
+        for (int s = tid; s < S; s += NT) { s_order[s] = s; s_ccls[s] = s; }
+        for (int k = tid; k <= S; k += NT) s_cs[k] = k;
+        // the matrix paid between layers 0 and 1; with one matrix per layer, matrix l sits in buffer l & 1
+        const int32_t* const T = T0 + (a.trans_layer ? a.trans_layer : 0);
+        int32_t* const dst = tsm + (a.trans_layer ? tfull : 0);
+        for (int x = tid; x < tfull; x += NT) {
+            const int r = x / a.SP, s = x - r * a.SP;
+            const int v = (s < S && Li > 1) ? (staged ? stage[r * S + s] : T[r * S + s]) : 0;
+            dst[x] = v;
+            if (a.trans_layer) tsm[x] = 0;                      // pad columns of the other buffer stay 0
+        }
+    }
+    int st = 0;
+    __syncthreads();                                            // s_all, classes; the staged matrix is no longer read
+    if (s_all.bad) st = GALV_STATUS_BAD_INPUT;
+    else if (s_all.sum + (long long)(Li - 1) * s_all.tmax >= (long long)kInf) st = GALV_STATUS_OVERFLOW_RISK;
+    const bool run = st == 0 && (classes || dense);
+    if (rank == 0 && tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run; }
+
+    // The halo: columns left of this CTA's own that its gathers reach, as many as the largest shift asks for or as fit;
+    // a multiple of 32.  Below column 0 it holds +inf.
+    const int H = max(0, min((s_all.mmax + 31) & ~31, (gints / Kc - W) & ~31)), P = W + H;
+
+    // ---- layer 0 gathers from an all-zero state: C[0] = time where mem fits
+    auto prepare = [&](int l, int base) -> int {                // records of layer l by one warp; returns the new frontier
+        const int slot = l % 3;
+        const int32_t* const rm = raw + (l & 3) * 2 * S;
+        int least = M + 1, most = 0;
+        for (int e = lane; e < S; e += 32) {
+            const int s = s_order[e];
+            const int mem = rm[s];
+            const bool fits = mem <= M;                         // else +inf everywhere: no shift, time +inf
+            const int shift = fits ? mem : 0;
+            rec[slot * S + e] = make_int4((s_ccls[s] * P + H - shift) * 4, fits ? rm[S + s] : kInf, shift | (s << 24), s * a.m_pitch * 4);
+            least = min(least, mem);
+            most = max(most, shift);
+        }
+        least = __reduce_min_sync(0xffffffffu, least);
+        most = __reduce_max_sync(0xffffffffu, most);
+        const int f = min(base + least, M + 1);
+        if (lane == 0) { s_front[slot] = f; s_reach[slot] = most; }
+        return f;
+    };
+    auto fetch = [&](int l) {
+        int32_t* const rm = raw + (l & 3) * 2 * S;
+        for (int s = lane; s < S; s += 32) {
+            cp_async_4(rm + s, mq + (size_t)l * S + s);
+            cp_async_4(rm + S + s, tq + (size_t)l * S + s);
+        }
+    };
+    int front = 0;
+    if (run) {
+        if (warp == NW) {
+            fetch(0);
+            if (Li > 1) fetch(1);
+            cp_async_commit();
+            if (Li > 2) fetch(2);
+            cp_async_commit();
+            cp_async_wait<1>();
+            __syncwarp();
+            front = prepare(0, 0);
+            if (Li > 1) front = prepare(1, front);
+        } else {
+            for (int k = 0; k < Kc; ++k)
+                for (int x = tid; x < P; x += NW * 32) {
+                    g0[k * P + x] = rank * W + x >= H ? 0 : kInf;           // column rank*W + x - H
+                    if (x < H) g0[gints + k * P + x] = kInf;
+                    if (ARG) {
+                        a0[k * P + x] = 255;
+                        if (x < H) a0[gints + k * P + x] = 255;
+                    }
+                }
+        }
+    }
+    layer_barrier(CL);                                          // also: nobody leaves while its partial sums are being read
+    if (!run) return;
+
+    if (warp == NW) {
+        // ---------------------------------------------------------------- service warp
+        for (int l = 0; l + 1 < Li; ++l) {
+            if (l + 3 < Li) fetch(l + 3);
+            cp_async_commit();
+            if (a.trans_layer && l + 2 < Li) {                  // matrix l + 1 is in use in this layer
+                const int32_t* const T = T0 + (size_t)(l + 2) * a.trans_layer;
+                int32_t* const dst = tsm + ((l & 1) ? tfull : 0);
+                for (int x = lane; x < S * S; x += 32) {
+                    const int r = x / S, s = x - r * S;
+                    cp_async_4(dst + r * a.SP + s, T + x);
+                }
+            }
+            cp_async_commit();
+            if (l + 2 < Li) {
+                cp_async_wait<2>();                             // the rows of layer l + 2, asked for a layer ago
+                __syncwarp();
+                front = prepare(l + 2, front);
+            }
+            if (a.trans_layer) cp_async_wait<0>();
+            layer_barrier(CL);
+        }
+    } else {
+        Ctx c;
+        c.S = S; c.M = M; c.W = W; c.H = H; c.P = P; c.G = W / 32; c.CL = CL; c.rank = rank; c.Li = Li; c.m_pitch = a.m_pitch; c.Kr = Kr; c.Kc = Kc;
+        c.tmax = s_all.tmax; c.SP = a.SP; c.NW = NW; c.gints = gints;
+        c.g0 = g0; c.a0 = a0; c.rec = rec; c.front = s_front; c.reach = s_reach; c.tsm = tsm; c.tmat = a.trans_layer ? tfull : 0;
+        c.cs = s_cs; c.cdelta = s_cdelta;
+        c.slice = (size_t)S * a.m_pitch;
+        c.C = STORE ? a.C + (size_t)i * Lmax * c.slice : nullptr;
+        c.A = ARG ? a.A + (size_t)i * Lmax * c.slice : nullptr;
+        c.C_last = a.C_last + (size_t)i * c.slice;
+        // columns per lane: one group of 32 per warp while the warps last, then two, then four (a record fetched once
+        // serves them all)
+        const int per = (c.G + NW - 1) / NW;
+        if (classes) {
+            if (K <= 4) {
+                if (per >= 3 && !ARG) run_layers<4, 4, false, STORE, ARG>(c, warp, lane);
+                else if (per >= 2) run_layers<4, 2, false, STORE, ARG>(c, warp, lane);
+                else run_layers<4, 1, false, STORE, ARG>(c, warp, lane);
+            } else if (K <= 8) {
+                if (per >= 3 && !ARG) run_layers<8, 4, false, STORE, ARG>(c, warp, lane);
+                else if (per >= 2) run_layers<8, 2, false, STORE, ARG>(c, warp, lane);
+                else run_layers<8, 1, false, STORE, ARG>(c, warp, lane);
+            } else {
+                if (per >= 2) run_layers<16, 2, false, STORE, ARG>(c, warp, lane);
+                else run_layers<16, 1, false, STORE, ARG>(c, warp, lane);
+            }
+        } else {
+            if (per >= 2 && !ARG) run_layers<32, 2, true, STORE, ARG>(c, warp, lane);
+            else run_layers<32, 1, true, STORE, ARG>(c, warp, lane);
+        }
+    }
+    if (CL > 1) layer_barrier(CL);                              // nobody's shared memory goes away while it is being read
 }
-
-}  // namespace
 
 // ---------------------------------------------------------------- host side
 
-namespace {
-
-typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                    const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                    CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// Tensor map of an int32 table [rows][m_pitch] seen as [rows][m_pitch / 32][32], box [box_rows][box_groups][32].
-cudaError_t encode_table_3d(CUtensorMap* map, void* base, size_t rows, int m_pitch, int box_rows, int box_groups)
+typedef void (*RsKernel)(const RsArgs);
+RsKernel kernel_of(bool store, bool arg)
 {
-    static PFN_encodeTiled fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q);
-        if (e != cudaSuccess) return e;
-        if (q != cudaDriverEntryPointSuccess || !p) return cudaErrorNotSupported;
-        fn = reinterpret_cast<PFN_encodeTiled>(p);
-    }
-    const cuuint64_t dims[3] = {32, (cuuint64_t)(m_pitch / 32), (cuuint64_t)rows};
-    const cuuint64_t strides[2] = {128, (cuuint64_t)m_pitch * 4};
-    const cuuint32_t box[3] = {32, (cuuint32_t)box_groups, (cuuint32_t)box_rows};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_INT32, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+    return store ? (arg ? resident_kernel<true, true> : resident_kernel<true, false>)
+                 : (arg ? resident_kernel<false, true> : resident_kernel<false, false>);
 }
 
-template <int TM>
-cudaError_t launch_cluster(const ClArgs& a, const ClPlan& p, const CUtensorMap& mc, const CUtensorMap& ml, cudaStream_t st, int* max_clusters)
+cudaError_t launch_resident(RsKernel k, const RsArgs& a, const RsPlan& p, cudaStream_t st, int* max_clusters)
 {
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
@@ -485,151 +797,127 @@ cudaError_t launch_cluster(const ClArgs& a, const ClPlan& p, const CUtensorMap& 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, cluster_search_kernel<TM>, &cfg);
-    return cudaLaunchKernelEx(&cfg, cluster_search_kernel<TM>, a, mc, ml);
-}
-
-cudaError_t launch_any(const ClArgs& a, const ClPlan& p, const CUtensorMap& mc, const CUtensorMap& ml, cudaStream_t st, int* max_clusters)
-{
-    switch (p.tm) {
-    case 2: return launch_cluster<2>(a, p, mc, ml, st, max_clusters);
-    case 3: return launch_cluster<3>(a, p, mc, ml, st, max_clusters);
-    default: return launch_cluster<4>(a, p, mc, ml, st, max_clusters);
-    }
+    if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, k, &cfg);
+    return cudaLaunchKernelEx(&cfg, k, a);
 }
 
 // Clusters of this plan's size and resources the device can hold at once (asked once per kind of launch).
-int max_active_clusters(const galv_ctx* ctx, const ClPlan& p)
+int max_active_clusters(const galv_ctx* ctx, const RsPlan& p, bool store, bool arg)
 {
     static std::map<unsigned long long, int> cache;          // shared by all contexts of the process
     static std::mutex cache_mutex;
     std::lock_guard<std::mutex> lock(cache_mutex);
-    const unsigned long long key = ((unsigned long long)ctx->device << 48) | ((unsigned long long)p.cl << 40) |
-                                   ((unsigned long long)p.tm << 36) | ((unsigned long long)p.nw << 28) | (unsigned long long)((p.smem + 1023) / 1024);
+    const unsigned long long key = ((unsigned long long)ctx->device << 48) | ((unsigned long long)p.cl << 40) | ((unsigned long long)store << 37) |
+                                   ((unsigned long long)arg << 36) | ((unsigned long long)p.nw << 28) | (unsigned long long)((p.smem + 1023) / 1024);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
-    ClArgs a{};
+    RsArgs a{};
     a.B = 1;
-    CUtensorMap m{};
     int n = 0;
-    if (launch_any(a, p, m, m, nullptr, &n) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+    if (launch_resident(kernel_of(store, arg), a, p, nullptr, &n) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
     cache[key] = n;
     return n;
 }
 
-// Register-tile height for g column groups per CTA: the one that gives the busiest warp the least work (units are
-// dealt out to at most 12 warps), then the busiest scheduler, then the smaller tile (more, smaller units spread the
-// cost of the tiles that straddle two CTAs).  Returns the busiest scheduler's work in units of 8*S*2 cycles.
-int tile_cost(int g, int nsg, int* tm_out)
+// Shared memory of a launch beside its state.
+long long fixed_smem(const galv_shape* sh, bool dense)
 {
-    int best_tm = 4, best_warp = 1 << 30, best_sched = 1 << 30;
-    for (int tm = 4; tm >= 2; --tm) {
-        const int units = (g + tm - 1) / tm * nsg;
-        int nw = (units + 3) & ~3;
-        if (nw > 12) nw = 12;
-        const int warp = (units + nw - 1) / nw * tm;
-        const int sched = (units + 3) / 4 * tm;
-        if (warp < best_warp || (warp == best_warp && sched <= best_sched)) { best_warp = warp; best_sched = sched; best_tm = tm; }
+    const int S = sh->S, SP = (S + 3) & ~3;
+    const long long t = dense ? (long long)S * SP * ((sh->flags & GALV_TRANS_PER_LAYER) ? 2 : 1) : 0;
+    return (t > kClassMax * kClassMax ? t : kClassMax * kClassMax) * 4 + (long long)3 * S * 16 + (long long)8 * S * 4 + 128;
+}
+
+// The best cluster size for a state of `rows` rows at least; false when none fits.
+bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, RsPlan* out, double* est)
+{
+    const int S = sh->S, Gt = sh->m_pitch / 32;
+    const bool store = (sh->flags & GALV_STORE_C_FULL) != 0, arg = (sh->flags & GALV_STORE_ARGMIN) != 0;
+    const int want = (sh->flags >> 16) & 31;                  // GALV_CLUSTER_SIZE(n): only clusters of n CTAs
+    const int per_word = arg ? 10 : 8;                        // two buffers of words, with argmin bytes beside
+    const long long words = ((long long)ctx->smem_optin - kStaticSmem - fixed_smem(sh, dense)) / per_word;
+    // halo to plan for: a few times what an even share of the budget gives a layer
+    long long halo = 4ll * sh->M / sh->Lmax;
+    if (halo < 64) halo = 64;
+    if (halo > sh->M) halo = sh->M;
+    bool found = false;
+    for (int cl = 1; cl <= ctx->max_cluster; ++cl) {
+        if (want && cl != want) continue;
+        const int g = (Gt + cl - 1) / cl;
+        if (cl > 1 && (g < 2 || g * (cl - 1) >= Gt)) continue;      // no CTA without columns
+        const int w = g * 32;
+        RsPlan p;
+        std::memset(&p, 0, sizeof(p));
+        p.cl = cl; p.w = w; p.dense = dense;
+        p.nw = g < kMaxWarps ? g : kMaxWarps;
+        long long gi = (long long)(dense && S > kClassMax ? S : kClassMax) * (w + ((sh->M + 32) & ~31));    // all that could be used
+        if (gi > words) gi = words;
+        p.gints = (int)(gi & ~31ll);
+        if ((long long)rows * w > p.gints) continue;
+        p.smem = (int)(p.gints * (long long)per_word + fixed_smem(sh, dense));
+        const int slots = max_active_clusters(ctx, p, store, arg);
+        if (slots < 1) continue;
+        // SM cycles a layer: the issue of the columns' work, the store port (32 bytes a clock), the latency of one warp's
+        // walk over the strategies, and the barrier
+        const double issue = g * (S * 7.0 + 120.0) / 2.2, port = store ? g * S * 4.0 : 0.0;
+        const double chain = S * 12.0 + 500.0;
+        double t = issue > port ? issue : port;
+        if (t < chain) t = chain;
+        t += cl == 1 ? 150.0 : (cl > 8 ? 1200.0 : 900.0);
+        const double share = (double)(sh->B < slots ? sh->B : slots) * cl / ctx->num_sms;      // several CTAs on an SM share its issue slots
+        if (share > 1.0) t *= share;
+        t *= (sh->B + slots - 1) / slots;
+        if (cl > 1 && (long long)rows * (w + halo) > p.gints) t *= 4.0;            // shifts beyond the halo take the slow way
+        if (!found || t < *est) {
+            found = true;
+            *est = t;
+            p.sorted = sh->B > slots && sh->B <= kMaxSortedB;
+            *out = p;
+        }
     }
-    *tm_out = best_tm;
-    return best_sched;
+    return found;
 }
 
 }  // namespace
 
-// Whether the cluster kernel can run this shape, and how: CTAs per cluster, columns per CTA, register tile.
-bool galv_cluster_plan(const galv_ctx* ctx, const galv_shape* sh, ClPlan* out)
+int galv_cluster_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
 {
-    std::memset(out, 0, sizeof(*out));
-    if (sh->flags & (GALV_STORE_ARGMIN | GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_DEBUG_WITHHOLD_LOAD | GALV_KERNEL_NO_CLUSTER))
-        return false;
-    const int S = sh->S, Gt = sh->m_pitch / 32;
-    if (S > 32 * kRowsPerLane) return false;
-    if ((long long)sh->B * sh->Lmax * S >= (1ll << 31)) return false;       // row coordinates of the table store are 32-bit
-    const int nsg = (S + 7) / 8, sp8 = nsg * 8;
-    const int nT = (sh->flags & GALV_TRANS_PER_LAYER) ? 2 : 1;
-    const int budget = ctx->smem_optin - 4096;               // static shared memory of the kernel, rounded up
-    // Candidates: every cluster size that gives each CTA at least 96 columns and leaves none without columns.
-    // Estimated SM cycles per layer of a cluster, fitted to measurements on B200: the add-min issue time of the
-    // busiest scheduler, stretched by the per-cell work beside it (push, fill, shared-memory loads: about 24
-    // add-mins' worth per cell), plus what a layer costs whatever its size (barrier, drain of the pushes that
-    // cross CTAs, start): about 3000 cycles, some more for clusters beyond 12 CTAs.  With more instances than the
-    // device holds clusters the batch takes several rounds; on its own the kernel is chosen only when one round
-    // does (a batch that needs rounds is better off on the tiled kernels, whose SMs never wait on a barrier).
-    double best_time = 0.0;
-    bool found = false;
-    const int want_cl = (sh->flags >> 16) & 31;              // GALV_CLUSTER_SIZE(n): only clusters of n CTAs
-    const bool forced = (sh->flags & GALV_KERNEL_CLUSTER) != 0 || want_cl != 0;
-    for (int cl = ctx->max_cluster; cl >= 1; --cl) {
-        if (want_cl && cl != want_cl) continue;
-        const int g = (Gt + cl - 1) / cl;
-        if (cl > 1 && (g < 3 || g * (cl - 1) >= Gt)) continue;
-        const long long smem = (long long)2 * S * g * 32 * 4 + (long long)nT * S * sp8 * 4 + (long long)2 * ((g + 1) / 2) * sp8 * 16 + (long long)2 * sp8 * 4 + 16 + 512 + 64;
-        if (smem > budget) break;                            // smaller clusters need more per CTA
-        ClPlan p;
-        std::memset(&p, 0, sizeof(p));
-        p.cl = cl; p.g = g; p.w = g * 32; p.nsg = nsg; p.sp8 = sp8;
-        const int cost = tile_cost(g, nsg, &p.tm);
-        p.nct = (g + p.tm - 1) / p.tm;
-        p.units = p.nct * nsg;
-        p.nw = (p.units + 3) & ~3;                           // a multiple of 4: the SM's four schedulers get the same share
-        if (p.nw > 12) p.nw = 12;
-        p.smem = (int)smem;
-        const int slots = max_active_clusters(ctx, p);
-        if (slots < 1) continue;
-        if (!forced && sh->B > slots) continue;
-        const double rounds = (double)((sh->B + slots - 1) / slots);
-        const double active = (double)(sh->B < slots ? sh->B : slots) * cl;     // CTAs resident at once
-        const double share = active > ctx->num_sms ? active / ctx->num_sms : 1.0;   // ... of which this many share an SM's ALUs
-        const double t = rounds * ((double)cost * 16.0 * S * (1.0 + 24.0 / S) * share + 3000.0 + (cl > 12 ? 800.0 : 0.0));
-        if (!found || t < best_time) {
-            best_time = t;
-            found = true;
-            p.sorted = sh->B > slots;                        // more clusters than fit at once: the longest instances first
-            *out = p;
-        }
+    if (sh->flags & (GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_DEBUG_WITHHOLD_LOAD | GALV_KERNEL_NO_CLUSTER)) return 0;
+    if (sh->S > kMaxS || (long long)sh->S * sh->m_pitch >= (1ll << 29)) return 0;      // row offsets are 32-bit
+    if (ctx->plan_valid && std::memcmp(&ctx->plan_shape, sh, sizeof(*sh)) == 0) {       // the shape of the last call
+        plans[0] = ctx->plans[0]; plans[1] = ctx->plans[1];
+        return ctx->plan_launches;
     }
-    if (!found) return false;
-    if (out->sorted && sh->B > kMaxSortedB) return false;
-    return true;
+    double td = 0.0, tc = 0.0;
+    int n = 0;
+    const bool d = best_plan(ctx, sh, sh->S, true, &plans[1], &td);
+    const bool c = !(sh->flags & GALV_TRANS_PER_LAYER) && sh->S > 12 && best_plan(ctx, sh, 12, false, &plans[0], &tc);
+    if (d && (!c || td <= tc * 1.15)) { plans[0] = plans[1]; n = 1; }
+    else if (c) n = d ? 2 : 1;
+    ctx->plan_shape = *sh; ctx->plans[0] = plans[0]; ctx->plans[1] = plans[1]; ctx->plan_launches = n; ctx->plan_valid = 1;
+    return n;
 }
 
 cudaError_t galv_cluster_configure(galv_ctx* ctx)
 {
-    const int bytes = ctx->smem_optin - 4096;
-    cudaError_t e = cudaFuncSetAttribute(cluster_search_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(cluster_search_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(cluster_search_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    // clusters of up to 16 CTAs where the device allows them (beyond the portable 8)
-    ctx->max_cluster = 8;
-    if (cudaFuncSetAttribute(cluster_search_kernel<2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaFuncSetAttribute(cluster_search_kernel<3>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaFuncSetAttribute(cluster_search_kernel<4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
-        ctx->max_cluster = 16;
-    else
-        (void)cudaGetLastError();
+    ctx->max_cluster = 16;                                     // beyond the portable 8 where the device allows it
+    for (int k = 0; k < 4; ++k) {
+        const RsKernel f = kernel_of(k & 1, (k & 2) != 0);
+        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin - kStaticSmem);
+        if (e != cudaSuccess) return e;
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) { (void)cudaGetLastError(); ctx->max_cluster = 8; }
+    }
     return cudaSuccess;
 }
 
-cudaError_t galv_cluster_launch(galv_ctx* ctx, const galv_shape* sh, const ClPlan& p, const DpArgs& d, cudaStream_t st)
+cudaError_t galv_cluster_launch(const RsPlan& p, int second, const DpArgs& d, cudaStream_t st)
 {
-    ClArgs a;
+    RsArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
-    a.CL = p.cl; a.W = p.w; a.G = p.g; a.NSG = p.nsg; a.SP8 = p.sp8; a.nct = p.nct; a.units = p.units; a.sorted = p.sorted;
+    a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second;
+    a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept
+    a.path_value = (d.B <= kMaxSortedB && !d.A) ? 2 : 0;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
-    a.C = d.C; a.C_last = d.C_last; a.status = d.status; a.path = d.err;
-    (void)sh;
-    CUtensorMap mc, ml;
-    std::memset(&mc, 0, sizeof(mc));
-    cudaError_t e = encode_table_3d(&ml, d.C_last, (size_t)d.B * d.S, d.m_pitch, d.S, p.g);
-    if (e == cudaSuccess && d.C) e = encode_table_3d(&mc, d.C, (size_t)d.B * d.Lmax * d.S, d.m_pitch, d.S, p.g);
-    if (e != cudaSuccess) return e;
-    const int pk = ctx->prof_count % 64;
-    if (ctx->profiling) cudaEventRecord(ctx->pev[2 * pk], st);
-    e = launch_any(a, p, mc, ml, st, nullptr);
-    if (e != cudaSuccess) return e;
-    if (ctx->profiling) { cudaEventRecord(ctx->pev[2 * pk + 1], st); ++ctx->prof_count; }
-    return cudaGetLastError();
+    a.C = d.C; a.A = d.A; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done;
+    return launch_resident(kernel_of(d.C != nullptr, d.A != nullptr), a, p, st, nullptr);
 }

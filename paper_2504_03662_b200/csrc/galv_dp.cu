@@ -146,10 +146,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // is paid between layers l-1 and l, matrix 0 unused).
 __global__ void validate_kernel(int B, int Lmax, int S, int M, long long tl, const int32_t* __restrict__ L,
                                 const int32_t* __restrict__ time_q, const int32_t* __restrict__ mem_q,
-                                const int32_t* __restrict__ trans_q, int32_t* __restrict__ status,
+                                const int32_t* __restrict__ trans_q, int32_t* __restrict__ status, const int32_t* __restrict__ done,
                                 int32_t* __restrict__ maxmem, int32_t* __restrict__ minmem_l, int32_t* __restrict__ front)
 {
     const int i = blockIdx.x;
+    if (done && done[i]) return;                              // searched, or flagged, by the cluster kernel
     __shared__ long long s_sum;
     __shared__ int s_tmax, s_bad, s_mmax;
     if (threadIdx.x == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; s_mmax = 0; }
@@ -254,7 +255,7 @@ __device__ long long block_scan_1024(long long v, long long* warp_sums, long lon
 // istart[l] = work items (instance, tile, s-block) of layers 1 .. l-1: the items of all layers in one sequence.
 // tcount[l][t] = layers 1 .. l whose items include tile t.
 __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, int tmb, int ntiles_m, int nsb, const int32_t* __restrict__ L,
-                                const int32_t* __restrict__ status, int32_t* __restrict__ order, int32_t* __restrict__ nactive,
+                                const int32_t* __restrict__ status, const int32_t* __restrict__ done, int32_t* __restrict__ order, int32_t* __restrict__ nactive,
                                 int32_t* __restrict__ scratch, const int32_t* __restrict__ minmem_l, int32_t* __restrict__ ntiles,
                                 long long* __restrict__ istart, int32_t* __restrict__ tcount, int p16_possible,
                                 int32_t* __restrict__ maxmem)
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
     int32_t* hist = scratch;
     int32_t* fill = scratch + Lmax + 2;
     for (int i = threadIdx.x; i < B; i += blockDim.x)
-        if (status[i] == 0) atomicAdd(&hist[L[i]], 1);
+        if (status[i] == 0 && !(done && done[i])) atomicAdd(&hist[L[i]], 1);
     for (int l = threadIdx.x; l <= Lmax; l += blockDim.x) {
         int nt = 1;
         if (l < Lmax && minmem_l[l] <= M) nt = min(ntiles_m, (M - minmem_l[l]) / tmb + 1);
@@ -283,8 +284,9 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
         }
     }
     __syncthreads();
+    if (threadIdx.x == 0 && done && nactive[0] == 0) maxmem[2] = 2;      // nothing left for the tiled kernels
     for (int i = threadIdx.x; i < B; i += blockDim.x)
-        if (status[i] == 0) {
+        if (status[i] == 0 && !(done && done[i])) {
             const int Li = L[i];
             order[nactive[Li] + atomicAdd(&fill[Li], 1)] = i;   // instances longer than Li come first
         }
@@ -315,7 +317,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
 __global__ void base_layer_kernel(DpArgs a)
 {
     const int i = blockIdx.z, s = blockIdx.y;
-    if (a.status[i] != 0) return;
+    if (a.status[i] != 0 || (a.done && a.done[i])) return;
     const int tt = a.time_q[(size_t)i * a.Lmax * a.S + s];
     const int mm = a.mem_q[(size_t)i * a.Lmax * a.S + s];
     const size_t row = ((size_t)i * a.S + s) * a.m_pitch;
@@ -1593,7 +1595,7 @@ __global__ void __launch_bounds__((NSG * NMS + (P16 ? (DOM ? 7 : 5) : 4)) * 32, 
 __global__ void copy_last_kernel(DpArgs a)
 {
     const int i = blockIdx.y;
-    if (a.status[i] != 0) return;
+    if (a.status[i] != 0 || (a.done && a.done[i])) return;
     const int Li = a.L[i];
     const size_t slice = (size_t)a.S * a.m_pitch;
     const int32_t* src = a.C ? a.C + ((size_t)i * a.Lmax + (Li - 1)) * slice : a.roll + ((size_t)((Li - 1) & 1) * a.B + i) * slice;
@@ -1687,6 +1689,7 @@ WsLayout galv_ws_layout(const galv_shape* sh)
     WsLayout w;
     size_t off = 0;
     w.order = off;   off = align256(off + (size_t)sh->B * 4);
+    w.done = off;    off = align256(off + (size_t)sh->B * 4);
     w.nactive = off; off = align256(off + (size_t)(sh->Lmax + 1) * 4);
     w.scratch = off; off = align256(off + (size_t)4 * (sh->Lmax + 2) * 4);    // two int32 arrays, one 64-bit array
     w.err = off;     off = align256(off + 32);                 // error flag, largest mem, largest trans, path chosen, keyed argmin
@@ -1795,18 +1798,28 @@ cudaError_t galv_dp_configure(const galv_ctx* ctx)
     return cudaSuccess;
 }
 
-cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& a, cudaStream_t st)
+cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& args, cudaStream_t st)
 {
     cudaError_t e;
+    DpArgs a = args;
     const int B = a.B, Lmax = a.Lmax, S = a.S;
+    const int pk = ctx->prof_count % 64;
+    if (ctx->profiling) cudaEventRecord(ctx->pev[2 * pk], st);
     {
-        // Small batches: one cluster per instance, the whole search in one launch (no workspace but the path flag).
-        ClPlan cp;
-        if (galv_cluster_plan(ctx, sh, &cp)) {
-            e = galv_cluster_launch(ctx, sh, cp, a, st);
-            if (e == cudaSuccess) return e;
-            (void)cudaGetLastError();                        // the clusters cannot be placed on this device right now: tiled kernels
+        // One cluster per instance wherever its state fits shared memory.  What the launches leave alone (known on the
+        // device only) goes to the tiled kernels, which then find their schedule shorter, or empty.
+        RsPlan rp[2];
+        const int n = galv_cluster_plan(ctx, sh, rp);
+        int launched = 0;
+        while (launched < n) {
+            if (galv_cluster_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now
+            ++launched;
         }
+        if (launched && launched == n && rp[n - 1].dense) {
+            if (ctx->profiling) { cudaEventRecord(ctx->pev[2 * pk + 1], st); ++ctx->prof_count; }
+            return cudaSuccess;
+        }
+        if (!launched) a.done = nullptr;
     }
     e = cudaMemsetAsync(a.scratch, 0, (size_t)4 * (Lmax + 2) * 4, st);      // histogram, fill and work counters
     if (e != cudaSuccess) return e;
@@ -1827,9 +1840,9 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& a,
     // The packed 16-bit kernel is launched as well when the shape allows it; which of the two runs is decided on
     // the device, where the largest transition entry is known (the other one returns at once).
     const int will_p16 = persistent && pl.p16 && !(sh->flags & GALV_KERNEL_NO_PACKED);
-    validate_kernel<<<B, 128, 0, st>>>(B, Lmax, S, a.M, (long long)a.trans_layer, a.L, a.time_q, a.mem_q, a.trans_q, a.status, a.err + 1, a.minmem_l,
+    validate_kernel<<<B, 128, 0, st>>>(B, Lmax, S, a.M, (long long)a.trans_layer, a.L, a.time_q, a.mem_q, a.trans_q, a.status, a.done, a.err + 1, a.minmem_l,
                                        (sh->flags & GALV_SKIP_INFEASIBLE) ? a.front : nullptr);
-    schedule_kernel<<<1, 1024, 0, st>>>(B, Lmax, a.M, pl.tmb, pl.ntiles_m, pl.nsb, a.L, a.status, a.order, a.nactive, a.scratch,
+    schedule_kernel<<<1, 1024, 0, st>>>(B, Lmax, a.M, pl.tmb, pl.ntiles_m, pl.nsb, a.L, a.status, a.done, a.order, a.nactive, a.scratch,
                                          a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.err + 1);
     auto base_layer = [&]() {
         int gx = (a.m_pitch + 255) / 256;
@@ -1838,6 +1851,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& a,
             DpArgs s = a;
             const int nb = (B - b0 < 65535) ? B - b0 : 65535;
             s.L += b0; s.status += b0;
+            if (s.done) s.done += b0;
             s.time_q += (size_t)b0 * Lmax * S; s.mem_q += (size_t)b0 * Lmax * S;
             if (s.C) s.C += (size_t)b0 * Lmax * S * a.m_pitch;
             if (s.A) s.A += (size_t)b0 * Lmax * S * a.m_pitch;
@@ -1893,8 +1907,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& a,
         ap.tile_done = a.tile_done;
         if ((e = cudaMemsetAsync(a.tile_done, 0, (size_t)B * pl.ntiles_m * 4, st)) != cudaSuccess) return e;
     }
-    const int pk = ctx->prof_count % 64;
-    if (ctx->profiling) cudaEventRecord(ctx->pev[2 * pk], st);
+    if (ctx->profiling && !a.done) cudaEventRecord(ctx->pev[2 * pk], st);      // the span covers the cluster kernel where it was launched
     bool persistent_ran = false;
     if (key_multi) {
         e = launch_tiled<true>(ap, pl, 1, Lmax, st, maps);
@@ -1942,6 +1955,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& a,
         DpArgs c = a;
         const int nb = (B - b0 < 65535) ? B - b0 : 65535;
         c.L += b0; c.status += b0;
+        if (c.done) c.done += b0;
         if (c.C) c.C += (size_t)b0 * Lmax * S * a.m_pitch;
         c.C_last += (size_t)b0 * S * a.m_pitch;
         c.roll += (size_t)b0 * S * a.m_pitch;
