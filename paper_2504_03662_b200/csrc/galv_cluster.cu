@@ -32,6 +32,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 #include "galv_internal.h"
 
@@ -82,21 +83,42 @@ __device__ __forceinline__ int ld_cluster_u8(uint32_t addr) {
     asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return (int)v;
 }
-__device__ __forceinline__ void st_cluster(uint32_t addr, int v) { asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-__device__ __forceinline__ void st_cluster_u8(uint32_t addr, int v) { asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// everyone's shared-memory writes of this layer are visible to the cluster
-__device__ __forceinline__ void layer_barrier(int CL) {
+// barrier of the CTA whose parties stand at different places in the code
+__device__ __forceinline__ void cta_barrier() {
     __syncwarp();                                              // the aligned forms want the whole warp together
-    if (CL == 1) {
-        asm volatile("bar.sync 0;" ::: "memory");              // the service warp meets it at another place in the code
-    } else {
-        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
+    asm volatile("bar.sync 0;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void whole_barrier(int CL) {
+    if (CL == 1) cta_barrier();
+    else { cluster_arrive(); cluster_wait(); }
+}
+// bytes of this CTA's shared memory to the same cluster's CTA that `dst` and `bar` lie in; counted on its mbarrier
+__device__ __forceinline__ void bulk_to_cta(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_init(uint32_t bar) { asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory"); }
+__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
 }
 __device__ __forceinline__ void cp_async_4(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
@@ -127,24 +149,94 @@ struct Ctx {
     uint8_t* A;
     int32_t* C_last;
     size_t slice;
+    uint32_t bars;             // address of the two mbarriers the halo's bytes are counted on (even, odd layers)
+    uint32_t halo_bytes;       // bytes of halo that arrive a layer
+    bool strict;               // some shift reaches beyond the halo: layers end with the full cluster barrier
+    int* late;                 // set when a bounded wait ran out
 };
+
+// End of a layer, by every warp of the CTA.  The state of layer l+1 is complete in this CTA; its last columns go to the
+// halo of the CTAs further up that hold them, one bulk copy (through the TMA unit) a row and CTA, the warps sharing the
+// rows: plain stores through the cluster window took about 100 cycles a warp store, 13 thousand a layer for 7 rows of
+// 608 columns.  Then the wait for this CTA's own halo.
+// The cluster barrier only keeps the buffers apart: an arrival says that this CTA has gathered from the older buffer
+// and received its halo, and it is waited for a layer later, before the copies that overwrite that buffer are issued.
+// With shifts beyond the halo other CTAs' state is read as well, and the barrier is waited for at once.
+constexpr int kWaitPolls = 1 << 20;                            // try_wait sleeps in hardware between polls: about a second
+template <bool ARG>
+__device__ __forceinline__ void end_layer(const Ctx& c, int l, int warp, int lane)
+{
+    if (c.CL == 1) { cta_barrier(); return; }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");            // plain stores of the state, read next by bulk copies
+    cta_barrier();
+    if (!c.strict) cluster_wait();
+    const uint32_t gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints), bar = c.bars + 8u * (l & 1);
+    const uint32_t an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
+    if (lane == 0)
+        for (int d = c.rank + 1, low = c.W - c.H; d < c.CL && low < c.W; ++d, low += c.W) {
+            // CTA d holds the columns from d*W - H on: this CTA's local columns from `low` on
+            const int from = max(low, 0), n = c.W - from, delta = c.cdelta[d];
+            const int at = c.H + from, to = at - (d - c.rank) * c.W;
+            for (int k = warp; k < c.Kc; k += c.NW + 1) {
+                bulk_to_cta(gn + (uint32_t)(delta + (k * c.P + to) * 4), gn + (uint32_t)(k * c.P + at) * 4u, (uint32_t)n * 4u, bar + (uint32_t)delta);
+                if (ARG) bulk_to_cta(an + (uint32_t)(delta + k * c.P + to), an + (uint32_t)(k * c.P + at), (uint32_t)n, bar + (uint32_t)delta);
+            }
+        }
+    if (c.halo_bytes) {
+        if (warp == c.NW && lane == 0) mbar_expect(bar, c.halo_bytes);
+        const uint32_t parity = (uint32_t)(l >> 1) & 1u;
+        int polls = 0;
+        while (!mbar_try(bar, parity))
+            if (++polls > kWaitPolls || *(volatile int*)c.late) { *(volatile int*)c.late = 1; break; }
+    }
+    cluster_arrive();
+    if (c.strict) cluster_wait();
+}
 
 // Record of (layer, strategy): x = byte offset, from the start of the state, of the cell column 0 of this CTA reads
 // (the row of the strategy's column class, shifted by mem); y = time (kInf: mem exceeds the budget, the row is +inf);
 // z = mem | strategy << 24; w = byte offset of the strategy's row in the table.
 //
-// G at the columns that column `col` of this CTA (and those 32, 64, ... after it) reads.  FAR: the layer has shifts
-// beyond the halo, whose cells are read from the CTA that owns them.
+// Shared-memory accesses of the layer loop go through 32-bit addresses and are written in batches, loads first: the table
+// stores between two strategies would otherwise hold the next strategy's loads back (they could alias for all the
+// compiler knows), and a strategy would cost the latency of its whole chain (220 cycles) instead of a share of it.
+__device__ __forceinline__ int lds(uint32_t a) {
+    int v;
+    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ int lds_at(uint32_t a) {
+    int v;
+    asm volatile("ld.shared.s32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
+    return v;
+}
+__device__ __forceinline__ int lds_u8(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+    return (int)v;
+}
+__device__ __forceinline__ int4 lds4(uint32_t a) {
+    int4 v;
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts(uint32_t a, int v) { asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+__device__ __forceinline__ void sts_u8(uint32_t a, int v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+
+// G at the columns that column `col` of this CTA (and those 32, 64, ... after it) reads; ga: the state's address plus
+// 4 * col.  FAR: the layer has shifts beyond the halo, whose cells are read from the CTA that owns them.
 template <int TM, bool FAR>
-__device__ __forceinline__ void gather(const Ctx& c, const int32_t* Gp, const int4 r, int col, int (&g)[TM])
+__device__ __forceinline__ void gather(const Ctx& c, uint32_t ga, const int4 r, int col, int (&g)[TM])
 {
     const int mem = r.z & 0xffffff;
     if (!FAR || mem <= c.H) {
-        const int32_t* p = reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(Gp + col) + r.x);
-#pragma unroll
-        for (int j = 0; j < TM; ++j) g[j] = p[j * 32];
+        const uint32_t a = ga + (uint32_t)r.x;
+        g[0] = lds(a);
+        if (TM > 1) g[1 % TM] = lds_at<128>(a);
+        if (TM > 2) { g[2 % TM] = lds_at<256>(a); g[3 % TM] = lds_at<384>(a); }
     } else {
-        const uint32_t row = smem_addr(Gp) + (uint32_t)r.x + (uint32_t)mem * 4u;
+        const uint32_t row = ga - 4u * (uint32_t)col + (uint32_t)r.x + (uint32_t)mem * 4u;
 #pragma unroll
         for (int j = 0; j < TM; ++j) {
             const int src = c.rank * c.W + col + 32 * j - mem;
@@ -154,16 +246,16 @@ __device__ __forceinline__ void gather(const Ctx& c, const int32_t* Gp, const in
         }
     }
 }
-// ... and their argmin entries
+// ... and their argmin entries; aa: the argmin state's address plus col
 template <int TM, bool FAR>
-__device__ __forceinline__ void gather_arg(const Ctx& c, const uint8_t* Ap, const int4 r, int col, int (&a)[TM])
+__device__ __forceinline__ void gather_arg(const Ctx& c, uint32_t aa, const int4 r, int col, int (&a)[TM])
 {
     const int mem = r.z & 0xffffff, off = r.x >> 2;
     if (!FAR || mem <= c.H) {
 #pragma unroll
-        for (int j = 0; j < TM; ++j) a[j] = Ap[off + col + j * 32];
+        for (int j = 0; j < TM; ++j) a[j] = lds_u8(aa + (uint32_t)(off + 32 * j));
     } else {
-        const uint32_t row = smem_addr(Ap) + (uint32_t)(off + mem);
+        const uint32_t row = aa - (uint32_t)col + (uint32_t)(off + mem);
 #pragma unroll
         for (int j = 0; j < TM; ++j) {
             const int src = c.rank * c.W + col + 32 * j - mem;
@@ -174,68 +266,114 @@ __device__ __forceinline__ void gather_arg(const Ctx& c, const uint8_t* Ap, cons
     }
 }
 
-// Values of one state row for the tile: into this CTA's columns, and into the halo of every CTA further up that holds them.
+// Values of one state row for the tile.
 template <int TM, bool ARG>
-__device__ __forceinline__ void emit(const Ctx& c, int32_t* Gn, uint8_t* An, int k, int colb, int lane, const int (&v)[TM], const int (&a)[TM])
+__device__ __forceinline__ void emit(const Ctx& c, uint32_t gn, uint32_t an, int k, int colb, int lane, const int (&v)[TM], const int (&a)[TM])
 {
     const int at = k * c.P + c.H + colb + lane;
 #pragma unroll
-    for (int j = 0; j < TM; ++j)
-        if (colb + 32 * j < c.W) {
-            Gn[at + 32 * j] = v[j];
-            if (ARG) An[at + 32 * j] = (uint8_t)a[j];
-        }
-    for (int d = c.rank + 1, low = c.W - c.H; d < c.CL && colb + 32 * TM > low; ++d, low += c.W) {
-        // CTA d holds the columns from d*W - H on: this CTA's local columns from `low` on
-        const uint32_t ga = smem_addr(Gn) + (uint32_t)(c.cdelta[d] + (at - (d - c.rank) * c.W) * 4);
-        const uint32_t aa = ARG ? smem_addr(An) + (uint32_t)(c.cdelta[d] + at - (d - c.rank) * c.W) : 0u;
-#pragma unroll
-        for (int j = 0; j < TM; ++j)
-            if (colb + 32 * j >= low && colb + 32 * j < c.W) {
-                st_cluster(ga + 128u * j, v[j]);
-                if (ARG) st_cluster_u8(aa + 32u * j, a[j]);
-            }
+    for (int j = 0; j < TM; ++j) {
+        sts(gn + (uint32_t)(at + 32 * j) * 4u, v[j]);
+        if (ARG) sts_u8(an + (uint32_t)(at + 32 * j), a[j]);
     }
+}
+
+// Where a tile's values go in the table.
+template <bool STORE, bool ARG>
+struct Out {
+    char* C;               // the tile's first column plus this lane, strategy 0
+    uint8_t* A;
+    bool whole;            // every column of the tile is a budget column
+    int cols;              // columns of the tile that exist in the table, less this lane
+    int budget;            // ... that are budget columns, less this lane
+    template <int TM>
+    __device__ __forceinline__ void put(const int4 r, const int (&v)[TM], const int (&a)[TM]) const
+    {
+        if (STORE) {
+            int32_t* const p = reinterpret_cast<int32_t*>(C + (uint32_t)r.w);
+            if (whole) {
+#pragma unroll
+                for (int j = 0; j < TM; ++j) p[32 * j] = v[j];
+            } else {                                           // +inf in the pad columns beyond the budget
+#pragma unroll
+                for (int j = 0; j < TM; ++j)
+                    if (32 * j < cols) p[32 * j] = 32 * j < budget ? v[j] : kInf;
+            }
+        }
+        if (ARG) {
+            uint8_t* const p = A + ((uint32_t)r.w >> 2);
+#pragma unroll
+            for (int j = 0; j < TM; ++j)
+                if (whole || 32 * j < cols) p[32 * j] = (uint8_t)((whole || 32 * j < budget) && v[j] < kInf ? a[j] : 255);
+        }
+    }
+};
+
+// U strategies, from record address ra on: their C values to the table, their smallest into h (with ARG: whose it is).
+template <int U, int TM, bool STORE, bool ARG, bool FAR>
+__device__ __forceinline__ void scan(const Ctx& c, const Out<STORE, ARG>& out, uint32_t ra, uint32_t ga, uint32_t aa, int col, int (&h)[TM], int (&hs)[TM])
+{
+    int4 r[U];
+    int v[U][TM], a[ARG ? U : 1][TM];
+#pragma unroll
+    for (int u = 0; u < U; ++u) r[u] = lds4(ra + 16u * u);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        gather<TM, FAR>(c, ga, r[u], col, v[u]);
+        if (ARG) gather_arg<TM, FAR>(c, aa, r[u], col, a[ARG ? u : 0]);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int j = 0; j < TM; ++j) {
+            if (STORE || ARG) {
+                v[u][j] = __viaddmin_s32(v[u][j], r[u].y, kInf);
+                if (ARG) hs[j] = v[u][j] < h[j] ? r[u].z >> 24 : hs[j];    // ascending strategies: the lowest keeps a tie
+                h[j] = min(h[j], v[u][j]);
+            } else {
+                h[j] = __viaddmin_s32(v[u][j], r[u].y, h[j]);
+            }
+        }
+        if (STORE || ARG) out.template put<TM>(r[u], v[u], a[ARG ? u : 0]);
+    }
+}
+
+// Which of U strategies are alive in some column of the tile, as bits.
+template <int U, int TM, bool FAR>
+__device__ __forceinline__ uint32_t alive(const Ctx& c, uint32_t ra, uint32_t ga, int col, const int (&thr)[TM])
+{
+    int4 r[U];
+    int v[U][TM];
+    uint32_t bits = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) r[u] = lds4(ra + 16u * u);
+#pragma unroll
+    for (int u = 0; u < U; ++u) gather<TM, FAR>(c, ga, r[u], col, v[u]);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        bool live = false;
+#pragma unroll
+        for (int j = 0; j < TM; ++j) live = live || __viaddmin_s32(v[u][j], r[u].y, kInf) <= thr[j];
+        if (__any_sync(0xffffffffu, live)) bits |= 1u << u;
+    }
+    return bits;
 }
 
 // One layer of one tile of TM x 32 columns.  KC: rows of the next state held in accumulators (PRUNE: per block of rows).
 template <int KC, int TM, bool PRUNE, bool STORE, bool ARG, bool FAR>
 __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
 {
-    const int slot = l % 3;
-    const int4* const rec = c.rec + slot * c.S;
-    const int32_t* const Gp = c.g0 + (l & 1) * c.gints;
-    int32_t* const Gn = c.g0 + ((l + 1) & 1) * c.gints;
-    const uint8_t* const Ap = ARG ? c.a0 + (l & 1) * c.gints : nullptr;
-    uint8_t* const An = ARG ? c.a0 + ((l + 1) & 1) * c.gints : nullptr;
+    const int slot = l % 3, col = colb + lane;
+    const uint32_t ra = smem_addr(c.rec + slot * c.S);
+    const uint32_t ga = smem_addr(c.g0 + (l & 1) * c.gints + col), gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints);
+    const uint32_t aa = ARG ? smem_addr(c.a0 + (l & 1) * c.gints + col) : 0u, an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
     const int colg = c.rank * c.W + colb;                      // the tile's first budget column
-    char* const Cl = STORE ? reinterpret_cast<char*>(c.C + (size_t)l * c.slice + colg + lane) : nullptr;
-    uint8_t* const Al = ARG ? c.A + (size_t)l * c.slice + colg + lane : nullptr;
-    const bool whole = colg + 32 * TM - 1 <= c.M && colb + 32 * TM <= c.W;     // every column of the tile is a budget column of this CTA
-    const int last_col = min(c.m_pitch - c.rank * c.W, c.W);   // local columns that exist in the table
-
-    // what goes to the table: +inf in the pad columns beyond the budget
-    auto put = [&](const int4 r, const int (&v)[TM]) {
-        if (STORE) {
-            int32_t* const p = reinterpret_cast<int32_t*>(Cl + (uint32_t)r.w);
-            if (whole) {
-#pragma unroll
-                for (int j = 0; j < TM; ++j) p[32 * j] = v[j];
-            } else {
-#pragma unroll
-                for (int j = 0; j < TM; ++j)
-                    if (colb + 32 * j < last_col) p[32 * j] = colg + lane + 32 * j <= c.M ? v[j] : kInf;
-            }
-        }
-        if (ARG) {
-            int a[TM];
-            gather_arg<TM, FAR>(c, Ap, r, colb + lane, a);
-            uint8_t* const p = Al + ((uint32_t)r.w >> 2);
-#pragma unroll
-            for (int j = 0; j < TM; ++j)
-                if (colb + 32 * j < last_col) p[32 * j] = (uint8_t)(colg + lane + 32 * j <= c.M && v[j] < kInf ? a[j] : 255);
-        }
-    };
+    Out<STORE, ARG> out;
+    out.C = STORE ? reinterpret_cast<char*>(c.C + (size_t)l * c.slice + colg + lane) : nullptr;
+    out.A = ARG ? c.A + (size_t)l * c.slice + colg + lane : nullptr;
+    out.whole = colg + 32 * TM - 1 <= c.M;
+    out.cols = c.m_pitch - colg - lane;
+    out.budget = c.M + 1 - colg - lane;
 
     if (colg + 32 * TM - 1 < c.front[slot]) {                  // nothing finite in the tile
         int inf[TM], none[TM];
@@ -243,16 +381,8 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
         for (int j = 0; j < TM; ++j) { inf[j] = kInf; none[j] = 255; }
         if (STORE || ARG)
 #pragma unroll 4
-            for (int e = 0; e < c.S; ++e) {
-                const uint32_t row = (uint32_t)rec[e].w;
-#pragma unroll
-                for (int j = 0; j < TM; ++j)
-                    if (colb + 32 * j < last_col) {
-                        if (STORE) reinterpret_cast<int32_t*>(Cl + row)[32 * j] = kInf;
-                        if (ARG) Al[(row >> 2) + 32 * j] = 255;
-                    }
-            }
-        for (int k = 0; k < c.Kc; ++k) emit<TM, ARG>(c, Gn, An, k, colb, lane, inf, none);
+            for (int e = 0; e < c.S; ++e) out.template put<TM>(make_int4(0, 0, 0, e * c.m_pitch * 4), inf, none);
+        for (int k = 0; k < c.Kc; ++k) emit<TM, ARG>(c, gn, an, k, colb, lane, inf, none);
         return;
     }
 
@@ -263,43 +393,33 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
 #pragma unroll
             for (int j = 0; j < TM; ++j) { acc[k][j] = kInf; if (ARG) arg[k][j] = 255; }
         int e = 0;
+        const uint32_t ta = smem_addr(c.tsm);
         for (int k = 0; k < c.Kr; ++k) {
             const int end = c.cs[k + 1];
-            int h[TM], hs[ARG ? TM : 1];
+            int h[TM], hs[TM];
 #pragma unroll
-            for (int j = 0; j < TM; ++j) { h[j] = kInf; if (ARG) hs[j] = 255; }
-#pragma unroll 4
-            for (; e < end; ++e) {
-                const int4 r = rec[e];
-                int g[TM];
-                gather<TM, FAR>(c, Gp, r, colb + lane, g);
-                if (STORE || ARG) {
-                    int v[TM];
+            for (int j = 0; j < TM; ++j) { h[j] = kInf; hs[j] = 255; }
+            int4 t4[KC / 4];
 #pragma unroll
-                    for (int j = 0; j < TM; ++j) {
-                        v[j] = __viaddmin_s32(g[j], r.y, kInf);
-                        if (ARG) hs[j] = v[j] < h[j] ? r.z >> 24 : hs[j];  // ascending strategies: the lowest keeps a tie
-                        h[j] = min(h[j], v[j]);
-                    }
-                    put(r, v);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < TM; ++j) h[j] = __viaddmin_s32(g[j], r.y, h[j]);
-                }
+            for (int q = 0; q < KC / 4; ++q) t4[q] = lds4(ta + (uint32_t)(k * kClassMax + 4 * q) * 4u);
+            if (!FAR) {
+                for (; e + 4 <= end; e += 4) scan<4, TM, STORE, ARG, FAR>(c, out, ra + 16u * e, ga, aa, col, h, hs);
+                if (e + 2 <= end) { scan<2, TM, STORE, ARG, FAR>(c, out, ra + 16u * e, ga, aa, col, h, hs); e += 2; }
+                if (e < end) { scan<1, TM, STORE, ARG, FAR>(c, out, ra + 16u * e, ga, aa, col, h, hs); ++e; }
+            } else {
+                for (; e < end; ++e) scan<1, TM, STORE, ARG, FAR>(c, out, ra + 16u * e, ga, aa, col, h, hs);
             }
-            const int4* const T4 = reinterpret_cast<const int4*>(c.tsm + k * kClassMax);
 #pragma unroll
             for (int q = 0; q < KC / 4; ++q) {
-                const int4 t4 = T4[q];
-                const int t[4] = {t4.x, t4.y, t4.z, t4.w};
+                const int t[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
 #pragma unroll
                 for (int j = 0; j < TM; ++j)
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         if (ARG) {
-                            const int cand = h[j] + t[u], old = acc[4 * q + u][j], oa = arg[4 * q + u][j];
+                            const int cand = h[j] + t[u], old = acc[4 * q + u][j], oa = arg[ARG ? 4 * q + u : 0][j];
                             const bool better = cand < old || (cand == old && hs[j] < oa);
-                            if (better && h[j] < kInf) { acc[4 * q + u][j] = cand; arg[4 * q + u][j] = hs[j]; }
+                            if (better && h[j] < kInf) { acc[4 * q + u][j] = cand; arg[ARG ? 4 * q + u : 0][j] = hs[j]; }
                         } else {
                             acc[4 * q + u][j] = __viaddmin_s32(h[j], t[u], acc[4 * q + u][j]);
                         }
@@ -308,50 +428,51 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
         }
 #pragma unroll
         for (int k = 0; k < KC; ++k)
-            if (k < c.Kc) emit<TM, ARG>(c, Gn, An, k, colb, lane, acc[k], arg[ARG ? k : 0]);
+            if (k < c.Kc) emit<TM, ARG>(c, gn, an, k, colb, lane, acc[k], arg[ARG ? k : 0]);
     } else {
-        int thr[TM];
+        int thr[TM], dummy[TM];
 #pragma unroll
-        for (int j = 0; j < TM; ++j) thr[j] = kInf;
-#pragma unroll 4
-        for (int s = 0; s < c.S; ++s) {
-            const int4 r = rec[s];
-            int v[TM];
-            gather<TM, FAR>(c, Gp, r, colb + lane, v);
-#pragma unroll
-            for (int j = 0; j < TM; ++j) {
-                v[j] = __viaddmin_s32(v[j], r.y, kInf);
-                thr[j] = min(thr[j], v[j]);
-            }
-            put(r, v);
-        }
+        for (int j = 0; j < TM; ++j) { thr[j] = kInf; dummy[j] = 255; }
+        int s = 0;
+        if (!FAR)
+            for (; s + 4 <= c.S; s += 4) scan<4, TM, STORE, ARG, FAR>(c, out, ra + 16u * s, ga, aa, col, thr, dummy);
+        for (; s < c.S; ++s) scan<1, TM, STORE, ARG, FAR>(c, out, ra + 16u * s, ga, aa, col, thr, dummy);
         // a candidate beyond the column's best plus the largest entry cannot win; a column without a finite value
         // keeps nothing alive
 #pragma unroll
         for (int j = 0; j < TM; ++j) thr[j] = thr[j] < kInf ? thr[j] + c.tmax : -1;
-        const int32_t* const T = c.tsm + (((l + 1) & 1) ? c.tmat : 0);
+        uint32_t live[kMaxS / 32];
+#pragma unroll
+        for (int b = 0; b < kMaxS / 32; ++b) {
+            live[b] = 0;
+            if (32 * b < c.S) {
+                const int n = min(32, c.S - 32 * b);
+                int q = 0;
+                if (!FAR)
+                    for (; q + 4 <= n; q += 4) live[b] |= alive<4, TM, FAR>(c, ra + 16u * (32 * b + q), ga, col, thr) << q;
+                for (; q < n; ++q) live[b] |= alive<1, TM, FAR>(c, ra + 16u * (32 * b + q), ga, col, thr) << q;
+            }
+        }
+        const uint32_t ta = smem_addr(c.tsm + (((l + 1) & 1) ? c.tmat : 0));
         for (int cb = 0; cb < c.S; cb += KC) {
             int acc[KC][TM], arg[ARG ? KC : 1][TM];
 #pragma unroll
             for (int k = 0; k < KC; ++k)
 #pragma unroll
                 for (int j = 0; j < TM; ++j) { acc[k][j] = kInf; if (ARG) arg[k][j] = 255; }
-#pragma unroll 2
-            for (int s = 0; s < c.S; ++s) {
-                const int4 r = rec[s];
-                int v[TM];
-                gather<TM, FAR>(c, Gp, r, colb + lane, v);
-                bool live = false;
 #pragma unroll
-                for (int j = 0; j < TM; ++j) {
-                    v[j] = __viaddmin_s32(v[j], r.y, kInf);
-                    live = live || v[j] <= thr[j];
-                }
-                if (__any_sync(0xffffffffu, live)) {
-                    const int4* const T4 = reinterpret_cast<const int4*>(T + s * c.SP + cb);
+            for (int b = 0; b < kMaxS / 32; ++b)
+                for (uint32_t m = live[b]; m; m &= m - 1) {
+                    const int q = 32 * b + __ffs(m) - 1;
+                    const int4 r = lds4(ra + 16u * q);
+                    const uint32_t t0 = ta + (uint32_t)(q * c.SP + cb) * 4u;
+                    int v[TM];
+                    gather<TM, FAR>(c, ga, r, col, v);
 #pragma unroll
-                    for (int q = 0; q < KC / 4; ++q) {
-                        const int4 t4 = T4[q];
+                    for (int j = 0; j < TM; ++j) v[j] = __viaddmin_s32(v[j], r.y, kInf);
+#pragma unroll
+                    for (int w = 0; w < KC / 4; ++w) {
+                        const int4 t4 = lds4(t0 + 16u * w);
                         const int t[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
                         for (int j = 0; j < TM; ++j)
@@ -359,70 +480,79 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
                             for (int u = 0; u < 4; ++u) {
                                 if (ARG) {
                                     const int cand = v[j] + t[u];
-                                    if (v[j] < kInf && cand < acc[4 * q + u][j]) { acc[4 * q + u][j] = cand; arg[4 * q + u][j] = s; }
+                                    if (v[j] < kInf && cand < acc[4 * w + u][j]) { acc[4 * w + u][j] = cand; arg[ARG ? 4 * w + u : 0][j] = q; }
                                 } else {
-                                    acc[4 * q + u][j] = __viaddmin_s32(v[j], t[u], acc[4 * q + u][j]);
+                                    acc[4 * w + u][j] = __viaddmin_s32(v[j], t[u], acc[4 * w + u][j]);
                                 }
                             }
                     }
                 }
-            }
 #pragma unroll
             for (int k = 0; k < KC; ++k)
-                if (cb + k < c.S) emit<TM, ARG>(c, Gn, An, cb + k, colb, lane, acc[k], arg[ARG ? k : 0]);
+                if (cb + k < c.S) emit<TM, ARG>(c, gn, an, cb + k, colb, lane, acc[k], arg[ARG ? k : 0]);
         }
     }
 }
 
 // The last layer hands nothing on: its values go to the table and to C_last.
-template <bool STORE, bool ARG>
+template <bool STORE, bool ARG, bool FAR>
 __device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lane)
 {
-    const int slot = l % 3;
-    const int4* const rec = c.rec + slot * c.S;
-    const int32_t* const Gp = c.g0 + (l & 1) * c.gints;
-    const uint8_t* const Ap = ARG ? c.a0 + (l & 1) * c.gints : nullptr;
+    const int slot = l % 3, col = colb + lane;
+    const uint32_t ra = smem_addr(c.rec + slot * c.S), ga = smem_addr(c.g0 + (l & 1) * c.gints + col);
+    const uint32_t aa = ARG ? smem_addr(c.a0 + (l & 1) * c.gints + col) : 0u;
     const int colg = c.rank * c.W + colb, m = colg + lane;
     if (colg >= c.m_pitch) return;                             // m_pitch is a multiple of 32: a group exists whole or not at all
     const bool pad = m > c.M;
-    auto step = [&](const int4 r, int g, int a) {
-        const int v = pad ? kInf : __viaddmin_s32(g, r.y, kInf);
-        const size_t row = ((uint32_t)r.w >> 2) + (size_t)m;
-        if (STORE) c.C[(size_t)l * c.slice + row] = v;
-        c.C_last[row] = v;
-        if (ARG) c.A[(size_t)l * c.slice + row] = (uint8_t)(v < kInf ? a : 255);
+    auto steps = [&](auto count, int e) {
+        constexpr int U = decltype(count)::value;
+        int4 r[U];
+        int g[U][1], a[U][1];
+#pragma unroll
+        for (int u = 0; u < U; ++u) r[u] = lds4(ra + 16u * (e + u));
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            gather<1, FAR>(c, ga, r[u], col, g[u]);
+            if (ARG) gather_arg<1, FAR>(c, aa, r[u], col, a[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int v = pad ? kInf : __viaddmin_s32(g[u][0], r[u].y, kInf);
+            const size_t row = ((uint32_t)r[u].w >> 2) + (size_t)m;
+            if (STORE) c.C[(size_t)l * c.slice + row] = v;
+            c.C_last[row] = v;
+            if (ARG) c.A[(size_t)l * c.slice + row] = (uint8_t)(v < kInf ? a[u][0] : 255);
+        }
     };
-    int g[1], a[1] = {255};
-    if (c.reach[slot] <= c.H) {
-#pragma unroll 4
-        for (int e = 0; e < c.S; ++e) {
-            const int4 r = rec[e];
-            gather<1, false>(c, Gp, r, colb + lane, g);
-            if (ARG) gather_arg<1, false>(c, Ap, r, colb + lane, a);
-            step(r, g[0], a[0]);
-        }
-    } else {
-        for (int e = 0; e < c.S; ++e) {
-            const int4 r = rec[e];
-            gather<1, true>(c, Gp, r, colb + lane, g);
-            if (ARG) gather_arg<1, true>(c, Ap, r, colb + lane, a);
-            step(r, g[0], a[0]);
-        }
-    }
+    int e = 0;
+    if (!FAR)
+        for (; e + 4 <= c.S; e += 4) steps(std::integral_constant<int, 4>(), e);
+    for (; e < c.S; ++e) steps(std::integral_constant<int, 1>(), e);
 }
 
+// A warp owns a run of column groups, the warps' runs differ by one group at most, and takes them TM at a time, then
+// one at a time.
 template <int KC, int TM, bool PRUNE, bool STORE, bool ARG>
 __device__ __forceinline__ void run_layers(const Ctx& c, int warp, int lane)
 {
+    const int g0 = c.G * warp / c.NW, g1 = c.G * (warp + 1) / c.NW;
     for (int l = 0; l + 1 < c.Li; ++l) {
+        int g = g0;
         if (c.reach[l % 3] <= c.H) {
-            for (int g = warp * TM; g < c.G; g += c.NW * TM) tile<KC, TM, PRUNE, STORE, ARG, false>(c, l, g * 32, lane);
+            if (TM > 1)
+                for (; g + TM <= g1; g += TM) tile<KC, TM, PRUNE, STORE, ARG, false>(c, l, g * 32, lane);
+            if (TM > 2 && g + 2 <= g1) { tile<KC, 2, PRUNE, STORE, ARG, false>(c, l, g * 32, lane); g += 2; }
+            for (; g < g1; ++g) tile<KC, 1, PRUNE, STORE, ARG, false>(c, l, g * 32, lane);
         } else {
-            for (int g = warp; g < c.G; g += c.NW) tile<KC, 1, PRUNE, STORE, ARG, true>(c, l, g * 32, lane);
+            for (; g < g1; ++g) tile<KC, 1, PRUNE, STORE, ARG, true>(c, l, g * 32, lane);
         }
-        layer_barrier(c.CL);
+        end_layer<ARG>(c, l, warp, lane);
     }
-    for (int g = warp; g < c.G; g += c.NW) last_tile<STORE, ARG>(c, c.Li - 1, g * 32, lane);
+    if (c.reach[(c.Li - 1) % 3] <= c.H) {
+        for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, false>(c, c.Li - 1, g * 32, lane);
+    } else {
+        for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, true>(c, c.Li - 1, g * 32, lane);
+    }
 }
 
 // Cluster c takes instance c (the c-th longest when `sorted`).  Warps 0..NW-1 compute, the last warp fetches the
@@ -435,6 +565,8 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     __shared__ int s_rrep[kMaxS], s_crep[kMaxS], s_rcls[kMaxS], s_ccls[kMaxS], s_order[kMaxS], s_cs[kMaxS + 1];
     __shared__ int s_cdelta[16], s_front[3], s_reach[3], s_inst, s_K[2];
     __shared__ struct { long long sum; int tmax, bad, mmax; } s_part, s_all;
+    __shared__ __align__(8) unsigned long long s_bar[2];
+    __shared__ int s_late;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x, NW = (NT >> 5) - 1;
     const int CL = a.CL, rank = CL > 1 ? (int)cluster_rank() : 0, cid = blockIdx.x / CL;
@@ -486,6 +618,11 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     const bool staged = !a.trans_layer && (long long)S * S <= (long long)2 * gints;
     if (tid == 0) { s_part.sum = 0; s_part.tmax = 0; s_part.bad = 0; s_part.mmax = 0; }
     for (int x = tid; x < kMaxS; x += NT) { s_u.h.rh[x] = 0; s_u.h.ch[x] = 0; }
+    if (tid == 0) {
+        s_late = 0;
+        mbar_init(smem_addr(&s_bar[0])); mbar_init(smem_addr(&s_bar[1]));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     if (tid < 16) s_cdelta[tid] = CL > 1 ? (int)(map_to_rank(smem_addr(g0), (uint32_t)min(tid, CL - 1)) - smem_addr(g0)) : 0;
     __syncthreads();
     {
@@ -530,7 +667,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
             if (bad) atomicOr(&s_part.bad, 1);
         }
     }
-    layer_barrier(CL);
+    whole_barrier(CL);
     if (warp == 0) {
         long long sum = 0;
         int tmax = 0, bad = 0, mmax = 0;
@@ -714,9 +851,24 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                 }
         }
     }
-    layer_barrier(CL);                                          // also: nobody leaves while its partial sums are being read
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");            // bulk copies write over the halo's initial values
+    whole_barrier(CL);                                          // also: nobody leaves while its partial sums are being read
     if (!run) return;
 
+    Ctx c;
+    c.S = S; c.M = M; c.W = W; c.H = H; c.P = P; c.G = W / 32; c.CL = CL; c.rank = rank; c.Li = Li; c.m_pitch = a.m_pitch; c.Kr = Kr; c.Kc = Kc;
+    c.tmax = s_all.tmax; c.SP = a.SP; c.NW = NW; c.gints = gints;
+    c.g0 = g0; c.a0 = a0; c.rec = rec; c.front = s_front; c.reach = s_reach; c.tsm = tsm; c.tmat = a.trans_layer ? tfull : 0;
+    c.cs = s_cs; c.cdelta = s_cdelta;
+    c.slice = (size_t)S * a.m_pitch;
+    c.C = STORE ? a.C + (size_t)i * Lmax * c.slice : nullptr;
+    c.A = ARG ? a.A + (size_t)i * Lmax * c.slice : nullptr;
+    c.C_last = a.C_last + (size_t)i * c.slice;
+    c.bars = smem_addr(&s_bar[0]);
+    c.halo_bytes = (uint32_t)(Kc * min(H, rank * W)) * (ARG ? 5u : 4u);
+    c.strict = s_all.mmax > H;
+    c.late = &s_late;
+    if (CL > 1 && !c.strict) cluster_arrive();                  // nobody has read anything yet: the first copies may come
     if (warp == NW) {
         // ---------------------------------------------------------------- service warp
         for (int l = 0; l + 1 < Li; ++l) {
@@ -737,28 +889,18 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                 front = prepare(l + 2, front);
             }
             if (a.trans_layer) cp_async_wait<0>();
-            layer_barrier(CL);
+            end_layer<ARG>(c, l, warp, lane);
         }
     } else {
-        Ctx c;
-        c.S = S; c.M = M; c.W = W; c.H = H; c.P = P; c.G = W / 32; c.CL = CL; c.rank = rank; c.Li = Li; c.m_pitch = a.m_pitch; c.Kr = Kr; c.Kc = Kc;
-        c.tmax = s_all.tmax; c.SP = a.SP; c.NW = NW; c.gints = gints;
-        c.g0 = g0; c.a0 = a0; c.rec = rec; c.front = s_front; c.reach = s_reach; c.tsm = tsm; c.tmat = a.trans_layer ? tfull : 0;
-        c.cs = s_cs; c.cdelta = s_cdelta;
-        c.slice = (size_t)S * a.m_pitch;
-        c.C = STORE ? a.C + (size_t)i * Lmax * c.slice : nullptr;
-        c.A = ARG ? a.A + (size_t)i * Lmax * c.slice : nullptr;
-        c.C_last = a.C_last + (size_t)i * c.slice;
-        // columns per lane: one group of 32 per warp while the warps last, then two, then four (a record fetched once
-        // serves them all)
+        // columns per lane: a record fetched once serves up to four groups of 32
         const int per = (c.G + NW - 1) / NW;
         if (classes) {
             if (K <= 4) {
-                if (per >= 3 && !ARG) run_layers<4, 4, false, STORE, ARG>(c, warp, lane);
+                if (per >= 4 && !ARG) run_layers<4, ARG ? 1 : 4, false, STORE, ARG>(c, warp, lane);
                 else if (per >= 2) run_layers<4, 2, false, STORE, ARG>(c, warp, lane);
                 else run_layers<4, 1, false, STORE, ARG>(c, warp, lane);
             } else if (K <= 8) {
-                if (per >= 3 && !ARG) run_layers<8, 4, false, STORE, ARG>(c, warp, lane);
+                if (per >= 4 && !ARG) run_layers<8, ARG ? 1 : 4, false, STORE, ARG>(c, warp, lane);
                 else if (per >= 2) run_layers<8, 2, false, STORE, ARG>(c, warp, lane);
                 else run_layers<8, 1, false, STORE, ARG>(c, warp, lane);
             } else {
@@ -766,11 +908,16 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                 else run_layers<16, 1, false, STORE, ARG>(c, warp, lane);
             }
         } else {
-            if (per >= 2 && !ARG) run_layers<32, 2, true, STORE, ARG>(c, warp, lane);
+            if (per >= 2 && !ARG) run_layers<32, ARG ? 1 : 2, true, STORE, ARG>(c, warp, lane);
             else run_layers<32, 1, true, STORE, ARG>(c, warp, lane);
         }
     }
-    if (CL > 1) layer_barrier(CL);                              // nobody's shared memory goes away while it is being read
+    if (CL > 1) {
+        if (!c.strict) cluster_wait();
+        whole_barrier(CL);                                      // nobody's shared memory goes away while it is being read
+        if (rank == 0 && tid == 0 && s_late) a.path[0] = 1;
+    }
+    if (s_late && tid == 0) atomicOr(reinterpret_cast<int*>(a.status + i), GALV_STATUS_TIMEOUT);
 }
 
 // ---------------------------------------------------------------- host side
