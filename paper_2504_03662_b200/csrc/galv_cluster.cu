@@ -97,6 +97,11 @@ __device__ __forceinline__ void cluster_arrive() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
+// an arrival that orders nothing: a release would wait for the table stores in flight
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_wait() {
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -166,22 +171,23 @@ constexpr int kWaitPolls = 1 << 20;                            // try_wait sleep
 template <bool ARG>
 __device__ __forceinline__ void end_layer(const Ctx& c, int l, int warp, int lane)
 {
-    if (c.CL == 1) { cta_barrier(); return; }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");            // plain stores of the state, read next by bulk copies
     cta_barrier();
+    if (c.CL == 1) return;
     if (!c.strict) cluster_wait();
-    const uint32_t gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints), bar = c.bars + 8u * (l & 1);
-    const uint32_t an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
-    if (lane == 0)
+    const uint32_t bar = c.bars + 8u * (l & 1);
+    if (warp == c.NW) {
+        const uint32_t gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints), an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // plain stores of the state, read next by bulk copies
         for (int d = c.rank + 1, low = c.W - c.H; d < c.CL && low < c.W; ++d, low += c.W) {
             // CTA d holds the columns from d*W - H on: this CTA's local columns from `low` on
             const int from = max(low, 0), n = c.W - from, delta = c.cdelta[d];
             const int at = c.H + from, to = at - (d - c.rank) * c.W;
-            for (int k = warp; k < c.Kc; k += c.NW + 1) {
+            for (int k = lane; k < c.Kc; k += 32) {
                 bulk_to_cta(gn + (uint32_t)(delta + (k * c.P + to) * 4), gn + (uint32_t)(k * c.P + at) * 4u, (uint32_t)n * 4u, bar + (uint32_t)delta);
                 if (ARG) bulk_to_cta(an + (uint32_t)(delta + k * c.P + to), an + (uint32_t)(k * c.P + at), (uint32_t)n, bar + (uint32_t)delta);
             }
         }
+    }
     if (c.halo_bytes) {
         if (warp == c.NW && lane == 0) mbar_expect(bar, c.halo_bytes);
         const uint32_t parity = (uint32_t)(l >> 1) & 1u;
@@ -189,8 +195,8 @@ __device__ __forceinline__ void end_layer(const Ctx& c, int l, int warp, int lan
         while (!mbar_try(bar, parity))
             if (++polls > kWaitPolls || *(volatile int*)c.late) { *(volatile int*)c.late = 1; break; }
     }
-    cluster_arrive();
-    if (c.strict) cluster_wait();
+    if (c.strict) { cluster_arrive(); cluster_wait(); }
+    else cluster_arrive_relaxed();
 }
 
 // Record of (layer, strategy): x = byte offset, from the start of the state, of the cell column 0 of this CTA reads
