@@ -143,12 +143,14 @@ struct Ctx {
     int S, M, W, H, P, G, CL, rank, Li, m_pitch, Kr, Kc, tmax, SP, NW, gints;
     int32_t* g0;               // [2][gints] state of this layer / the next: rows of P = H + W columns
     uint8_t* a0;               // [2][gints] its argmin (argmin table only)
-    const int4* rec;           // [3][S] ring of per-layer records, strategies in class order
+    uint32_t rec;              // address of the ring of per-layer records: three slots of RB bytes
+    int S2;                    // record entries a slot
+    int n_all;                 // strategies of a slot's records, pads included
     const int* front;          // [3] no column below it holds a finite value in this layer
     const int* reach;          // [3] the layer's largest shift
     const int32_t* tsm;        // transition entries: [16][16] by class, or [S][SP] (two of them with one matrix per layer)
     int tmat;                  // entries of one full matrix when there is one per layer, else 0
-    const int* cs;             // [Kr + 1] first record of each class
+    const int* cs;             // [3][kClassMax + 1] first record of each class
     const int* cdelta;         // [16] cluster-window address of CTA d minus this CTA's own shared address
     int32_t* C;                // this instance's table
     uint8_t* A;
@@ -199,10 +201,13 @@ __device__ __forceinline__ void end_layer(const Ctx& c, int l, int warp, int lan
     else cluster_arrive_relaxed();
 }
 
-// Record of (layer, strategy): x = byte offset, from the start of the state, of the cell column 0 of this CTA reads
-// (the row of the strategy's column class, shifted by mem); y = time (kInf: mem exceeds the budget, the row is +inf);
-// z = mem | strategy << 24; w = byte offset of the strategy's row in the table.
-//
+// Records of a layer, one entry per strategy in class order, three arrays of S2 entries each (a slot of the ring):
+//   int2 (x, time)  x = byte offset, from the start of the state, of the cell that column 0 of this CTA reads (the row of
+//                   the strategy's column class, shifted by mem); time = kInf where mem exceeds the budget (+inf row)
+//   int  row        byte offset of the strategy's row in the table
+//   int  who        mem | strategy << 24
+// A class has an even number of entries (the last one may stand twice: it stores the same values again, and a minimum
+// does not change), so entries are read two to a 128-bit load, and four at a time from one address.
 // Shared-memory accesses of the layer loop go through 32-bit addresses and are written in batches, loads first: the table
 // stores between two strategies would otherwise hold the next strategy's loads back (they could alias for all the
 // compiler knows), and a strategy would cost the latency of its whole chain (220 cycles) instead of a share of it.
@@ -230,19 +235,28 @@ __device__ __forceinline__ int4 lds4(uint32_t a) {
 __device__ __forceinline__ void sts(uint32_t a, int v) { asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ void sts_u8(uint32_t a, int v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 
+template <int OFF>
+__device__ __forceinline__ int4 lds4_at(uint32_t a) {
+    int4 v;
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4+%5];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a), "n"(OFF));
+    return v;
+}
+template <int TM, int J = 0>
+__device__ __forceinline__ void lds_row(uint32_t a, int (&g)[TM]) {
+    g[J] = lds_at<128 * J>(a);
+    if constexpr (J + 1 < TM) lds_row<TM, J + 1>(a, g);
+}
+
 // G at the columns that column `col` of this CTA (and those 32, 64, ... after it) reads; ga: the state's address plus
 // 4 * col.  FAR: the layer has shifts beyond the halo, whose cells are read from the CTA that owns them.
 template <int TM, bool FAR>
-__device__ __forceinline__ void gather(const Ctx& c, uint32_t ga, const int4 r, int col, int (&g)[TM])
+__device__ __forceinline__ void gather(const Ctx& c, uint32_t ga, int x, int who, int col, int (&g)[TM])
 {
-    const int mem = r.z & 0xffffff;
+    const int mem = who & 0xffffff;
     if (!FAR || mem <= c.H) {
-        const uint32_t a = ga + (uint32_t)r.x;
-        g[0] = lds(a);
-        if (TM > 1) g[1 % TM] = lds_at<128>(a);
-        if (TM > 2) { g[2 % TM] = lds_at<256>(a); g[3 % TM] = lds_at<384>(a); }
+        lds_row<TM>(ga + (uint32_t)x, g);
     } else {
-        const uint32_t row = ga - 4u * (uint32_t)col + (uint32_t)r.x + (uint32_t)mem * 4u;
+        const uint32_t row = ga - 4u * (uint32_t)col + (uint32_t)x + (uint32_t)mem * 4u;
 #pragma unroll
         for (int j = 0; j < TM; ++j) {
             const int src = c.rank * c.W + col + 32 * j - mem;
@@ -254,9 +268,9 @@ __device__ __forceinline__ void gather(const Ctx& c, uint32_t ga, const int4 r, 
 }
 // ... and their argmin entries; aa: the argmin state's address plus col
 template <int TM, bool FAR>
-__device__ __forceinline__ void gather_arg(const Ctx& c, uint32_t aa, const int4 r, int col, int (&a)[TM])
+__device__ __forceinline__ void gather_arg(const Ctx& c, uint32_t aa, int x, int who, int col, int (&a)[TM])
 {
-    const int mem = r.z & 0xffffff, off = r.x >> 2;
+    const int mem = who & 0xffffff, off = x >> 2;
     if (!FAR || mem <= c.H) {
 #pragma unroll
         for (int j = 0; j < TM; ++j) a[j] = lds_u8(aa + (uint32_t)(off + 32 * j));
@@ -293,10 +307,10 @@ struct Out {
     int cols;              // columns of the tile that exist in the table, less this lane
     int budget;            // ... that are budget columns, less this lane
     template <int TM>
-    __device__ __forceinline__ void put(const int4 r, const int (&v)[TM], const int (&a)[TM]) const
+    __device__ __forceinline__ void put(uint32_t row, const int (&v)[TM], const int (&a)[TM]) const
     {
         if (STORE) {
-            int32_t* const p = reinterpret_cast<int32_t*>(C + (uint32_t)r.w);
+            int32_t* const p = reinterpret_cast<int32_t*>(C + row);
             if (whole) {
 #pragma unroll
                 for (int j = 0; j < TM; ++j) p[32 * j] = v[j];
@@ -307,7 +321,7 @@ struct Out {
             }
         }
         if (ARG) {
-            uint8_t* const p = A + ((uint32_t)r.w >> 2);
+            uint8_t* const p = A + (row >> 2);
 #pragma unroll
             for (int j = 0; j < TM; ++j)
                 if (whole || 32 * j < cols) p[32 * j] = (uint8_t)((whole || 32 * j < budget) && v[j] < kInf ? a[j] : 255);
@@ -315,51 +329,80 @@ struct Out {
     }
 };
 
-// U strategies, from record address ra on: their C values to the table, their smallest into h (with ARG: whose it is).
-template <int U, int TM, bool STORE, bool ARG, bool FAR>
-__device__ __forceinline__ void scan(const Ctx& c, const Out<STORE, ARG>& out, uint32_t ra, uint32_t ga, uint32_t aa, int col, int (&h)[TM], int (&hs)[TM])
+// U entries' records, from entry address ra (of the (x, time) array) on.
+template <int U>
+struct Recs { int x[U], t[U], row[U], who[U]; };
+template <int U, bool ROW, bool WHO>
+__device__ __forceinline__ void fetch_recs(const Ctx& c, uint32_t ra, uint32_t rowa, Recs<U>& r)
 {
-    int4 r[U];
-    int v[U][TM], a[ARG ? U : 1][TM];
+    if constexpr (U >= 2) {
+        const int4 p = lds4_at<0>(ra);
+        r.x[0] = p.x; r.t[0] = p.y; r.x[1] = p.z; r.t[1] = p.w;
+        if constexpr (U == 4) {
+            const int4 q = lds4_at<16>(ra);
+            r.x[2 % U] = q.x; r.t[2 % U] = q.y; r.x[3 % U] = q.z; r.t[3 % U] = q.w;
+        }
+    } else {
+        r.x[0] = lds_at<0>(ra); r.t[0] = lds_at<4>(ra);
+    }
 #pragma unroll
-    for (int u = 0; u < U; ++u) r[u] = lds4(ra + 16u * u);
+    for (int u = 0; u < U; ++u) { r.row[u] = 0; r.who[u] = 0; }
+    if (ROW) {
+        r.row[0] = lds_at<0>(rowa);
+        if constexpr (U >= 2) r.row[1 % U] = lds_at<4>(rowa);
+        if constexpr (U == 4) { r.row[2 % U] = lds_at<8>(rowa); r.row[3 % U] = lds_at<12>(rowa); }
+    }
+    if (WHO) {
+        const uint32_t w = rowa + 4u * c.S2;
+        r.who[0] = lds_at<0>(w);
+        if constexpr (U >= 2) r.who[1 % U] = lds_at<4>(w);
+        if constexpr (U == 4) { r.who[2 % U] = lds_at<8>(w); r.who[3 % U] = lds_at<12>(w); }
+    }
+}
+
+// U strategies: their C values to the table, their smallest into h (with ARG: whose it is).
+template <int U, int TM, bool STORE, bool ARG, bool FAR>
+__device__ __forceinline__ void scan(const Ctx& c, const Out<STORE, ARG>& out, uint32_t ra, uint32_t rowa, uint32_t ga, uint32_t aa, int col, int (&h)[TM], int (&hs)[TM])
+{
+    Recs<U> r;
+    int v[U][TM], a[ARG ? U : 1][TM];
+    fetch_recs<U, STORE || ARG, ARG || FAR>(c, ra, rowa, r);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        gather<TM, FAR>(c, ga, r[u], col, v[u]);
-        if (ARG) gather_arg<TM, FAR>(c, aa, r[u], col, a[ARG ? u : 0]);
+        gather<TM, FAR>(c, ga, r.x[u], r.who[u], col, v[u]);
+        if (ARG) gather_arg<TM, FAR>(c, aa, r.x[u], r.who[u], col, a[ARG ? u : 0]);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
 #pragma unroll
         for (int j = 0; j < TM; ++j) {
             if (STORE || ARG) {
-                v[u][j] = __viaddmin_s32(v[u][j], r[u].y, kInf);
-                if (ARG) hs[j] = v[u][j] < h[j] ? r[u].z >> 24 : hs[j];    // ascending strategies: the lowest keeps a tie
+                v[u][j] = __viaddmin_s32(v[u][j], r.t[u], kInf);
+                if (ARG) hs[j] = v[u][j] < h[j] ? r.who[u] >> 24 : hs[j];  // ascending strategies: the lowest keeps a tie
                 h[j] = min(h[j], v[u][j]);
             } else {
-                h[j] = __viaddmin_s32(v[u][j], r[u].y, h[j]);
+                h[j] = __viaddmin_s32(v[u][j], r.t[u], h[j]);
             }
         }
-        if (STORE || ARG) out.template put<TM>(r[u], v[u], a[ARG ? u : 0]);
+        if (STORE || ARG) out.template put<TM>((uint32_t)r.row[u], v[u], a[ARG ? u : 0]);
     }
 }
 
 // Which of U strategies are alive in some column of the tile, as bits.
 template <int U, int TM, bool FAR>
-__device__ __forceinline__ uint32_t alive(const Ctx& c, uint32_t ra, uint32_t ga, int col, const int (&thr)[TM])
+__device__ __forceinline__ uint32_t alive(const Ctx& c, uint32_t ra, uint32_t rowa, uint32_t ga, int col, const int (&thr)[TM])
 {
-    int4 r[U];
+    Recs<U> r;
     int v[U][TM];
     uint32_t bits = 0;
+    fetch_recs<U, false, FAR>(c, ra, rowa, r);
 #pragma unroll
-    for (int u = 0; u < U; ++u) r[u] = lds4(ra + 16u * u);
-#pragma unroll
-    for (int u = 0; u < U; ++u) gather<TM, FAR>(c, ga, r[u], col, v[u]);
+    for (int u = 0; u < U; ++u) gather<TM, FAR>(c, ga, r.x[u], r.who[u], col, v[u]);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         bool live = false;
 #pragma unroll
-        for (int j = 0; j < TM; ++j) live = live || __viaddmin_s32(v[u][j], r[u].y, kInf) <= thr[j];
+        for (int j = 0; j < TM; ++j) live = live || __viaddmin_s32(v[u][j], r.t[u], kInf) <= thr[j];
         if (__any_sync(0xffffffffu, live)) bits |= 1u << u;
     }
     return bits;
@@ -370,7 +413,7 @@ template <int KC, int TM, bool PRUNE, bool STORE, bool ARG, bool FAR>
 __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
 {
     const int slot = l % 3, col = colb + lane;
-    const uint32_t ra = smem_addr(c.rec + slot * c.S);
+    const uint32_t ra = c.rec + (uint32_t)(slot * c.S2) * 16u, rowa = ra + (uint32_t)c.S2 * 8u;
     const uint32_t ga = smem_addr(c.g0 + (l & 1) * c.gints + col), gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints);
     const uint32_t aa = ARG ? smem_addr(c.a0 + (l & 1) * c.gints + col) : 0u, an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
     const int colg = c.rank * c.W + colb;                      // the tile's first budget column
@@ -387,7 +430,7 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
         for (int j = 0; j < TM; ++j) { inf[j] = kInf; none[j] = 255; }
         if (STORE || ARG)
 #pragma unroll 4
-            for (int e = 0; e < c.S; ++e) out.template put<TM>(make_int4(0, 0, 0, e * c.m_pitch * 4), inf, none);
+            for (int e = 0; e < c.S; ++e) out.template put<TM>((uint32_t)(e * c.m_pitch) * 4u, inf, none);
         for (int k = 0; k < c.Kc; ++k) emit<TM, ARG>(c, gn, an, k, colb, lane, inf, none);
         return;
     }
@@ -399,22 +442,19 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
 #pragma unroll
             for (int j = 0; j < TM; ++j) { acc[k][j] = kInf; if (ARG) arg[k][j] = 255; }
         int e = 0;
+        const int* const cs = c.cs + slot * (kClassMax + 1);
         const uint32_t ta = smem_addr(c.tsm);
         for (int k = 0; k < c.Kr; ++k) {
-            const int end = c.cs[k + 1];
+            const int end = cs[k + 1];
             int h[TM], hs[TM];
 #pragma unroll
             for (int j = 0; j < TM; ++j) { h[j] = kInf; hs[j] = 255; }
             int4 t4[KC / 4];
 #pragma unroll
             for (int q = 0; q < KC / 4; ++q) t4[q] = lds4(ta + (uint32_t)(k * kClassMax + 4 * q) * 4u);
-            if (!FAR) {
-                for (; e + 4 <= end; e += 4) scan<4, TM, STORE, ARG, FAR>(c, out, ra + 16u * e, ga, aa, col, h, hs);
-                if (e + 2 <= end) { scan<2, TM, STORE, ARG, FAR>(c, out, ra + 16u * e, ga, aa, col, h, hs); e += 2; }
-                if (e < end) { scan<1, TM, STORE, ARG, FAR>(c, out, ra + 16u * e, ga, aa, col, h, hs); ++e; }
-            } else {
-                for (; e < end; ++e) scan<1, TM, STORE, ARG, FAR>(c, out, ra + 16u * e, ga, aa, col, h, hs);
-            }
+            constexpr int U = FAR ? 1 : TM > 3 ? 2 : 4;
+            for (; e + U <= end; e += U) scan<U, TM, STORE, ARG, FAR>(c, out, ra + 8u * e, rowa + 4u * e, ga, aa, col, h, hs);
+            if (U == 4 && e < end) { scan<2, TM, STORE, ARG, FAR>(c, out, ra + 8u * e, rowa + 4u * e, ga, aa, col, h, hs); e += 2; }
 #pragma unroll
             for (int q = 0; q < KC / 4; ++q) {
                 const int t[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
@@ -441,8 +481,8 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
         for (int j = 0; j < TM; ++j) { thr[j] = kInf; dummy[j] = 255; }
         int s = 0;
         if (!FAR)
-            for (; s + 4 <= c.S; s += 4) scan<4, TM, STORE, ARG, FAR>(c, out, ra + 16u * s, ga, aa, col, thr, dummy);
-        for (; s < c.S; ++s) scan<1, TM, STORE, ARG, FAR>(c, out, ra + 16u * s, ga, aa, col, thr, dummy);
+            for (; s + 4 <= c.S; s += 4) scan<4, TM, STORE, ARG, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
+        for (; s < c.S; ++s) scan<1, TM, STORE, ARG, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
         // a candidate beyond the column's best plus the largest entry cannot win; a column without a finite value
         // keeps nothing alive
 #pragma unroll
@@ -455,8 +495,8 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
                 const int n = min(32, c.S - 32 * b);
                 int q = 0;
                 if (!FAR)
-                    for (; q + 4 <= n; q += 4) live[b] |= alive<4, TM, FAR>(c, ra + 16u * (32 * b + q), ga, col, thr) << q;
-                for (; q < n; ++q) live[b] |= alive<1, TM, FAR>(c, ra + 16u * (32 * b + q), ga, col, thr) << q;
+                    for (; q + 4 <= n; q += 4) live[b] |= alive<4, TM, FAR>(c, ra + 8u * (32 * b + q), rowa + 4u * (32 * b + q), ga, col, thr) << q;
+                for (; q < n; ++q) live[b] |= alive<1, TM, FAR>(c, ra + 8u * (32 * b + q), rowa + 4u * (32 * b + q), ga, col, thr) << q;
             }
         }
         const uint32_t ta = smem_addr(c.tsm + (((l + 1) & 1) ? c.tmat : 0));
@@ -470,12 +510,13 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
             for (int b = 0; b < kMaxS / 32; ++b)
                 for (uint32_t m = live[b]; m; m &= m - 1) {
                     const int q = 32 * b + __ffs(m) - 1;
-                    const int4 r = lds4(ra + 16u * q);
+                    Recs<1> r;
+                    fetch_recs<1, false, FAR>(c, ra + 8u * q, rowa + 4u * q, r);
                     const uint32_t t0 = ta + (uint32_t)(q * c.SP + cb) * 4u;
                     int v[TM];
-                    gather<TM, FAR>(c, ga, r, col, v);
+                    gather<TM, FAR>(c, ga, r.x[0], r.who[0], col, v);
 #pragma unroll
-                    for (int j = 0; j < TM; ++j) v[j] = __viaddmin_s32(v[j], r.y, kInf);
+                    for (int j = 0; j < TM; ++j) v[j] = __viaddmin_s32(v[j], r.t[0], kInf);
 #pragma unroll
                     for (int w = 0; w < KC / 4; ++w) {
                         const int4 t4 = lds4(t0 + 16u * w);
@@ -505,26 +546,25 @@ template <bool STORE, bool ARG, bool FAR>
 __device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lane)
 {
     const int slot = l % 3, col = colb + lane;
-    const uint32_t ra = smem_addr(c.rec + slot * c.S), ga = smem_addr(c.g0 + (l & 1) * c.gints + col);
+    const uint32_t ra = c.rec + (uint32_t)(slot * c.S2) * 16u, rowa = ra + (uint32_t)c.S2 * 8u, ga = smem_addr(c.g0 + (l & 1) * c.gints + col);
     const uint32_t aa = ARG ? smem_addr(c.a0 + (l & 1) * c.gints + col) : 0u;
     const int colg = c.rank * c.W + colb, m = colg + lane;
     if (colg >= c.m_pitch) return;                             // m_pitch is a multiple of 32: a group exists whole or not at all
     const bool pad = m > c.M;
     auto steps = [&](auto count, int e) {
         constexpr int U = decltype(count)::value;
-        int4 r[U];
+        Recs<U> r;
         int g[U][1], a[U][1];
-#pragma unroll
-        for (int u = 0; u < U; ++u) r[u] = lds4(ra + 16u * (e + u));
+        fetch_recs<U, true, ARG || FAR>(c, ra + 8u * e, rowa + 4u * e, r);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            gather<1, FAR>(c, ga, r[u], col, g[u]);
-            if (ARG) gather_arg<1, FAR>(c, aa, r[u], col, a[u]);
+            gather<1, FAR>(c, ga, r.x[u], r.who[u], col, g[u]);
+            if (ARG) gather_arg<1, FAR>(c, aa, r.x[u], r.who[u], col, a[u]);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int v = pad ? kInf : __viaddmin_s32(g[u][0], r[u].y, kInf);
-            const size_t row = ((uint32_t)r[u].w >> 2) + (size_t)m;
+            const int v = pad ? kInf : __viaddmin_s32(g[u][0], r.t[u], kInf);
+            const size_t row = ((uint32_t)r.row[u] >> 2) + (size_t)m;
             if (STORE) c.C[(size_t)l * c.slice + row] = v;
             c.C_last[row] = v;
             if (ARG) c.A[(size_t)l * c.slice + row] = (uint8_t)(v < kInf ? a[u][0] : 255);
@@ -532,23 +572,34 @@ __device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lan
     };
     int e = 0;
     if (!FAR)
-        for (; e + 4 <= c.S; e += 4) steps(std::integral_constant<int, 4>(), e);
-    for (; e < c.S; ++e) steps(std::integral_constant<int, 1>(), e);
+        for (; e + 4 <= c.n_all; e += 4) steps(std::integral_constant<int, 4>(), e);
+    for (; e < c.n_all; ++e) steps(std::integral_constant<int, 1>(), e);
 }
 
-// A warp owns a run of column groups, the warps' runs differ by one group at most, and takes them TM at a time, then
-// one at a time.
-template <int KC, int TM, bool PRUNE, bool STORE, bool ARG>
+// `n` column groups from group g on, as one tile.
+template <int KC, int MAX, bool PRUNE, bool STORE, bool ARG>
+__device__ __forceinline__ void tile_of(const Ctx& c, int l, int g, int n, int lane)
+{
+    if constexpr (MAX > 1) {
+        if (n < MAX) { tile_of<KC, MAX - 1, PRUNE, STORE, ARG>(c, l, g, n, lane); return; }
+    }
+    tile<KC, MAX, PRUNE, STORE, ARG, false>(c, l, g * 32, lane);
+}
+
+// A warp owns a run of column groups (the warps' runs differ by one group at most) and takes it as one tile, or as
+// several of about the same width when it is wider than MAX groups: a record fetched once serves them all.
+template <int KC, int MAX, bool PRUNE, bool STORE, bool ARG>
 __device__ __forceinline__ void run_layers(const Ctx& c, int warp, int lane)
 {
     const int g0 = c.G * warp / c.NW, g1 = c.G * (warp + 1) / c.NW;
     for (int l = 0; l + 1 < c.Li; ++l) {
         int g = g0;
         if (c.reach[l % 3] <= c.H) {
-            if (TM > 1)
-                for (; g + TM <= g1; g += TM) tile<KC, TM, PRUNE, STORE, ARG, false>(c, l, g * 32, lane);
-            if (TM > 2 && g + 2 <= g1) { tile<KC, 2, PRUNE, STORE, ARG, false>(c, l, g * 32, lane); g += 2; }
-            for (; g < g1; ++g) tile<KC, 1, PRUNE, STORE, ARG, false>(c, l, g * 32, lane);
+            for (int left = (g1 - g0 + MAX - 1) / MAX; left > 0; --left) {
+                const int n = (g1 - g + left - 1) / left;
+                tile_of<KC, MAX, PRUNE, STORE, ARG>(c, l, g, n, lane);
+                g += n;
+            }
         } else {
             for (; g < g1; ++g) tile<KC, 1, PRUNE, STORE, ARG, true>(c, l, g * 32, lane);
         }
@@ -568,7 +619,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ union { int L[kMaxSortedB]; struct { uint32_t rh[kMaxS], ch[kMaxS]; } h; } s_u;
-    __shared__ int s_rrep[kMaxS], s_crep[kMaxS], s_rcls[kMaxS], s_ccls[kMaxS], s_order[kMaxS], s_cs[kMaxS + 1];
+    __shared__ int s_rrep[kMaxS], s_crep[kMaxS], s_rcls[kMaxS], s_ccls[kMaxS], s_order[kMaxS + kClassMax], s_cs[3 * (kClassMax + 1)], s_first[kClassMax + 1];
     __shared__ int s_cdelta[16], s_front[3], s_reach[3], s_inst, s_K[2];
     __shared__ struct { long long sum; int tmax, bad, mmax; } s_part, s_all;
     __shared__ __align__(8) unsigned long long s_bar[2];
@@ -583,9 +634,10 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     const int tfull = S * a.SP;
     int32_t* const tsm = g0 + 2 * gints;                                                   // [16][16] or [1|2][S][SP]
     const int tints = max(kClassMax * kClassMax, (a.trans_layer ? 2 : 1) * tfull);
-    int4* const rec = reinterpret_cast<int4*>(tsm + tints);                                // [3][S]
-    int32_t* const raw = reinterpret_cast<int32_t*>(rec + 3 * S);                          // [4][2][S] mem, time rows as they come
-    uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * S);                           // [2][gints] argmin of the state
+    const int S2 = (S + kClassMax + 3) & ~3;
+    int32_t* const rec = tsm + tints;                                                      // [3] slots of S2 x (int2, int, int)
+    int32_t* const raw = rec + 3 * 4 * S2;                                                 // [4][2][S] mem, time rows as they come
+    uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * ((S + 3) & ~3));                           // [2][gints] argmin of the state
 
     if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = a.path_value; }
 
@@ -764,17 +816,29 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     const bool dense = !classes && a.SP > 0 && S * W <= gints;
     const int Kr = classes ? s_K[0] : S, Kc = classes ? s_K[1] : S;
     if (classes) {
-        // strategies in class order, ascending inside a class
+        // strategies in class order, ascending inside a class; a class of an odd number has its last one twice
+        for (int k = tid; k <= Kr; k += NT) s_first[k] = 0;
+        __syncthreads();
+        for (int s = tid; s < S; s += NT) atomicAdd(&s_first[s_rcls[s]], 1);
+        __syncthreads();
+        if (warp == 0) {
+            const int n = lane < Kr ? s_first[lane] : 0;
+            int at = (n + 1) & ~1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, at, o);
+                if (lane >= o) at += v;
+            }
+            if (lane < Kr) s_first[lane] = at - ((n + 1) & ~1);
+            if (lane == Kr - 1) s_first[Kr] = at;
+        }
+        __syncthreads();
         for (int s = tid; s < S; s += NT) {
             const int me = s_rcls[s];
-            int pos = 0;
-            for (int o = 0; o < S; ++o) pos += s_rcls[o] < me || (s_rcls[o] == me && o < s);
-            s_order[pos] = s;
-        }
-        for (int k = tid; k <= Kr; k += NT) {
-            int n = 0;
-            for (int o = 0; o < S; ++o) n += s_rcls[o] < k;
-            s_cs[k] = n;
+            int before = 0, size = 0;
+            for (int o = 0; o < S; ++o) { size += s_rcls[o] == me; before += s_rcls[o] == me && o < s; }
+            s_order[s_first[me] + before] = s;
+            if (before == size - 1 && (size & 1)) s_order[s_first[me] + size] = s;
         }
         for (int x = tid; x < kClassMax * kClassMax; x += NT) tsm[x] = 0;
         __syncthreads();
@@ -784,7 +848,6 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                     if (s_crep[s] == s) tsm[s_rcls[r] * kClassMax + s_ccls[s]] = stage[r * S + s];
     } else if (dense) {
         for (int s = tid; s < S; s += NT) { s_order[s] = s; s_ccls[s] = s; }
-        for (int k = tid; k <= S; k += NT) s_cs[k] = k;
         // the matrix paid between layers 0 and 1; with one matrix per layer, matrix l sits in buffer l & 1
         const int32_t* const T = T0 + (a.trans_layer ? a.trans_layer : 0);
         int32_t* const dst = tsm + (a.trans_layer ? tfull : 0);
@@ -806,20 +869,25 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     // a multiple of 32.  Below column 0 it holds +inf.
     const int H = max(0, min((s_all.mmax + 31) & ~31, (gints / Kc - W) & ~31)), P = W + H;
 
+    const int n_all = classes ? s_first[Kr] : S;
     // ---- layer 0 gathers from an all-zero state: C[0] = time where mem fits
     auto prepare = [&](int l, int base) -> int {                // records of layer l by one warp; returns the new frontier
         const int slot = l % 3;
         const int32_t* const rm = raw + (l & 3) * 2 * S;
+        int32_t* const rs = rec + slot * 4 * S2;
         int least = M + 1, most = 0;
-        for (int e = lane; e < S; e += 32) {
+        for (int e = lane; e < n_all; e += 32) {
             const int s = s_order[e];
             const int mem = rm[s];
             const bool fits = mem <= M;                         // else +inf everywhere: no shift, time +inf
             const int shift = fits ? mem : 0;
-            rec[slot * S + e] = make_int4((s_ccls[s] * P + H - shift) * 4, fits ? rm[S + s] : kInf, shift | (s << 24), s * a.m_pitch * 4);
+            reinterpret_cast<int2*>(rs)[e] = make_int2((s_ccls[s] * P + H - shift) * 4, fits ? rm[S + s] : kInf);
+            rs[2 * S2 + e] = s * a.m_pitch * 4;
+            rs[3 * S2 + e] = shift | (s << 24);
             least = min(least, mem);
             most = max(most, shift);
         }
+        if (classes && lane <= Kr) s_cs[slot * (kClassMax + 1) + lane] = s_first[lane];
         least = __reduce_min_sync(0xffffffffu, least);
         most = __reduce_max_sync(0xffffffffu, most);
         const int f = min(base + least, M + 1);
@@ -864,7 +932,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     Ctx c;
     c.S = S; c.M = M; c.W = W; c.H = H; c.P = P; c.G = W / 32; c.CL = CL; c.rank = rank; c.Li = Li; c.m_pitch = a.m_pitch; c.Kr = Kr; c.Kc = Kc;
     c.tmax = s_all.tmax; c.SP = a.SP; c.NW = NW; c.gints = gints;
-    c.g0 = g0; c.a0 = a0; c.rec = rec; c.front = s_front; c.reach = s_reach; c.tsm = tsm; c.tmat = a.trans_layer ? tfull : 0;
+    c.g0 = g0; c.a0 = a0; c.rec = smem_addr(rec); c.S2 = S2; c.n_all = n_all; c.front = s_front; c.reach = s_reach; c.tsm = tsm; c.tmat = a.trans_layer ? tfull : 0;
     c.cs = s_cs; c.cdelta = s_cdelta;
     c.slice = (size_t)S * a.m_pitch;
     c.C = STORE ? a.C + (size_t)i * Lmax * c.slice : nullptr;
@@ -898,24 +966,12 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
             end_layer<ARG>(c, l, warp, lane);
         }
     } else {
-        // columns per lane: a record fetched once serves up to four groups of 32
-        const int per = (c.G + NW - 1) / NW;
         if (classes) {
-            if (K <= 4) {
-                if (per >= 4 && !ARG) run_layers<4, ARG ? 1 : 4, false, STORE, ARG>(c, warp, lane);
-                else if (per >= 2) run_layers<4, 2, false, STORE, ARG>(c, warp, lane);
-                else run_layers<4, 1, false, STORE, ARG>(c, warp, lane);
-            } else if (K <= 8) {
-                if (per >= 4 && !ARG) run_layers<8, ARG ? 1 : 4, false, STORE, ARG>(c, warp, lane);
-                else if (per >= 2) run_layers<8, 2, false, STORE, ARG>(c, warp, lane);
-                else run_layers<8, 1, false, STORE, ARG>(c, warp, lane);
-            } else {
-                if (per >= 2) run_layers<16, 2, false, STORE, ARG>(c, warp, lane);
-                else run_layers<16, 1, false, STORE, ARG>(c, warp, lane);
-            }
+            if (K <= 4) run_layers<4, ARG ? 2 : 6, false, STORE, ARG>(c, warp, lane);
+            else if (K <= 8) run_layers<8, ARG ? 2 : 6, false, STORE, ARG>(c, warp, lane);
+            else run_layers<16, ARG ? 1 : 3, false, STORE, ARG>(c, warp, lane);
         } else {
-            if (per >= 2 && !ARG) run_layers<32, ARG ? 1 : 2, true, STORE, ARG>(c, warp, lane);
-            else run_layers<32, 1, true, STORE, ARG>(c, warp, lane);
+            run_layers<32, ARG ? 1 : 2, true, STORE, ARG>(c, warp, lane);
         }
     }
     if (CL > 1) {
@@ -977,7 +1033,7 @@ long long fixed_smem(const galv_shape* sh, bool dense)
 {
     const int S = sh->S, SP = (S + 3) & ~3;
     const long long t = dense ? (long long)S * SP * ((sh->flags & GALV_TRANS_PER_LAYER) ? 2 : 1) : 0;
-    return (t > kClassMax * kClassMax ? t : kClassMax * kClassMax) * 4 + (long long)3 * S * 16 + (long long)8 * S * 4 + 128;
+    return (t > kClassMax * kClassMax ? t : kClassMax * kClassMax) * 4 + (long long)3 * 16 * ((S + kClassMax + 3) & ~3) + (long long)8 * SP * 4 + 128;
 }
 
 // The best cluster size for a state of `rows` rows at least; false when none fits.
