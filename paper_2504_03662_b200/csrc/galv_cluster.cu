@@ -29,6 +29,8 @@
 // launch's shared memory is left alone and marked in done[]; a second launch with larger clusters or the tiled kernels
 // take it.
 
+#include <cuda.h>
+
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -50,6 +52,7 @@ struct RsArgs {
     int CL;            // CTAs per cluster
     int W;             // budget columns per CTA (multiple of 32)
     int gints;         // words of one state buffer: rows of W columns and their halo
+    int stage_at;      // word offset of the collected rows
     int SP;            // row pitch of the full transition matrix in shared memory; 0: no room for unstructured matrices
     int sorted;        // clusters take the instances longest first
     int second;        // only the instances the first launch left alone
@@ -110,6 +113,15 @@ __device__ __forceinline__ void whole_barrier(int CL) {
     if (CL == 1) cta_barrier();
     else { cluster_arrive(); cluster_wait(); }
 }
+// One box [S][W / 32][32] from shared memory to element coordinates (0, g0, row0) of the table behind `map`, seen as
+// [rows][m_pitch / 32][32]; what lies beyond the tensor's edge (the last CTA's columns past m_pitch) is not written.
+__device__ __forceinline__ void tensor_store_3d(const CUtensorMap* map, const void* src, int g0, int row0) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                 ::"l"(map), "r"(0), "r"(g0), "r"(row0), "r"(smem_addr(src)) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // bytes of this CTA's shared memory to the same cluster's CTA that `dst` and `bar` lie in; counted on its mbarrier
 __device__ __forceinline__ void bulk_to_cta(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -143,15 +155,18 @@ struct Ctx {
     int S, M, W, H, P, G, CL, rank, Li, m_pitch, Kr, Kc, tmax, SP, NW, gints;
     int32_t* g0;               // [2][gints] state of this layer / the next: rows of P = H + W columns
     uint8_t* a0;               // [2][gints] its argmin (argmin table only)
-    uint32_t rec;              // address of the ring of per-layer records: three slots of RB bytes
+    uint32_t rec;              // address of the per-layer records: four slots of 24 * S2 bytes
+    const int* slot;           // [4] the slot of layer l is slot[l & 3] (layers with the same rows share one)
     int S2;                    // record entries a slot
     int n_all;                 // strategies of a slot's records, pads included
-    const int* front;          // [3] no column below it holds a finite value in this layer
-    const int* reach;          // [3] the layer's largest shift
+    const int* front;          // [4] no column below front[l & 3] holds a finite value in layer l
+    const int* reach;          // [4] largest shift of a slot's layer
     const int32_t* tsm;        // transition entries: [16][16] by class, or [S][SP] (two of them with one matrix per layer)
     int tmat;                  // entries of one full matrix when there is one per layer, else 0
-    const int* cs;             // [3][kClassMax + 1] first record of each class
+    const int* cs;             // [kClassMax + 1] first record of each class
+    const int* csp;            // [4][kClassMax + 1] the same in the list of the records that can matter
     const int* cdelta;         // [16] cluster-window address of CTA d minus this CTA's own shared address
+    int32_t* stage;            // [2][S][W] collected rows
     int32_t* C;                // this instance's table
     uint8_t* A;
     int32_t* C_last;
@@ -171,7 +186,7 @@ struct Ctx {
 // With shifts beyond the halo other CTAs' state is read as well, and the barrier is waited for at once.
 constexpr int kWaitPolls = 1 << 20;                            // try_wait sleeps in hardware between polls: about a second
 template <bool ARG>
-__device__ __forceinline__ void end_layer(const Ctx& c, int l, int warp, int lane)
+__device__ __forceinline__ void send_halo(const Ctx& c, int l, int warp, int lane)
 {
     cta_barrier();
     if (c.CL == 1) return;
@@ -190,6 +205,12 @@ __device__ __forceinline__ void end_layer(const Ctx& c, int l, int warp, int lan
             }
         }
     }
+}
+template <bool ARG>
+__device__ __forceinline__ void await_halo(const Ctx& c, int l, int warp, int lane)
+{
+    if (c.CL == 1) return;
+    const uint32_t bar = c.bars + 8u * (l & 1);
     if (c.halo_bytes) {
         if (warp == c.NW && lane == 0) mbar_expect(bar, c.halo_bytes);
         const uint32_t parity = (uint32_t)(l >> 1) & 1u;
@@ -206,6 +227,9 @@ __device__ __forceinline__ void end_layer(const Ctx& c, int l, int warp, int lan
 //                   the strategy's column class, shifted by mem); time = kInf where mem exceeds the budget (+inf row)
 //   int  row        byte offset of the strategy's row in the table
 //   int  who        mem | strategy << 24
+//   int2 (x, time)  of the strategies that can be the smallest of their class in some column: a strategy whose column
+//                   class, too, has a member that needs no more memory and no more time never is (G does not rise
+//                   with the budget).  ZeRO stages and checkpointing mostly differ in memory alone: about half drop out.
 // A class has an even number of entries (the last one may stand twice: it stores the same values again, and a minimum
 // does not change), so entries are read two to a 128-bit load, and four at a time from one address.
 // Shared-memory accesses of the layer loop go through 32-bit addresses and are written in batches, loads first: the table
@@ -299,9 +323,13 @@ __device__ __forceinline__ void emit(const Ctx& c, uint32_t gn, uint32_t an, int
 }
 
 // Where a tile's values go in the table.
-template <bool STORE, bool ARG>
+// STAGE: the rows of a layer are collected in shared memory ([S][W], two layers in turn) and leave with one bulk tensor
+// store the service warp issues.  A table store of a warp holds the load / store unit for four cycles and more, and the
+// loads of the next strategies, which the layer's chain of latencies consists of, queue up behind it.
+template <bool STORE, bool ARG, bool STAGE>
 struct Out {
-    char* C;               // the tile's first column plus this lane, strategy 0
+    uint32_t stage;        // the tile's first column plus this lane, strategy 0, in the collected rows
+    char* C;               // ... in the table
     uint8_t* A;
     bool whole;            // every column of the tile is a budget column
     int cols;              // columns of the tile that exist in the table, less this lane
@@ -309,7 +337,10 @@ struct Out {
     template <int TM>
     __device__ __forceinline__ void put(uint32_t row, const int (&v)[TM], const int (&a)[TM]) const
     {
-        if (STORE) {
+        if (STAGE) {
+#pragma unroll
+            for (int j = 0; j < TM; ++j) sts(stage + row + 128u * j, whole || 32 * j < budget ? v[j] : kInf);
+        } else if (STORE) {
             int32_t* const p = reinterpret_cast<int32_t*>(C + row);
             if (whole) {
 #pragma unroll
@@ -361,8 +392,8 @@ __device__ __forceinline__ void fetch_recs(const Ctx& c, uint32_t ra, uint32_t r
 }
 
 // U strategies: their C values to the table, their smallest into h (with ARG: whose it is).
-template <int U, int TM, bool STORE, bool ARG, bool FAR>
-__device__ __forceinline__ void scan(const Ctx& c, const Out<STORE, ARG>& out, uint32_t ra, uint32_t rowa, uint32_t ga, uint32_t aa, int col, int (&h)[TM], int (&hs)[TM])
+template <int U, int TM, bool STORE, bool ARG, bool STAGE, bool FAR>
+__device__ __forceinline__ void scan(const Ctx& c, const Out<STORE, ARG, STAGE>& out, uint32_t ra, uint32_t rowa, uint32_t ga, uint32_t aa, int col, int (&h)[TM], int (&hs)[TM])
 {
     Recs<U> r;
     int v[U][TM], a[ARG ? U : 1][TM];
@@ -409,28 +440,29 @@ __device__ __forceinline__ uint32_t alive(const Ctx& c, uint32_t ra, uint32_t ro
 }
 
 // One layer of one tile of TM x 32 columns.  KC: rows of the next state held in accumulators (PRUNE: per block of rows).
-template <int KC, int TM, bool PRUNE, bool STORE, bool ARG, bool FAR>
+template <int KC, int TM, bool PRUNE, bool STORE, bool ARG, bool STAGE, bool FAR>
 __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
 {
-    const int slot = l % 3, col = colb + lane;
-    const uint32_t ra = c.rec + (uint32_t)(slot * c.S2) * 16u, rowa = ra + (uint32_t)c.S2 * 8u;
+    const int slot = c.slot[l & 3], col = colb + lane;
+    const uint32_t ra = c.rec + (uint32_t)(slot * c.S2) * 24u, rowa = ra + (uint32_t)c.S2 * 8u;
     const uint32_t ga = smem_addr(c.g0 + (l & 1) * c.gints + col), gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints);
     const uint32_t aa = ARG ? smem_addr(c.a0 + (l & 1) * c.gints + col) : 0u, an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
     const int colg = c.rank * c.W + colb;                      // the tile's first budget column
-    Out<STORE, ARG> out;
+    Out<STORE, ARG, STAGE> out;
+    out.stage = STAGE ? smem_addr(c.stage + (l & 1) * c.S * c.W + col) : 0u;
     out.C = STORE ? reinterpret_cast<char*>(c.C + (size_t)l * c.slice + colg + lane) : nullptr;
     out.A = ARG ? c.A + (size_t)l * c.slice + colg + lane : nullptr;
     out.whole = colg + 32 * TM - 1 <= c.M;
     out.cols = c.m_pitch - colg - lane;
     out.budget = c.M + 1 - colg - lane;
 
-    if (colg + 32 * TM - 1 < c.front[slot]) {                  // nothing finite in the tile
+    if (colg + 32 * TM - 1 < c.front[l & 3]) {                  // nothing finite in the tile
         int inf[TM], none[TM];
 #pragma unroll
         for (int j = 0; j < TM; ++j) { inf[j] = kInf; none[j] = 255; }
         if (STORE || ARG)
 #pragma unroll 4
-            for (int e = 0; e < c.S; ++e) out.template put<TM>((uint32_t)(e * c.m_pitch) * 4u, inf, none);
+            for (int e = 0; e < c.S; ++e) out.template put<TM>((uint32_t)(e * (STAGE ? c.W : c.m_pitch)) * 4u, inf, none);
         for (int k = 0; k < c.Kc; ++k) emit<TM, ARG>(c, gn, an, k, colb, lane, inf, none);
         return;
     }
@@ -442,7 +474,10 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
 #pragma unroll
             for (int j = 0; j < TM; ++j) { acc[k][j] = kInf; if (ARG) arg[k][j] = 255; }
         int e = 0;
-        const int* const cs = c.cs + slot * (kClassMax + 1);
+        // without a table to write, only the strategies that can matter
+        constexpr bool kAll = STORE || ARG || FAR;
+        const int* const cs = kAll ? c.cs : c.csp + slot * (kClassMax + 1);
+        const uint32_t la = kAll ? ra : ra + (uint32_t)c.S2 * 16u;
         const uint32_t ta = smem_addr(c.tsm);
         for (int k = 0; k < c.Kr; ++k) {
             const int end = cs[k + 1];
@@ -452,9 +487,9 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
             int4 t4[KC / 4];
 #pragma unroll
             for (int q = 0; q < KC / 4; ++q) t4[q] = lds4(ta + (uint32_t)(k * kClassMax + 4 * q) * 4u);
-            constexpr int U = FAR ? 1 : TM > 3 ? 2 : 4;
-            for (; e + U <= end; e += U) scan<U, TM, STORE, ARG, FAR>(c, out, ra + 8u * e, rowa + 4u * e, ga, aa, col, h, hs);
-            if (U == 4 && e < end) { scan<2, TM, STORE, ARG, FAR>(c, out, ra + 8u * e, rowa + 4u * e, ga, aa, col, h, hs); e += 2; }
+            constexpr int U = FAR ? 1 : TM > 4 && STORE ? 2 : 4;
+            for (; e + U <= end; e += U) scan<U, TM, STORE, ARG, STAGE, FAR>(c, out, la + 8u * e, rowa + 4u * e, ga, aa, col, h, hs);
+            if (U == 4 && e < end) { scan<2, TM, STORE, ARG, STAGE, FAR>(c, out, la + 8u * e, rowa + 4u * e, ga, aa, col, h, hs); e += 2; }
 #pragma unroll
             for (int q = 0; q < KC / 4; ++q) {
                 const int t[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
@@ -481,8 +516,8 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
         for (int j = 0; j < TM; ++j) { thr[j] = kInf; dummy[j] = 255; }
         int s = 0;
         if (!FAR)
-            for (; s + 4 <= c.S; s += 4) scan<4, TM, STORE, ARG, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
-        for (; s < c.S; ++s) scan<1, TM, STORE, ARG, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
+            for (; s + 4 <= c.S; s += 4) scan<4, TM, STORE, ARG, STAGE, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
+        for (; s < c.S; ++s) scan<1, TM, STORE, ARG, STAGE, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
         // a candidate beyond the column's best plus the largest entry cannot win; a column without a finite value
         // keeps nothing alive
 #pragma unroll
@@ -542,11 +577,12 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
 }
 
 // The last layer hands nothing on: its values go to the table and to C_last.
-template <bool STORE, bool ARG, bool FAR>
+template <bool STORE, bool ARG, bool STAGE, bool FAR>
 __device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lane)
 {
-    const int slot = l % 3, col = colb + lane;
-    const uint32_t ra = c.rec + (uint32_t)(slot * c.S2) * 16u, rowa = ra + (uint32_t)c.S2 * 8u, ga = smem_addr(c.g0 + (l & 1) * c.gints + col);
+    const uint32_t sa = STAGE ? smem_addr(c.stage + (l & 1) * c.S * c.W + colb + lane) : 0u;
+    const int slot = c.slot[l & 3], col = colb + lane;
+    const uint32_t ra = c.rec + (uint32_t)(slot * c.S2) * 24u, rowa = ra + (uint32_t)c.S2 * 8u, ga = smem_addr(c.g0 + (l & 1) * c.gints + col);
     const uint32_t aa = ARG ? smem_addr(c.a0 + (l & 1) * c.gints + col) : 0u;
     const int colg = c.rank * c.W + colb, m = colg + lane;
     if (colg >= c.m_pitch) return;                             // m_pitch is a multiple of 32: a group exists whole or not at all
@@ -564,6 +600,7 @@ __device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lan
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int v = pad ? kInf : __viaddmin_s32(g[u][0], r.t[u], kInf);
+            if (STAGE) { sts(sa + (uint32_t)r.row[u], v); continue; }
             const size_t row = ((uint32_t)r.row[u] >> 2) + (size_t)m;
             if (STORE) c.C[(size_t)l * c.slice + row] = v;
             c.C_last[row] = v;
@@ -577,50 +614,52 @@ __device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lan
 }
 
 // `n` column groups from group g on, as one tile.
-template <int KC, int MAX, bool PRUNE, bool STORE, bool ARG>
+template <int KC, int MAX, bool PRUNE, bool STORE, bool ARG, bool STAGE>
 __device__ __forceinline__ void tile_of(const Ctx& c, int l, int g, int n, int lane)
 {
     if constexpr (MAX > 1) {
-        if (n < MAX) { tile_of<KC, MAX - 1, PRUNE, STORE, ARG>(c, l, g, n, lane); return; }
+        if (n < MAX) { tile_of<KC, MAX - 1, PRUNE, STORE, ARG, STAGE>(c, l, g, n, lane); return; }
     }
-    tile<KC, MAX, PRUNE, STORE, ARG, false>(c, l, g * 32, lane);
+    tile<KC, MAX, PRUNE, STORE, ARG, STAGE, false>(c, l, g * 32, lane);
 }
 
 // A warp owns a run of column groups (the warps' runs differ by one group at most) and takes it as one tile, or as
 // several of about the same width when it is wider than MAX groups: a record fetched once serves them all.
-template <int KC, int MAX, bool PRUNE, bool STORE, bool ARG>
+template <int KC, int MAX, bool PRUNE, bool STORE, bool ARG, bool STAGE>
 __device__ __forceinline__ void run_layers(const Ctx& c, int warp, int lane)
 {
     const int g0 = c.G * warp / c.NW, g1 = c.G * (warp + 1) / c.NW;
     for (int l = 0; l + 1 < c.Li; ++l) {
         int g = g0;
-        if (c.reach[l % 3] <= c.H) {
+        if (c.reach[c.slot[l & 3]] <= c.H) {
             for (int left = (g1 - g0 + MAX - 1) / MAX; left > 0; --left) {
                 const int n = (g1 - g + left - 1) / left;
-                tile_of<KC, MAX, PRUNE, STORE, ARG>(c, l, g, n, lane);
+                tile_of<KC, MAX, PRUNE, STORE, ARG, STAGE>(c, l, g, n, lane);
                 g += n;
             }
         } else {
-            for (; g < g1; ++g) tile<KC, 1, PRUNE, STORE, ARG, true>(c, l, g * 32, lane);
+            for (; g < g1; ++g) tile<KC, 1, PRUNE, STORE, ARG, STAGE, true>(c, l, g * 32, lane);
         }
-        end_layer<ARG>(c, l, warp, lane);
+        send_halo<ARG>(c, l, warp, lane);
+        await_halo<ARG>(c, l, warp, lane);
     }
-    if (c.reach[(c.Li - 1) % 3] <= c.H) {
-        for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, false>(c, c.Li - 1, g * 32, lane);
+    if (c.reach[c.slot[(c.Li - 1) & 3]] <= c.H) {
+        for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, STAGE, false>(c, c.Li - 1, g * 32, lane);
     } else {
-        for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, true>(c, c.Li - 1, g * 32, lane);
+        for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, STAGE, true>(c, c.Li - 1, g * 32, lane);
     }
 }
 
 // Cluster c takes instance c (the c-th longest when `sorted`).  Warps 0..NW-1 compute, the last warp fetches the
 // layers' mem / time rows (and with one matrix per layer the matrices) ahead and turns them into records.
-template <bool STORE, bool ARG>
-__global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const RsArgs a)
+template <bool STORE, bool ARG, bool STAGE>
+__global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const RsArgs a, const __grid_constant__ CUtensorMap map_c,
+                                                                           const __grid_constant__ CUtensorMap map_last)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ union { int L[kMaxSortedB]; struct { uint32_t rh[kMaxS], ch[kMaxS]; } h; } s_u;
-    __shared__ int s_rrep[kMaxS], s_crep[kMaxS], s_rcls[kMaxS], s_ccls[kMaxS], s_order[kMaxS + kClassMax], s_cs[3 * (kClassMax + 1)], s_first[kClassMax + 1];
-    __shared__ int s_cdelta[16], s_front[3], s_reach[3], s_inst, s_K[2];
+    __shared__ int s_rrep[kMaxS], s_crep[kMaxS], s_rcls[kMaxS], s_ccls[kMaxS], s_order[kMaxS + kClassMax], s_csp[4 * (kClassMax + 1)], s_first[kClassMax + 1], s_cnt[kClassMax];
+    __shared__ int s_cdelta[16], s_front[4], s_reach[4], s_slot[4], s_inst, s_K[2];
     __shared__ struct { long long sum; int tmax, bad, mmax; } s_part, s_all;
     __shared__ __align__(8) unsigned long long s_bar[2];
     __shared__ int s_late;
@@ -635,8 +674,9 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     int32_t* const tsm = g0 + 2 * gints;                                                   // [16][16] or [1|2][S][SP]
     const int tints = max(kClassMax * kClassMax, (a.trans_layer ? 2 : 1) * tfull);
     const int S2 = (S + kClassMax + 3) & ~3;
-    int32_t* const rec = tsm + tints;                                                      // [3] slots of S2 x (int2, int, int)
-    int32_t* const raw = rec + 3 * 4 * S2;                                                 // [4][2][S] mem, time rows as they come
+    int32_t* const rec = tsm + tints;                                                      // [4] slots of S2 x (int2, int, int, int2)
+    int32_t* const raw = rec + 4 * 6 * S2;                                                 // [4][2][S] mem, time rows as they come
+    int32_t* const stage_rows = reinterpret_cast<int32_t*>(smem_raw) + a.stage_at;         // [2][S][W] rows on their way to the table
     uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * ((S + 3) & ~3));                           // [2][gints] argmin of the state
 
     if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = a.path_value; }
@@ -829,7 +869,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                 const int v = __shfl_up_sync(0xffffffffu, at, o);
                 if (lane >= o) at += v;
             }
-            if (lane < Kr) s_first[lane] = at - ((n + 1) & ~1);
+            if (lane < Kr) { s_first[lane] = at - ((n + 1) & ~1); s_cnt[lane] = n; }
             if (lane == Kr - 1) s_first[Kr] = at;
         }
         __syncthreads();
@@ -870,28 +910,82 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     const int H = max(0, min((s_all.mmax + 31) & ~31, (gints / Kc - W) & ~31)), P = W + H;
 
     const int n_all = classes ? s_first[Kr] : S;
+    const bool strict = s_all.mmax > H;                         // some shift reaches beyond the halo
     // ---- layer 0 gathers from an all-zero state: C[0] = time where mem fits
     auto prepare = [&](int l, int base) -> int {                // records of layer l by one warp; returns the new frontier
-        const int slot = l % 3;
         const int32_t* const rm = raw + (l & 3) * 2 * S;
-        int32_t* const rs = rec + slot * 4 * S2;
-        int least = M + 1, most = 0;
-        for (int e = lane; e < n_all; e += 32) {
-            const int s = s_order[e];
-            const int mem = rm[s];
-            const bool fits = mem <= M;                         // else +inf everywhere: no shift, time +inf
-            const int shift = fits ? mem : 0;
-            reinterpret_cast<int2*>(rs)[e] = make_int2((s_ccls[s] * P + H - shift) * 4, fits ? rm[S + s] : kInf);
-            rs[2 * S2 + e] = s * a.m_pitch * 4;
-            rs[3 * S2 + e] = shift | (s << 24);
-            least = min(least, mem);
-            most = max(most, shift);
+        // a layer with the rows of one of the two before it takes that one's records
+        int slot = -1, least = M + 1;
+        for (int back = 1; back <= 2 && back <= l && slot < 0; ++back) {
+            const int32_t* const ro = raw + ((l - back) & 3) * 2 * S;
+            int diff = 0;
+            for (int x = lane; x < 2 * S; x += 32) diff |= rm[x] != ro[x];
+            if (!__any_sync(0xffffffffu, diff)) slot = s_slot[(l - back) & 3];
         }
-        if (classes && lane <= Kr) s_cs[slot * (kClassMax + 1) + lane] = s_first[lane];
+        if (slot < 0) {
+            // not one of the three layers before: the oldest may still be on its way to the table
+            unsigned used = 0;
+            for (int back = 1; back <= 3 && back <= l; ++back) used |= 1u << s_slot[(l - back) & 3];
+            slot = __ffs(~used) - 1;
+            int32_t* const rs = rec + slot * 6 * S2;
+            int most = 0;
+            for (int e = lane; e < n_all; e += 32) {
+                const int s = s_order[e];
+                const int mem = rm[s];
+                const bool fits = mem <= M;                     // else +inf everywhere: no shift, time +inf
+                const int shift = fits ? mem : 0;
+                reinterpret_cast<int2*>(rs)[e] = make_int2((s_ccls[s] * P + H - shift) * 4, fits ? rm[S + s] : kInf);
+                rs[2 * S2 + e] = s * (STAGE ? W : a.m_pitch) * 4;
+                rs[3 * S2 + e] = shift | (s << 24);
+                most = max(most, shift);
+            }
+            most = __reduce_max_sync(0xffffffffu, most);
+            if (lane == 0) s_reach[slot] = most;
+            if (classes && !STORE && !ARG) {
+                // the strategies that can matter, class by class
+                __syncwarp();
+                int2* const keep = reinterpret_cast<int2*>(rs + 4 * S2);
+                const int2* const all = reinterpret_cast<const int2*>(rs);
+                int at = 0;
+                for (int k = 0; k < Kr; ++k) {
+                    if (lane == 0) s_csp[slot * (kClassMax + 1) + k] = at;
+                    const int first = s_first[k], n = s_cnt[k];
+                    int2 lastkept = make_int2(0, 0);
+                    int kept = 0;
+                    for (int b = 0; b < n; b += 32) {
+                        const int p = b + lane;
+                        bool in = p < n;
+                        int2 me = make_int2(0, kInf);
+                        if (in) {
+                            me = all[first + p];
+                            in = me.y < kInf;
+                            const int mm = rm[s_order[first + p]], mc = s_ccls[s_order[first + p]];
+                            for (int q = 0; q < n && in; ++q) {
+                                const int so = s_order[first + q];
+                                const int om = rm[so], ot = rm[S + so];
+                                if (s_ccls[so] == mc && om <= mm && ot <= me.y && (om < mm || ot < me.y || q < p)) in = false;
+                            }
+                        }
+                        const unsigned b1 = __ballot_sync(0xffffffffu, in);
+                        if (in) keep[at + kept + __popc(b1 & ((1u << lane) - 1))] = me;
+                        if (b1) {
+                            const int src = 31 - __clz(b1);
+                            lastkept.x = __shfl_sync(0xffffffffu, me.x, src);
+                            lastkept.y = __shfl_sync(0xffffffffu, me.y, src);
+                        }
+                        kept += __popc(b1);
+                    }
+                    if ((kept & 1) && lane == 0) keep[at + kept] = lastkept;
+                    at += (kept + 1) & ~1;
+                }
+                if (lane == 0) s_csp[slot * (kClassMax + 1) + Kr] = at;
+            }
+        }
+        for (int s = lane; s < S; s += 32) least = min(least, rm[s]);
         least = __reduce_min_sync(0xffffffffu, least);
-        most = __reduce_max_sync(0xffffffffu, most);
         const int f = min(base + least, M + 1);
-        if (lane == 0) { s_front[slot] = f; s_reach[slot] = most; }
+        if (lane == 0) { s_front[l & 3] = f; s_slot[l & 3] = slot; }
+        __syncwarp();
         return f;
     };
     auto fetch = [&](int l) {
@@ -932,15 +1026,15 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     Ctx c;
     c.S = S; c.M = M; c.W = W; c.H = H; c.P = P; c.G = W / 32; c.CL = CL; c.rank = rank; c.Li = Li; c.m_pitch = a.m_pitch; c.Kr = Kr; c.Kc = Kc;
     c.tmax = s_all.tmax; c.SP = a.SP; c.NW = NW; c.gints = gints;
-    c.g0 = g0; c.a0 = a0; c.rec = smem_addr(rec); c.S2 = S2; c.n_all = n_all; c.front = s_front; c.reach = s_reach; c.tsm = tsm; c.tmat = a.trans_layer ? tfull : 0;
-    c.cs = s_cs; c.cdelta = s_cdelta;
+    c.g0 = g0; c.a0 = a0; c.stage = stage_rows; c.rec = smem_addr(rec); c.S2 = S2; c.n_all = n_all; c.front = s_front; c.reach = s_reach; c.tsm = tsm; c.tmat = a.trans_layer ? tfull : 0;
+    c.cs = s_first; c.csp = s_csp; c.slot = s_slot; c.cdelta = s_cdelta;
     c.slice = (size_t)S * a.m_pitch;
     c.C = STORE ? a.C + (size_t)i * Lmax * c.slice : nullptr;
     c.A = ARG ? a.A + (size_t)i * Lmax * c.slice : nullptr;
     c.C_last = a.C_last + (size_t)i * c.slice;
     c.bars = smem_addr(&s_bar[0]);
     c.halo_bytes = (uint32_t)(Kc * min(H, rank * W)) * (ARG ? 5u : 4u);
-    c.strict = s_all.mmax > H;
+    c.strict = strict;
     c.late = &s_late;
     if (CL > 1 && !c.strict) cluster_arrive();                  // nobody has read anything yet: the first copies may come
     if (warp == NW) {
@@ -963,16 +1057,40 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                 front = prepare(l + 2, front);
             }
             if (a.trans_layer) cp_async_wait<0>();
-            end_layer<ARG>(c, l, warp, lane);
+            if (STAGE) {
+                if (lane == 0) bulk_wait_read();                // layer l - 1 has left its buffer, which layer l + 1 fills
+                __syncwarp();
+            }
+            send_halo<ARG>(c, l, warp, lane);
+            if (STAGE && lane == 0) {
+                if (CL == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                tensor_store_3d(&map_c, c.stage + (l & 1) * S * W, rank * (W / 32), (i * Lmax + l) * S);
+                bulk_commit();
+            }
+            await_halo<ARG>(c, l, warp, lane);
+        }
+        if (STAGE) {
+            if (lane == 0) bulk_wait_read();
+            cta_barrier();                                      // the last layer's rows are collected
+            if (lane == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                const int l = Li - 1;
+                tensor_store_3d(&map_c, c.stage + (l & 1) * S * W, rank * (W / 32), (i * Lmax + l) * S);
+                tensor_store_3d(&map_last, c.stage + (l & 1) * S * W, rank * (W / 32), i * S);
+                bulk_commit();
+                bulk_wait_all();
+            }
+            __syncwarp();
         }
     } else {
         if (classes) {
-            if (K <= 4) run_layers<4, ARG ? 2 : 6, false, STORE, ARG>(c, warp, lane);
-            else if (K <= 8) run_layers<8, ARG ? 2 : 6, false, STORE, ARG>(c, warp, lane);
-            else run_layers<16, ARG ? 1 : 3, false, STORE, ARG>(c, warp, lane);
+            if (K <= 4) run_layers<4, ARG ? 2 : 6, false, STORE, ARG, STAGE>(c, warp, lane);
+            else if (K <= 8) run_layers<8, ARG ? 2 : 6, false, STORE, ARG, STAGE>(c, warp, lane);
+            else run_layers<16, ARG ? 1 : 3, false, STORE, ARG, STAGE>(c, warp, lane);
         } else {
-            run_layers<32, ARG ? 1 : 2, true, STORE, ARG>(c, warp, lane);
+            run_layers<32, ARG ? 1 : 2, true, STORE, ARG, STAGE>(c, warp, lane);
         }
+        if (STAGE) cta_barrier();                               // the last layer's rows are collected
     }
     if (CL > 1) {
         if (!c.strict) cluster_wait();
@@ -984,14 +1102,40 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
 
 // ---------------------------------------------------------------- host side
 
-typedef void (*RsKernel)(const RsArgs);
-RsKernel kernel_of(bool store, bool arg)
+typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                    const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                    CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// Tensor map of an int32 table [rows][m_pitch] seen as [rows][m_pitch / 32][32], box [box_rows][box_groups][32].
+cudaError_t encode_table_3d(CUtensorMap* map, void* base, size_t rows, int m_pitch, int box_rows, int box_groups)
 {
-    return store ? (arg ? resident_kernel<true, true> : resident_kernel<true, false>)
-                 : (arg ? resident_kernel<false, true> : resident_kernel<false, false>);
+    static PFN_encodeTiled fn = nullptr;
+    if (!fn) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q);
+        if (e != cudaSuccess) return e;
+        if (q != cudaDriverEntryPointSuccess || !p) return cudaErrorNotSupported;
+        fn = reinterpret_cast<PFN_encodeTiled>(p);
+    }
+    const cuuint64_t dims[3] = {32, (cuuint64_t)(m_pitch / 32), (cuuint64_t)rows};
+    const cuuint64_t strides[2] = {128, (cuuint64_t)m_pitch * 4};
+    const cuuint32_t box[3] = {32, (cuuint32_t)box_groups, (cuuint32_t)box_rows};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_INT32, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t launch_resident(RsKernel k, const RsArgs& a, const RsPlan& p, cudaStream_t st, int* max_clusters)
+typedef void (*RsKernel)(const RsArgs, const CUtensorMap, const CUtensorMap);
+RsKernel kernel_of(bool store, bool arg, bool stage)
+{
+    if (stage) return resident_kernel<true, false, true>;
+    return store ? (arg ? resident_kernel<true, true, false> : resident_kernel<true, false, false>)
+                 : (arg ? resident_kernel<false, true, false> : resident_kernel<false, false, false>);
+}
+
+cudaError_t launch_resident(RsKernel k, const RsArgs& a, const RsPlan& p, const CUtensorMap& mc, const CUtensorMap& ml, cudaStream_t st, int* max_clusters)
 {
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
@@ -1007,7 +1151,7 @@ cudaError_t launch_resident(RsKernel k, const RsArgs& a, const RsPlan& p, cudaSt
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, k, &cfg);
-    return cudaLaunchKernelEx(&cfg, k, a);
+    return cudaLaunchKernelEx(&cfg, k, a, mc, ml);
 }
 
 // Clusters of this plan's size and resources the device can hold at once (asked once per kind of launch).
@@ -1016,14 +1160,15 @@ int max_active_clusters(const galv_ctx* ctx, const RsPlan& p, bool store, bool a
     static std::map<unsigned long long, int> cache;          // shared by all contexts of the process
     static std::mutex cache_mutex;
     std::lock_guard<std::mutex> lock(cache_mutex);
-    const unsigned long long key = ((unsigned long long)ctx->device << 48) | ((unsigned long long)p.cl << 40) | ((unsigned long long)store << 37) |
+    const unsigned long long key = ((unsigned long long)ctx->device << 48) | ((unsigned long long)p.cl << 40) | ((unsigned long long)p.stage << 38) | ((unsigned long long)store << 37) |
                                    ((unsigned long long)arg << 36) | ((unsigned long long)p.nw << 28) | (unsigned long long)((p.smem + 1023) / 1024);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     RsArgs a{};
     a.B = 1;
     int n = 0;
-    if (launch_resident(kernel_of(store, arg), a, p, nullptr, &n) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+    CUtensorMap m{};
+    if (launch_resident(kernel_of(store, arg, p.stage), a, p, m, m, nullptr, &n) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
     cache[key] = n;
     return n;
 }
@@ -1033,7 +1178,7 @@ long long fixed_smem(const galv_shape* sh, bool dense)
 {
     const int S = sh->S, SP = (S + 3) & ~3;
     const long long t = dense ? (long long)S * SP * ((sh->flags & GALV_TRANS_PER_LAYER) ? 2 : 1) : 0;
-    return (t > kClassMax * kClassMax ? t : kClassMax * kClassMax) * 4 + (long long)3 * 16 * ((S + kClassMax + 3) & ~3) + (long long)8 * SP * 4 + 128;
+    return (t > kClassMax * kClassMax ? t : kClassMax * kClassMax) * 4 + (long long)4 * 24 * ((S + kClassMax + 3) & ~3) + (long long)8 * SP * 4 + 256;
 }
 
 // The best cluster size for a state of `rows` rows at least; false when none fits.
@@ -1058,11 +1203,19 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
         std::memset(&p, 0, sizeof(p));
         p.cl = cl; p.w = w; p.dense = dense;
         p.nw = g < kMaxWarps ? g : kMaxWarps;
+        // rows collected in shared memory where there is room for them beside the state (a tensor box has 256 entries a
+        // side at most) and where a layer is a chain of latencies rather than a stream of stores
+        const long long collected = (long long)2 * S * w * 4;
+        p.stage = store && !arg && g <= 2 * kMaxWarps && (long long)rows * (w + (cl > 1 ? halo : 0)) * per_word + collected <= words * per_word &&
+                  (long long)sh->B * sh->Lmax * S < (1ll << 31);
+        const long long room = p.stage ? words - collected / per_word : words;
         long long gi = (long long)(dense && S > kClassMax ? S : kClassMax) * (w + ((sh->M + 32) & ~31));    // all that could be used
-        if (gi > words) gi = words;
+        if (gi > room) gi = room;
         p.gints = (int)(gi & ~31ll);
         if ((long long)rows * w > p.gints) continue;
         p.smem = (int)(p.gints * (long long)per_word + fixed_smem(sh, dense));
+        p.stage_at = (p.smem + 127) / 128 * 32;
+        if (p.stage) p.smem = p.stage_at * 4 + (int)collected;
         const int slots = max_active_clusters(ctx, p, store, arg);
         if (slots < 1) continue;
         // SM cycles a layer: the issue of the columns' work, the store port (32 bytes a clock), the latency of one warp's
@@ -1109,8 +1262,8 @@ int galv_cluster_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
 cudaError_t galv_cluster_configure(galv_ctx* ctx)
 {
     ctx->max_cluster = 16;                                     // beyond the portable 8 where the device allows it
-    for (int k = 0; k < 4; ++k) {
-        const RsKernel f = kernel_of(k & 1, (k & 2) != 0);
+    for (int k = 0; k < 5; ++k) {
+        const RsKernel f = kernel_of(k & 1, (k & 2) != 0, k == 4);
         cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin - kStaticSmem);
         if (e != cudaSuccess) return e;
         if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) { (void)cudaGetLastError(); ctx->max_cluster = 8; }
@@ -1128,5 +1281,14 @@ cudaError_t galv_cluster_launch(const RsPlan& p, int second, const DpArgs& d, cu
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
     a.C = d.C; a.A = d.A; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done;
-    return launch_resident(kernel_of(d.C != nullptr, d.A != nullptr), a, p, st, nullptr);
+    a.stage_at = p.stage_at;
+    CUtensorMap mc, ml;
+    std::memset(&mc, 0, sizeof(mc));
+    std::memset(&ml, 0, sizeof(ml));
+    if (p.stage) {
+        cudaError_t e = encode_table_3d(&ml, d.C_last, (size_t)d.B * d.S, d.m_pitch, d.S, p.w / 32);
+        if (e == cudaSuccess) e = encode_table_3d(&mc, d.C, (size_t)d.B * d.Lmax * d.S, d.m_pitch, d.S, p.w / 32);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_resident(kernel_of(d.C != nullptr, d.A != nullptr, p.stage), a, p, mc, ml, st, nullptr);
 }

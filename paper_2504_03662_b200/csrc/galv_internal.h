@@ -16,6 +16,8 @@ struct RsPlan {
     int dense;     // the state of an unstructured matrix (S rows and the matrix itself) fits: every instance can run
     int smem;      // dynamic shared memory bytes
     int sorted;    // clusters take the instances longest first
+    int stage;     // a layer's rows are collected in shared memory and leave with one tensor store
+    int stage_at;  // word offset of the collected rows
 };
 
 struct galv_ctx {
