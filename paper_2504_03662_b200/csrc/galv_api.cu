@@ -106,6 +106,7 @@ int galv_create(galv_ctx** out, int device_ordinal)
     if (cur != device_ordinal) cudaSetDevice(device_ordinal);
     e = galv_dp_configure(ctx);
     if (e == cudaSuccess) e = galv_cluster_configure(ctx);
+    if (e == cudaSuccess) e = galv_resident_configure(ctx);
     for (auto& ev : ctx->pev)
         if (e == cudaSuccess) e = cudaEventCreate(&ev);
     if (cur >= 0 && cur != device_ordinal) cudaSetDevice(cur);

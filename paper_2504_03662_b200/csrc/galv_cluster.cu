@@ -1,33 +1,25 @@
-// The whole recurrence of one instance on the SMs of one thread-block cluster, its state kept in shared memory.
+// Small batches: one thread-block cluster per search instance, the table slice kept in shared memory.
 //
-//   C[l][m][s] = time(l,s) + G[l][m - mem(l,s)][s],   G[l][m][s] = min_{s'} ( C[l-1][m][s'] + trans(s',s) )
+//   C[l][m][s] = time(l,s) + min_{s'} ( C[l-1][m-mem(l,s)][s'] + trans(s',s) )
 //
-// (Section 3 of the paper: dynamic-programming search over a performance model; Sections 3-4: it runs again while
-// the job runs.)
+// (Section 3 of the paper: the selector searches again while the job runs, one model at a time;
+// Section 4: the manager's step.  Such a re-search is a batch of one to a few dozen instances.)
 //
-// What a layer hands to the next one is G, and G has one row per DISTINCT COLUMN of the transition matrix: strategies
-// with equal columns have equal G.  Strategies with equal ROWS enter the minimum with the same offset, so only the
-// smallest of them matters.  A matrix that prices a move between layouts (tensor-parallel degree, sequence
-// parallelism) has a handful of distinct rows and columns however many strategies there are (8 among 64, 4 among 24):
-// a cell then costs one addition, one minimum over its class and its store instead of S add-mins, and the state of an
-// instance shrinks from S to 8 rows.  The kernel finds the classes itself, by comparing the matrix's rows and columns
-// word by word (hashes only propose), so nothing is assumed about where a matrix comes from.
-// A matrix without such structure keeps all S rows.  Then a candidate C[l-1][m][s'] that lies more than the largest
-// transition entry above its column's best can neither win nor tie (the best row gives a candidate at most that entry
-// above itself), so a warp relaxes only the rows that are alive in one of its columns.
+// With fewer work items per layer than the GPU has SMs the tiled kernel's step is a chain of dependent
+// layers, each link paying a trip through L2 and a gpu-scope publish.  Here the chain never leaves the
+// SMs: the budget columns of ONE instance are split over the CTAs of a cluster (CTA r owns columns
+// r*W .. r*W+W-1), each CTA keeps its columns of the previous layer, all S rows, in shared memory,
+// computes G[s][m'] = min_{s'}(Cprev[s'][m'] + T[s'][s]) for its own columns m' (no halo: G does not
+// depend on mem) and PUSHES time + G to where it belongs, column m' + mem(l,s) of the next layer's
+// buffer, which lies in its own shared memory or in that of a CTA further up: a plain store into
+// distributed shared memory.  One hardware cluster barrier per layer (release / acquire) ends the
+// layer.  Cells no column maps to (m < mem(l,s)) are written +inf by the CTA that owns them.
+// The finished slice of a layer goes to the table in HBM by ONE tensor-map bulk store (TMA) straight
+// from the shared-memory buffer, issued by a service warp while the other warps compute the next layer.
 //
-// The budget columns are split over the CTAs of the cluster: CTA r owns columns r*W .. r*W+W-1 and keeps their G in two
-// buffers (this layer's, the next one's), with a halo of H columns to their left: C is produced by GATHERING G at
-// m - mem(l,s), from this CTA's own shared memory as long as the shift stays within the halo.  Whoever computes a column
-// writes it to its own buffer and into the halo of the CTAs further up that hold it (distributed shared memory; a store
-// is fired and forgotten, while reading the cells from their owner instead puts a round trip on every gather's chain:
-// 8.4 us a layer on one instance of 24 strategies over 16 CTAs).  A layer ends with one cluster barrier (a block barrier
-// where the cluster is one CTA).  No spin-waits, no cooperative launch, no cluster multicast, no workspace but a word per
-// instance and the path flag; the tables go out as full 128-byte lines and are never read back.
-//
-// Validation is the kernel's own (same rules and status bits as everywhere).  An instance whose state does not fit this
-// launch's shared memory is left alone and marked in done[]; a second launch with larger clusters or the tiled kernels
-// take it.
+// The kernel validates its instance itself, writes the base layer, every layer and C_last: the
+// whole search is one launch.  No spin-waits anywhere: the cluster barrier is a hardware barrier
+// among co-scheduled CTAs, and clusters never wait on one another.  No cluster multicast.
 
 #include <cuda.h>
 
@@ -38,83 +30,61 @@
 
 #include "galv_internal.h"
 
+
 namespace {
 
 constexpr int kInf = GALV_INF;
 constexpr int kMaxSortedB = 512;          // instances whose lengths fit the ranking scratch below
-constexpr int kMaxS = 128;
-constexpr int kMaxWarps = 15;             // compute warps per CTA (with the service warp 512 threads: 128 registers each)
-constexpr int kStaticSmem = 5632;         // the kernel's static shared memory, rounded up
-constexpr int kClassMax = 16;             // classes beyond which the matrix counts as unstructured
+constexpr int kRowsPerLane = 4;           // strategies per lane of the service warp: S <= 128
 
-struct RsArgs {
+struct ClArgs {
     int B, Lmax, S, M, m_pitch;
     int CL;            // CTAs per cluster
     int W;             // budget columns per CTA (multiple of 32)
-    int gints;         // words of one state buffer: rows of W columns and their halo
-    int stage_at;      // word offset of the collected rows
-    int SP;            // row pitch of the full transition matrix in shared memory; 0: no room for unstructured matrices
+    int G;             // W / 32
+    int NSG;           // ceil(S / 8)
+    int SP8;           // NSG * 8: row pitch of the trans matrix in shared memory
+    int nct;           // column tiles of 32*TM columns per CTA
+    int units;         // nct * NSG work units per CTA and layer
     int sorted;        // clusters take the instances longest first
-    int second;        // only the instances the first launch left alone
-    int path_value;    // what galv_dp_search_path reports
     const int32_t* L;
     const int32_t* time_q;
     const int32_t* mem_q;
     const int32_t* trans_q;
     long long trans_inst, trans_layer;
     int32_t* C;        // full table or NULL
-    uint8_t* A;        // argmin table or NULL
     int32_t* C_last;
     int32_t* status;
     int32_t* path;     // [4] device flags of the search: error, -, -, kernel that ran
-    int32_t* done;     // [B] 1: this instance needs nothing more
+    const int32_t* done;   // [B] instances that need nothing more, or NULL
 };
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
+// 3-D view of a table for the tensor-map store: [rows of S strategies per (instance, layer)][m_pitch / 32][32].
+// A CTA's slice [S][G][32] in shared memory is then one box.
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+// address of the same shared-memory location in the CTA of rank `rank` of this cluster
 __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ int ld_cluster(uint32_t addr) {
-    int v;
-    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
+__device__ __forceinline__ void st_cluster(uint32_t addr, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-__device__ __forceinline__ int ld_cluster_u8(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return (int)v;
+__device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();                                              // the aligned forms want the whole warp together
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// barrier of the CTA whose parties stand at different places in the code
-__device__ __forceinline__ void cta_barrier() {
-    __syncwarp();                                              // the aligned forms want the whole warp together
-    asm volatile("bar.sync 0;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_arrive() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-// an arrival that orders nothing: a release would wait for the table stores in flight
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-    __syncwarp();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void whole_barrier(int CL) {
-    if (CL == 1) cta_barrier();
-    else { cluster_arrive(); cluster_wait(); }
-}
-// One box [S][W / 32][32] from shared memory to element coordinates (0, g0, row0) of the table behind `map`, seen as
-// [rows][m_pitch / 32][32]; what lies beyond the tensor's edge (the last CTA's columns past m_pitch) is not written.
+// One box [S][G][32] from shared memory to element coordinates (0, g0, row0) of the table behind `map`;
+// what lies beyond the tensor's edge (the last CTA's columns past m_pitch) is not written.
 __device__ __forceinline__ void tensor_store_3d(const CUtensorMap* map, const void* src, int g0, int row0) {
     asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
                  ::"l"(map), "r"(0), "r"(g0), "r"(row0), "r"(smem_addr(src)) : "memory");
@@ -122,578 +92,84 @@ __device__ __forceinline__ void tensor_store_3d(const CUtensorMap* map, const vo
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// bytes of this CTA's shared memory to the same cluster's CTA that `dst` and `bar` lie in; counted on its mbarrier
-__device__ __forceinline__ void bulk_to_cta(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar) { asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory"); }
-__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
+
 __device__ __forceinline__ void cp_async_4(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ uint32_t mix(uint32_t v, uint32_t k) {
-    v = (v ^ (k * 0x9E3779B1u)) * 0x85EBCA6Bu;
-    v ^= v >> 15;
-    v *= 0xC2B2AE35u;
-    return v ^ (v >> 13);
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// What the push of one (column tile, strategy) needs, derived once per layer and CTA by the service warp.
+// Column m' of strategy s belongs at column m' + mem(l,s); for the tile that starts at this CTA's column colb:
+//   x = CTA of the cluster that receives the tile's first column (-1: nothing of the tile lands inside the budget),
+//   y = offset of that first column inside the receiving CTA's columns, z = time(l,s),
+//   w = kWholeTile when all nj*32 columns land in CTA x, else the largest offset that still lands inside the
+//       budget (the tile then straddles two CTAs or the budget's edge and every column is checked).
+// mem is clamped to M+1: nothing it shifts by lands inside the budget.  Pad strategies (s >= S) get x = -1.
+constexpr int kWholeTile = 0x7fffffff;
+__device__ __forceinline__ int4 tile_record(bool real, int mem, int time, int M, int W, int rank, int colb, int ncols) {
+    const int mc = mem < M + 1 ? mem : M + 1;
+    const int q = mc / W;
+    int d = rank + q, xb = colb + (mc - q * W);
+    if (xb >= W) { xb -= W; ++d; }
+    const int lim = M - d * W;
+    if (!real || lim < xb) return make_int4(-1, 0, time, 0);
+    const bool whole = xb + ncols <= W && xb + ncols - 1 <= lim;
+    return make_int4(d, xb, time, whole ? kWholeTile : lim);
+}
+// cells of this CTA's own columns that no column maps to (m < mem): written +inf
+__device__ __forceinline__ int fill_count(bool real, int mem, int M, int W, int rank) {
+    const int mc = mem < M + 1 ? mem : M + 1;
+    const int nf = mc - rank * W;
+    return !real ? 0 : (nf < 0 ? 0 : (nf > W ? W : nf));
 }
 
-// Everything the layer loop needs; lives in registers (all members are uniform over the CTA).
-struct Ctx {
-    int S, M, W, H, P, G, CL, rank, Li, m_pitch, Kr, Kc, tmax, SP, NW, gints;
-    int32_t* g0;               // [2][gints] state of this layer / the next: rows of P = H + W columns
-    uint8_t* a0;               // [2][gints] its argmin (argmin table only)
-    uint32_t rec;              // address of the per-layer records: four slots of 24 * S2 bytes
-    const int* slot;           // [4] the slot of layer l is slot[l & 3] (layers with the same rows share one)
-    int S2;                    // record entries a slot
-    int n_all;                 // strategies of a slot's records, pads included
-    const int* front;          // [4] no column below front[l & 3] holds a finite value in layer l
-    const int* reach;          // [4] largest shift of a slot's layer
-    const int32_t* tsm;        // transition entries: [16][16] by class, or [S][SP] (two of them with one matrix per layer)
-    int tmat;                  // entries of one full matrix when there is one per layer, else 0
-    const int* cs;             // [kClassMax + 1] first record of each class
-    const int* csp;            // [4][kClassMax + 1] the same in the list of the records that can matter
-    const int* cdelta;         // [16] cluster-window address of CTA d minus this CTA's own shared address
-    int32_t* stage;            // [2][S][W] collected rows
-    int32_t* C;                // this instance's table
-    uint8_t* A;
-    int32_t* C_last;
-    size_t slice;
-    uint32_t bars;             // address of the two mbarriers the halo's bytes are counted on (even, odd layers)
-    uint32_t halo_bytes;       // bytes of halo that arrive a layer
-    bool strict;               // some shift reaches beyond the halo: layers end with the full cluster barrier
-    int* late;                 // set when a bounded wait ran out
-};
-
-// End of a layer, by every warp of the CTA.  The state of layer l+1 is complete in this CTA; its last columns go to the
-// halo of the CTAs further up that hold them, one bulk copy (through the TMA unit) a row and CTA, the warps sharing the
-// rows: plain stores through the cluster window took about 100 cycles a warp store, 13 thousand a layer for 7 rows of
-// 608 columns.  Then the wait for this CTA's own halo.
-// The cluster barrier only keeps the buffers apart: an arrival says that this CTA has gathered from the older buffer
-// and received its halo, and it is waited for a layer later, before the copies that overwrite that buffer are issued.
-// With shifts beyond the halo other CTAs' state is read as well, and the barrier is waited for at once.
-constexpr int kWaitPolls = 1 << 20;                            // try_wait sleeps in hardware between polls: about a second
-template <bool ARG>
-__device__ __forceinline__ void send_halo(const Ctx& c, int l, int warp, int lane)
-{
-    cta_barrier();
-    if (c.CL == 1) return;
-    if (!c.strict) cluster_wait();
-    const uint32_t bar = c.bars + 8u * (l & 1);
-    if (warp == c.NW) {
-        const uint32_t gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints), an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // plain stores of the state, read next by bulk copies
-        for (int d = c.rank + 1, low = c.W - c.H; d < c.CL && low < c.W; ++d, low += c.W) {
-            // CTA d holds the columns from d*W - H on: this CTA's local columns from `low` on
-            const int from = max(low, 0), n = c.W - from, delta = c.cdelta[d];
-            const int at = c.H + from, to = at - (d - c.rank) * c.W;
-            for (int k = lane; k < c.Kc; k += 32) {
-                bulk_to_cta(gn + (uint32_t)(delta + (k * c.P + to) * 4), gn + (uint32_t)(k * c.P + at) * 4u, (uint32_t)n * 4u, bar + (uint32_t)delta);
-                if (ARG) bulk_to_cta(an + (uint32_t)(delta + k * c.P + to), an + (uint32_t)(k * c.P + at), (uint32_t)n, bar + (uint32_t)delta);
-            }
-        }
-    }
-}
-template <bool ARG>
-__device__ __forceinline__ void await_halo(const Ctx& c, int l, int warp, int lane)
-{
-    if (c.CL == 1) return;
-    const uint32_t bar = c.bars + 8u * (l & 1);
-    if (c.halo_bytes) {
-        if (warp == c.NW && lane == 0) mbar_expect(bar, c.halo_bytes);
-        const uint32_t parity = (uint32_t)(l >> 1) & 1u;
-        int polls = 0;
-        while (!mbar_try(bar, parity))
-            if (++polls > kWaitPolls || *(volatile int*)c.late) { *(volatile int*)c.late = 1; break; }
-    }
-    if (c.strict) { cluster_arrive(); cluster_wait(); }
-    else cluster_arrive_relaxed();
-}
-
-// Records of a layer, one entry per strategy in class order, three arrays of S2 entries each (a slot of the ring):
-//   int2 (x, time)  x = byte offset, from the start of the state, of the cell that column 0 of this CTA reads (the row of
-//                   the strategy's column class, shifted by mem); time = kInf where mem exceeds the budget (+inf row)
-//   int  row        byte offset of the strategy's row in the table
-//   int  who        mem | strategy << 24
-//   int2 (x, time)  of the strategies that can be the smallest of their class in some column: a strategy whose column
-//                   class, too, has a member that needs no more memory and no more time never is (G does not rise
-//                   with the budget).  ZeRO stages and checkpointing mostly differ in memory alone: about half drop out.
-// A class has an even number of entries (the last one may stand twice: it stores the same values again, and a minimum
-// does not change), so entries are read two to a 128-bit load, and four at a time from one address.
-// Shared-memory accesses of the layer loop go through 32-bit addresses and are written in batches, loads first: the table
-// stores between two strategies would otherwise hold the next strategy's loads back (they could alias for all the
-// compiler knows), and a strategy would cost the latency of its whole chain (220 cycles) instead of a share of it.
-__device__ __forceinline__ int lds(uint32_t a) {
-    int v;
-    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
-    return v;
-}
-template <int OFF>
-__device__ __forceinline__ int lds_at(uint32_t a) {
-    int v;
-    asm volatile("ld.shared.s32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(OFF));
-    return v;
-}
-__device__ __forceinline__ int lds_u8(uint32_t a) {
-    uint32_t v;
-    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
-    return (int)v;
-}
-__device__ __forceinline__ int4 lds4(uint32_t a) {
-    int4 v;
-    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-    return v;
-}
-__device__ __forceinline__ void sts(uint32_t a, int v) { asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
-__device__ __forceinline__ void sts_u8(uint32_t a, int v) { asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
-
-template <int OFF>
-__device__ __forceinline__ int4 lds4_at(uint32_t a) {
-    int4 v;
-    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4+%5];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a), "n"(OFF));
-    return v;
-}
-template <int TM, int J = 0>
-__device__ __forceinline__ void lds_row(uint32_t a, int (&g)[TM]) {
-    g[J] = lds_at<128 * J>(a);
-    if constexpr (J + 1 < TM) lds_row<TM, J + 1>(a, g);
-}
-
-// G at the columns that column `col` of this CTA (and those 32, 64, ... after it) reads; ga: the state's address plus
-// 4 * col.  FAR: the layer has shifts beyond the halo, whose cells are read from the CTA that owns them.
-template <int TM, bool FAR>
-__device__ __forceinline__ void gather(const Ctx& c, uint32_t ga, int x, int who, int col, int (&g)[TM])
-{
-    const int mem = who & 0xffffff;
-    if (!FAR || mem <= c.H) {
-        lds_row<TM>(ga + (uint32_t)x, g);
-    } else {
-        const uint32_t row = ga - 4u * (uint32_t)col + (uint32_t)x + (uint32_t)mem * 4u;
-#pragma unroll
-        for (int j = 0; j < TM; ++j) {
-            const int src = c.rank * c.W + col + 32 * j - mem;
-            const int o = src / c.W;
-            g[j] = kInf;
-            if (src >= 0 && col + 32 * j < c.W) g[j] = ld_cluster(row + (uint32_t)((src - o * c.W) * 4 + c.cdelta[o]));
-        }
-    }
-}
-// ... and their argmin entries; aa: the argmin state's address plus col
-template <int TM, bool FAR>
-__device__ __forceinline__ void gather_arg(const Ctx& c, uint32_t aa, int x, int who, int col, int (&a)[TM])
-{
-    const int mem = who & 0xffffff, off = x >> 2;
-    if (!FAR || mem <= c.H) {
-#pragma unroll
-        for (int j = 0; j < TM; ++j) a[j] = lds_u8(aa + (uint32_t)(off + 32 * j));
-    } else {
-        const uint32_t row = aa - (uint32_t)col + (uint32_t)(off + mem);
-#pragma unroll
-        for (int j = 0; j < TM; ++j) {
-            const int src = c.rank * c.W + col + 32 * j - mem;
-            const int o = src / c.W;
-            a[j] = 255;
-            if (src >= 0 && col + 32 * j < c.W) a[j] = ld_cluster_u8(row + (uint32_t)(src - o * c.W + c.cdelta[o]));
-        }
-    }
-}
-
-// Values of one state row for the tile.
-template <int TM, bool ARG>
-__device__ __forceinline__ void emit(const Ctx& c, uint32_t gn, uint32_t an, int k, int colb, int lane, const int (&v)[TM], const int (&a)[TM])
-{
-    const int at = k * c.P + c.H + colb + lane;
-#pragma unroll
-    for (int j = 0; j < TM; ++j) {
-        sts(gn + (uint32_t)(at + 32 * j) * 4u, v[j]);
-        if (ARG) sts_u8(an + (uint32_t)(at + 32 * j), a[j]);
-    }
-}
-
-// Where a tile's values go in the table.
-// STAGE: the rows of a layer are collected in shared memory ([S][W], two layers in turn) and leave with one bulk tensor
-// store the service warp issues.  A table store of a warp holds the load / store unit for four cycles and more, and the
-// loads of the next strategies, which the layer's chain of latencies consists of, queue up behind it.
-template <bool STORE, bool ARG, bool STAGE>
-struct Out {
-    uint32_t stage;        // the tile's first column plus this lane, strategy 0, in the collected rows
-    char* C;               // ... in the table
-    uint8_t* A;
-    bool whole;            // every column of the tile is a budget column
-    int cols;              // columns of the tile that exist in the table, less this lane
-    int budget;            // ... that are budget columns, less this lane
-    template <int TM>
-    __device__ __forceinline__ void put(uint32_t row, const int (&v)[TM], const int (&a)[TM]) const
-    {
-        if (STAGE) {
-#pragma unroll
-            for (int j = 0; j < TM; ++j) sts(stage + row + 128u * j, whole || 32 * j < budget ? v[j] : kInf);
-        } else if (STORE) {
-            int32_t* const p = reinterpret_cast<int32_t*>(C + row);
-            if (whole) {
-#pragma unroll
-                for (int j = 0; j < TM; ++j) p[32 * j] = v[j];
-            } else {                                           // +inf in the pad columns beyond the budget
-#pragma unroll
-                for (int j = 0; j < TM; ++j)
-                    if (32 * j < cols) p[32 * j] = 32 * j < budget ? v[j] : kInf;
-            }
-        }
-        if (ARG) {
-            uint8_t* const p = A + (row >> 2);
-#pragma unroll
-            for (int j = 0; j < TM; ++j)
-                if (whole || 32 * j < cols) p[32 * j] = (uint8_t)((whole || 32 * j < budget) && v[j] < kInf ? a[j] : 255);
-        }
-    }
-};
-
-// U entries' records, from entry address ra (of the (x, time) array) on.
-template <int U>
-struct Recs { int x[U], t[U], row[U], who[U]; };
-template <int U, bool ROW, bool WHO>
-__device__ __forceinline__ void fetch_recs(const Ctx& c, uint32_t ra, uint32_t rowa, Recs<U>& r)
-{
-    if constexpr (U >= 2) {
-        const int4 p = lds4_at<0>(ra);
-        r.x[0] = p.x; r.t[0] = p.y; r.x[1] = p.z; r.t[1] = p.w;
-        if constexpr (U == 4) {
-            const int4 q = lds4_at<16>(ra);
-            r.x[2 % U] = q.x; r.t[2 % U] = q.y; r.x[3 % U] = q.z; r.t[3 % U] = q.w;
-        }
-    } else {
-        r.x[0] = lds_at<0>(ra); r.t[0] = lds_at<4>(ra);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) { r.row[u] = 0; r.who[u] = 0; }
-    if (ROW) {
-        r.row[0] = lds_at<0>(rowa);
-        if constexpr (U >= 2) r.row[1 % U] = lds_at<4>(rowa);
-        if constexpr (U == 4) { r.row[2 % U] = lds_at<8>(rowa); r.row[3 % U] = lds_at<12>(rowa); }
-    }
-    if (WHO) {
-        const uint32_t w = rowa + 4u * c.S2;
-        r.who[0] = lds_at<0>(w);
-        if constexpr (U >= 2) r.who[1 % U] = lds_at<4>(w);
-        if constexpr (U == 4) { r.who[2 % U] = lds_at<8>(w); r.who[3 % U] = lds_at<12>(w); }
-    }
-}
-
-// U strategies: their C values to the table, their smallest into h (with ARG: whose it is).
-template <int U, int TM, bool STORE, bool ARG, bool STAGE, bool FAR>
-__device__ __forceinline__ void scan(const Ctx& c, const Out<STORE, ARG, STAGE>& out, uint32_t ra, uint32_t rowa, uint32_t ga, uint32_t aa, int col, int (&h)[TM], int (&hs)[TM])
-{
-    Recs<U> r;
-    int v[U][TM], a[ARG ? U : 1][TM];
-    fetch_recs<U, STORE || ARG, ARG || FAR>(c, ra, rowa, r);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        gather<TM, FAR>(c, ga, r.x[u], r.who[u], col, v[u]);
-        if (ARG) gather_arg<TM, FAR>(c, aa, r.x[u], r.who[u], col, a[ARG ? u : 0]);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-#pragma unroll
-        for (int j = 0; j < TM; ++j) {
-            if (STORE || ARG) {
-                v[u][j] = __viaddmin_s32(v[u][j], r.t[u], kInf);
-                if (ARG) hs[j] = v[u][j] < h[j] ? r.who[u] >> 24 : hs[j];  // ascending strategies: the lowest keeps a tie
-                h[j] = min(h[j], v[u][j]);
-            } else {
-                h[j] = __viaddmin_s32(v[u][j], r.t[u], h[j]);
-            }
-        }
-        if (STORE || ARG) out.template put<TM>((uint32_t)r.row[u], v[u], a[ARG ? u : 0]);
-    }
-}
-
-// Which of U strategies are alive in some column of the tile, as bits.
-template <int U, int TM, bool FAR>
-__device__ __forceinline__ uint32_t alive(const Ctx& c, uint32_t ra, uint32_t rowa, uint32_t ga, int col, const int (&thr)[TM])
-{
-    Recs<U> r;
-    int v[U][TM];
-    uint32_t bits = 0;
-    fetch_recs<U, false, FAR>(c, ra, rowa, r);
-#pragma unroll
-    for (int u = 0; u < U; ++u) gather<TM, FAR>(c, ga, r.x[u], r.who[u], col, v[u]);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        bool live = false;
-#pragma unroll
-        for (int j = 0; j < TM; ++j) live = live || __viaddmin_s32(v[u][j], r.t[u], kInf) <= thr[j];
-        if (__any_sync(0xffffffffu, live)) bits |= 1u << u;
-    }
-    return bits;
-}
-
-// One layer of one tile of TM x 32 columns.  KC: rows of the next state held in accumulators (PRUNE: per block of rows).
-template <int KC, int TM, bool PRUNE, bool STORE, bool ARG, bool STAGE, bool FAR>
-__device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
-{
-    const int slot = c.slot[l & 3], col = colb + lane;
-    const uint32_t ra = c.rec + (uint32_t)(slot * c.S2) * 24u, rowa = ra + (uint32_t)c.S2 * 8u;
-    const uint32_t ga = smem_addr(c.g0 + (l & 1) * c.gints + col), gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints);
-    const uint32_t aa = ARG ? smem_addr(c.a0 + (l & 1) * c.gints + col) : 0u, an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
-    const int colg = c.rank * c.W + colb;                      // the tile's first budget column
-    Out<STORE, ARG, STAGE> out;
-    out.stage = STAGE ? smem_addr(c.stage + (l & 1) * c.S * c.W + col) : 0u;
-    out.C = STORE ? reinterpret_cast<char*>(c.C + (size_t)l * c.slice + colg + lane) : nullptr;
-    out.A = ARG ? c.A + (size_t)l * c.slice + colg + lane : nullptr;
-    out.whole = colg + 32 * TM - 1 <= c.M;
-    out.cols = c.m_pitch - colg - lane;
-    out.budget = c.M + 1 - colg - lane;
-
-    if (colg + 32 * TM - 1 < c.front[l & 3]) {                  // nothing finite in the tile
-        int inf[TM], none[TM];
-#pragma unroll
-        for (int j = 0; j < TM; ++j) { inf[j] = kInf; none[j] = 255; }
-        if (STORE || ARG)
-#pragma unroll 4
-            for (int e = 0; e < c.S; ++e) out.template put<TM>((uint32_t)(e * (STAGE ? c.W : c.m_pitch)) * 4u, inf, none);
-        for (int k = 0; k < c.Kc; ++k) emit<TM, ARG>(c, gn, an, k, colb, lane, inf, none);
-        return;
-    }
-
-    if (!PRUNE) {
-        int acc[KC][TM], arg[ARG ? KC : 1][TM];
-#pragma unroll
-        for (int k = 0; k < KC; ++k)
-#pragma unroll
-            for (int j = 0; j < TM; ++j) { acc[k][j] = kInf; if (ARG) arg[k][j] = 255; }
-        int e = 0;
-        // without a table to write, only the strategies that can matter
-        constexpr bool kAll = STORE || ARG || FAR;
-        const int* const cs = kAll ? c.cs : c.csp + slot * (kClassMax + 1);
-        const uint32_t la = kAll ? ra : ra + (uint32_t)c.S2 * 16u;
-        const uint32_t ta = smem_addr(c.tsm);
-        for (int k = 0; k < c.Kr; ++k) {
-            const int end = cs[k + 1];
-            int h[TM], hs[TM];
-#pragma unroll
-            for (int j = 0; j < TM; ++j) { h[j] = kInf; hs[j] = 255; }
-            int4 t4[KC / 4];
-#pragma unroll
-            for (int q = 0; q < KC / 4; ++q) t4[q] = lds4(ta + (uint32_t)(k * kClassMax + 4 * q) * 4u);
-            constexpr int U = FAR ? 1 : TM > 4 && STORE ? 2 : 4;
-            for (; e + U <= end; e += U) scan<U, TM, STORE, ARG, STAGE, FAR>(c, out, la + 8u * e, rowa + 4u * e, ga, aa, col, h, hs);
-            if (U == 4 && e < end) { scan<2, TM, STORE, ARG, STAGE, FAR>(c, out, la + 8u * e, rowa + 4u * e, ga, aa, col, h, hs); e += 2; }
-#pragma unroll
-            for (int q = 0; q < KC / 4; ++q) {
-                const int t[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
-#pragma unroll
-                for (int j = 0; j < TM; ++j)
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        if (ARG) {
-                            const int cand = h[j] + t[u], old = acc[4 * q + u][j], oa = arg[ARG ? 4 * q + u : 0][j];
-                            const bool better = cand < old || (cand == old && hs[j] < oa);
-                            if (better && h[j] < kInf) { acc[4 * q + u][j] = cand; arg[ARG ? 4 * q + u : 0][j] = hs[j]; }
-                        } else {
-                            acc[4 * q + u][j] = __viaddmin_s32(h[j], t[u], acc[4 * q + u][j]);
-                        }
-                    }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < KC; ++k)
-            if (k < c.Kc) emit<TM, ARG>(c, gn, an, k, colb, lane, acc[k], arg[ARG ? k : 0]);
-    } else {
-        int thr[TM], dummy[TM];
-#pragma unroll
-        for (int j = 0; j < TM; ++j) { thr[j] = kInf; dummy[j] = 255; }
-        int s = 0;
-        if (!FAR)
-            for (; s + 4 <= c.S; s += 4) scan<4, TM, STORE, ARG, STAGE, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
-        for (; s < c.S; ++s) scan<1, TM, STORE, ARG, STAGE, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
-        // a candidate beyond the column's best plus the largest entry cannot win; a column without a finite value
-        // keeps nothing alive
-#pragma unroll
-        for (int j = 0; j < TM; ++j) thr[j] = thr[j] < kInf ? thr[j] + c.tmax : -1;
-        uint32_t live[kMaxS / 32];
-#pragma unroll
-        for (int b = 0; b < kMaxS / 32; ++b) {
-            live[b] = 0;
-            if (32 * b < c.S) {
-                const int n = min(32, c.S - 32 * b);
-                int q = 0;
-                if (!FAR)
-                    for (; q + 4 <= n; q += 4) live[b] |= alive<4, TM, FAR>(c, ra + 8u * (32 * b + q), rowa + 4u * (32 * b + q), ga, col, thr) << q;
-                for (; q < n; ++q) live[b] |= alive<1, TM, FAR>(c, ra + 8u * (32 * b + q), rowa + 4u * (32 * b + q), ga, col, thr) << q;
-            }
-        }
-        const uint32_t ta = smem_addr(c.tsm + (((l + 1) & 1) ? c.tmat : 0));
-        for (int cb = 0; cb < c.S; cb += KC) {
-            int acc[KC][TM], arg[ARG ? KC : 1][TM];
-#pragma unroll
-            for (int k = 0; k < KC; ++k)
-#pragma unroll
-                for (int j = 0; j < TM; ++j) { acc[k][j] = kInf; if (ARG) arg[k][j] = 255; }
-#pragma unroll
-            for (int b = 0; b < kMaxS / 32; ++b)
-                for (uint32_t m = live[b]; m; m &= m - 1) {
-                    const int q = 32 * b + __ffs(m) - 1;
-                    Recs<1> r;
-                    fetch_recs<1, false, FAR>(c, ra + 8u * q, rowa + 4u * q, r);
-                    const uint32_t t0 = ta + (uint32_t)(q * c.SP + cb) * 4u;
-                    int v[TM];
-                    gather<TM, FAR>(c, ga, r.x[0], r.who[0], col, v);
-#pragma unroll
-                    for (int j = 0; j < TM; ++j) v[j] = __viaddmin_s32(v[j], r.t[0], kInf);
-#pragma unroll
-                    for (int w = 0; w < KC / 4; ++w) {
-                        const int4 t4 = lds4(t0 + 16u * w);
-                        const int t[4] = {t4.x, t4.y, t4.z, t4.w};
-#pragma unroll
-                        for (int j = 0; j < TM; ++j)
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                if (ARG) {
-                                    const int cand = v[j] + t[u];
-                                    if (v[j] < kInf && cand < acc[4 * w + u][j]) { acc[4 * w + u][j] = cand; arg[ARG ? 4 * w + u : 0][j] = q; }
-                                } else {
-                                    acc[4 * w + u][j] = __viaddmin_s32(v[j], t[u], acc[4 * w + u][j]);
-                                }
-                            }
-                    }
-                }
-#pragma unroll
-            for (int k = 0; k < KC; ++k)
-                if (cb + k < c.S) emit<TM, ARG>(c, gn, an, cb + k, colb, lane, acc[k], arg[ARG ? k : 0]);
-        }
-    }
-}
-
-// The last layer hands nothing on: its values go to the table and to C_last.
-template <bool STORE, bool ARG, bool STAGE, bool FAR>
-__device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lane)
-{
-    const uint32_t sa = STAGE ? smem_addr(c.stage + (l & 1) * c.S * c.W + colb + lane) : 0u;
-    const int slot = c.slot[l & 3], col = colb + lane;
-    const uint32_t ra = c.rec + (uint32_t)(slot * c.S2) * 24u, rowa = ra + (uint32_t)c.S2 * 8u, ga = smem_addr(c.g0 + (l & 1) * c.gints + col);
-    const uint32_t aa = ARG ? smem_addr(c.a0 + (l & 1) * c.gints + col) : 0u;
-    const int colg = c.rank * c.W + colb, m = colg + lane;
-    if (colg >= c.m_pitch) return;                             // m_pitch is a multiple of 32: a group exists whole or not at all
-    const bool pad = m > c.M;
-    auto steps = [&](auto count, int e) {
-        constexpr int U = decltype(count)::value;
-        Recs<U> r;
-        int g[U][1], a[U][1];
-        fetch_recs<U, true, ARG || FAR>(c, ra + 8u * e, rowa + 4u * e, r);
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            gather<1, FAR>(c, ga, r.x[u], r.who[u], col, g[u]);
-            if (ARG) gather_arg<1, FAR>(c, aa, r.x[u], r.who[u], col, a[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int v = pad ? kInf : __viaddmin_s32(g[u][0], r.t[u], kInf);
-            if (STAGE) { sts(sa + (uint32_t)r.row[u], v); continue; }
-            const size_t row = ((uint32_t)r.row[u] >> 2) + (size_t)m;
-            if (STORE) c.C[(size_t)l * c.slice + row] = v;
-            c.C_last[row] = v;
-            if (ARG) c.A[(size_t)l * c.slice + row] = (uint8_t)(v < kInf ? a[u][0] : 255);
-        }
-    };
-    int e = 0;
-    if (!FAR)
-        for (; e + 4 <= c.n_all; e += 4) steps(std::integral_constant<int, 4>(), e);
-    for (; e < c.n_all; ++e) steps(std::integral_constant<int, 1>(), e);
-}
-
-// `n` column groups from group g on, as one tile.
-template <int KC, int MAX, bool PRUNE, bool STORE, bool ARG, bool STAGE>
-__device__ __forceinline__ void tile_of(const Ctx& c, int l, int g, int n, int lane)
-{
-    if constexpr (MAX > 1) {
-        if (n < MAX) { tile_of<KC, MAX - 1, PRUNE, STORE, ARG, STAGE>(c, l, g, n, lane); return; }
-    }
-    tile<KC, MAX, PRUNE, STORE, ARG, STAGE, false>(c, l, g * 32, lane);
-}
-
-// A warp owns a run of column groups (the warps' runs differ by one group at most) and takes it as one tile, or as
-// several of about the same width when it is wider than MAX groups: a record fetched once serves them all.
-template <int KC, int MAX, bool PRUNE, bool STORE, bool ARG, bool STAGE>
-__device__ __forceinline__ void run_layers(const Ctx& c, int warp, int lane)
-{
-    const int g0 = c.G * warp / c.NW, g1 = c.G * (warp + 1) / c.NW;
-    for (int l = 0; l + 1 < c.Li; ++l) {
-        int g = g0;
-        if (c.reach[c.slot[l & 3]] <= c.H) {
-            for (int left = (g1 - g0 + MAX - 1) / MAX; left > 0; --left) {
-                const int n = (g1 - g + left - 1) / left;
-                tile_of<KC, MAX, PRUNE, STORE, ARG, STAGE>(c, l, g, n, lane);
-                g += n;
-            }
-        } else {
-            for (; g < g1; ++g) tile<KC, 1, PRUNE, STORE, ARG, STAGE, true>(c, l, g * 32, lane);
-        }
-        send_halo<ARG>(c, l, warp, lane);
-        await_halo<ARG>(c, l, warp, lane);
-    }
-    if (c.reach[c.slot[(c.Li - 1) & 3]] <= c.H) {
-        for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, STAGE, false>(c, c.Li - 1, g * 32, lane);
-    } else {
-        for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, STAGE, true>(c, c.Li - 1, g * 32, lane);
-    }
-}
-
-// Cluster c takes instance c (the c-th longest when `sorted`).  Warps 0..NW-1 compute, the last warp fetches the
-// layers' mem / time rows (and with one matrix per layer the matrices) ahead and turns them into records.
-template <bool STORE, bool ARG, bool STAGE>
-__global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const RsArgs a, const __grid_constant__ CUtensorMap map_c,
-                                                                           const __grid_constant__ CUtensorMap map_last)
+// One cluster per instance (cluster c takes the c-th longest when `sorted`), CTA `rank` of the cluster owns
+// budget columns rank*W .. rank*W+W-1.  Dynamic shared memory: two buffers [S][W] of table values (previous
+// and next layer, swapping), the transition matrix [S][SP8] (two of them with one matrix per layer), the push
+// records of this layer and the next (one per column tile and strategy), the fill counts, and a dump row for the
+// stores of strategies that land nowhere.  Warps 0..NW-1 compute: warp w takes work units w, w+NW, ...; a unit is
+// 32*TM columns x 8 strategies, one fused add-min per relaxation, accumulators in registers.  The last warp
+// is the service warp: it sends the finished layer to the table (one tensor-map store), prepares the next
+// layer's records and, with one matrix per layer, fetches the next matrix.
+template <int TM>
+__global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, const __grid_constant__ CUtensorMap map_c,
+                                                                const __grid_constant__ CUtensorMap map_last)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ union { int L[kMaxSortedB]; struct { uint32_t rh[kMaxS], ch[kMaxS]; } h; } s_u;
-    __shared__ int s_rrep[kMaxS], s_crep[kMaxS], s_rcls[kMaxS], s_ccls[kMaxS], s_order[kMaxS + kClassMax], s_csp[4 * (kClassMax + 1)], s_first[kClassMax + 1], s_cnt[kClassMax];
-    __shared__ int s_cdelta[16], s_front[4], s_reach[4], s_slot[4], s_inst, s_K[2];
-    __shared__ struct { long long sum; int tmax, bad, mmax; } s_part, s_all;
-    __shared__ __align__(8) unsigned long long s_bar[2];
-    __shared__ int s_late;
+    __shared__ int s_L[kMaxSortedB];
+    __shared__ int s_inst, s_tmax, s_bad;
+    __shared__ long long s_sum;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x, NW = (NT >> 5) - 1;
-    const int CL = a.CL, rank = CL > 1 ? (int)cluster_rank() : 0, cid = blockIdx.x / CL;
-    const int S = a.S, M = a.M, W = a.W, Lmax = a.Lmax, gints = a.gints;
+    const int CL = a.CL, rank = (int)cluster_rank(), cid = blockIdx.x / CL;
+    const int S = a.S, M = a.M, W = a.W, SP8 = a.SP8, Lmax = a.Lmax;
 
-    // ---- shared memory
-    int32_t* const g0 = reinterpret_cast<int32_t*>(smem_raw);                              // [2][gints]
-    const int tfull = S * a.SP;
-    int32_t* const tsm = g0 + 2 * gints;                                                   // [16][16] or [1|2][S][SP]
-    const int tints = max(kClassMax * kClassMax, (a.trans_layer ? 2 : 1) * tfull);
-    const int S2 = (S + kClassMax + 3) & ~3;
-    int32_t* const rec = tsm + tints;                                                      // [4] slots of S2 x (int2, int, int, int2)
-    int32_t* const raw = rec + 4 * 6 * S2;                                                 // [4][2][S] mem, time rows as they come
-    int32_t* const stage_rows = reinterpret_cast<int32_t*>(smem_raw) + a.stage_at;         // [2][S][W] rows on their way to the table
-    uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * ((S + 3) & ~3));                           // [2][gints] argmin of the state
+    int32_t* const buf0 = reinterpret_cast<int32_t*>(smem_raw);
+    int32_t* const buf1 = buf0 + S * W;
+    int32_t* const tsm = buf1 + S * W;
+    const int tmat = S * SP8;
+    const int nrec = a.nct * SP8;
+    int4* const rows = reinterpret_cast<int4*>(tsm + (a.trans_layer ? 2 : 1) * tmat);     // [2][nct][SP8] push records
+    int* const fillc = reinterpret_cast<int*>(rows + 2 * nrec);                            // [2][SP8] leading cells of each row to fill with +inf
+    int* const fillmax = fillc + 2 * SP8;                                                  // [2] the largest of them (padded to 4 ints)
+    int32_t* const dump = fillmax + 4;                                                     // [32 * TM] where stores of skipped strategies go
+    int* const cdelta = dump + 32 * TM;                                                    // [16] cluster-window address of CTA d minus this CTA's own shared address
 
-    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = a.path_value; }
+    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = 2; }      // no error flag to raise; the cluster kernel ran
 
     // ---- which instance: clusters are dispatched in order, so the longest instances go first
     int i = cid;
     if (a.sorted) {
         for (int j = tid; j < a.B; j += NT) {
             const int v = a.L[j];
-            s_u.L[j] = (v < 1 || v > Lmax) ? 0 : v;
+            s_L[j] = (v < 1 || v > Lmax) ? 0 : v;
         }
         __syncthreads();
         for (int j = tid; j < a.B; j += NT) {
-            const int Lj = s_u.L[j];
+            const int Lj = s_L[j];
             int before = 0;
             for (int k = 0; k < a.B; ++k) {
-                const int Lk = s_u.L[k];
+                const int Lk = s_L[k];
                 before += (Lk > Lj) || (Lk == Lj && k < j);
             }
             if (before == cid) s_inst = j;
@@ -701,406 +177,274 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
         __syncthreads();
         i = s_inst;
     }
-    if (a.second && a.done[i]) return;
+
+    if (a.done && a.done[i]) return;
+    // ---- validation (every CTA of the cluster comes to the same result: nobody is left waiting at a barrier)
+    if (tid == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; }
+    __syncthreads();
     const int Li = a.L[i];
     if (Li < 1 || Li > Lmax) {
-        if (rank == 0 && tid == 0) { a.status[i] = GALV_STATUS_BAD_INPUT; a.done[i] = 1; }
+        if (rank == 0 && tid == 0) a.status[i] = GALV_STATUS_BAD_INPUT;
         return;
     }
     const int32_t* const tq = a.time_q + (size_t)i * Lmax * S;
     const int32_t* const mq = a.mem_q + (size_t)i * Lmax * S;
     const int32_t* const T0 = a.trans_q + (size_t)i * a.trans_inst;
-
-    // ---- validation: the CTAs of the cluster share the layers (and matrices); one matrix per instance is staged whole
-    int32_t* const stage = g0;                                 // the state is not in use yet
-    const bool staged = !a.trans_layer && (long long)S * S <= (long long)2 * gints;
-    if (tid == 0) { s_part.sum = 0; s_part.tmax = 0; s_part.bad = 0; s_part.mmax = 0; }
-    for (int x = tid; x < kMaxS; x += NT) { s_u.h.rh[x] = 0; s_u.h.ch[x] = 0; }
-    if (tid == 0) {
-        s_late = 0;
-        mbar_init(smem_addr(&s_bar[0])); mbar_init(smem_addr(&s_bar[1]));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (tid < 16) s_cdelta[tid] = CL > 1 ? (int)(map_to_rank(smem_addr(g0), (uint32_t)min(tid, CL - 1)) - smem_addr(g0)) : 0;
-    __syncthreads();
     {
         long long sum = 0;
-        int bad = 0, tmax = 0, mmax = 0;                        // mmax: the largest shift that stays inside the budget
-        for (int l = rank * (NW + 1) + warp; l < Li; l += CL * (NW + 1)) {      // a warp per layer: largest time of the layer
+        int bad = 0, tmax = 0;
+        for (int l = warp; l < Li; l += NW + 1) {             // a warp per layer: largest time of the layer
             int mx = 0;
             for (int s = lane; s < S; s += 32) {
                 const int tv = tq[l * S + s], mv = mq[l * S + s];
                 bad |= (tv < 0) | (mv < 0);
                 mx = max(mx, tv);
-                mmax = max(mmax, mv <= M ? mv : 0);
             }
             mx = __reduce_max_sync(0xffffffffu, mx);
             if (lane == 0) sum += mx;
         }
-        if (a.trans_layer) {
-            const long long nx = (long long)(Li - 1) * S * S;                     // matrix 0 is unused
-            const int32_t* const x = T0 + (size_t)S * S;
-#pragma unroll 4
-            for (long long k = (long long)rank * NT + tid; k < nx; k += (long long)CL * NT) {
-                const int v = x[k];
-                bad |= v < 0;
-                tmax = max(tmax, v);
-            }
-        } else {
-#pragma unroll 4
-            for (int k = tid; k < S * S; k += NT) {
-                const int v = T0[k];
-                bad |= v < 0;
-                tmax = max(tmax, v);
-                if (staged) stage[k] = v;
-            }
+        const int xl0 = a.trans_layer ? 1 : 0, xl1 = a.trans_layer ? Li : 1;       // matrices in use
+        const long long nx = (long long)(xl1 - xl0) * S * S;
+        const int32_t* x = T0 + (size_t)xl0 * S * S;
+        for (long long k = tid; k < nx; k += NT) {
+            const int v = x[k];
+            bad |= (v < 0);
+            tmax = max(tmax, v);
         }
         tmax = __reduce_max_sync(0xffffffffu, tmax);
-        mmax = __reduce_max_sync(0xffffffffu, mmax);
         bad = __any_sync(0xffffffffu, bad != 0);
         if (lane == 0) {
-            if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(&s_part.sum), static_cast<unsigned long long>(sum));
-            atomicMax(&s_part.tmax, tmax);
-            atomicMax(&s_part.mmax, mmax);
-            if (bad) atomicOr(&s_part.bad, 1);
+            if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(&s_sum), static_cast<unsigned long long>(sum));
+            atomicMax(&s_tmax, tmax);
+            if (bad) atomicOr(&s_bad, 1);
         }
     }
-    whole_barrier(CL);
-    if (warp == 0) {
-        long long sum = 0;
-        int tmax = 0, bad = 0, mmax = 0;
-        if (CL == 1) {
-            sum = s_part.sum; tmax = s_part.tmax; bad = s_part.bad; mmax = s_part.mmax;
-        } else {
-            if (lane < CL) {
-                const uint32_t p = map_to_rank(smem_addr(&s_part), (uint32_t)lane);
-                sum = (long long)(((unsigned long long)(uint32_t)ld_cluster(p + 4) << 32) | (uint32_t)ld_cluster(p));
-                tmax = ld_cluster(p + 8);
-                bad = ld_cluster(p + 12);
-                mmax = ld_cluster(p + 16);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            tmax = __reduce_max_sync(0xffffffffu, tmax);
-            mmax = __reduce_max_sync(0xffffffffu, mmax);
-            bad = __any_sync(0xffffffffu, bad != 0);
-        }
-        if (lane == 0) { s_all.sum = sum; s_all.tmax = tmax; s_all.bad = bad; s_all.mmax = mmax; }
+    __syncthreads();
+    {
+        int st = 0;
+        if (s_bad) st = GALV_STATUS_BAD_INPUT;
+        else if (s_sum + (long long)(Li - 1) * s_tmax >= (long long)kInf) st = GALV_STATUS_OVERFLOW_RISK;
+        if (rank == 0 && tid == 0) a.status[i] = st;
+        if (st) return;                                        // flagged: tables left untouched
     }
 
-    // ---- classes of equal rows and equal columns
-    int K = S;                                                  // unstructured unless found otherwise
-    if (staged) {
-        // a sum of mixed words per row and per column proposes twins ...
-        for (int r = warp; r < S; r += NW + 1) {
-            uint32_t h = 0;
-            for (int s = lane; s < S; s += 32) h += mix((uint32_t)stage[r * S + s], (uint32_t)s);
-            h = __reduce_add_sync(0xffffffffu, h);
-            if (lane == 0) s_u.h.rh[r] = h;
-        }
-        const int parts = max(1, NT / S);
-        for (int x = tid; x < parts * S; x += NT) {
-            const int s = x % S, p = x / S;
-            uint32_t h = 0;
-            for (int r = p; r < S; r += parts) h += mix((uint32_t)stage[r * S + s], (uint32_t)r);
-            atomicAdd(&s_u.h.ch[s], h);
-        }
-        __syncthreads();
-        for (int x = tid; x < 2 * S; x += NT) {
-            const uint32_t* const hh = x < S ? s_u.h.rh : s_u.h.ch;
-            const int s = x < S ? x : x - S;
-            int o = 0;
-            while (hh[o] != hh[s]) ++o;                         // ends at s itself at the latest
-            (x < S ? s_rrep : s_crep)[s] = o;
-            (x < S ? s_rcls : s_ccls)[s] = 0;                   // for now: words that differ
-        }
-        __syncthreads();
-        // ... and a comparison of all their words decides
-        for (int r = warp; r < S; r += NW + 1) {
-            const int o = s_rrep[r];
-            int diff = 0;
-            for (int s = lane; s < S; s += 32) diff |= stage[r * S + s] != stage[o * S + s];
-            if (__any_sync(0xffffffffu, diff) && lane == 0) s_rcls[r] = 1;
-        }
-        for (int x = tid; x < parts * S; x += NT) {
-            const int s = x % S, p = x / S, o = s_crep[s];
-            int diff = 0;
-            for (int r = p; r < S; r += parts) diff |= stage[r * S + s] != stage[r * S + o];
-            if (diff) s_ccls[s] = 1;
-        }
-        __syncthreads();
-        for (int s = tid; s < S; s += NT) {
-            if (s_rcls[s]) s_rrep[s] = s;
-            if (s_ccls[s]) s_crep[s] = s;
-        }
-        __syncthreads();
-        // class numbers in the order of the classes' first members
-        for (int x = tid; x < 2 * S; x += NT) {
-            const int* const rep = x < S ? s_rrep : s_crep;
-            const int s = x < S ? x : x - S, me = rep[s];
-            int k = 0;
-            for (int o = 0; o < me; ++o) k += rep[o] == o;
-            (x < S ? s_rcls : s_ccls)[s] = k;
-        }
-        if (warp < 2) {                                         // there are at least two warps
-            const int* const rep = warp == 0 ? s_rrep : s_crep;
-            int k = 0;
-            for (int s = lane; s < S; s += 32) k += rep[s] == s;
-            k = __reduce_add_sync(0xffffffffu, k);
-            if (lane == 0) s_K[warp] = k;
-        }
-        __syncthreads();
-        K = max(s_K[0], s_K[1]);
-    }
-    const bool classes = staged && K <= kClassMax && s_K[1] * W <= gints;
-    const bool dense = !classes && a.SP > 0 && S * W <= gints;
-    const int Kr = classes ? s_K[0] : S, Kc = classes ? s_K[1] : S;
-    if (classes) {
-        // strategies in class order, ascending inside a class; a class of an odd number has its last one twice
-        for (int k = tid; k <= Kr; k += NT) s_first[k] = 0;
-        __syncthreads();
-        for (int s = tid; s < S; s += NT) atomicAdd(&s_first[s_rcls[s]], 1);
-        __syncthreads();
-        if (warp == 0) {
-            const int n = lane < Kr ? s_first[lane] : 0;
-            int at = (n + 1) & ~1;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, at, o);
-                if (lane >= o) at += v;
-            }
-            if (lane < Kr) { s_first[lane] = at - ((n + 1) & ~1); s_cnt[lane] = n; }
-            if (lane == Kr - 1) s_first[Kr] = at;
-        }
-        __syncthreads();
-        for (int s = tid; s < S; s += NT) {
-            const int me = s_rcls[s];
-            int before = 0, size = 0;
-            for (int o = 0; o < S; ++o) { size += s_rcls[o] == me; before += s_rcls[o] == me && o < s; }
-            s_order[s_first[me] + before] = s;
-            if (before == size - 1 && (size & 1)) s_order[s_first[me] + size] = s;
-        }
-        for (int x = tid; x < kClassMax * kClassMax; x += NT) tsm[x] = 0;
-        __syncthreads();
-        for (int r = warp; r < S; r += NW + 1)
-            if (s_rrep[r] == r)
-                for (int s = lane; s < S; s += 32)
-                    if (s_crep[s] == s) tsm[s_rcls[r] * kClassMax + s_ccls[s]] = stage[r * S + s];
-    } else if (dense) {
-        for (int s = tid; s < S; s += NT) { s_order[s] = s; s_ccls[s] = s; }
-        // the matrix paid between layers 0 and 1; with one matrix per layer, matrix l sits in buffer l & 1
-        const int32_t* const T = T0 + (a.trans_layer ? a.trans_layer : 0);
-        int32_t* const dst = tsm + (a.trans_layer ? tfull : 0);
-        for (int x = tid; x < tfull; x += NT) {
-            const int r = x / a.SP, s = x - r * a.SP;
-            const int v = (s < S && Li > 1) ? (staged ? stage[r * S + s] : T[r * S + s]) : 0;
-            dst[x] = v;
-            if (a.trans_layer) tsm[x] = 0;                      // pad columns of the other buffer stay 0
-        }
-    }
-    int st = 0;
-    __syncthreads();                                            // s_all, classes; the staged matrix is no longer read
-    if (s_all.bad) st = GALV_STATUS_BAD_INPUT;
-    else if (s_all.sum + (long long)(Li - 1) * s_all.tmax >= (long long)kInf) st = GALV_STATUS_OVERFLOW_RISK;
-    const bool run = st == 0 && (classes || dense);
-    if (rank == 0 && tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run; }
+    const int col_g0 = rank * W;                               // first budget column of this CTA
 
-    // The halo: columns left of this CTA's own that its gathers reach, as many as the largest shift asks for or as fit;
-    // a multiple of 32.  Below column 0 it holds +inf.
-    const int H = max(0, min((s_all.mmax + 31) & ~31, (gints / Kc - W) & ~31)), P = W + H;
-
-    const int n_all = classes ? s_first[Kr] : S;
-    const bool strict = s_all.mmax > H;                         // some shift reaches beyond the halo
-    // ---- layer 0 gathers from an all-zero state: C[0] = time where mem fits
-    auto prepare = [&](int l, int base) -> int {                // records of layer l by one warp; returns the new frontier
-        const int32_t* const rm = raw + (l & 3) * 2 * S;
-        // a layer with the rows of one of the two before it takes that one's records
-        int slot = -1, least = M + 1;
-        for (int back = 1; back <= 2 && back <= l && slot < 0; ++back) {
-            const int32_t* const ro = raw + ((l - back) & 3) * 2 * S;
-            int diff = 0;
-            for (int x = lane; x < 2 * S; x += 32) diff |= rm[x] != ro[x];
-            if (!__any_sync(0xffffffffu, diff)) slot = s_slot[(l - back) & 3];
+    // ---- layer 0, the records of layer 1, the transition matrix
+    // the push records and fill count of strategy s (raw mem / time given) into half `h` of the two arrays
+    auto prepare_one = [&](int h, int s, int mem, int time) -> int {                       // returns the row's fill count
+        const bool real = s < S;
+        const int nf = fill_count(real, mem, M, W, rank);
+        fillc[h * SP8 + s] = nf;
+        for (int ct = 0; ct < a.nct; ++ct) {
+            const int left = a.G - ct * TM;
+            rows[h * nrec + ct * SP8 + s] = tile_record(real, mem, time, M, W, rank, ct * 32 * TM, 32 * (left < TM ? left : TM));
         }
-        if (slot < 0) {
-            // not one of the three layers before: the oldest may still be on its way to the table
-            unsigned used = 0;
-            for (int back = 1; back <= 3 && back <= l; ++back) used |= 1u << s_slot[(l - back) & 3];
-            slot = __ffs(~used) - 1;
-            int32_t* const rs = rec + slot * 6 * S2;
-            int most = 0;
-            for (int e = lane; e < n_all; e += 32) {
-                const int s = s_order[e];
-                const int mem = rm[s];
-                const bool fits = mem <= M;                     // else +inf everywhere: no shift, time +inf
-                const int shift = fits ? mem : 0;
-                reinterpret_cast<int2*>(rs)[e] = make_int2((s_ccls[s] * P + H - shift) * 4, fits ? rm[S + s] : kInf);
-                rs[2 * S2 + e] = s * (STAGE ? W : a.m_pitch) * 4;
-                rs[3 * S2 + e] = shift | (s << 24);
-                most = max(most, shift);
-            }
-            most = __reduce_max_sync(0xffffffffu, most);
-            if (lane == 0) s_reach[slot] = most;
-            if (classes && !STORE && !ARG) {
-                // the strategies that can matter, class by class
-                __syncwarp();
-                int2* const keep = reinterpret_cast<int2*>(rs + 4 * S2);
-                const int2* const all = reinterpret_cast<const int2*>(rs);
-                int at = 0;
-                for (int k = 0; k < Kr; ++k) {
-                    if (lane == 0) s_csp[slot * (kClassMax + 1) + k] = at;
-                    const int first = s_first[k], n = s_cnt[k];
-                    int2 lastkept = make_int2(0, 0);
-                    int kept = 0;
-                    for (int b = 0; b < n; b += 32) {
-                        const int p = b + lane;
-                        bool in = p < n;
-                        int2 me = make_int2(0, kInf);
-                        if (in) {
-                            me = all[first + p];
-                            in = me.y < kInf;
-                            const int mm = rm[s_order[first + p]], mc = s_ccls[s_order[first + p]];
-                            for (int q = 0; q < n && in; ++q) {
-                                const int so = s_order[first + q];
-                                const int om = rm[so], ot = rm[S + so];
-                                if (s_ccls[so] == mc && om <= mm && ot <= me.y && (om < mm || ot < me.y || q < p)) in = false;
-                            }
-                        }
-                        const unsigned b1 = __ballot_sync(0xffffffffu, in);
-                        if (in) keep[at + kept + __popc(b1 & ((1u << lane) - 1))] = me;
-                        if (b1) {
-                            const int src = 31 - __clz(b1);
-                            lastkept.x = __shfl_sync(0xffffffffu, me.x, src);
-                            lastkept.y = __shfl_sync(0xffffffffu, me.y, src);
-                        }
-                        kept += __popc(b1);
-                    }
-                    if ((kept & 1) && lane == 0) keep[at + kept] = lastkept;
-                    at += (kept + 1) & ~1;
-                }
-                if (lane == 0) s_csp[slot * (kClassMax + 1) + Kr] = at;
-            }
-        }
-        for (int s = lane; s < S; s += 32) least = min(least, rm[s]);
-        least = __reduce_min_sync(0xffffffffu, least);
-        const int f = min(base + least, M + 1);
-        if (lane == 0) { s_front[l & 3] = f; s_slot[l & 3] = slot; }
-        __syncwarp();
-        return f;
+        return nf;
     };
-    auto fetch = [&](int l) {
-        int32_t* const rm = raw + (l & 3) * 2 * S;
-        for (int s = lane; s < S; s += 32) {
-            cp_async_4(rm + s, mq + (size_t)l * S + s);
-            cp_async_4(rm + S + s, tq + (size_t)l * S + s);
+    // ... of a whole layer by one warp: lane k takes strategies k, k+32, ...
+    auto prepare_layer = [&](int h, const int (&m)[kRowsPerLane], const int (&t)[kRowsPerLane]) {
+        int most = 0;
+#pragma unroll
+        for (int j = 0; j < kRowsPerLane; ++j)
+            if (lane + 32 * j < SP8) most = max(most, prepare_one(h, lane + 32 * j, m[j], t[j]));
+        most = __reduce_max_sync(0xffffffffu, most);
+        if (lane == 0) fillmax[h] = most;
+    };
+    // layers 0 and 1 straight from global memory, a warp each (nothing is being stored yet)
+    if (warp <= 1 && warp < Li) {
+        int m0[kRowsPerLane], t0[kRowsPerLane];
+#pragma unroll
+        for (int j = 0; j < kRowsPerLane; ++j) {
+            const int s = lane + 32 * j;
+            m0[j] = s < S ? mq[warp * S + s] : 0;
+            t0[j] = s < S ? tq[warp * S + s] : 0;
+        }
+        prepare_layer(warp, m0, t0);
+    }
+    for (int x = tid; x < 32 * TM; x += NT) dump[x] = 0;
+    // where the other CTAs' buffers lie in the cluster window: asked once, not once per store (the mapping is an
+    // offset per CTA; asking inside the push puts its latency on every strategy's chain of branches)
+    if (tid < 16) cdelta[tid] = (int)(map_to_rank(smem_addr(buf0), (uint32_t)min(tid, CL - 1)) - smem_addr(buf0));
+    {
+        const int32_t* T = T0 + (a.trans_layer ? a.trans_layer : 0);       // matrix 1 is paid between layers 0 and 1
+        int32_t* dst = tsm + (a.trans_layer ? tmat : 0);                    // per layer: matrix l sits in tsm[l & 1]
+        for (int e = tid; e < tmat; e += NT) {
+            const int k = e / SP8, c = e - k * SP8;
+            dst[e] = (c < S && Li > 1) ? T[k * S + c] : 0;
+            if (a.trans_layer) tsm[e] = 0;                                  // pad columns of the other buffer stay 0
+        }
+    }
+    __syncthreads();
+    for (int s = warp; s < S; s += NW + 1) {
+        const int t0 = rows[s].z;                                           // time(0,s) sits in every record of s
+        const int nf = fillc[s];
+        for (int x = lane; x < W; x += 32) {
+            const bool pad = col_g0 + x > M;
+            buf0[s * W + x] = (pad || x < nf) ? kInf : t0;
+            if (pad) buf1[s * W + x] = kInf;                                // pad columns are never written again
+        }
+    }
+    // Service warp: raw mem / time rows of the layer after next, lane k keeps strategies k, k+32, ... (S <= 128).
+    // They are fetched a whole layer before they are needed and BEFORE that layer's table store is issued: a
+    // global load issued while the SM's bulk stores are in flight comes back after thousands of cycles.
+    int raw_m[kRowsPerLane], raw_t[kRowsPerLane];
+    auto fetch_rows = [&](int lay, int (&m)[kRowsPerLane], int (&t)[kRowsPerLane]) {
+#pragma unroll
+        for (int j = 0; j < kRowsPerLane; ++j) {
+            const int s = lane + 32 * j;
+            m[j] = s < S ? mq[lay * S + s] : 0;
+            t[j] = s < S ? tq[lay * S + s] : 0;
         }
     };
-    int front = 0;
-    if (run) {
+    if (warp == NW && Li > 2) fetch_rows(2, raw_m, raw_t);
+    // every CTA of the cluster has started and holds its layer 0 before anyone writes into a neighbour
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");            // layer 0 goes to the table by a bulk store
+    cluster_barrier();
+
+    for (int l = 1; l < Li; ++l) {
+        const int32_t* const X = (l & 1) ? buf0 : buf1;                     // layer l-1
+        int32_t* const Y = (l & 1) ? buf1 : buf0;                           // layer l
+        const int4* const rl = rows + (l & 1) * nrec;
+        const int32_t* const Tl = tsm + ((a.trans_layer && (l & 1)) ? tmat : 0);
+
         if (warp == NW) {
-            fetch(0);
-            if (Li > 1) fetch(1);
-            cp_async_commit();
-            if (Li > 2) fetch(2);
-            cp_async_commit();
-            cp_async_wait<1>();
-            __syncwarp();
-            front = prepare(0, 0);
-            if (Li > 1) front = prepare(1, front);
+            // ------------------------------------------------------------ service warp
+            // first the loads: rows of layer l+2, and with one matrix per layer the matrix of layer l+1
+            int next_m[kRowsPerLane], next_t[kRowsPerLane];
+            if (l + 2 < Li) fetch_rows(l + 2, next_m, next_t);
+            if (l + 1 < Li && a.trans_layer) {
+                const int32_t* T = T0 + (size_t)(l + 1) * a.trans_layer;
+                int32_t* dst = tsm + (((l + 1) & 1) ? tmat : 0);
+                for (int e = lane; e < S * S; e += 32) {
+                    const int k = e / S, c = e - k * S;
+                    cp_async_4(dst + k * SP8 + c, T + e);
+                }
+            }
+            // layer l-1 is complete in X: to the table while this layer is computed
+            if (a.C && lane == 0) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");    // the buffer was written by plain stores
+                tensor_store_3d(&map_c, X, rank * a.G, (i * Lmax + (l - 1)) * S);
+                bulk_commit();
+            }
+            // the records of layer l+1 from the rows fetched a layer ago
+            if (l + 1 < Li) prepare_layer((l + 1) & 1, raw_m, raw_t);
+#pragma unroll
+            for (int j = 0; j < kRowsPerLane; ++j) { raw_m[j] = next_m[j]; raw_t[j] = next_t[j]; }
+            if (l + 1 < Li && a.trans_layer) cp_async_wait_all();
+            if (a.C && lane == 0) bulk_wait_read();                         // X may be overwritten from the next barrier on
         } else {
-            for (int k = 0; k < Kc; ++k)
-                for (int x = tid; x < P; x += NW * 32) {
-                    g0[k * P + x] = rank * W + x >= H ? 0 : kInf;           // column rank*W + x - H
-                    if (x < H) g0[gints + k * P + x] = kInf;
-                    if (ARG) {
-                        a0[k * P + x] = 255;
-                        if (x < H) a0[gints + k * P + x] = 255;
+            // ------------------------------------------------------------ compute warps
+            // cells of this CTA's columns that no column maps to in this layer (m < mem(l,s): the first fillc[s] of
+            // row s): the compute warps share the columns, each takes every strategy in turn (independent predicated
+            // stores; a loop per strategy would be a chain of dependent steps)
+            {
+                const int* const fc = fillc + (l & 1) * SP8;
+                const int most = fillmax[l & 1];
+                for (int x = warp * 32 + lane; x < most; x += NW * 32) {
+#pragma unroll 4
+                    for (int s = 0; s < S; ++s)
+                        if (x < fc[s]) Y[s * W + x] = kInf;
+                }
+            }
+            const uint32_t ybase = smem_addr(Y);
+            for (int unit = warp; unit < a.units; unit += NW) {
+                const int ct = unit / a.NSG, sg = unit - ct * a.NSG;
+                const int colb = ct * (32 * TM);
+                int nj = a.G - ct * TM;                                     // 32-column groups of this tile that exist
+                nj = nj > TM ? TM : nj;
+                int acc[TM][8];
+#pragma unroll
+                for (int j = 0; j < TM; ++j)
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc[j][u] = kInf;
+                const int32_t* pc = X + colb + lane;
+                const int32_t* pt = Tl + sg * 8;
+                int k = 0;
+                auto steps = [&](auto ku) {
+                    constexpr int K = decltype(ku)::value;
+                    for (; k + K <= S; k += K) {
+#pragma unroll
+                        for (int kk = 0; kk < K; ++kk) {
+                            int c[TM];
+#pragma unroll
+                            for (int j = 0; j < TM; ++j) c[j] = pc[kk * W + j * 32];
+                            const int4 t0 = *reinterpret_cast<const int4*>(pt + kk * SP8);
+                            const int4 t1 = *reinterpret_cast<const int4*>(pt + kk * SP8 + 4);
+                            const int t[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+#pragma unroll
+                            for (int j = 0; j < TM; ++j)
+#pragma unroll
+                                for (int u = 0; u < 8; ++u) acc[j][u] = __viaddmin_s32(c[j], t[u], acc[j][u]);
+                        }
+                        pc += K * W;
+                        pt += K * SP8;
+                    }
+                };
+                steps(std::integral_constant<int, 8>());
+                steps(std::integral_constant<int, 1>());
+                // push: column m' of strategy s belongs at column m' + mem(l,s): in this CTA's buffer or in one further up.
+                // All eight records first; when every strategy either stays at home in one piece or lands nowhere, the
+                // stores go out in one run without a branch (those that land nowhere go to a dump row).
+                int4 r[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) r[u] = rl[ct * SP8 + sg * 8 + u];
+                bool plain = nj == TM;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) plain = plain && (r[u].x < 0 || (r[u].x == rank && r[u].w == kWholeTile));
+                int32_t* const yl = Y + (sg * 8) * W + lane;
+                if (plain) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        int32_t* const y = r[u].x < 0 ? dump + lane : yl + u * W + r[u].y;
+#pragma unroll
+                        for (int j = 0; j < TM; ++j) y[j * 32] = __viaddmin_s32(acc[j][u], r[u].z, kInf);    // +inf stays +inf
+                    }
+                } else {
+                    // Some strategy's tile leaves the CTA or straddles two: the whole unit goes through the cluster window
+                    // (what stays at home too), one predicated store a register and no branch - a chain of branches per
+                    // strategy cost the warps that own such tiles three times the time of the stores themselves.
+                    // A whole tile has w = the largest int: its columns pass the test against w and lie below W.
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int dx = r[u].x < 0 ? 0 : r[u].x;
+                        const uint32_t row = ybase + (uint32_t)((sg * 8 + u) * W) * 4u;
+                        const uint32_t ra0 = row + (uint32_t)cdelta[dx];
+                        const uint32_t ra1 = row + (uint32_t)cdelta[min(dx + 1, CL - 1)] - (uint32_t)W * 4u;
+                        const bool lands = r[u].x >= 0;
+#pragma unroll
+                        for (int j = 0; j < TM; ++j)
+                            if (j < nj) {
+                                const int x = r[u].y + j * 32 + lane;
+                                const int v = __viaddmin_s32(acc[j][u], r[u].z, kInf);
+                                if (lands && x <= r[u].w) st_cluster((x < W ? ra0 : ra1) + (uint32_t)x * 4u, v);
+                            }
                     }
                 }
+            }
         }
+        // What this thread stored into shared memory, its own CTA's or a neighbour's, is read next by the bulk store of
+        // the CTA that owns it (async proxy): the writer orders it for that proxy before the barrier that publishes it.
+        asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
+        cluster_barrier();                                                  // layer l is complete everywhere
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");            // bulk copies write over the halo's initial values
-    whole_barrier(CL);                                          // also: nobody leaves while its partial sums are being read
-    if (!run) return;
 
-    Ctx c;
-    c.S = S; c.M = M; c.W = W; c.H = H; c.P = P; c.G = W / 32; c.CL = CL; c.rank = rank; c.Li = Li; c.m_pitch = a.m_pitch; c.Kr = Kr; c.Kc = Kc;
-    c.tmax = s_all.tmax; c.SP = a.SP; c.NW = NW; c.gints = gints;
-    c.g0 = g0; c.a0 = a0; c.stage = stage_rows; c.rec = smem_addr(rec); c.S2 = S2; c.n_all = n_all; c.front = s_front; c.reach = s_reach; c.tsm = tsm; c.tmat = a.trans_layer ? tfull : 0;
-    c.cs = s_first; c.csp = s_csp; c.slot = s_slot; c.cdelta = s_cdelta;
-    c.slice = (size_t)S * a.m_pitch;
-    c.C = STORE ? a.C + (size_t)i * Lmax * c.slice : nullptr;
-    c.A = ARG ? a.A + (size_t)i * Lmax * c.slice : nullptr;
-    c.C_last = a.C_last + (size_t)i * c.slice;
-    c.bars = smem_addr(&s_bar[0]);
-    c.halo_bytes = (uint32_t)(Kc * min(H, rank * W)) * (ARG ? 5u : 4u);
-    c.strict = strict;
-    c.late = &s_late;
-    if (CL > 1 && !c.strict) cluster_arrive();                  // nobody has read anything yet: the first copies may come
-    if (warp == NW) {
-        // ---------------------------------------------------------------- service warp
-        for (int l = 0; l + 1 < Li; ++l) {
-            if (l + 3 < Li) fetch(l + 3);
-            cp_async_commit();
-            if (a.trans_layer && l + 2 < Li) {                  // matrix l + 1 is in use in this layer
-                const int32_t* const T = T0 + (size_t)(l + 2) * a.trans_layer;
-                int32_t* const dst = tsm + ((l & 1) ? tfull : 0);
-                for (int x = lane; x < S * S; x += 32) {
-                    const int r = x / S, s = x - r * S;
-                    cp_async_4(dst + r * a.SP + s, T + x);
-                }
-            }
-            cp_async_commit();
-            if (l + 2 < Li) {
-                cp_async_wait<2>();                             // the rows of layer l + 2, asked for a layer ago
-                __syncwarp();
-                front = prepare(l + 2, front);
-            }
-            if (a.trans_layer) cp_async_wait<0>();
-            if (STAGE) {
-                if (lane == 0) bulk_wait_read();                // layer l - 1 has left its buffer, which layer l + 1 fills
-                __syncwarp();
-            }
-            send_halo<ARG>(c, l, warp, lane);
-            if (STAGE && lane == 0) {
-                if (CL == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                tensor_store_3d(&map_c, c.stage + (l & 1) * S * W, rank * (W / 32), (i * Lmax + l) * S);
-                bulk_commit();
-            }
-            await_halo<ARG>(c, l, warp, lane);
-        }
-        if (STAGE) {
-            if (lane == 0) bulk_wait_read();
-            cta_barrier();                                      // the last layer's rows are collected
-            if (lane == 0) {
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                const int l = Li - 1;
-                tensor_store_3d(&map_c, c.stage + (l & 1) * S * W, rank * (W / 32), (i * Lmax + l) * S);
-                tensor_store_3d(&map_last, c.stage + (l & 1) * S * W, rank * (W / 32), i * S);
-                bulk_commit();
-                bulk_wait_all();
-            }
-            __syncwarp();
-        }
-    } else {
-        if (classes) {
-            if (K <= 4) run_layers<4, ARG ? 2 : 6, false, STORE, ARG, STAGE>(c, warp, lane);
-            else if (K <= 8) run_layers<8, ARG ? 2 : 6, false, STORE, ARG, STAGE>(c, warp, lane);
-            else run_layers<16, ARG ? 1 : 3, false, STORE, ARG, STAGE>(c, warp, lane);
-        } else {
-            run_layers<32, ARG ? 1 : 2, true, STORE, ARG, STAGE>(c, warp, lane);
-        }
-        if (STAGE) cta_barrier();                               // the last layer's rows are collected
+    // ---- the last layer: to the table and to C_last
+    if (warp == NW && lane == 0) {
+        const int32_t* const F = ((Li - 1) & 1) ? buf1 : buf0;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (a.C) tensor_store_3d(&map_c, F, rank * a.G, (i * Lmax + (Li - 1)) * S);
+        tensor_store_3d(&map_last, F, rank * a.G, i * S);
+        bulk_commit();
+        bulk_wait_all();
     }
-    if (CL > 1) {
-        if (!c.strict) cluster_wait();
-        whole_barrier(CL);                                      // nobody's shared memory goes away while it is being read
-        if (rank == 0 && tid == 0 && s_late) a.path[0] = 1;
-    }
-    if (s_late && tid == 0) atomicOr(reinterpret_cast<int*>(a.status + i), GALV_STATUS_TIMEOUT);
 }
 
+}  // namespace
+
 // ---------------------------------------------------------------- host side
+
+namespace {
 
 typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                     const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -1127,15 +471,8 @@ cudaError_t encode_table_3d(CUtensorMap* map, void* base, size_t rows, int m_pit
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-typedef void (*RsKernel)(const RsArgs, const CUtensorMap, const CUtensorMap);
-RsKernel kernel_of(bool store, bool arg, bool stage)
-{
-    if (stage) return resident_kernel<true, false, true>;
-    return store ? (arg ? resident_kernel<true, true, false> : resident_kernel<true, false, false>)
-                 : (arg ? resident_kernel<false, true, false> : resident_kernel<false, false, false>);
-}
-
-cudaError_t launch_resident(RsKernel k, const RsArgs& a, const RsPlan& p, const CUtensorMap& mc, const CUtensorMap& ml, cudaStream_t st, int* max_clusters)
+template <int TM>
+cudaError_t launch_cluster(const ClArgs& a, const ClPlan& p, const CUtensorMap& mc, const CUtensorMap& ml, cudaStream_t st, int* max_clusters)
 {
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
@@ -1150,145 +487,147 @@ cudaError_t launch_resident(RsKernel k, const RsArgs& a, const RsPlan& p, const 
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, k, &cfg);
-    return cudaLaunchKernelEx(&cfg, k, a, mc, ml);
+    if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, cluster_search_kernel<TM>, &cfg);
+    return cudaLaunchKernelEx(&cfg, cluster_search_kernel<TM>, a, mc, ml);
+}
+
+cudaError_t launch_any(const ClArgs& a, const ClPlan& p, const CUtensorMap& mc, const CUtensorMap& ml, cudaStream_t st, int* max_clusters)
+{
+    switch (p.tm) {
+    case 2: return launch_cluster<2>(a, p, mc, ml, st, max_clusters);
+    case 3: return launch_cluster<3>(a, p, mc, ml, st, max_clusters);
+    default: return launch_cluster<4>(a, p, mc, ml, st, max_clusters);
+    }
 }
 
 // Clusters of this plan's size and resources the device can hold at once (asked once per kind of launch).
-int max_active_clusters(const galv_ctx* ctx, const RsPlan& p, bool store, bool arg)
+int max_active_clusters(const galv_ctx* ctx, const ClPlan& p)
 {
     static std::map<unsigned long long, int> cache;          // shared by all contexts of the process
     static std::mutex cache_mutex;
     std::lock_guard<std::mutex> lock(cache_mutex);
-    const unsigned long long key = ((unsigned long long)ctx->device << 48) | ((unsigned long long)p.cl << 40) | ((unsigned long long)p.stage << 38) | ((unsigned long long)store << 37) |
-                                   ((unsigned long long)arg << 36) | ((unsigned long long)p.nw << 28) | (unsigned long long)((p.smem + 1023) / 1024);
+    const unsigned long long key = ((unsigned long long)ctx->device << 48) | ((unsigned long long)p.cl << 40) |
+                                   ((unsigned long long)p.tm << 36) | ((unsigned long long)p.nw << 28) | (unsigned long long)((p.smem + 1023) / 1024);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
-    RsArgs a{};
+    ClArgs a{};
     a.B = 1;
-    int n = 0;
     CUtensorMap m{};
-    if (launch_resident(kernel_of(store, arg, p.stage), a, p, m, m, nullptr, &n) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+    int n = 0;
+    if (launch_any(a, p, m, m, nullptr, &n) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
     cache[key] = n;
     return n;
 }
 
-// Shared memory of a launch beside its state.
-long long fixed_smem(const galv_shape* sh, bool dense)
+// Register-tile height for g column groups per CTA: the one that gives the busiest warp the least work (units are
+// dealt out to at most 12 warps), then the busiest scheduler, then the smaller tile (more, smaller units spread the
+// cost of the tiles that straddle two CTAs).  Returns the busiest scheduler's work in units of 8*S*2 cycles.
+int tile_cost(int g, int nsg, int* tm_out)
 {
-    const int S = sh->S, SP = (S + 3) & ~3;
-    const long long t = dense ? (long long)S * SP * ((sh->flags & GALV_TRANS_PER_LAYER) ? 2 : 1) : 0;
-    return (t > kClassMax * kClassMax ? t : kClassMax * kClassMax) * 4 + (long long)4 * 24 * ((S + kClassMax + 3) & ~3) + (long long)8 * SP * 4 + 256;
-}
-
-// The best cluster size for a state of `rows` rows at least; false when none fits.
-bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, RsPlan* out, double* est)
-{
-    const int S = sh->S, Gt = sh->m_pitch / 32;
-    const bool store = (sh->flags & GALV_STORE_C_FULL) != 0, arg = (sh->flags & GALV_STORE_ARGMIN) != 0;
-    const int want = (sh->flags >> 16) & 31;                  // GALV_CLUSTER_SIZE(n): only clusters of n CTAs
-    const int per_word = arg ? 10 : 8;                        // two buffers of words, with argmin bytes beside
-    const long long words = ((long long)ctx->smem_optin - kStaticSmem - fixed_smem(sh, dense)) / per_word;
-    // halo to plan for: a few times what an even share of the budget gives a layer
-    long long halo = 4ll * sh->M / sh->Lmax;
-    if (halo < 64) halo = 64;
-    if (halo > sh->M) halo = sh->M;
-    bool found = false;
-    for (int cl = 1; cl <= ctx->max_cluster; ++cl) {
-        if (want && cl != want) continue;
-        const int g = (Gt + cl - 1) / cl;
-        if (cl > 1 && (g < 2 || g * (cl - 1) >= Gt)) continue;      // no CTA without columns
-        const int w = g * 32;
-        RsPlan p;
-        std::memset(&p, 0, sizeof(p));
-        p.cl = cl; p.w = w; p.dense = dense;
-        p.nw = g < kMaxWarps ? g : kMaxWarps;
-        // rows collected in shared memory where there is room for them beside the state (a tensor box has 256 entries a
-        // side at most) and where a layer is a chain of latencies rather than a stream of stores
-        const long long collected = (long long)2 * S * w * 4;
-        p.stage = store && !arg && g <= 2 * kMaxWarps && (long long)rows * (w + (cl > 1 ? halo : 0)) * per_word + collected <= words * per_word &&
-                  (long long)sh->B * sh->Lmax * S < (1ll << 31);
-        const long long room = p.stage ? words - collected / per_word : words;
-        long long gi = (long long)(dense && S > kClassMax ? S : kClassMax) * (w + ((sh->M + 32) & ~31));    // all that could be used
-        if (gi > room) gi = room;
-        p.gints = (int)(gi & ~31ll);
-        if ((long long)rows * w > p.gints) continue;
-        p.smem = (int)(p.gints * (long long)per_word + fixed_smem(sh, dense));
-        p.stage_at = (p.smem + 127) / 128 * 32;
-        if (p.stage) p.smem = p.stage_at * 4 + (int)collected;
-        const int slots = max_active_clusters(ctx, p, store, arg);
-        if (slots < 1) continue;
-        // SM cycles a layer: the issue of the columns' work, the store port (32 bytes a clock), the latency of one warp's
-        // walk over the strategies, and the barrier
-        const double issue = g * (S * 7.0 + 120.0) / 2.2, port = store ? g * S * 4.0 : 0.0;
-        const double chain = S * 12.0 + 500.0;
-        double t = issue > port ? issue : port;
-        if (t < chain) t = chain;
-        t += cl == 1 ? 150.0 : (cl > 8 ? 1200.0 : 900.0);
-        const double share = (double)(sh->B < slots ? sh->B : slots) * cl / ctx->num_sms;      // several CTAs on an SM share its issue slots
-        if (share > 1.0) t *= share;
-        t *= (sh->B + slots - 1) / slots;
-        if (cl > 1 && (long long)rows * (w + halo) > p.gints) t *= 4.0;            // shifts beyond the halo take the slow way
-        if (!found || t < *est) {
-            found = true;
-            *est = t;
-            p.sorted = sh->B > slots && sh->B <= kMaxSortedB;
-            *out = p;
-        }
+    int best_tm = 4, best_warp = 1 << 30, best_sched = 1 << 30;
+    for (int tm = 4; tm >= 2; --tm) {
+        const int units = (g + tm - 1) / tm * nsg;
+        int nw = (units + 3) & ~3;
+        if (nw > 12) nw = 12;
+        const int warp = (units + nw - 1) / nw * tm;
+        const int sched = (units + 3) / 4 * tm;
+        if (warp < best_warp || (warp == best_warp && sched <= best_sched)) { best_warp = warp; best_sched = sched; best_tm = tm; }
     }
-    return found;
+    *tm_out = best_tm;
+    return best_sched;
 }
 
 }  // namespace
 
-int galv_cluster_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
+// Whether the cluster kernel can run this shape, and how: CTAs per cluster, columns per CTA, register tile.
+bool galv_cluster_plan(const galv_ctx* ctx, const galv_shape* sh, ClPlan* out)
 {
-    if (sh->flags & (GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_DEBUG_WITHHOLD_LOAD | GALV_KERNEL_NO_CLUSTER)) return 0;
-    if (sh->S > kMaxS || (long long)sh->S * sh->m_pitch >= (1ll << 29)) return 0;      // row offsets are 32-bit
-    if (ctx->plan_valid && std::memcmp(&ctx->plan_shape, sh, sizeof(*sh)) == 0) {       // the shape of the last call
-        plans[0] = ctx->plans[0]; plans[1] = ctx->plans[1];
-        return ctx->plan_launches;
+    std::memset(out, 0, sizeof(*out));
+    if (sh->flags & (GALV_STORE_ARGMIN | GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_DEBUG_WITHHOLD_LOAD | GALV_KERNEL_NO_CLUSTER))
+        return false;
+    const int S = sh->S, Gt = sh->m_pitch / 32;
+    if (S > 32 * kRowsPerLane) return false;
+    if ((long long)sh->B * sh->Lmax * S >= (1ll << 31)) return false;       // row coordinates of the table store are 32-bit
+    const int nsg = (S + 7) / 8, sp8 = nsg * 8;
+    const int nT = (sh->flags & GALV_TRANS_PER_LAYER) ? 2 : 1;
+    const int budget = ctx->smem_optin - 4096;               // static shared memory of the kernel, rounded up
+    // Candidates: every cluster size that gives each CTA at least 96 columns and leaves none without columns.
+    // Estimated SM cycles per layer of a cluster, fitted to measurements on B200: the add-min issue time of the
+    // busiest scheduler, stretched by the per-cell work beside it (push, fill, shared-memory loads: about 24
+    // add-mins' worth per cell), plus what a layer costs whatever its size (barrier, drain of the pushes that
+    // cross CTAs, start): about 3000 cycles, some more for clusters beyond 12 CTAs.  With more instances than the
+    // device holds clusters the batch takes several rounds; on its own the kernel is chosen only when one round
+    // does (a batch that needs rounds is better off on the tiled kernels, whose SMs never wait on a barrier).
+    double best_time = 0.0;
+    bool found = false;
+    const int want_cl = (sh->flags >> 16) & 31;              // GALV_CLUSTER_SIZE(n): only clusters of n CTAs
+    const bool forced = (sh->flags & GALV_KERNEL_CLUSTER) != 0 || want_cl != 0;
+    for (int cl = ctx->max_cluster; cl >= 1; --cl) {
+        if (want_cl && cl != want_cl) continue;
+        const int g = (Gt + cl - 1) / cl;
+        if (cl > 1 && (g < 3 || g * (cl - 1) >= Gt)) continue;
+        const long long smem = (long long)2 * S * g * 32 * 4 + (long long)nT * S * sp8 * 4 + (long long)2 * ((g + 1) / 2) * sp8 * 16 + (long long)2 * sp8 * 4 + 16 + 512 + 64;
+        if (smem > budget) break;                            // smaller clusters need more per CTA
+        ClPlan p;
+        std::memset(&p, 0, sizeof(p));
+        p.cl = cl; p.g = g; p.w = g * 32; p.nsg = nsg; p.sp8 = sp8;
+        const int cost = tile_cost(g, nsg, &p.tm);
+        p.nct = (g + p.tm - 1) / p.tm;
+        p.units = p.nct * nsg;
+        p.nw = (p.units + 3) & ~3;                           // a multiple of 4: the SM's four schedulers get the same share
+        if (p.nw > 12) p.nw = 12;
+        p.smem = (int)smem;
+        const int slots = max_active_clusters(ctx, p);
+        if (slots < 1) continue;
+        if (!forced && sh->B > slots) continue;
+        const double rounds = (double)((sh->B + slots - 1) / slots);
+        const double active = (double)(sh->B < slots ? sh->B : slots) * cl;     // CTAs resident at once
+        const double share = active > ctx->num_sms ? active / ctx->num_sms : 1.0;   // ... of which this many share an SM's ALUs
+        const double t = rounds * ((double)cost * 16.0 * S * (1.0 + 24.0 / S) * share + 3000.0 + (cl > 12 ? 800.0 : 0.0));
+        if (!found || t < best_time) {
+            best_time = t;
+            found = true;
+            p.sorted = sh->B > slots;                        // more clusters than fit at once: the longest instances first
+            *out = p;
+        }
     }
-    double td = 0.0, tc = 0.0;
-    int n = 0;
-    const bool d = best_plan(ctx, sh, sh->S, true, &plans[1], &td);
-    const bool c = !(sh->flags & GALV_TRANS_PER_LAYER) && sh->S > 12 && best_plan(ctx, sh, 12, false, &plans[0], &tc);
-    if (d && (!c || td <= tc * 1.15)) { plans[0] = plans[1]; n = 1; }
-    else if (c) n = d ? 2 : 1;
-    ctx->plan_shape = *sh; ctx->plans[0] = plans[0]; ctx->plans[1] = plans[1]; ctx->plan_launches = n; ctx->plan_valid = 1;
-    return n;
+    if (!found) return false;
+    if (out->sorted && sh->B > kMaxSortedB) return false;
+    return true;
 }
 
 cudaError_t galv_cluster_configure(galv_ctx* ctx)
 {
-    ctx->max_cluster = 16;                                     // beyond the portable 8 where the device allows it
-    for (int k = 0; k < 5; ++k) {
-        const RsKernel f = kernel_of(k & 1, (k & 2) != 0, k == 4);
-        cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin - kStaticSmem);
-        if (e != cudaSuccess) return e;
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) { (void)cudaGetLastError(); ctx->max_cluster = 8; }
-    }
+    const int bytes = ctx->smem_optin - 4096;
+    cudaError_t e = cudaFuncSetAttribute(cluster_search_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cluster_search_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(cluster_search_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    // clusters of up to 16 CTAs where the device allows them (beyond the portable 8)
+    ctx->max_cluster = 8;
+    if (cudaFuncSetAttribute(cluster_search_kernel<2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(cluster_search_kernel<3>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(cluster_search_kernel<4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+        ctx->max_cluster = 16;
+    else
+        (void)cudaGetLastError();
     return cudaSuccess;
 }
 
-cudaError_t galv_cluster_launch(const RsPlan& p, int second, const DpArgs& d, cudaStream_t st)
+cudaError_t galv_cluster_launch(galv_ctx* ctx, const galv_shape* sh, const ClPlan& p, const DpArgs& d, cudaStream_t st)
 {
-    RsArgs a;
+    ClArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
-    a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second;
-    a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept
-    a.path_value = (d.B <= kMaxSortedB && !d.A) ? 2 : 0;
+    a.CL = p.cl; a.W = p.w; a.G = p.g; a.NSG = p.nsg; a.SP8 = p.sp8; a.nct = p.nct; a.units = p.units; a.sorted = p.sorted;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
-    a.C = d.C; a.A = d.A; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done;
-    a.stage_at = p.stage_at;
+    a.C = d.C; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done;
+    (void)sh;
     CUtensorMap mc, ml;
     std::memset(&mc, 0, sizeof(mc));
-    std::memset(&ml, 0, sizeof(ml));
-    if (p.stage) {
-        cudaError_t e = encode_table_3d(&ml, d.C_last, (size_t)d.B * d.S, d.m_pitch, d.S, p.w / 32);
-        if (e == cudaSuccess) e = encode_table_3d(&mc, d.C, (size_t)d.B * d.Lmax * d.S, d.m_pitch, d.S, p.w / 32);
-        if (e != cudaSuccess) return e;
-    }
-    return launch_resident(kernel_of(d.C != nullptr, d.A != nullptr, p.stage), a, p, mc, ml, st, nullptr);
+    cudaError_t e = encode_table_3d(&ml, d.C_last, (size_t)d.B * d.S, d.m_pitch, d.S, p.g);
+    if (e == cudaSuccess && d.C) e = encode_table_3d(&mc, d.C, (size_t)d.B * d.Lmax * d.S, d.m_pitch, d.S, p.g);
+    if (e != cudaSuccess) return e;
+    (void)ctx;
+    return launch_any(a, p, mc, ml, st, nullptr);
 }

@@ -1806,29 +1806,42 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     const int pk = ctx->prof_count % 64;
     if (ctx->profiling) cudaEventRecord(ctx->pev[2 * pk], st);
     {
-        // One cluster per instance wherever its state fits shared memory.  What the launches leave alone (known on the
-        // device only) goes to the tiled kernels, which then find their schedule shorter, or empty.
-        RsPlan rp[2];
-        const int n = galv_cluster_plan(ctx, sh, rp);
-        int launched = 0;
-        while (launched < n) {
-            if (galv_cluster_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now
-            ++launched;
-        }
-        if (launched && launched == n && rp[n - 1].dense) {
+        // The state between layers kept in shared memory wherever it fits.  What these launches leave alone is known on
+        // the device only: it goes to the pushing cluster kernel (small batches) or to the tiled kernels, which find
+        // their schedule shorter, or empty.
+        auto finished = [&]() {
             if (ctx->profiling) { cudaEventRecord(ctx->pev[2 * pk + 1], st); ++ctx->prof_count; }
             return cudaSuccess;
+        };
+        RsPlan rp[2];
+        const int n = galv_resident_plan(ctx, sh, rp);
+        int launched = 0;
+        while (launched < n) {
+            if (galv_resident_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now
+            ++launched;
         }
+        if (launched && launched == n && rp[n - 1].dense) return finished();
         if (!launched) a.done = nullptr;
+        ClPlan cp;
+        if (galv_cluster_plan(ctx, sh, &cp)) {
+            if (galv_cluster_launch(ctx, sh, cp, a, st) == cudaSuccess) return finished();
+            (void)cudaGetLastError();                        // the clusters cannot be placed on this device right now: tiled kernels
+        }
     }
     e = cudaMemsetAsync(a.scratch, 0, (size_t)4 * (Lmax + 2) * 4, st);      // histogram, fill and work counters
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(a.err, 0, 32, st);                       // error flag, largest mem, largest trans, path, keyed
     if (e != cudaSuccess) return e;
     const bool reference = (sh->flags & GALV_KERNEL_REFERENCE) != 0;
+    // Matrices that come this far are unstructured.  Without an argmin table the rows that cannot win are left out unasked
+    // (GALV_KERNEL_NO_CLUSTER takes the tiled kernels as the other flags say): 1024 instances of 48 layers, S = 32, 2048
+    // columns 7.8 -> 4.6 ms, 300 of S = 64 7.7 -> 4.1; with one, the loop on keys does about as well without (1.69 / 1.73).
+    galv_shape planned = *sh;
+    if (!a.A && S <= 64 && !(sh->flags & (GALV_KERNEL_NO_CLUSTER | GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_DEBUG_WITHHOLD_LOAD)))
+        planned.flags |= GALV_SKIP_DOMINATED;
     DpPlan pl;
     std::memset(&pl, 0, sizeof(pl));
-    if (!reference && !galv_dp_make_plan(ctx, sh, &pl)) return cudaErrorInvalidConfiguration;
+    if (!reference && !galv_dp_make_plan(ctx, &planned, &pl)) return cudaErrorInvalidConfiguration;
     if (reference) { pl.tmb = 256; pl.ntiles_m = (a.M + 256) / 256; }
     e = cudaMemsetAsync(a.minmem_l, 0x7f, (size_t)(Lmax + 1) * 4, st);
     if (e != cudaSuccess) return e;
@@ -1894,7 +1907,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     }
     DpArgs ap = a;
     ap.withhold = (sh->flags & GALV_DEBUG_WITHHOLD_LOAD) != 0;
-    ap.skip_dom = (sh->flags & GALV_SKIP_DOMINATED) != 0;
+    ap.skip_dom = (planned.flags & GALV_SKIP_DOMINATED) != 0;
     ap.keyed = keyed_possible;
     if (!(sh->flags & GALV_SKIP_INFEASIBLE)) ap.front = nullptr;
     ap.tile_done = nullptr;

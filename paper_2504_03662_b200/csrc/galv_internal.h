@@ -7,7 +7,7 @@
 
 #include "galv.h"
 
-// How the cluster kernel (one thread-block cluster per instance, its state in shared memory) cuts an instance.
+// How the resident kernel (one thread-block cluster per instance, the state between layers in shared memory) cuts an instance.
 struct RsPlan {
     int cl;        // CTAs per cluster
     int w;         // budget columns per CTA (multiple of 32)
@@ -16,6 +16,7 @@ struct RsPlan {
     int dense;     // the state of an unstructured matrix (S rows and the matrix itself) fits: every instance can run
     int smem;      // dynamic shared memory bytes
     int sorted;    // clusters take the instances longest first
+    int halo_fits, rounds;
     int stage;     // a layer's rows are collected in shared memory and leave with one tensor store
     int stage_at;  // word offset of the collected rows
 };
@@ -24,11 +25,12 @@ struct galv_ctx {
     int device;
     int num_sms;
     int smem_optin;      // max dynamic shared memory per block (bytes)
+    int max_resident;    // the same for the resident kernel
     int max_cluster;     // largest thread-block cluster the cluster kernel may be launched with (8 portable, 16 where allowed)
     int profiling;       // record an event pair around the layer launches of every search
     int prof_count;      // searches profiled since profiling was switched on
     cudaEvent_t pev[2 * 64];   // ring of event pairs: search k uses pev[2*(k%64)], pev[2*(k%64)+1]
-    galv_shape plan_shape;     // the cluster kernel's plan for the shape of the last search
+    galv_shape plan_shape;     // the resident kernel's plan for the shape of the last search
     RsPlan plans[2];
     int plan_launches, plan_valid;
     char err[512];
@@ -85,7 +87,7 @@ struct DpArgs {
     int32_t* ntiles;     // [Lmax+1] tiles per instance that can store anything in layer l
     int32_t* tcount;     // [Lmax][ntiles_m] layers 1..l whose items include tile t
     int32_t* status;
-    int32_t* done;       // [B] instances the cluster kernel has finished, or NULL when it was not launched
+    int32_t* done;       // [B] instances the resident kernel has finished, or NULL when it was not launched
     int withhold;        // test hook: CTA 0 never loads its first chunk, so that the bounded waits run out
     int skip_dom;        // packed path: leave out row pairs that cannot win in any column of a warp group's tile
 };
@@ -98,9 +100,27 @@ struct WsLayout { size_t order, done, nactive, scratch, err, minmem_l, ntiles, i
 WsLayout galv_ws_layout(const galv_shape* sh);
 
 // launches to make (0: the shape is left to the tiled kernels); the last one takes every instance when it is dense
-int galv_cluster_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2]);
+int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2]);
+cudaError_t galv_resident_configure(galv_ctx* ctx);
+cudaError_t galv_resident_launch(const RsPlan& plan, int second, const struct DpArgs& a, cudaStream_t st);
+
+// How the pushing cluster kernel (small batches of unstructured matrices: one thread-block cluster per instance) cuts an instance.
+struct ClPlan {
+    int cl;        // CTAs per cluster
+    int w;         // budget columns per CTA (multiple of 32)
+    int g;         // w / 32
+    int nsg;       // ceil(S / 8)
+    int sp8;       // nsg * 8
+    int tm;        // 32-column groups per warp register tile
+    int nct;       // column tiles per CTA
+    int units;     // nct * nsg work units per CTA and layer
+    int nw;        // warps per CTA
+    int smem;      // dynamic shared memory bytes
+    int sorted;    // clusters take the instances longest first
+};
+bool galv_cluster_plan(const galv_ctx* ctx, const galv_shape* sh, ClPlan* plan);
 cudaError_t galv_cluster_configure(galv_ctx* ctx);
-cudaError_t galv_cluster_launch(const RsPlan& plan, int second, const struct DpArgs& a, cudaStream_t st);
+cudaError_t galv_cluster_launch(galv_ctx* ctx, const galv_shape* sh, const ClPlan& plan, const struct DpArgs& a, cudaStream_t st);
 
 bool galv_dp_make_plan(const galv_ctx* ctx, const galv_shape* sh, DpPlan* plan);
 cudaError_t galv_dp_configure(const galv_ctx* ctx);
