@@ -46,7 +46,7 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Device arena of galv_search_host.
-struct Arena { size_t L, layers, strat, inst, time_q, mem_q, trans_q, C, A, C_last, opt, plan, used, status, ws, total; };
+struct Arena { size_t L, map, layers, strat, inst, time_q, mem_q, trans_q, C, A, C_last, opt, plan, used, status, ws, total; };
 
 Arena arena_layout(const galv_shape* sh, bool with_model)
 {
@@ -55,6 +55,7 @@ Arena arena_layout(const galv_shape* sh, bool with_model)
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
     a.L = take(B * 4);
+    a.map = take(B * S * 4);
     a.layers = take(with_model ? B * Lm * sizeof(galv_layer_desc) : 0);
     a.strat = take(with_model ? S * sizeof(galv_strategy_desc) : 0);
     a.inst = take(with_model ? B * sizeof(galv_inst_params) : 0);
@@ -80,6 +81,10 @@ int galv_set_error(galv_ctx* ctx, int code, const char* text)
     if (ctx) std::snprintf(ctx->err, sizeof(ctx->err), "%s", text);
     return code;
 }
+
+static int dp_search(galv_ctx* ctx, const galv_shape* sh, const int32_t* L, const int32_t* time_q, const int32_t* mem_q,
+                     const int32_t* trans_q, int32_t* C, uint8_t* A, int32_t* C_last, int32_t* lean_map, void* workspace,
+                     size_t workspace_bytes, int32_t* status, void* stream);
 
 extern "C" {
 
@@ -180,6 +185,15 @@ int galv_dp_search(galv_ctx* ctx, const galv_shape* sh, const int32_t* L, const 
                    const int32_t* mem_q, const int32_t* trans_q, int32_t* C, uint8_t* A, int32_t* C_last,
                    void* workspace, size_t workspace_bytes, int32_t* status, void* stream)
 {
+    return dp_search(ctx, sh, L, time_q, mem_q, trans_q, C, A, C_last, nullptr, workspace, workspace_bytes, status, stream);
+}
+
+}  // extern "C"
+
+static int dp_search(galv_ctx* ctx, const galv_shape* sh, const int32_t* L, const int32_t* time_q, const int32_t* mem_q,
+                     const int32_t* trans_q, int32_t* C, uint8_t* A, int32_t* C_last, int32_t* lean_map, void* workspace,
+                     size_t workspace_bytes, int32_t* status, void* stream)
+{
     GALV_RANGE("galv_dp_search");
     if (!ctx) return GALV_ERR_INVALID_ARG;
     if (!shape_ok(sh)) { set_err(ctx, "galv_dp_search: shape outside limits"); return GALV_ERR_INVALID_ARG; }
@@ -210,6 +224,7 @@ int galv_dp_search(galv_ctx* ctx, const galv_shape* sh, const int32_t* L, const 
     a.roll = reinterpret_cast<int32_t*>(ws + w.roll);
     a.order = reinterpret_cast<int32_t*>(ws + w.order);
     a.done = reinterpret_cast<int32_t*>(ws + w.done);
+    a.lean_map = lean_map;
     a.nactive = reinterpret_cast<int32_t*>(ws + w.nactive);
     a.scratch = reinterpret_cast<int32_t*>(ws + w.scratch);
     a.work = reinterpret_cast<unsigned long long*>(a.scratch + 2 * (sh->Lmax + 2));
@@ -229,6 +244,8 @@ int galv_dp_search(galv_ctx* ctx, const galv_shape* sh, const int32_t* L, const 
     cudaError_t e = galv_dp_launch(ctx, sh, a, (cudaStream_t)stream);
     return e == cudaSuccess ? GALV_OK : cuda_fail(ctx, "galv_dp_search", e);
 }
+
+extern "C" {
 
 int galv_dp_search_path(galv_ctx* ctx, const galv_shape* sh, const void* workspace, int32_t* packed, void* stream)
 {
@@ -259,7 +276,7 @@ int galv_backtrack(galv_ctx* ctx, const galv_shape* sh, const int32_t* L, const 
         set_err(ctx, "galv_backtrack: a plan needs the argmin table A or the full table C");
         return GALV_ERR_INVALID_ARG;
     }
-    cudaError_t e = galv_backtrack_launch(sh, L, time_q, mem_q, trans_q, C, A, C_last, budget, opt_cost, plan,
+    cudaError_t e = galv_backtrack_launch(sh, L, time_q, mem_q, trans_q, C, A, C_last, nullptr, budget, opt_cost, plan,
                                           mem_used, status, (cudaStream_t)stream);
     return e == cudaSuccess ? GALV_OK : cuda_fail(ctx, "galv_backtrack", e);
 }
@@ -331,12 +348,16 @@ int galv_search_host(galv_ctx* ctx, const galv_shape* sh, const int32_t* L, cons
     int32_t* d_C = (sh->flags & GALV_STORE_C_FULL) ? reinterpret_cast<int32_t*>(d + ar.C) : nullptr;
     uint8_t* d_A = (sh->flags & GALV_STORE_ARGMIN) ? reinterpret_cast<uint8_t*>(d + ar.A) : nullptr;
     int32_t* d_last = reinterpret_cast<int32_t*>(d + ar.C_last);
-    rc = galv_dp_search(ctx, sh, d_L, d_tq, d_mq, d_xq, d_C, d_A, d_last, d + ar.ws, ar.total - ar.ws, d_status, stream);
+    // The table never leaves the arena: where only it is kept, the walk can do with the states between the layers (7 rows
+    // of them for 64 strategies), and the resident kernel leaves those in its place: 128 instances of the heterogeneous
+    // stack write 4.7 GB instead of 43.
+    int32_t* const d_map = d_C && !d_A ? reinterpret_cast<int32_t*>(d + ar.map) : nullptr;
+    if (d_map && (e = cudaMemsetAsync(d_map, 0xff, B * S * 4, st)) != cudaSuccess) return cuda_fail(ctx, "galv_search_host", e);
+    rc = dp_search(ctx, sh, d_L, d_tq, d_mq, d_xq, d_C, d_A, d_last, d_map, d + ar.ws, ar.total - ar.ws, d_status, stream);
     if (rc != GALV_OK) return rc;
-    rc = galv_backtrack(ctx, sh, d_L, d_tq, d_mq, d_xq, d_C, d_A, d_last, nullptr,
-                        reinterpret_cast<int32_t*>(d + ar.opt), reinterpret_cast<int32_t*>(d + ar.plan),
-                        reinterpret_cast<int32_t*>(d + ar.used), d_status, stream);
-    if (rc != GALV_OK) return rc;
+    e = galv_backtrack_launch(sh, d_L, d_tq, d_mq, d_xq, d_C, d_A, d_last, d_map, nullptr, reinterpret_cast<int32_t*>(d + ar.opt),
+                              reinterpret_cast<int32_t*>(d + ar.plan), reinterpret_cast<int32_t*>(d + ar.used), d_status, st);
+    if (e != cudaSuccess) return cuda_fail(ctx, "galv_search_host (plan)", e);
 #define GALV_D2H(dst, src_off, bytes)                                                              \
     if ((e = cudaMemcpyAsync((dst), d + (src_off), (bytes), cudaMemcpyDeviceToHost, st)) != cudaSuccess) \
         return cuda_fail(ctx, "galv_search_host (copy out)", e)

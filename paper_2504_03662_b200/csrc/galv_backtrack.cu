@@ -28,7 +28,7 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
                                  const int32_t* __restrict__ L, const int32_t* __restrict__ time_q,
                                  const int32_t* __restrict__ mem_q, const int32_t* __restrict__ trans_q,
                                  const int32_t* __restrict__ C, const uint8_t* __restrict__ A,
-                                 const int32_t* __restrict__ C_last, const int32_t* __restrict__ budget,
+                                 const int32_t* __restrict__ C_last, const int32_t* __restrict__ lean_map, const int32_t* __restrict__ budget,
                                  int32_t* __restrict__ opt_cost, int32_t* __restrict__ plan,
                                  int32_t* __restrict__ mem_used, int32_t* __restrict__ status)
 {
@@ -83,12 +83,23 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
     // candidate of the step before), and the mem / time rows of the next layer down are fetched, whole,
     // while this layer's candidates are in flight; lane k%32 keeps entries k, k+32, ... (S <= 256).
     int cur = opt;                                             // C[l][m][s] of the cell the walk stands on
-    int mrow[NJ], trow[NJ];
+    int mrow[NJ], trow[NJ], mnext[NJ], tnext[NJ];              // rows of layers l and l-1
+    // the resident kernel's states in place of the table: state row of each of this lane's strategies, rows a layer
+    const bool lean = !A && lean_map && lean_map[(size_t)i * S] >= 0;
+    int crow[NJ], rows = 0;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        crow[j] = lean && lane + 32 * j < S ? lean_map[(size_t)i * S + lane + 32 * j] : 0;
+        rows = max(rows, crow[j] + 1);
+    }
+    rows = __reduce_max_sync(0xffffffffu, rows);
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
         mrow[j] = k < S ? mq[(Li - 1) * S + k] : 0;
         trow[j] = k < S ? tq[(Li - 1) * S + k] : 0;
+        mnext[j] = k < S && Li > 1 ? mq[(Li - 2) * S + k] : 0;
+        tnext[j] = k < S && Li > 1 ? tq[(Li - 2) * S + k] : 0;
     }
     for (int l = Li - 1; l >= 0; --l) {
         if (lane == 0) pl[l] = s;
@@ -107,10 +118,11 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
         }
         if (l == 0) break;
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) {                          // rows of layer l-1, needed one step from now
+        for (int j = 0; j < NJ; ++j) {                          // rows of layer l-2 asked for, a step before the walk gets there
             const int k = lane + 32 * j;
-            mrow[j] = k < S ? mq[(l - 1) * S + k] : 0;
-            trow[j] = k < S ? tq[(l - 1) * S + k] : 0;
+            mrow[j] = mnext[j]; trow[j] = tnext[j];
+            mnext[j] = k < S && l > 1 ? mq[(l - 2) * S + k] : 0;
+            tnext[j] = k < S && l > 1 ? tq[(l - 2) * S + k] : 0;
         }
         int sp;
         if (A) {
@@ -125,7 +137,14 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
 #pragma unroll
             for (int j = 0; j < NJ; ++j) {
                 const int k = lane + 32 * j;
-                cv[j] = k < S ? prev[(size_t)k * m_pitch] : kInf;
+                if (lean) {
+                    // value of strategy k in layer l-1: its time on top of the state at the column its memory leaves
+                    const int src = m - mm - mrow[j];
+                    const int g = k < S && src >= 0 ? (l > 1 ? C[(size_t)i * Lmax * slice + ((size_t)(l - 1) * rows + crow[j]) * m_pitch + src] : 0) : kInf;
+                    cv[j] = g < kInf ? g + trow[j] : kInf;
+                } else {
+                    cv[j] = k < S ? prev[(size_t)k * m_pitch] : kInf;
+                }
                 tv[j] = k < S ? T[k * S + s] : 0;
             }
 #pragma unroll
@@ -155,14 +174,14 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
 
 cudaError_t galv_backtrack_launch(const galv_shape* sh, const int32_t* L, const int32_t* time_q,
                                   const int32_t* mem_q, const int32_t* trans_q, const int32_t* C,
-                                  const uint8_t* A, const int32_t* C_last, const int32_t* budget,
+                                  const uint8_t* A, const int32_t* C_last, const int32_t* lean_map, const int32_t* budget,
                                   int32_t* opt_cost, int32_t* plan, int32_t* mem_used, int32_t* status,
                                   cudaStream_t st)
 {
     const int warps = 4;
     const dim3 grid((sh->B + warps - 1) / warps), block(warps * 32);
 #define GALV_WALK(NJ) backtrack_kernel<NJ><<<grid, block, 0, st>>>( \
-        sh->B, sh->Lmax, sh->S, sh->M, sh->m_pitch, galv_trans_inst(sh), galv_trans_layer(sh), L, time_q, mem_q, trans_q, C, A, C_last, budget, \
+        sh->B, sh->Lmax, sh->S, sh->M, sh->m_pitch, galv_trans_inst(sh), galv_trans_layer(sh), L, time_q, mem_q, trans_q, C, A, C_last, lean_map, budget, \
         opt_cost, plan, mem_used, status)
     if (sh->S <= 32) GALV_WALK(1);
     else if (sh->S <= 64) GALV_WALK(2);

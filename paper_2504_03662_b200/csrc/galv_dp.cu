@@ -1814,7 +1814,9 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
             return cudaSuccess;
         };
         RsPlan rp[2];
-        const int n = galv_resident_plan(ctx, sh, rp);
+        galv_shape kept = *sh;
+        if (a.lean_map) kept.flags &= ~GALV_STORE_C_FULL;
+        const int n = galv_resident_plan(ctx, &kept, rp);
         int launched = 0;
         while (launched < n) {
             if (galv_resident_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now

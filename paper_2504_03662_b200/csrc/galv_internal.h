@@ -87,6 +87,8 @@ struct DpArgs {
     int32_t* ntiles;     // [Lmax+1] tiles per instance that can store anything in layer l
     int32_t* tcount;     // [Lmax][ntiles_m] layers 1..l whose items include tile t
     int32_t* status;
+    int32_t* lean_map;   // host entry point (nobody sees the table): [B][S] state row of each strategy where the resident kernel has left
+                         // the states between the layers in C in place of its values; -1 where C holds the values.  Else NULL
     int32_t* done;       // [B] instances the resident kernel has finished, or NULL when it was not launched
     int withhold;        // test hook: CTA 0 never loads its first chunk, so that the bounded waits run out
     int skip_dom;        // packed path: leave out row pairs that cannot win in any column of a warp group's tile
@@ -129,7 +131,7 @@ inline long long galv_trans_layer(const galv_shape* sh) { return (sh->flags & GA
 inline long long galv_trans_inst(const galv_shape* sh) { return (long long)sh->S * sh->S * ((sh->flags & GALV_TRANS_PER_LAYER) ? sh->Lmax : 1); }
 cudaError_t galv_backtrack_launch(const galv_shape* sh, const int32_t* L, const int32_t* time_q,
                                   const int32_t* mem_q, const int32_t* trans_q, const int32_t* C,
-                                  const uint8_t* A, const int32_t* C_last, const int32_t* budget,
+                                  const uint8_t* A, const int32_t* C_last, const int32_t* lean_map, const int32_t* budget,
                                   int32_t* opt_cost, int32_t* plan, int32_t* mem_used, int32_t* status,
                                   cudaStream_t st);
 cudaError_t galv_costs_launch(const galv_shape* sh, const int32_t* L, const galv_layer_desc* layers,

@@ -63,6 +63,8 @@ struct RsArgs {
     const int32_t* trans_q;
     long long trans_inst, trans_layer;
     int32_t* C;        // full table or NULL
+    int32_t* states;   // in place of the table, when nobody sees it: the states between the layers, [Lmax][rows][m_pitch] per instance; or NULL
+    int32_t* map;      // [B][S] state row of each strategy, with `states`
     uint8_t* A;        // argmin table or NULL
     int32_t* C_last;
     int32_t* status;
@@ -168,6 +170,7 @@ struct Ctx {
     const int* cdelta;         // [16] cluster-window address of CTA d minus this CTA's own shared address
     int32_t* stage;            // [2][S][W] collected rows
     int32_t* C;                // this instance's table
+    int32_t* states;           // ... or the states between its layers, or NULL
     uint8_t* A;
     int32_t* C_last;
     size_t slice;
@@ -311,14 +314,21 @@ __device__ __forceinline__ void gather_arg(const Ctx& c, uint32_t aa, int x, int
 }
 
 // Values of one state row for the tile.
-template <int TM, bool ARG>
-__device__ __forceinline__ void emit(const Ctx& c, uint32_t gn, uint32_t an, int k, int colb, int lane, const int (&v)[TM], const int (&a)[TM])
+template <int TM, bool ARG, bool KEEP>
+__device__ __forceinline__ void emit(const Ctx& c, int l, uint32_t gn, uint32_t an, int k, int colb, int lane, const int (&v)[TM], const int (&a)[TM])
 {
     const int at = k * c.P + c.H + colb + lane;
 #pragma unroll
     for (int j = 0; j < TM; ++j) {
         sts(gn + (uint32_t)(at + 32 * j) * 4u, v[j]);
         if (ARG) sts_u8(an + (uint32_t)(at + 32 * j), a[j]);
+    }
+    if (KEEP && c.states) {
+        const int m = c.rank * c.W + colb + lane;
+        int32_t* const p = c.states + ((size_t)(l + 1) * c.Kc + k) * c.m_pitch + m;
+#pragma unroll
+        for (int j = 0; j < TM; ++j)
+            if (m + 32 * j < c.m_pitch) p[32 * j] = v[j];
     }
 }
 
@@ -463,7 +473,7 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
         if (STORE || ARG)
 #pragma unroll 4
             for (int e = 0; e < c.S; ++e) out.template put<TM>((uint32_t)(e * (STAGE ? c.W : c.m_pitch)) * 4u, inf, none);
-        for (int k = 0; k < c.Kc; ++k) emit<TM, ARG>(c, gn, an, k, colb, lane, inf, none);
+        for (int k = 0; k < c.Kc; ++k) emit<TM, ARG, !STORE && !ARG>(c, l, gn, an, k, colb, lane, inf, none);
         return;
     }
 
@@ -570,7 +580,7 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
         }
 #pragma unroll
         for (int k = 0; k < KC; ++k)
-            if (k < c.Kc) emit<TM, ARG>(c, gn, an, k, colb, lane, acc[k], arg[ARG ? k : 0]);
+            if (k < c.Kc) emit<TM, ARG, !STORE && !ARG>(c, l, gn, an, k, colb, lane, acc[k], arg[ARG ? k : 0]);
     } else {
         int thr[TM], dummy[TM];
 #pragma unroll
@@ -632,7 +642,7 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
                 }
 #pragma unroll
             for (int k = 0; k < KC; ++k)
-                if (cb + k < c.S) emit<TM, ARG>(c, gn, an, cb + k, colb, lane, acc[k], arg[ARG ? k : 0]);
+                if (cb + k < c.S) emit<TM, ARG, !STORE && !ARG>(c, l, gn, an, cb + k, colb, lane, acc[k], arg[ARG ? k : 0]);
         }
     }
 }
@@ -1096,6 +1106,9 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     c.cs = s_first; c.csp = s_csp; c.slot = s_slot; c.cdelta = s_cdelta;
     c.slice = (size_t)S * a.m_pitch;
     c.C = STORE ? a.C + (size_t)i * Lmax * c.slice : nullptr;
+    c.states = a.states ? a.states + (size_t)i * Lmax * c.slice : nullptr;
+    if (a.states && rank == 0)
+        for (int s = tid; s < S; s += NT) a.map[(size_t)i * S + s] = s_ccls[s];
     c.A = ARG ? a.A + (size_t)i * Lmax * c.slice : nullptr;
     c.C_last = a.C_last + (size_t)i * c.slice;
     c.bars = smem_addr(&s_bar[0]);
@@ -1299,9 +1312,12 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
         t *= p.rounds > 3 ? (double)sh->B / slots + 0.5 : p.rounds;          // ragged batches fill the last round
         p.halo_fits = cl == 1 || (long long)rows * (w + halo) <= p.gints;
         if (!p.halo_fits) t *= 4.0;                            // shifts beyond the halo take the slow way
-        if (!found || t < *est) {
+        // Of two sizes that come out about the same the finer one: ragged batches, whose lengths the host does not know,
+        // fill the SMs better with it (64 instances of 1 to 96 layers: 0.79 ms on clusters of 2, 0.51 on clusters of 4;
+        // with 96 layers each 0.79 and 0.94).
+        if (!found || t < *est * (out->rounds == 1 && p.rounds <= 2 && sh->B > 1 ? 1.12 : 1.0)) {
             found = true;
-            *est = t;
+            *est = t < *est || *est == 0.0 ? t : *est;
             p.sorted = sh->B > slots && sh->B <= kMaxSortedB;
             *out = p;
         }
@@ -1329,7 +1345,7 @@ int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
     // argmin table, where only the tiled kernels compete, one instance 0.27 against 0.78 ms.
     bool d = (sh->S <= 32 || arg || forced) && best_plan(ctx, sh, sh->S, true, &plans[1], &td);
     if (d && !forced) d = plans[1].halo_fits && plans[1].rounds == 1;
-    const bool c = !(sh->flags & GALV_TRANS_PER_LAYER) && sh->S > 8 && best_plan(ctx, sh, sh->S < 12 ? sh->S : 12, false, &plans[0], &tc);
+    const bool c = !(sh->flags & GALV_TRANS_PER_LAYER) && sh->S > 8 && best_plan(ctx, sh, sh->S < 9 ? sh->S : 9, false, &plans[0], &tc);
     if (d && (!c || forced || td <= tc * 1.3)) { plans[0] = plans[1]; n = 1; }
     else if (c) n = d ? 2 : 1;
     ctx->plan_shape = *sh; ctx->plans[0] = plans[0]; ctx->plans[1] = plans[1]; ctx->plan_launches = n; ctx->plan_valid = 1;
@@ -1357,7 +1373,9 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
     a.path_value = (d.B <= kMaxSortedB && !d.A) ? 2 : 0;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
-    a.C = d.C; a.A = d.A; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done;
+    const bool lean = d.lean_map != nullptr;
+    a.C = lean ? nullptr : d.C; a.states = lean ? d.C : nullptr; a.map = d.lean_map;
+    a.A = d.A; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done;
     a.stage_at = p.stage_at;
     CUtensorMap mc, ml;
     std::memset(&mc, 0, sizeof(mc));
@@ -1367,5 +1385,5 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
         if (e == cudaSuccess) e = encode_table_3d(&mc, d.C, (size_t)d.B * d.Lmax * d.S, d.m_pitch, d.S, p.w / 32);
         if (e != cudaSuccess) return e;
     }
-    return launch_resident(kernel_of(d.C != nullptr, d.A != nullptr, p.stage), a, p, mc, ml, st, nullptr);
+    return launch_resident(kernel_of(a.C != nullptr, d.A != nullptr, p.stage), a, p, mc, ml, st, nullptr);
 }
