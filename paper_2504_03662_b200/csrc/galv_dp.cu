@@ -272,7 +272,17 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
         if (l < Lmax && minmem_l[l] <= M) nt = min(ntiles_m, (M - minmem_l[l]) / tmb + 1);
         ntiles[l] = max(1, nt);
     }
+    __shared__ int s_any;
+    if (threadIdx.x == 0) s_any = 0;
     __syncthreads();
+    for (int l = threadIdx.x; l <= Lmax; l += blockDim.x)
+        if (hist[l]) s_any = 1;
+    __syncthreads();
+    if (done && !s_any) {                              // every instance is finished: an empty schedule
+        for (int l = threadIdx.x; l <= Lmax; l += blockDim.x) { nactive[l] = 0; istart[l] = 0; }
+        if (threadIdx.x == 0) maxmem[2] = 2;
+        return;
+    }
     {
         long long carry = 0, total;                    // instances with L > l: a sum from the top layer down
         for (int base = 0; base <= Lmax; base += 1024) {
@@ -284,7 +294,6 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0 && done && nactive[0] == 0) maxmem[2] = 2;      // nothing left for the tiled kernels
     for (int i = threadIdx.x; i < B; i += blockDim.x)
         if (status[i] == 0 && !(done && done[i])) {
             const int Li = L[i];
@@ -316,8 +325,10 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
 // C[0][s][m] = time(0,s) if mem(0,s) <= m else INF; pad columns INF; A = 255.
 __global__ void base_layer_kernel(DpArgs a)
 {
-    const int i = blockIdx.z, s = blockIdx.y;
-    if (a.status[i] != 0 || (a.done && a.done[i])) return;
+    // with most instances finished elsewhere (done) a few blocks look after many rows, else a block has one
+    for (int row_at = blockIdx.y; row_at < a.B * a.S; row_at += gridDim.y) {
+    const int i = row_at / a.S, s = row_at - i * a.S;
+    if (a.status[i] != 0 || (a.done && a.done[i])) continue;
     const int tt = a.time_q[(size_t)i * a.Lmax * a.S + s];
     const int mm = a.mem_q[(size_t)i * a.Lmax * a.S + s];
     const size_t row = ((size_t)i * a.S + s) * a.m_pitch;
@@ -327,6 +338,7 @@ __global__ void base_layer_kernel(DpArgs a)
         const int v = (m <= a.M && mm <= m) ? tt : kInf;
         out[m] = v;
         if (ao) ao[m] = 255;
+    }
     }
 }
 
@@ -1862,18 +1874,10 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     auto base_layer = [&]() {
         int gx = (a.m_pitch + 255) / 256;
         if (gx > 8) gx = 8;
-        for (int b0 = 0; b0 < B; b0 += 65535) {           // grid.z limit
-            DpArgs s = a;
-            const int nb = (B - b0 < 65535) ? B - b0 : 65535;
-            s.L += b0; s.status += b0;
-            if (s.done) s.done += b0;
-            s.time_q += (size_t)b0 * Lmax * S; s.mem_q += (size_t)b0 * Lmax * S;
-            if (s.C) s.C += (size_t)b0 * Lmax * S * a.m_pitch;
-            if (s.A) s.A += (size_t)b0 * Lmax * S * a.m_pitch;
-            s.C_last += (size_t)b0 * S * a.m_pitch;
-            s.roll += (size_t)b0 * S * a.m_pitch;
-            base_layer_kernel<<<dim3(gx, S, nb), 256, 0, st>>>(s);
-        }
+        long long rows = (long long)B * S;
+        const long long most = a.done ? 4 * 148 / gx : 65535; // grid.y limit
+        if (rows > most) rows = most;
+        base_layer_kernel<<<dim3(gx, (unsigned)rows), 256, 0, st>>>(a);
     };
     base_layer();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1975,7 +1979,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         c.C_last += (size_t)b0 * S * a.m_pitch;
         c.roll += (size_t)b0 * S * a.m_pitch;
         size_t per = ((size_t)S * a.m_pitch / 4 + 255) / 256;
-        if (per > 64) per = 64;
+        if (per > (a.done ? 8 : 64)) per = a.done ? 8 : 64;
         copy_last_kernel<<<dim3((unsigned)per, nb), 256, 0, st>>>(c);
     }
     finalize_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, a.err, a.status);

@@ -145,12 +145,6 @@ __device__ __forceinline__ void cp_async_4(void* dst, const void* src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ uint32_t mix(uint32_t v, uint32_t k) {
-    v = (v ^ (k * 0x9E3779B1u)) * 0x85EBCA6Bu;
-    v ^= v >> 15;
-    v *= 0xC2B2AE35u;
-    return v ^ (v >> 13);
-}
 
 // Everything the layer loop needs; lives in registers (all members are uniform over the CTA).
 struct Ctx {
@@ -728,8 +722,8 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                                                                            const __grid_constant__ CUtensorMap map_last)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ union { int L[kMaxSortedB]; struct { uint32_t rh[kMaxS], ch[kMaxS]; } h; } s_u;
-    __shared__ int s_rrep[kMaxS], s_crep[kMaxS], s_rcls[kMaxS], s_ccls[kMaxS], s_order[kMaxS + kClassMax], s_csp[4 * (kClassMax + 1)], s_first[kClassMax + 1], s_cnt[kClassMax];
+    __shared__ int s_len[kMaxSortedB], s_twin[2 * kMaxS], s_root[2 * kClassMax];
+    __shared__ int s_ccls[kMaxS], s_order[kMaxS + kClassMax], s_csp[4 * (kClassMax + 1)], s_first[kClassMax + 1], s_cnt[kClassMax];
     __shared__ int s_cdelta[16], s_front[4], s_reach[4], s_slot[4], s_inst, s_K[2];
     __shared__ struct { long long sum; int tmax, bad, mmax; } s_part, s_all;
     __shared__ __align__(8) unsigned long long s_bar[2];
@@ -757,14 +751,14 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     if (a.sorted) {
         for (int j = tid; j < a.B; j += NT) {
             const int v = a.L[j];
-            s_u.L[j] = (v < 1 || v > Lmax) ? 0 : v;
+            s_len[j] = (v < 1 || v > Lmax) ? 0 : v;
         }
         __syncthreads();
         for (int j = tid; j < a.B; j += NT) {
-            const int Lj = s_u.L[j];
+            const int Lj = s_len[j];
             int before = 0;
             for (int k = 0; k < a.B; ++k) {
-                const int Lk = s_u.L[k];
+                const int Lk = s_len[k];
                 before += (Lk > Lj) || (Lk == Lj && k < j);
             }
             if (before == cid) s_inst = j;
@@ -784,9 +778,23 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
 
     // ---- validation: the CTAs of the cluster share the layers (and matrices); one matrix per instance is staged whole
     int32_t* const stage = g0;                                 // the state is not in use yet
-    const bool staged = !a.trans_layer && (long long)S * S <= (long long)2 * gints;
+    const int TP = S | 1;                                       // odd pitch: columns are read without bank conflicts too
+    const bool staged = !a.trans_layer && (long long)S * TP <= (long long)2 * gints;
+    auto fetch = [&](int l) {
+        int32_t* const rm = raw + (l & 3) * 2 * S;
+        for (int s = lane; s < S; s += 32) {
+            cp_async_4(rm + s, mq + (size_t)l * S + s);
+            cp_async_4(rm + S + s, tq + (size_t)l * S + s);
+        }
+    };
+    if (warp == NW) {                                           // the first layers' rows are under way while the rest is looked at
+        fetch(0);
+        if (Li > 1) fetch(1);
+        cp_async_commit();
+        if (Li > 2) fetch(2);
+        cp_async_commit();
+    }
     if (tid == 0) { s_part.sum = 0; s_part.tmax = 0; s_part.bad = 0; s_part.mmax = 0; }
-    for (int x = tid; x < kMaxS; x += NT) { s_u.h.rh[x] = 0; s_u.h.ch[x] = 0; }
     if (tid == 0) {
         s_late = 0;
         mbar_init(smem_addr(&s_bar[0])); mbar_init(smem_addr(&s_bar[1]));
@@ -823,7 +831,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                 const int v = T0[k];
                 bad |= v < 0;
                 tmax = max(tmax, v);
-                if (staged) stage[k] = v;
+                if (staged) { const int q = k / S; stage[q * TP + k - q * S] = v; }
             }
         }
         tmax = __reduce_max_sync(0xffffffffu, tmax);
@@ -836,7 +844,86 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
             if (bad) atomicOr(&s_part.bad, 1);
         }
     }
-    whole_barrier(CL);
+    __syncthreads();                                            // the partial results and the staged matrix
+    if (CL > 1) cluster_arrive();
+
+    // ---- classes of equal rows and equal columns
+    int K = S;                                                  // unstructured unless found otherwise
+    if (staged) {
+        // the nearest earlier twin of every row (0 .. S-1) and column (S .. 2S-1), compared word by word, a warp each
+        auto twins = [&](auto words) {
+            constexpr int N = decltype(words)::value;
+            for (int x = warp; x < 2 * S; x += NW + 1) {
+                const bool row = x < S;
+                const int me = row ? x : x - S, step = row ? TP : 1, word = row ? 1 : TP;      // from one row / column, or word, to the next
+                int w[N];
+#pragma unroll
+                for (int j = 0; j < N; ++j) w[j] = lane + 32 * j < S ? stage[me * step + (lane + 32 * j) * word] : 0;
+                int twin = me;
+                for (int o = me - 1; o >= 0; --o) {
+                    bool diff = false;
+#pragma unroll
+                    for (int j = 0; j < N; ++j)
+                        if (lane + 32 * j < S) diff |= stage[o * step + (lane + 32 * j) * word] != w[j];
+                    if (!__any_sync(0xffffffffu, diff)) { twin = o; break; }
+                }
+                if (lane == 0) s_twin[x] = twin;
+            }
+        };
+        if (S <= 32) twins(std::integral_constant<int, 1>());
+        else if (S <= 64) twins(std::integral_constant<int, 2>());
+        else twins(std::integral_constant<int, kMaxS / 32>());
+        __syncthreads();
+        // a class is the twins that lead back to the same first; classes are numbered in the order of their firsts, and
+        // the strategies put into the order of their rows' classes: one warp for the rows, one for the columns
+        if (warp < 2) {
+            volatile int* const tw = s_twin + (warp == 0 ? 0 : S);
+            for (int span = 1; span < S; span <<= 1) {          // pointer jumping: any value read is an ancestor
+                for (int s = lane; s < S; s += 32) tw[s] = tw[tw[s]];
+                __syncwarp();
+            }
+            unsigned first[kMaxS / 32];                         // which strategies open a class
+            int k = 0, cls[kMaxS / 32];
+#pragma unroll
+            for (int j = 0; j < kMaxS / 32; ++j) {
+                const int s = lane + 32 * j;
+                first[j] = __ballot_sync(0xffffffffu, s < S && tw[s] == s);
+                k += __popc(first[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < kMaxS / 32; ++j) {
+                const int s = lane + 32 * j, root = s < S ? tw[s] : 0;
+                int n = 0;
+#pragma unroll
+                for (int q = 0; q < kMaxS / 32; ++q) n += __popc(first[q] & (q < (root >> 5) ? ~0u : q == (root >> 5) ? (1u << (root & 31)) - 1u : 0u));
+                cls[j] = s < S ? n : -1;
+                if (s < S && warp == 1) s_ccls[s] = n;
+                if (s < S && root == s && n < kClassMax) s_root[warp * kClassMax + n] = s;
+            }
+            if (lane == 0) s_K[warp] = k;
+            if (warp == 0 && k <= kClassMax) {
+                // ascending inside a class; a class of an odd number has its last one twice
+                int at = 0;
+                for (int q = 0; q < k; ++q) {
+                    int n = 0;
+#pragma unroll
+                    for (int j = 0; j < kMaxS / 32; ++j) {
+                        const unsigned in = __ballot_sync(0xffffffffu, cls[j] == q);
+                        const int pos = at + n + __popc(in & ((1u << lane) - 1u));
+                        if (cls[j] == q) s_order[pos + 1] = lane + 32 * j;             // the next entry's owner overwrites it, if there is one
+                        __syncwarp();
+                        if (cls[j] == q) s_order[pos] = lane + 32 * j;
+                        __syncwarp();
+                        n += __popc(in);
+                    }
+                    if (lane == 0) { s_first[q] = at; s_cnt[q] = n; }
+                    at += (n + 1) & ~1;
+                }
+                if (lane == 0) s_first[k] = at;
+            }
+        }
+    }
+    if (CL > 1) cluster_wait();                                 // everybody's partial results
     if (warp == 0) {
         long long sum = 0;
         int tmax = 0, bad = 0, mmax = 0;
@@ -858,105 +945,16 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
         }
         if (lane == 0) { s_all.sum = sum; s_all.tmax = tmax; s_all.bad = bad; s_all.mmax = mmax; }
     }
-
-    // ---- classes of equal rows and equal columns
-    int K = S;                                                  // unstructured unless found otherwise
-    if (staged) {
-        // a sum of mixed words per row and per column proposes twins ...
-        for (int r = warp; r < S; r += NW + 1) {
-            uint32_t h = 0;
-            for (int s = lane; s < S; s += 32) h += mix((uint32_t)stage[r * S + s], (uint32_t)s);
-            h = __reduce_add_sync(0xffffffffu, h);
-            if (lane == 0) s_u.h.rh[r] = h;
-        }
-        const int parts = max(1, NT / S);
-        for (int x = tid; x < parts * S; x += NT) {
-            const int s = x % S, p = x / S;
-            uint32_t h = 0;
-            for (int r = p; r < S; r += parts) h += mix((uint32_t)stage[r * S + s], (uint32_t)r);
-            atomicAdd(&s_u.h.ch[s], h);
-        }
-        __syncthreads();
-        for (int x = tid; x < 2 * S; x += NT) {
-            const uint32_t* const hh = x < S ? s_u.h.rh : s_u.h.ch;
-            const int s = x < S ? x : x - S;
-            int o = 0;
-            while (hh[o] != hh[s]) ++o;                         // ends at s itself at the latest
-            (x < S ? s_rrep : s_crep)[s] = o;
-            (x < S ? s_rcls : s_ccls)[s] = 0;                   // for now: words that differ
-        }
-        __syncthreads();
-        // ... and a comparison of all their words decides
-        for (int r = warp; r < S; r += NW + 1) {
-            const int o = s_rrep[r];
-            int diff = 0;
-            for (int s = lane; s < S; s += 32) diff |= stage[r * S + s] != stage[o * S + s];
-            if (__any_sync(0xffffffffu, diff) && lane == 0) s_rcls[r] = 1;
-        }
-        for (int x = tid; x < parts * S; x += NT) {
-            const int s = x % S, p = x / S, o = s_crep[s];
-            int diff = 0;
-            for (int r = p; r < S; r += parts) diff |= stage[r * S + s] != stage[r * S + o];
-            if (diff) s_ccls[s] = 1;
-        }
-        __syncthreads();
-        for (int s = tid; s < S; s += NT) {
-            if (s_rcls[s]) s_rrep[s] = s;
-            if (s_ccls[s]) s_crep[s] = s;
-        }
-        __syncthreads();
-        // class numbers in the order of the classes' first members
-        for (int x = tid; x < 2 * S; x += NT) {
-            const int* const rep = x < S ? s_rrep : s_crep;
-            const int s = x < S ? x : x - S, me = rep[s];
-            int k = 0;
-            for (int o = 0; o < me; ++o) k += rep[o] == o;
-            (x < S ? s_rcls : s_ccls)[s] = k;
-        }
-        if (warp < 2) {                                         // there are at least two warps
-            const int* const rep = warp == 0 ? s_rrep : s_crep;
-            int k = 0;
-            for (int s = lane; s < S; s += 32) k += rep[s] == s;
-            k = __reduce_add_sync(0xffffffffu, k);
-            if (lane == 0) s_K[warp] = k;
-        }
-        __syncthreads();
-        K = max(s_K[0], s_K[1]);
-    }
+    __syncthreads();
+    if (staged) K = max(s_K[0], s_K[1]);
     const bool classes = staged && K <= kClassMax && s_K[1] * W <= gints;
     const bool dense = !classes && a.SP > 0 && S * W <= gints;
     const int Kr = classes ? s_K[0] : S, Kc = classes ? s_K[1] : S;
     if (classes) {
-        // strategies in class order, ascending inside a class; a class of an odd number has its last one twice
-        for (int k = tid; k <= Kr; k += NT) s_first[k] = 0;
-        __syncthreads();
-        for (int s = tid; s < S; s += NT) atomicAdd(&s_first[s_rcls[s]], 1);
-        __syncthreads();
-        if (warp == 0) {
-            const int n = lane < Kr ? s_first[lane] : 0;
-            int at = (n + 1) & ~1;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, at, o);
-                if (lane >= o) at += v;
-            }
-            if (lane < Kr) { s_first[lane] = at - ((n + 1) & ~1); s_cnt[lane] = n; }
-            if (lane == Kr - 1) s_first[Kr] = at;
+        for (int x = tid; x < kClassMax * kClassMax; x += NT) {
+            const int k = x / kClassMax, q = x - k * kClassMax;
+            tsm[x] = k < Kr && q < Kc ? stage[s_root[k] * TP + s_root[kClassMax + q]] : 0;
         }
-        __syncthreads();
-        for (int s = tid; s < S; s += NT) {
-            const int me = s_rcls[s];
-            int before = 0, size = 0;
-            for (int o = 0; o < S; ++o) { size += s_rcls[o] == me; before += s_rcls[o] == me && o < s; }
-            s_order[s_first[me] + before] = s;
-            if (before == size - 1 && (size & 1)) s_order[s_first[me] + size] = s;
-        }
-        for (int x = tid; x < kClassMax * kClassMax; x += NT) tsm[x] = 0;
-        __syncthreads();
-        for (int r = warp; r < S; r += NW + 1)
-            if (s_rrep[r] == r)
-                for (int s = lane; s < S; s += 32)
-                    if (s_crep[s] == s) tsm[s_rcls[r] * kClassMax + s_ccls[s]] = stage[r * S + s];
     } else if (dense) {
         for (int s = tid; s < S; s += NT) { s_order[s] = s; s_ccls[s] = s; }
         // the matrix paid between layers 0 and 1; with one matrix per layer, matrix l sits in buffer l & 1
@@ -964,7 +962,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
         int32_t* const dst = tsm + (a.trans_layer ? tfull : 0);
         for (int x = tid; x < tfull; x += NT) {
             const int r = x / a.SP, s = x - r * a.SP;
-            const int v = (s < S && Li > 1) ? (staged ? stage[r * S + s] : T[r * S + s]) : 0;
+            const int v = (s < S && Li > 1) ? (staged ? stage[r * TP + s] : T[r * S + s]) : 0;
             dst[x] = v;
             if (a.trans_layer) tsm[x] = 0;                      // pad columns of the other buffer stay 0
         }
@@ -1064,21 +1062,9 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
         __syncwarp();
         return f;
     };
-    auto fetch = [&](int l) {
-        int32_t* const rm = raw + (l & 3) * 2 * S;
-        for (int s = lane; s < S; s += 32) {
-            cp_async_4(rm + s, mq + (size_t)l * S + s);
-            cp_async_4(rm + S + s, tq + (size_t)l * S + s);
-        }
-    };
     int front = 0;
     if (run) {
         if (warp == NW) {
-            fetch(0);
-            if (Li > 1) fetch(1);
-            cp_async_commit();
-            if (Li > 2) fetch(2);
-            cp_async_commit();
             cp_async_wait<1>();
             __syncwarp();
             front = prepare(0, 0);
@@ -1097,7 +1083,10 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");            // bulk copies write over the halo's initial values
     whole_barrier(CL);                                          // also: nobody leaves while its partial sums are being read
-    if (!run) return;
+    if (!run) {
+        if (warp == NW) cp_async_wait<0>();                     // nothing may land in shared memory that is no longer ours
+        return;
+    }
 
     Ctx c;
     c.S = S; c.M = M; c.W = W; c.H = H; c.P = P; c.G = W / 32; c.CL = CL; c.rank = rank; c.Li = Li; c.m_pitch = a.m_pitch; c.Kr = Kr; c.Kc = Kc;
@@ -1346,7 +1335,8 @@ int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
     bool d = (sh->S <= 32 || arg || forced) && best_plan(ctx, sh, sh->S, true, &plans[1], &td);
     if (d && !forced) d = plans[1].halo_fits && plans[1].rounds == 1;
     const bool c = !(sh->flags & GALV_TRANS_PER_LAYER) && sh->S > 8 && best_plan(ctx, sh, sh->S < 9 ? sh->S : 9, false, &plans[0], &tc);
-    if (d && (!c || forced || td <= tc * 1.3)) { plans[0] = plans[1]; n = 1; }
+    // a launch that takes every instance spares the ones after it, which find nothing to do (20 us, 40 thousand cycles)
+    if (d && (!c || forced || td * sh->Lmax <= tc * sh->Lmax * 1.05 + 40000.0)) { plans[0] = plans[1]; n = 1; }
     else if (c) n = d ? 2 : 1;
     ctx->plan_shape = *sh; ctx->plans[0] = plans[0]; ctx->plans[1] = plans[1]; ctx->plan_launches = n; ctx->plan_valid = 1;
     return n;
