@@ -30,17 +30,30 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
                                  const int32_t* __restrict__ C, const uint8_t* __restrict__ A,
                                  const int32_t* __restrict__ C_last, const int32_t* __restrict__ lean_map, const int32_t* __restrict__ budget,
                                  int32_t* __restrict__ opt_cost, int32_t* __restrict__ plan,
-                                 int32_t* __restrict__ mem_used, int32_t* __restrict__ status)
+                                 int32_t* __restrict__ mem_used, int32_t* __restrict__ status, const bool staged)
 {
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= B) return;
-    const int st0 = status[i] & ~GALV_STATUS_INFEASIBLE;
+    extern __shared__ int32_t s_trans[];                       // the instance's transition matrix, where it has one that fits
+    const int lane = threadIdx.x;
+    const int i = blockIdx.x;
+    // what does not depend on anything is asked for at once: every round trip to memory counts in a walk of a few dozen
+    const int Li = L[i], st_in = status[i], bud = budget ? budget[i] : M;
+    const size_t slice = (size_t)S * m_pitch;
+    const int32_t* const T0 = trans_q + (size_t)i * trans_inst;
+    if (staged) {
+        for (int k = lane; k < S * S; k += 32)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(s_trans + k)), "l"(T0 + k) : "memory");
+    }
+    unsigned long long key = ~0ull;                            // optimum at the budget: lowest s among the minima
+    for (int s = lane; s < S; s += 32) {
+        const unsigned long long k = ((unsigned long long)(unsigned)C_last[(size_t)i * slice + (size_t)s * m_pitch + min(max(bud, 0), M)] << 32) | (unsigned)s;
+        key = k < key ? k : key;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");           // the matrix
+    const int st0 = st_in & ~GALV_STATUS_INFEASIBLE;
     int32_t* pl = plan ? plan + (size_t)i * Lmax : nullptr;
     if (pl)
         for (int l = lane; l < Lmax; l += 32) pl[l] = -1;
     __syncwarp();          // lane 0 overwrites entries other lanes have just cleared
-    const int bud = budget ? budget[i] : M;
     // a search whose bounded waits ran out left void tables: not walked either
     const bool skip = (st0 & (GALV_STATUS_BAD_INPUT | GALV_STATUS_OVERFLOW_RISK | GALV_STATUS_TIMEOUT)) != 0 || bud < 0 || bud > M;
     if (skip) {
@@ -50,15 +63,6 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
             status[i] = st0 | ((bud < 0 || bud > M) ? GALV_STATUS_BAD_INPUT : 0);
         }
         return;
-    }
-    const int Li = L[i];
-    const size_t slice = (size_t)S * m_pitch;
-
-    // optimum at the budget: lowest s among the minima
-    unsigned long long key = ~0ull;
-    for (int s = lane; s < S; s += 32) {
-        const unsigned long long k = ((unsigned long long)(unsigned)C_last[(size_t)i * slice + (size_t)s * m_pitch + bud] << 32) | (unsigned)s;
-        key = k < key ? k : key;
     }
     key = warp_min_u64(key);
     const int opt = (int)(key >> 32);
@@ -76,7 +80,6 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
 
     const int32_t* tq = time_q + (size_t)i * Lmax * S;
     const int32_t* mq = mem_q + (size_t)i * Lmax * S;
-    const int32_t* T0 = trans_q + (size_t)i * trans_inst;
     int m = bud;
     long long used = 0;
     // One dependent memory round trip per layer: the cell's value is carried along (it is the chosen
@@ -101,22 +104,48 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
         mnext[j] = k < S && Li > 1 ? mq[(Li - 2) * S + k] : 0;
         tnext[j] = k < S && Li > 1 ? tq[(Li - 2) * S + k] : 0;
     }
-    for (int l = Li - 1; l >= 0; --l) {
-        if (lane == 0) pl[l] = s;
+    // mem and time of the strategy the walk stands on: from here on they come along with the winner of each step
+    int mm, tt;
+    {
         int msel = mrow[0], tsel = trow[0];
 #pragma unroll
         for (int j = 1; j < NJ; ++j) {
             msel = (s >> 5) == j ? mrow[j] : msel;
             tsel = (s >> 5) == j ? trow[j] : tsel;
         }
-        const int mm = __shfl_sync(0xffffffffu, msel, s & 31);
-        const int tt = __shfl_sync(0xffffffffu, tsel, s & 31);
+        mm = __shfl_sync(0xffffffffu, msel, s & 31);
+        tt = __shfl_sync(0xffffffffu, tsel, s & 31);
+    }
+    for (int l = Li - 1; l >= 0; --l) {
+        if (lane == 0) pl[l] = s;
         used += mm;
         if (mm > m) {                  // cannot happen on consistent tables: the cell would be +inf; never index below column 0
             if (lane == 0) status[i] = st0 | GALV_STATUS_BAD_INPUT;
             break;
         }
         if (l == 0) break;
+        int sp = 255;
+        int cv[NJ], tv[NJ];
+        if (A) {
+            sp = A[((size_t)i * Lmax + l) * slice + (size_t)s * m_pitch + m];
+        } else {
+            // every row's candidate is asked for before the first is looked at: one round trip to memory, not one per 32 rows
+            const int32_t* prev = C + ((size_t)i * Lmax + (l - 1)) * slice + (m - mm);
+            const int32_t* T = T0 + (size_t)l * trans_layer;       // paid between layers l-1 and l
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const int k = lane + 32 * j;
+                if (lean) {
+                    // value of strategy k in layer l-1: its time on top of the state at the column its memory leaves
+                    const int src = m - mm - mnext[j];
+                    const int g = k < S && src >= 0 ? (l > 1 ? C[(size_t)i * Lmax * slice + ((size_t)(l - 1) * rows + crow[j]) * m_pitch + src] : 0) : kInf;
+                    cv[j] = g < kInf ? g + tnext[j] : kInf;
+                } else {
+                    cv[j] = k < S ? prev[(size_t)k * m_pitch] : kInf;
+                }
+                tv[j] = k < S ? (staged ? s_trans[k * S + s] : T[k * S + s]) : 0;
+            }
+        }
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {                          // rows of layer l-2 asked for, a step before the walk gets there
             const int k = lane + 32 * j;
@@ -124,38 +153,28 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
             mnext[j] = k < S && l > 1 ? mq[(l - 2) * S + k] : 0;
             tnext[j] = k < S && l > 1 ? tq[(l - 2) * S + k] : 0;
         }
-        int sp;
+        m -= mm;
         if (A) {
-            sp = A[((size_t)i * Lmax + l) * slice + (size_t)s * m_pitch + m];
+            int msel = mrow[0], tsel = trow[0];
+#pragma unroll
+            for (int j = 1; j < NJ; ++j) {
+                msel = (sp >> 5) == j ? mrow[j] : msel;
+                tsel = (sp >> 5) == j ? trow[j] : tsel;
+            }
+            mm = __shfl_sync(0xffffffffu, msel, sp & 31);
+            tt = __shfl_sync(0xffffffffu, tsel, sp & 31);
         } else {
             const int target = cur - tt;
-            const int32_t* prev = C + ((size_t)i * Lmax + (l - 1)) * slice + (m - mm);
-            const int32_t* T = T0 + (size_t)l * trans_layer;       // paid between layers l-1 and l
-            sp = 255;
-            // every row's candidate is asked for before the first is looked at: one round trip to memory, not one per 32 rows
-            int cv[NJ], tv[NJ];
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int k = lane + 32 * j;
-                if (lean) {
-                    // value of strategy k in layer l-1: its time on top of the state at the column its memory leaves
-                    const int src = m - mm - mrow[j];
-                    const int g = k < S && src >= 0 ? (l > 1 ? C[(size_t)i * Lmax * slice + ((size_t)(l - 1) * rows + crow[j]) * m_pitch + src] : 0) : kInf;
-                    cv[j] = g < kInf ? g + trow[j] : kInf;
-                } else {
-                    cv[j] = k < S ? prev[(size_t)k * m_pitch] : kInf;
-                }
-                tv[j] = k < S ? T[k * S + s] : 0;
-            }
 #pragma unroll
             for (int j = 0; j < NJ; ++j) {
                 if (32 * j >= S) break;
-                const bool hit = (cv[j] < kInf) && (cv[j] + tv[j] == target);
-                const unsigned b = __ballot_sync(0xffffffffu, hit);
+                const unsigned b = __ballot_sync(0xffffffffu, cv[j] < kInf && cv[j] + tv[j] == target);
                 if (b) {
                     const int src = __ffs(b) - 1;
                     sp = 32 * j + src;
                     cur = __shfl_sync(0xffffffffu, cv[j], src);
+                    mm = __shfl_sync(0xffffffffu, mrow[j], src);
+                    tt = __shfl_sync(0xffffffffu, trow[j], src);
                     break;
                 }
             }
@@ -164,7 +183,6 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
             if (lane == 0) status[i] = st0 | GALV_STATUS_BAD_INPUT;
             break;
         }
-        m -= mm;
         s = sp;
     }
     if (lane == 0 && mem_used) mem_used[i] = (int32_t)used;
@@ -178,11 +196,12 @@ cudaError_t galv_backtrack_launch(const galv_shape* sh, const int32_t* L, const 
                                   int32_t* opt_cost, int32_t* plan, int32_t* mem_used, int32_t* status,
                                   cudaStream_t st)
 {
-    const int warps = 4;
-    const dim3 grid((sh->B + warps - 1) / warps), block(warps * 32);
-#define GALV_WALK(NJ) backtrack_kernel<NJ><<<grid, block, 0, st>>>( \
+    // a warp per instance, a CTA of its own; one matrix per instance is kept in shared memory (48 KB: S <= 110)
+    const bool staged = plan && !A && !(sh->flags & GALV_TRANS_PER_LAYER) && (size_t)sh->S * sh->S * 4 <= 48 * 1024;
+    const size_t smem = staged ? (size_t)sh->S * sh->S * 4 : 0;
+#define GALV_WALK(NJ) backtrack_kernel<NJ><<<sh->B, 32, smem, st>>>( \
         sh->B, sh->Lmax, sh->S, sh->M, sh->m_pitch, galv_trans_inst(sh), galv_trans_layer(sh), L, time_q, mem_q, trans_q, C, A, C_last, lean_map, budget, \
-        opt_cost, plan, mem_used, status)
+        opt_cost, plan, mem_used, status, staged)
     if (sh->S <= 32) GALV_WALK(1);
     else if (sh->S <= 64) GALV_WALK(2);
     else if (sh->S <= 128) GALV_WALK(4);

@@ -164,18 +164,21 @@ __global__ void validate_kernel(int B, int Lmax, int S, int M, long long tl, con
     int bad = 0, tmax = 0, mmax = 0;
     const int32_t* t = time_q + (size_t)i * Lmax * S;
     const int32_t* mq = mem_q + (size_t)i * Lmax * S;
-    for (int l = threadIdx.x; l < Li; l += blockDim.x) {
+    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    for (int l = threadIdx.x >> 5; l < Li; l += nwarps) {          // a warp per layer
         int mx = 0;
-        for (int s = 0; s < S; ++s) {
+        for (int s = lane; s < S; s += 32) {
             const int tv = t[l * S + s], mv = mq[l * S + s];
             bad |= (tv < 0) | (mv < 0);
             mx = max(mx, tv);
             mmax = max(mmax, mv);
         }
-        sum += mx;
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) sum += mx;
     }
     const int32_t* x = trans_q + (size_t)i * (tl ? (size_t)Lmax * S * S : (size_t)S * S);
     const int xl0 = tl ? 1 : 0, xl1 = tl ? Li : 1;            // matrices in use
+#pragma unroll 4
     for (long long k = threadIdx.x; k < (long long)(xl1 - xl0) * S * S; k += blockDim.x) {
         const int v = x[(size_t)xl0 * S * S + k];
         bad |= (v < 0);
@@ -200,11 +203,14 @@ __global__ void validate_kernel(int B, int Lmax, int S, int M, long long tl, con
     }
     __syncthreads();
     if (s_bad == 0) {
-        for (int l = threadIdx.x; l < Li; l += blockDim.x) {      // smallest mem of each layer over the valid instances
+        for (int l = threadIdx.x >> 5; l < Li; l += nwarps) {     // smallest mem of each layer over the valid instances
             int mn = 0x7fffffff;
-            for (int s = 0; s < S; ++s) mn = min(mn, mq[l * S + s]);
-            atomicMin(&minmem_l[l], mn);
-            if (front) front[(size_t)i * Lmax + l] = mn;
+            for (int s = lane; s < S; s += 32) mn = min(mn, mq[l * S + s]);
+            mn = __reduce_min_sync(0xffffffffu, mn);
+            if (lane == 0) {
+                atomicMin(&minmem_l[l], mn);
+                if (front) front[(size_t)i * Lmax + l] = mn;
+            }
         }
         if (front) {
             // feasibility frontier: no cell of layer l is finite below the sum of the layers' smallest mem
@@ -323,12 +329,9 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
 // ---------------------------------------------------------------- base layer
 
 // C[0][s][m] = time(0,s) if mem(0,s) <= m else INF; pad columns INF; A = 255.
-__global__ void base_layer_kernel(DpArgs a)
+__device__ __forceinline__ void base_row(const DpArgs& a, int i, int s)
 {
-    // with most instances finished elsewhere (done) a few blocks look after many rows, else a block has one
-    for (int row_at = blockIdx.y; row_at < a.B * a.S; row_at += gridDim.y) {
-    const int i = row_at / a.S, s = row_at - i * a.S;
-    if (a.status[i] != 0 || (a.done && a.done[i])) continue;
+    if (a.status[i] != 0 || (a.done && a.done[i])) return;
     const int tt = a.time_q[(size_t)i * a.Lmax * a.S + s];
     const int mm = a.mem_q[(size_t)i * a.Lmax * a.S + s];
     const size_t row = ((size_t)i * a.S + s) * a.m_pitch;
@@ -339,7 +342,13 @@ __global__ void base_layer_kernel(DpArgs a)
         out[m] = v;
         if (ao) ao[m] = 255;
     }
-    }
+}
+__global__ void base_layer_kernel(DpArgs a) { base_row(a, blockIdx.z, blockIdx.y); }
+// After the resident kernel, which leaves few instances or none: a few blocks look after all rows.
+__global__ void base_layer_rest_kernel(DpArgs a)
+{
+    if (a.nactive[0] == 0) return;
+    for (int r = blockIdx.y; r < a.B * a.S; r += gridDim.y) base_row(a, r / a.S, r % a.S);
 }
 
 // ---------------------------------------------------------------- reference layer kernel (one thread per cell)
@@ -1867,17 +1876,29 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     // The packed 16-bit kernel is launched as well when the shape allows it; which of the two runs is decided on
     // the device, where the largest transition entry is known (the other one returns at once).
     const int will_p16 = persistent && pl.p16 && !(sh->flags & GALV_KERNEL_NO_PACKED);
-    validate_kernel<<<B, 128, 0, st>>>(B, Lmax, S, a.M, (long long)a.trans_layer, a.L, a.time_q, a.mem_q, a.trans_q, a.status, a.done, a.err + 1, a.minmem_l,
+    // one matrix per layer is a thousand words a thread for 128 threads (96 instances of 40 layers, S = 44: 50 us)
+    validate_kernel<<<B, a.trans_layer || B <= 148 ? 512 : 128, 0, st>>>(B, Lmax, S, a.M, (long long)a.trans_layer, a.L, a.time_q, a.mem_q, a.trans_q, a.status, a.done, a.err + 1, a.minmem_l,
                                        (sh->flags & GALV_SKIP_INFEASIBLE) ? a.front : nullptr);
     schedule_kernel<<<1, 1024, 0, st>>>(B, Lmax, a.M, pl.tmb, pl.ntiles_m, pl.nsb, a.L, a.status, a.done, a.order, a.nactive, a.scratch,
                                          a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.err + 1);
     auto base_layer = [&]() {
         int gx = (a.m_pitch + 255) / 256;
         if (gx > 8) gx = 8;
-        long long rows = (long long)B * S;
-        const long long most = a.done ? 4 * 148 / gx : 65535; // grid.y limit
-        if (rows > most) rows = most;
-        base_layer_kernel<<<dim3(gx, (unsigned)rows), 256, 0, st>>>(a);
+        if (a.done) {
+            base_layer_rest_kernel<<<dim3(gx, (unsigned)(B < 8 ? B * S : 8 * 148 / gx)), 256, 0, st>>>(a);
+            return;
+        }
+        for (int b0 = 0; b0 < B; b0 += 65535) {           // grid.z limit
+            DpArgs s = a;
+            const int nb = (B - b0 < 65535) ? B - b0 : 65535;
+            s.L += b0; s.status += b0;
+            s.time_q += (size_t)b0 * Lmax * S; s.mem_q += (size_t)b0 * Lmax * S;
+            if (s.C) s.C += (size_t)b0 * Lmax * S * a.m_pitch;
+            if (s.A) s.A += (size_t)b0 * Lmax * S * a.m_pitch;
+            s.C_last += (size_t)b0 * S * a.m_pitch;
+            s.roll += (size_t)b0 * S * a.m_pitch;
+            base_layer_kernel<<<dim3(gx, S, nb), 256, 0, st>>>(s);
+        }
     };
     base_layer();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

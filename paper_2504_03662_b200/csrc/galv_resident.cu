@@ -1294,7 +1294,8 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
         const double work = g * (store ? S * 4.7 + 60.0 : S * 1.15 + 20.0);
         const double chain = S * (40.0 + 22.0 * width) + 400.0;
         double t = work > chain ? work : chain;
-        t += cl == 1 ? 200.0 : (cl > 8 ? 1500.0 : 1100.0);
+        if (store && !p.stage) t += S * 10.0;                  // loads wait behind stores
+        t += cl == 1 ? 200.0 : (cl > 8 ? 1250.0 : 1100.0);
         const double share = (double)(sh->B < slots ? sh->B : slots) * cl / ctx->num_sms;      // several CTAs on an SM share its issue slots
         if (share > 1.0) t *= share;
         p.rounds = (sh->B + slots - 1) / slots;
