@@ -66,13 +66,14 @@ extern "C" {
 #define GALV_KERNEL_NO_PACKED 4096 /* never take the packed 16-bit path (two relaxations per instruction on rebased
                                       costs; taken on its own when S <= 64, S % 4 == 0, no argmin table, all layers in
                                       one launch and every transition entry <= 32767; same results) */
-#define GALV_KERNEL_NO_CLUSTER 16384 /* never take the cluster kernel (small batches: one thread-block cluster per instance,
-                                        the table slice kept in shared memory; taken on its own when the device can hold
-                                        one cluster per instance at once, no argmin table is asked for, S <= 128 and the
-                                        slice fits in shared memory; same results) */
-#define GALV_KERNEL_CLUSTER 32768 /* take the cluster kernel whenever the shape allows it, also for batches that need
-                                     several rounds of clusters (at most 512 instances then) */
-#define GALV_CLUSTER_SIZE(n) (((n) & 31) << 16) /* the cluster kernel with clusters of n CTAs (1..16), where that size is possible
+#define GALV_KERNEL_NO_CLUSTER 16384 /* the tiled kernels only: never the resident kernel (one thread-block cluster per
+                                        instance, the state between layers kept in shared memory: one row per distinct
+                                        column of the transition matrix; taken on its own wherever that state fits,
+                                        S <= 128) nor the pushing cluster kernel (small batches of unstructured matrices,
+                                        the table slice kept in shared memory).  Same results */
+#define GALV_KERNEL_CLUSTER 32768 /* take one of the cluster kernels whenever the shape allows it, also for batches that need
+                                     several rounds of clusters */
+#define GALV_CLUSTER_SIZE(n) (((n) & 31) << 16) /* ... with clusters of n CTAs (1..16), where that size is possible
                                                    for the shape (by default the size is chosen from the shape, the batch
                                                    and what the device can hold at once) */
 #define GALV_DEBUG_WITHHOLD_LOAD 2048 /* test hook for the time-out path: one CTA never receives its first stage, every
@@ -86,7 +87,9 @@ extern "C" {
                                     are such in all 128 columns of a warp group's tile are left out of the inner
                                     loop.  Same tables (argmin table included); the work then depends on the spread
                                     of the costs.  Honoured when S <= 64 and, in the 32-bit loop, a tile's S rows fit
-                                    one stage; ignored elsewhere (GALV_KERNEL_REFERENCE among them). */
+                                    one stage; ignored elsewhere (GALV_KERNEL_REFERENCE among them).  Where the tiled
+                                    kernels run without an argmin table and without GALV_KERNEL_NO_CLUSTER they do so
+                                    unasked; the resident kernel always does. */
 
 typedef struct galv_ctx galv_ctx;
 
@@ -192,9 +195,10 @@ int galv_dp_search(galv_ctx* ctx, const galv_shape* shape, const int32_t* L,
 /*
  * Which kernel the most recent galv_dp_search on `workspace` ran: *packed = 1 for the tiled kernel
  * with the packed 16-bit inner loop (two relaxations per instruction; see GALV_KERNEL_NO_PACKED),
- * 0 for the tiled kernel with the 32-bit one, 2 for the cluster kernel (32-bit loop; see
- * GALV_KERNEL_NO_CLUSTER).  The choice between the two inner loops is made on the device; this
- * call waits for `stream` and reads the answer back (host pointer).
+ * 0 for 32-bit arithmetic in rounds over the batch (the tiled kernel with the 32-bit loop; the resident kernel on
+ * more than 512 instances or with an argmin table), 2 for the cluster kernels (see GALV_KERNEL_NO_CLUSTER).  Where the
+ * kernels take a batch between them, the one that took the last of it.  Part of the choice is made on the device;
+ * this call waits for `stream` and reads the answer back (host pointer).
  */
 int galv_dp_search_path(galv_ctx* ctx, const galv_shape* shape, const void* workspace, int32_t* packed, void* stream);
 
@@ -389,7 +393,8 @@ size_t galv_search_host_arena_bytes(const galv_ctx* ctx, const galv_shape* shape
  * Host pointers (pinned memory makes the copies asynchronous): L, layers, strat,
  * inst, or time_q/mem_q/trans_q; outputs opt_cost [B], plan [B][Lmax], mem_used [B],
  * status [B].  arena: device, 256-byte aligned, galv_search_host_arena_bytes bytes.
- * shape.flags selects the table mode as in galv_dp_search (tables live in the arena).
+ * shape.flags selects the table mode as in galv_dp_search.  What the arena holds afterwards is the library's own
+ * business: with the full table alone the kernels may leave the states between the layers in its place.
  */
 int galv_search_host(galv_ctx* ctx, const galv_shape* shape, const int32_t* L,
                      const galv_layer_desc* layers, int64_t layer_stride_B,

@@ -150,7 +150,7 @@ __global__ void validate_kernel(int B, int Lmax, int S, int M, long long tl, con
                                 int32_t* __restrict__ maxmem, int32_t* __restrict__ minmem_l, int32_t* __restrict__ front)
 {
     const int i = blockIdx.x;
-    if (done && done[i]) return;                              // searched, or flagged, by the cluster kernel
+    if (done && done[i] == 1) return;                              // searched, or flagged, by the cluster kernel
     __shared__ long long s_sum;
     __shared__ int s_tmax, s_bad, s_mmax;
     if (threadIdx.x == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; s_mmax = 0; }
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
     int32_t* hist = scratch;
     int32_t* fill = scratch + Lmax + 2;
     for (int i = threadIdx.x; i < B; i += blockDim.x)
-        if (status[i] == 0 && !(done && done[i])) atomicAdd(&hist[L[i]], 1);
+        if (status[i] == 0 && !(done && done[i] == 1)) atomicAdd(&hist[L[i]], 1);
     for (int l = threadIdx.x; l <= Lmax; l += blockDim.x) {
         int nt = 1;
         if (l < Lmax && minmem_l[l] <= M) nt = min(ntiles_m, (M - minmem_l[l]) / tmb + 1);
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
     }
     __syncthreads();
     for (int i = threadIdx.x; i < B; i += blockDim.x)
-        if (status[i] == 0 && !(done && done[i])) {
+        if (status[i] == 0 && !(done && done[i] == 1)) {
             const int Li = L[i];
             order[nactive[Li] + atomicAdd(&fill[Li], 1)] = i;   // instances longer than Li come first
         }
@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
 // C[0][s][m] = time(0,s) if mem(0,s) <= m else INF; pad columns INF; A = 255.
 __device__ __forceinline__ void base_row(const DpArgs& a, int i, int s)
 {
-    if (a.status[i] != 0 || (a.done && a.done[i])) return;
+    if (a.status[i] != 0 || (a.done && a.done[i] == 1)) return;
     const int tt = a.time_q[(size_t)i * a.Lmax * a.S + s];
     const int mm = a.mem_q[(size_t)i * a.Lmax * a.S + s];
     const size_t row = ((size_t)i * a.S + s) * a.m_pitch;
@@ -1616,7 +1616,7 @@ __global__ void __launch_bounds__((NSG * NMS + (P16 ? (DOM ? 7 : 5) : 4)) * 32, 
 __global__ void copy_last_kernel(DpArgs a)
 {
     const int i = blockIdx.y;
-    if (a.status[i] != 0 || (a.done && a.done[i])) return;
+    if (a.status[i] != 0 || (a.done && a.done[i] == 1)) return;
     const int Li = a.L[i];
     const size_t slice = (size_t)a.S * a.m_pitch;
     const int32_t* src = a.C ? a.C + ((size_t)i * a.Lmax + (Li - 1)) * slice : a.roll + ((size_t)((Li - 1) & 1) * a.B + i) * slice;
@@ -1837,7 +1837,13 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         RsPlan rp[2];
         galv_shape kept = *sh;
         if (a.lean_map) kept.flags &= ~GALV_STORE_C_FULL;
-        const int n = galv_resident_plan(ctx, &kept, rp);
+        ClPlan cp;
+        const bool pushing = galv_cluster_plan(ctx, sh, &cp);
+        // A short stack is over before the resident kernel has looked at its matrix: up to 16 layers the pushing cluster
+        // kernel alone, where it can (3 instances of 6 layers, S = 7: 21 us against 33; 10 layers, S = 18: 47 against 55;
+        // 14 layers of an analytic model, S = 16: 62 against 73).
+        const bool asked = (sh->flags & GALV_KERNEL_CLUSTER) != 0 || ((sh->flags >> 16) & 31) != 0;
+        const int n = pushing && Lmax <= 16 && !asked ? 0 : galv_resident_plan(ctx, &kept, rp);
         int launched = 0;
         while (launched < n) {
             if (galv_resident_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now
@@ -1845,8 +1851,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         }
         if (launched && launched == n && rp[n - 1].dense) return finished();
         if (!launched) a.done = nullptr;
-        ClPlan cp;
-        if (galv_cluster_plan(ctx, sh, &cp)) {
+        if (pushing) {
             if (galv_cluster_launch(ctx, sh, cp, a, st) == cudaSuccess) return finished();
             (void)cudaGetLastError();                        // the clusters cannot be placed on this device right now: tiled kernels
         }
@@ -1885,7 +1890,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         int gx = (a.m_pitch + 255) / 256;
         if (gx > 8) gx = 8;
         if (a.done) {
-            base_layer_rest_kernel<<<dim3(gx, (unsigned)(B < 8 ? B * S : 8 * 148 / gx)), 256, 0, st>>>(a);
+            base_layer_rest_kernel<<<dim3(gx, (unsigned)(B * (long long)S < 1024 ? B * S : 1024)), 256, 0, st>>>(a);
             return;
         }
         for (int b0 = 0; b0 < B; b0 += 65535) {           // grid.z limit

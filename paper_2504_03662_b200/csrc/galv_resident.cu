@@ -55,7 +55,8 @@ struct RsArgs {
     int stage_at;      // word offset of the collected rows
     int SP;            // row pitch of the full transition matrix in shared memory; 0: no room for unstructured matrices
     int sorted;        // clusters take the instances longest first
-    int second;        // only the instances the first launch left alone
+    int second;        // only the instances earlier launches left alone
+    int probed;        // done[] says which matrices are unstructured
     int path_value;    // what galv_dp_search_path reports
     const int32_t* L;
     const int32_t* time_q;
@@ -766,7 +767,9 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
         __syncthreads();
         i = s_inst;
     }
-    if (a.second && a.done[i]) return;
+    // finished before, or (no room here for an unstructured matrix) found to be one by the probe: nobody in the cluster
+    // writes the word before all have read it
+    if ((a.second && a.done[i] == 1) || (a.probed && a.done[i] == 2)) return;
     const int Li = a.L[i];
     if (Li < 1 || Li > Lmax) {
         if (rank == 0 && tid == 0) { a.status[i] = GALV_STATUS_BAD_INPUT; a.done[i] = 1; }
@@ -780,28 +783,6 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     int32_t* const stage = g0;                                 // the state is not in use yet
     const int TP = S | 1;                                       // odd pitch: columns are read without bank conflicts too
     const bool staged = !a.trans_layer && (long long)S * TP <= (long long)2 * gints;
-    if (a.SP == 0 && S > kClassMax) {
-        // No room for an unstructured matrix.  Of kClassMax + 1 rows two are equal if there are at most kClassMax classes:
-        // a matrix without a pair among its first rows is left alone before anything else is looked at (1024 instances
-        // of S = 32: 0.35 ms without this look, 0.03 with it).
-        constexpr int R = kClassMax + 1;
-        if (tid == 0) s_K[0] = 0;
-        for (int k = tid; k < R * S; k += NT) { const int q = k / S; stage[q * TP + k - q * S] = T0[k]; }
-        __syncthreads();
-        for (int x = warp; x < R * R; x += NW + 1) {
-            const int p = x / R, q = x - p * R;
-            if (p >= q) continue;
-            bool diff = false;
-            for (int s = lane; s < S; s += 32) diff |= stage[p * TP + s] != stage[q * TP + s];
-            if (!__any_sync(0xffffffffu, diff) && lane == 0) s_K[0] = 1;
-        }
-        __syncthreads();
-        if (!s_K[0]) {
-            if (rank == 0 && tid == 0) a.done[i] = 0;
-            return;
-        }
-        __syncthreads();
-    }
     auto fetch = [&](int l) {
         int32_t* const rm = raw + (l & 3) * 2 * S;
         for (int s = lane; s < S; s += 32) {
@@ -1190,6 +1171,31 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     if (s_late && tid == 0) atomicOr(reinterpret_cast<int*>(a.status + i), GALV_STATUS_TIMEOUT);
 }
 
+// Which matrices are worth the resident kernel's look: of kClassMax + 1 rows two are equal if there are at most kClassMax
+// classes.  done[i] = 2: no two of the first rows are.  A kernel of a few hundred instructions, as it is latency alone: the
+// same look inside the resident kernel cost a batch it turns away 15 us, most of them spent on fetching its code.
+__global__ void __launch_bounds__(256) probe_kernel(int B, int S, const int32_t* __restrict__ trans_q, long long trans_inst, int32_t* __restrict__ done)
+{
+    constexpr int R = kClassMax + 1;
+    __shared__ int32_t rows[R * kMaxS];
+    __shared__ int s_pair;
+    const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    const int32_t* const T = trans_q + (size_t)i * trans_inst;
+    if (tid == 0) s_pair = 0;
+    for (int k = tid; k < R * S; k += 256) rows[k] = T[k];
+    __syncthreads();
+    for (int x = tid >> 5; x < R * R; x += 8) {
+        const int p = x / R, q = x - p * R;
+        if (p >= q || s_pair) continue;
+        bool diff = false;
+        for (int s = lane; s < S; s += 32) diff |= rows[p * S + s] != rows[q * S + s];
+        if (!__any_sync(0xffffffffu, diff) && lane == 0) s_pair = 1;
+        __syncwarp();
+    }
+    __syncthreads();
+    if (tid == 0) done[i] = s_pair ? 0 : 2;
+}
+
 // ---------------------------------------------------------------- host side
 
 typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -1280,8 +1286,10 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
     const int want = (sh->flags >> 16) & 31;                  // GALV_CLUSTER_SIZE(n): only clusters of n CTAs
     const int per_word = arg ? 10 : 8;                        // two buffers of words, with argmin bytes beside
     const long long words = ((long long)ctx->smem_optin - kStaticSmem - fixed_smem(sh, dense)) / per_word;
-    // halo to plan for: a few times what an even share of the budget gives a layer
+    // halo to plan for: a few times what an even share of the budget gives a layer, and what large layers of the analytic
+    // models ask for (a fifth of 2880 columns, 600 of 8192); beyond it a layer takes the slow way
     long long halo = 4ll * sh->M / sh->Lmax;
+    if (!dense && halo < (sh->M / 5 < 600 ? sh->M / 5 : 600)) halo = sh->M / 5 < 600 ? sh->M / 5 : 600;
     if (halo < 64) halo = 64;
     if (halo > sh->M) halo = sh->M;
     bool found = false;
@@ -1297,7 +1305,7 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
         // rows collected in shared memory where there is room for them beside the state (a tensor box has 256 entries a
         // side at most) and where a layer is a chain of latencies rather than a stream of stores
         const long long collected = (long long)2 * S * w * 4;
-        p.stage = store && !arg && g <= 2 * kMaxWarps && (long long)rows * (w + (cl > 1 ? halo : 0)) * per_word + collected <= words * per_word &&
+        p.stage = store && !arg && g <= 2 * kMaxWarps && (long long)rows * (w + (cl > 1 ? (halo > sh->M / 5 ? halo : sh->M / 5) : 0)) * per_word + collected <= words * per_word &&
                   (long long)sh->B * sh->Lmax * S < (1ll << 31);
         const long long room = p.stage ? words - collected / per_word : words;
         long long gi = (long long)(dense && S > kClassMax ? S : kClassMax) * (w + ((sh->M + 32) & ~31));    // all that could be used
@@ -1382,6 +1390,8 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
     RsArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
     a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second;
+    a.probed = !p.dense && d.S > kClassMax && !second;
+    if (a.probed) probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.trans_q, d.trans_inst, d.done);
     a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept
     a.path_value = (d.B <= kMaxSortedB && !d.A) ? 2 : 0;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
