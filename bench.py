@@ -247,7 +247,7 @@ def cost_model_scaled(torch, galv, hbm_gbs, barrier, copies=8192):
 
 
 def launches_per_step(w, cluster: bool = False) -> int:
-    if cluster:                                   # the cost model's kernel, ONE cluster kernel for the whole search, backtrack
+    if cluster:                                   # the cost model's kernel, the resident kernel for the whole search, backtrack
         return (1 if w.has_model else 0) + 1 + 1
     # the cost model's kernel, validate + schedule + base layer, ONE cooperative launch over all layers,
     # copy-last + finalize, backtrack; where the shape allows the packed 16-bit path, the kernel that packs
@@ -367,20 +367,43 @@ def main():
     del sb
     torch.cuda.empty_cache()
 
-    # end to end through the host-buffer entry point: pinned host inputs -> device -> search -> host results
+    # end to end with the table kept: pinned host inputs -> device -> search -> host results; the host-buffer entry point,
+    # which keeps the states between the layers in the table's place, beside it
     e2e = None
     if not args.no_e2e:
-        hs = HostSearch(galv, w, gb.STORE_C_FULL)
-        for _ in range(args.warmup):
-            hs.run()
-        torch.cuda.synchronize(); barrier()
-        t0 = time.perf_counter()
-        for _ in range(args.steps):
-            hs.run()
-        torch.cuda.synchronize(); barrier()
-        te = max_over_ranks(time.perf_counter() - t0)
+        from paper_2504_03662_b200.search import SearchBuffers
+        sb = SearchBuffers(galv, w, gb.STORE_C_FULL)
+        ins = [getattr(sb, k) for k in (("L", "layers", "strat", "inst") if w.has_model else ("L", "time_q", "mem_q", "trans_q"))]
+        outs = [sb.opt_cost, sb.plan, sb.mem_used, sb.status]
+        h_in = [t.cpu().pin_memory() for t in ins]
+        h_out = [t.cpu().pin_memory() for t in outs]
+
+        def end_to_end():
+            for d, h in zip(ins, h_in):
+                d.copy_(h, non_blocking=True)
+            sb.step()
+            for h, d in zip(h_out, outs):
+                h.copy_(d, non_blocking=True)
+            torch.cuda.synchronize()
+
+        def timed(fn):
+            for _ in range(args.warmup):
+                fn()
+            torch.cuda.synchronize(); barrier()
+            t0 = time.perf_counter()
+            for _ in range(args.steps):
+                fn()
+            torch.cuda.synchronize(); barrier()
+            return max_over_ranks(time.perf_counter() - t0)
+
+        te = timed(end_to_end)
+        nbytes = lambda ts: sum(t.numel() * t.element_size() for t in ts)
         e2e = {"value": world * w.cells * args.steps / te, "unit": UNIT, "ms_per_step": te / args.steps * 1e3,
-               "h2d_bytes_per_step": hs.h2d, "d2h_bytes_per_step": hs.d2h}
+               "h2d_bytes_per_step": nbytes(h_in), "d2h_bytes_per_step": nbytes(h_out)}
+        del sb, ins, outs
+        torch.cuda.empty_cache()
+        hs = HostSearch(galv, w, gb.STORE_C_FULL)
+        e2e["host_entry_ms_per_step"] = timed(hs.run) / args.steps * 1e3
         del hs
         torch.cuda.empty_cache()
 
@@ -412,6 +435,27 @@ def main():
                                     + (" (two relaxations each in the packed 16-bit form)" if r["packed"] else "")},
     }
 
+    if r["cluster"]:
+        # The resident kernel does not relax S*S pairs a column: it keeps one state row per distinct column of the
+        # transition matrix and writes every cell of the table once.  Its bound is that write.
+        peaks = {}
+        try:
+            peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
+        except OSError:
+            pass
+        hbm_gbs = peaks.get("hbm_gbs", 6650.0)
+        written = 4 * int(np.sum(w.L)) * w.S * gb.make_shape(w.B, w.Lmax, w.S, w.M).m_pitch
+        line["roofline"].update({"bound": "hbm", "achieved": written / kernel_s / 1e9, "peak": hbm_gbs, "unit": "GB/s",
+                                 "frac": written / kernel_s / 1e9 / hbm_gbs, "traffic": None,
+                                 "traffic_unit": "bytes per launch", "algorithmic_bytes_per_launch": written,
+                                 "algorithmic_ops_per_launch": None,
+                                 "inner_loop": "one add and one class minimum a cell, 32-bit",
+                                 "relaxations_stood_for_of_alu_peak": achieved / ALU_PEAK_GOPS,
+                                 "kernel": "resident_kernel (one thread-block cluster per instance, the state between layers in shared memory)",
+                                 "peak_source": "measured copy bandwidth" if peaks else "fallback copy bandwidth"})
+        del line["roofline"]["frac_of_32bit_peak"]
+        achieved = line["roofline"]["achieved"]
+
     line["inputs_fnv1a64"] = input_checksums(w)
     line["kernel_variant"] = line["roofline"]["kernel"]
     if rank == 0:
@@ -422,14 +466,14 @@ def main():
         try:
             fused = galv.galv_probe_int_alu(0, 4096) / 1e9
             packed = galv.galv_probe_int_alu(3, 4096) / 1e9
-            rf["peak_measured"] = packed if r["packed"] else fused
+            rf["peak_measured"] = rf["peak"] if r["cluster"] else packed if r["packed"] else fused
             rf["frac_of_measured"] = achieved / rf["peak_measured"]
             rf["probe_fused_addmin_gops"] = fused
             rf["probe_packed_addmin_u16x2_gops"] = packed
             rf["probe_add_then_min_gops"] = galv.galv_probe_int_alu(1, 4096) / 1e9
             rf["probe_add_xor_2ops_gops"] = galv.galv_probe_int_alu(2, 4096) / 1e9
             rf["probe_min3_gops"] = galv.galv_probe_int_alu(4, 4096) / 1e9
-            rf["peak_measured_source"] = ("galv_probe_int_alu kind 3 (__viaddmin_u16x2, two relaxations per instruction)" if r["packed"]
+            rf["peak_measured_source"] = (rf["peak_source"] if r["cluster"] else "galv_probe_int_alu kind 3 (__viaddmin_u16x2, two relaxations per instruction)" if r["packed"]
                                           else "galv_probe_int_alu kind 0 (__viaddmin_s32)")
         except gb.GalvError as e:      # diagnostic only
             rf["peak_measured"] = None
@@ -437,14 +481,14 @@ def main():
         # HBM side of the roofline: every table cell written once and read once by the next layer
         from paper_2504_03662_b200.binding import make_shape
         pitch = make_shape(w.B, w.Lmax, w.S, w.M).m_pitch
-        hbm_bytes = 2 * 4 * int(np.sum(w.L)) * w.S * pitch
+        hbm_bytes = (1 if r["cluster"] else 2) * 4 * int(np.sum(w.L)) * w.S * pitch
         peaks = {}
         try:
             peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
         except OSError:
             pass
         hbm_gbs = peaks.get("hbm_gbs", 6650.0)
-        line["roofline"]["t_alu_ms"] = w.relaxations / (line["roofline"]["peak"] * 1e9) * 1e3
+        line["roofline"]["t_alu_ms"] = 0.0 if r["cluster"] else w.relaxations / (line["roofline"]["peak"] * 1e9) * 1e3
         line["roofline"]["t_hbm_ms"] = hbm_bytes / (hbm_gbs * 1e9) * 1e3
         line["roofline"]["hbm_peak"] = f"{hbm_gbs} GB/s " + ("of measured" if peaks else "of fallback")
         line["roofline"]["step_frac_of_bound"] = max(line["roofline"]["t_alu_ms"], line["roofline"]["t_hbm_ms"]) / (t / args.steps * 1e3)
