@@ -196,8 +196,9 @@ cudaError_t galv_backtrack_launch(const galv_shape* sh, const int32_t* L, const 
                                   int32_t* opt_cost, int32_t* plan, int32_t* mem_used, int32_t* status,
                                   cudaStream_t st)
 {
-    // a warp per instance, a CTA of its own; one matrix per instance is kept in shared memory (48 KB: S <= 110)
-    const bool staged = plan && !A && !(sh->flags & GALV_TRANS_PER_LAYER) && (size_t)sh->S * sh->S * 4 <= 48 * 1024;
+    // a warp per instance, a CTA of its own; one matrix per instance is kept in shared memory (48 KB: S <= 110; 48 layers of
+    // S = 48 69 -> 56 us), a small one stays in L1 anyway (24 layers of S = 24: 22.5 us so, 24 with the copy)
+    const bool staged = plan && !A && sh->S > 32 && !(sh->flags & GALV_TRANS_PER_LAYER) && (size_t)sh->S * sh->S * 4 <= 48 * 1024;
     const size_t smem = staged ? (size_t)sh->S * sh->S * 4 : 0;
 #define GALV_WALK(NJ) backtrack_kernel<NJ><<<sh->B, 32, smem, st>>>( \
         sh->B, sh->Lmax, sh->S, sh->M, sh->m_pitch, galv_trans_inst(sh), galv_trans_layer(sh), L, time_q, mem_q, trans_q, C, A, C_last, lean_map, budget, \

@@ -1841,9 +1841,10 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         const bool pushing = galv_cluster_plan(ctx, sh, &cp);
         // A short stack is over before the resident kernel has looked at its matrix: up to 16 layers the pushing cluster
         // kernel alone, where it can (3 instances of 6 layers, S = 7: 21 us against 33; 10 layers, S = 18: 47 against 55;
-        // 14 layers of an analytic model, S = 16: 62 against 73).
+        // 14 layers of an analytic model, S = 16: 62 against 73).  So do fewer than a thousand columns, a few warps' worth
+        // of work a layer (5 instances of 52 layers, S = 22, 126 columns: 136 against 185).
         const bool asked = (sh->flags & GALV_KERNEL_CLUSTER) != 0 || ((sh->flags >> 16) & 31) != 0;
-        const int n = pushing && Lmax <= 16 && !asked ? 0 : galv_resident_plan(ctx, &kept, rp);
+        const int n = pushing && (Lmax <= 16 || a.M < 1024) && !asked ? 0 : galv_resident_plan(ctx, &kept, rp);
         int launched = 0;
         while (launched < n) {
             if (galv_resident_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now

@@ -1303,9 +1303,10 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
         p.cl = cl; p.w = w; p.dense = dense;
         p.nw = g < kMaxWarps ? g : kMaxWarps;
         // rows collected in shared memory where there is room for them beside the state (a tensor box has 256 entries a
-        // side at most) and where a layer is a chain of latencies rather than a stream of stores
+        // side at most) and where a layer is a chain of latencies rather than a stream of stores; room for shifts of a third
+        // of the budget comes first (one instance of 50 layers whose shifts pass the halo: 436 us)
         const long long collected = (long long)2 * S * w * 4;
-        p.stage = store && !arg && g <= 2 * kMaxWarps && (long long)rows * (w + (cl > 1 ? (halo > sh->M / 5 ? halo : sh->M / 5) : 0)) * per_word + collected <= words * per_word &&
+        p.stage = store && !arg && g <= 2 * kMaxWarps && (long long)rows * (w + (cl > 1 ? (halo > sh->M / 3 ? halo : sh->M / 3) : 0)) * per_word + collected <= words * per_word &&
                   (long long)sh->B * sh->Lmax * S < (1ll << 31);
         const long long room = p.stage ? words - collected / per_word : words;
         long long gi = (long long)(dense && S > kClassMax ? S : kClassMax) * (w + ((sh->M + 32) & ~31));    // all that could be used
