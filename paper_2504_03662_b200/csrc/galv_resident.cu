@@ -11,7 +11,7 @@
 // parallelism) has a handful of distinct rows and columns however many strategies there are (8 among 64, 4 among 24):
 // a cell then costs one addition, one minimum over its class and its store instead of S add-mins, and the state of an
 // instance shrinks from S to 8 rows.  The kernel finds the classes itself, by comparing the matrix's rows and columns
-// word by word (hashes only propose), so nothing is assumed about where a matrix comes from.
+// word by word, so nothing is assumed about where a matrix comes from.
 // A matrix without such structure keeps all S rows.  Then a candidate C[l-1][m][s'] that lies more than the largest
 // transition entry above its column's best can neither win nor tie (the best row gives a candidate at most that entry
 // above itself), so a warp relaxes only the rows that are alive in one of its columns.
