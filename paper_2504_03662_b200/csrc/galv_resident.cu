@@ -1184,14 +1184,15 @@ __global__ void __launch_bounds__(256) probe_kernel(int B, int S, const int32_t*
     if (tid == 0) s_pair = 0;
     for (int k = tid; k < R * S; k += 256) rows[k] = T[k];
     __syncthreads();
-    for (int x = tid >> 5; x < R * R; x += 8) {
+    bool equal = false;                                         // the vote's answer: the same in all lanes, as the next vote needs it
+    for (int x = tid >> 5; x < R * R && !equal; x += 8) {
         const int p = x / R, q = x - p * R;
-        if (p >= q || s_pair) continue;
+        if (p >= q) continue;
         bool diff = false;
         for (int s = lane; s < S; s += 32) diff |= rows[p * S + s] != rows[q * S + s];
-        if (!__any_sync(0xffffffffu, diff) && lane == 0) s_pair = 1;
-        __syncwarp();
+        equal = !__any_sync(0xffffffffu, diff);
     }
+    if (equal && lane == 0) s_pair = 1;
     __syncthreads();
     if (tid == 0) done[i] = s_pair ? 0 : 2;
 }

@@ -71,3 +71,14 @@ def test_host_plans_from_states(orc, galv, B, S, rows):
             Li = int(w.L[i])
             assert res["opt_cost"][i] == ref[i]["opt_cost"] and res["status"][i] == ref[i]["status"], i
             assert (res["plan"][i, :Li] == ref[i]["plan"]).all() and res["mem_used"][i] == ref[i]["mem_used"], i
+
+
+@pytest.mark.parametrize("twins", [None, (0, 1), (15, 16), (0, 16), (0, 17), (38, 39)])
+def test_probe_of_the_first_rows(orc, galv, twins):
+    """Which of a matrix's first 17 rows are equal decides who searches the instance, never what is found: no pair, pairs
+    at both ends of the 17, pairs the probe does not look at.  (Its warps leave their loops at different pairs.)"""
+    w = inputs.random_tables(71, 4, 18, 40, 1100, ragged=True, mem_lo=0, mem_hi=150)
+    if twins:
+        w.trans_q[1::2, twins[1]] = w.trans_q[1::2, twins[0]]
+    for flags in (1, 0):
+        check_batch(orc, galv, w, flags)
