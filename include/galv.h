@@ -66,16 +66,19 @@ extern "C" {
 #define GALV_KERNEL_NO_PACKED 4096 /* never take the packed 16-bit path (two relaxations per instruction on rebased
                                       costs; taken on its own when S <= 64, S % 4 == 0, no argmin table, all layers in
                                       one launch and every transition entry <= 32767; same results) */
-#define GALV_KERNEL_NO_CLUSTER 16384 /* the tiled kernels only: never the resident kernel (one thread-block cluster per
+#define GALV_KERNEL_NO_CLUSTER 16384 /* the tiled kernels only: neither the resident kernel (one thread-block cluster per
                                         instance, the state between layers kept in shared memory: one row per distinct
-                                        column of the transition matrix; taken on its own wherever that state fits,
-                                        S <= 128) nor the pushing cluster kernel (small batches of unstructured matrices,
+                                        column of the transition matrix) nor the pushing cluster kernel (small batches,
                                         the table slice kept in shared memory).  Same results */
-#define GALV_KERNEL_CLUSTER 32768 /* take one of the cluster kernels whenever the shape allows it, also for batches that need
-                                     several rounds of clusters */
+#define GALV_KERNEL_CLUSTER 32768 /* the pushing cluster kernel whenever the shape allows it (S <= 128, no argmin table),
+                                     also for batches that need several rounds of clusters (at most 512 instances then);
+                                     never the resident kernel */
 #define GALV_CLUSTER_SIZE(n) (((n) & 31) << 16) /* ... with clusters of n CTAs (1..16), where that size is possible
                                                    for the shape (by default the size is chosen from the shape, the batch
-                                                   and what the device can hold at once) */
+                                                   and what the device can hold at once).  Beside GALV_KERNEL_RESIDENT
+                                                   the cluster size of that kernel */
+#define GALV_KERNEL_RESIDENT 2097152 /* the resident kernel whenever the shape allows it (S <= 128), also where another one
+                                        would be taken on its own; instances it has no room for go to the tiled kernels */
 #define GALV_DEBUG_WITHHOLD_LOAD 2048 /* test hook for the time-out path: one CTA never receives its first stage, every
                                          bounded wait that depends on it runs out (about a second each), status gets
                                          GALV_STATUS_TIMEOUT and the call's results are void; nothing faults or hangs */
@@ -195,10 +198,11 @@ int galv_dp_search(galv_ctx* ctx, const galv_shape* shape, const int32_t* L,
 /*
  * Which kernel the most recent galv_dp_search on `workspace` ran: *packed = 1 for the tiled kernel
  * with the packed 16-bit inner loop (two relaxations per instruction; see GALV_KERNEL_NO_PACKED),
- * 0 for 32-bit arithmetic in rounds over the batch (the tiled kernel with the 32-bit loop; the resident kernel on
- * more than 512 instances or with an argmin table), 2 for the cluster kernels (see GALV_KERNEL_NO_CLUSTER).  Where the
- * kernels take a batch between them, the one that took the last of it.  Part of the choice is made on the device;
- * this call waits for `stream` and reads the answer back (host pointer).
+ * 0 for the tiled kernel with the 32-bit one, 2 for the cluster kernels (one thread-block cluster per instance: the
+ * resident one, the pushing one, or the first and what it left alone the second; see GALV_KERNEL_CLUSTER,
+ * GALV_KERNEL_RESIDENT).  Where the tiled kernels took some of the batch, theirs.  With an argmin table always 0: the
+ * arithmetic is 32-bit in the tiled kernels and in the resident one, and this word does not say which of them ran.  Part
+ * of the choice is made on the device; this call waits for `stream` and reads the answer back (host pointer).
  */
 int galv_dp_search_path(galv_ctx* ctx, const galv_shape* shape, const void* workspace, int32_t* packed, void* stream);
 

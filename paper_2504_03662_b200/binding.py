@@ -20,12 +20,12 @@ STORE_C_FULL, STORE_ARGMIN, KERNEL_REFERENCE, KERNEL_PER_LAYER, SKIP_INFEASIBLE 
 SKIP_DOMINATED = 8192
 DEBUG_WITHHOLD_LOAD = 2048
 KERNEL_NO_PACKED = 4096
-KERNEL_NO_CLUSTER, KERNEL_CLUSTER = 16384, 32768
+KERNEL_NO_CLUSTER, KERNEL_CLUSTER, KERNEL_RESIDENT = 16384, 32768, 1 << 21
 PATH_TILED_32, PATH_TILED_PACKED, PATH_CLUSTER = 0, 1, 2
 
 
 def CLUSTER_SIZE(n: int) -> int:
-    """Flag bits that ask for the cluster kernel with clusters of n CTAs."""
+    """Flag bits that ask for the pushing cluster kernel (with KERNEL_RESIDENT: the resident kernel) with clusters of n CTAs."""
     return (n & 31) << 16
 TRANS_PER_LAYER = 4
 STATIC_WORKSPACE_BYTES = 1 << 20

@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
                                 const int32_t* __restrict__ status, const int32_t* __restrict__ done, int32_t* __restrict__ order, int32_t* __restrict__ nactive,
                                 int32_t* __restrict__ scratch, const int32_t* __restrict__ minmem_l, int32_t* __restrict__ ntiles,
                                 long long* __restrict__ istart, int32_t* __restrict__ tcount, int p16_possible,
-                                int32_t* __restrict__ maxmem)
+                                int path_done, int32_t* __restrict__ maxmem)
 {
     __shared__ long long warp_sums[32];
     // The packed 16-bit path needs every trans entry, and twice the largest plus one, to fit 16 bits.
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
     __syncthreads();
     if (done && !s_any) {                              // every instance is finished: an empty schedule
         for (int l = threadIdx.x; l <= Lmax; l += blockDim.x) { nactive[l] = 0; istart[l] = 0; }
-        if (threadIdx.x == 0) maxmem[2] = 2;
+        if (threadIdx.x == 0) maxmem[2] = path_done;
         return;
     }
     {
@@ -1838,13 +1838,15 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         galv_shape kept = *sh;
         if (a.lean_map) kept.flags &= ~GALV_STORE_C_FULL;
         ClPlan cp;
-        const bool pushing = galv_cluster_plan(ctx, sh, &cp);
+        const bool resident_asked = (sh->flags & GALV_KERNEL_RESIDENT) != 0;
+        const bool pushing_asked = !resident_asked && ((sh->flags & GALV_KERNEL_CLUSTER) != 0 || ((sh->flags >> 16) & 31) != 0);
+        const bool pushing = !resident_asked && galv_cluster_plan(ctx, sh, &cp);
         // A short stack is over before the resident kernel has looked at its matrix: up to 16 layers the pushing cluster
         // kernel alone, where it can (3 instances of 6 layers, S = 7: 21 us against 33; 10 layers, S = 18: 47 against 55;
         // 14 layers of an analytic model, S = 16: 62 against 73).  So do fewer than a thousand columns, a few warps' worth
         // of work a layer (5 instances of 52 layers, S = 22, 126 columns: 136 against 185).
-        const bool asked = (sh->flags & GALV_KERNEL_CLUSTER) != 0 || ((sh->flags >> 16) & 31) != 0;
-        const int n = pushing && (Lmax <= 16 || a.M < 1024) && !asked ? 0 : galv_resident_plan(ctx, &kept, rp);
+        const bool pushing_alone = pushing_asked || (pushing && (Lmax <= 16 || a.M < 1024));
+        const int n = pushing_alone ? 0 : galv_resident_plan(ctx, &kept, rp);
         int launched = 0;
         while (launched < n) {
             if (galv_resident_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now
@@ -1886,7 +1888,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     validate_kernel<<<B, a.trans_layer || B <= 148 ? 512 : 128, 0, st>>>(B, Lmax, S, a.M, (long long)a.trans_layer, a.L, a.time_q, a.mem_q, a.trans_q, a.status, a.done, a.err + 1, a.minmem_l,
                                        (sh->flags & GALV_SKIP_INFEASIBLE) ? a.front : nullptr);
     schedule_kernel<<<1, 1024, 0, st>>>(B, Lmax, a.M, pl.tmb, pl.ntiles_m, pl.nsb, a.L, a.status, a.done, a.order, a.nactive, a.scratch,
-                                         a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.err + 1);
+                                         a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.A ? 0 : 2, a.err + 1);
     auto base_layer = [&]() {
         int gx = (a.m_pitch + 255) / 256;
         if (gx > 8) gx = 8;

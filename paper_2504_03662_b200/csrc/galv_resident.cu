@@ -57,7 +57,6 @@ struct RsArgs {
     int sorted;        // clusters take the instances longest first
     int second;        // only the instances earlier launches left alone
     int probed;        // done[] says which matrices are unstructured
-    int path_value;    // what galv_dp_search_path reports
     const int32_t* L;
     const int32_t* time_q;
     const int32_t* mem_q;
@@ -745,7 +744,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     int32_t* const stage_rows = reinterpret_cast<int32_t*>(smem_raw) + a.stage_at;         // [2][S][W] rows on their way to the table
     uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * ((S + 3) & ~3));                           // [2][gints] argmin of the state
 
-    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = a.path_value; }
+    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = ARG ? 0 : 2; }
 
     // ---- which instance: clusters are dispatched in order, so the longest instances go first
     int i = cid;
@@ -1284,7 +1283,7 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
 {
     const int S = sh->S, Gt = sh->m_pitch / 32;
     const bool store = (sh->flags & GALV_STORE_C_FULL) != 0, arg = (sh->flags & GALV_STORE_ARGMIN) != 0;
-    const int want = (sh->flags >> 16) & 31;                  // GALV_CLUSTER_SIZE(n): only clusters of n CTAs
+    const int want = (sh->flags >> 16) & 31;                  // GALV_CLUSTER_SIZE(n) beside GALV_KERNEL_RESIDENT: only clusters of n CTAs
     const int per_word = arg ? 10 : 8;                        // two buffers of words, with argmin bytes beside
     const long long words = ((long long)ctx->smem_optin - kStaticSmem - fixed_smem(sh, dense)) / per_word;
     // halo to plan for: a few times what an even share of the budget gives a layer, and what large layers of the analytic
@@ -1359,7 +1358,7 @@ int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
     }
     double td = 0.0, tc = 0.0;
     int n = 0;
-    const bool forced = (sh->flags & GALV_KERNEL_CLUSTER) != 0 || ((sh->flags >> 16) & 31) != 0;
+    const bool forced = (sh->flags & GALV_KERNEL_RESIDENT) != 0;
     const bool arg = (sh->flags & GALV_STORE_ARGMIN) != 0;
     // Unstructured matrices, measured on 48 layers of 2048 columns: S = 32, 16 instances 238 us here against 304 in the
     // pushing cluster kernel; S = 64 on 4000 columns 1.3 ms against 0.69 (its rows leave no room for the halo); 74
@@ -1395,7 +1394,6 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
     a.probed = !p.dense && d.S > kClassMax && !second;
     if (a.probed) probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.trans_q, d.trans_inst, d.done);
     a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept
-    a.path_value = (d.B <= kMaxSortedB && !d.A) ? 2 : 0;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
     const bool lean = d.lean_map != nullptr;

@@ -1,6 +1,8 @@
 """The kernel that keeps the state between layers in shared memory: matrices with classes of equal rows and columns.
 
-Tables, optima and plans against the CPU oracle, exact: everything is integers.
+Tables, optima and plans against the CPU oracle, exact: everything is integers.  RES asks for this kernel at any size, and
+without the pushing cluster kernel behind it: the path is then 2 only if this kernel took every instance (with an argmin
+table it is 0 whichever kernel ran).
 """
 import numpy as np
 import pytest
@@ -9,6 +11,14 @@ from paper_2504_03662_b200 import inputs
 from tests.test_gpu_parity import check_batch, galv, oracle_search_many  # noqa: F401  (galv is a fixture)
 
 pytestmark = pytest.mark.gpu
+
+RES = 1 << 21                 # GALV_KERNEL_RESIDENT
+
+
+def check_resident(orc, galv, w, flags, **kw):
+    sb, res = check_batch(orc, galv, w, flags | RES, **kw)
+    assert galv.galv_dp_search_path(sb.shape, sb.workspace) == (0 if flags & 2 else 2)
+    return sb, res
 
 
 def classed(seed, B, Lmax, S, M, rows, cols, **kw):
@@ -30,7 +40,7 @@ def test_classes_of_equal_rows_and_columns(orc, galv, S, rows, cols, flags):
     w.mem_q[1, 2, : S // 2] = M + 3                              # rows that never fit
     w.time_q[2, 1, :] = 9                                        # ties: the lowest strategy must win
     w.mem_q[3, 0, :] = M // 2                                    # the lower half of every later column is +inf
-    check_batch(orc, galv, w, flags)
+    check_resident(orc, galv, w, flags)
 
 
 # columns per CTA against shifts: inside the CTA, into the halo, beyond it (read from the owner), from the last column
@@ -42,20 +52,25 @@ def test_shifts_across_the_cluster(orc, galv, n, M, mem_hi, S, classes):
     w = classed(40 + n, 3, 5, S, M, classes, classes, **kw) if classes else inputs.random_tables(40 + n, 3, 5, S, M, **kw)
     w.mem_q[0, 1, 0] = M
     for flags in (gb.STORE_C_FULL, 0, gb.STORE_ARGMIN):
-        check_batch(orc, galv, w, flags | gb.CLUSTER_SIZE(n))
+        check_resident(orc, galv, w, flags | gb.CLUSTER_SIZE(n))
 
 
-def test_some_instances_left_to_the_other_kernels(orc, galv):
+@pytest.mark.parametrize("S,M,path", [(40, 1100, 2),            # the pushing cluster kernel takes the rest
+                                      (64, 8200, 1)])           # ... has no room: the tiled kernels (packed loop) do
+def test_some_instances_left_to_the_other_kernels(orc, galv, S, M, path):
     """One batch with structured, unstructured and flagged matrices, too many strategies for an unstructured state."""
-    w = classed(7, 9, 6, 60, 3000, 6, 6, mem_lo=0, mem_hi=300, ragged=True)
+    w = classed(7, 7, 18, S, M, 6, 6, mem_lo=0, mem_hi=M // 10, ragged=True)
     rng = np.random.default_rng(1)
-    for i in (1, 4, 5):
-        w.trans_q[i] = rng.integers(0, 3000, (60, 60), np.int32)
+    for i in (1, 4):
+        w.trans_q[i] = rng.integers(0, 3000, (S, S), np.int32)
     w.trans_q[3, 2, 2] = -1
-    w.L[7] = 0
+    w.L[5] = 0
+    w.L[[0, 1]] = 18                                             # both kinds at full length
     for flags in (1, 0, 3):
-        sb, res = check_batch(orc, galv, w, flags, idx=[0, 1, 2, 4, 5, 6, 8])
-        assert res["status"][[3, 7]].tolist() == [2, 2]
+        sb, res = check_batch(orc, galv, w, flags, idx=[0, 1, 2, 4, 6])
+        assert res["status"][[3, 5]].tolist() == [2, 2]
+        if not flags & 2:
+            assert galv.galv_dp_search_path(sb.shape, sb.workspace) == path
 
 
 @pytest.mark.parametrize("B,S,rows", [(1, 24, 4), (40, 48, 8), (3, 64, 64), (5, 7, 7)])
@@ -63,7 +78,8 @@ def test_host_plans_from_states(orc, galv, B, S, rows):
     """The host entry point keeps the states between the layers where a table would be kept: same optima and plans."""
     from paper_2504_03662_b200.search import HostSearch
     w = classed(60 + B, B, 8, S, 900, rows, rows, mem_lo=0, mem_hi=200, ragged=True)
-    hs = HostSearch(galv, w, 1)
+    check_resident(orc, galv, w, 0, idx=[0])                     # without a table, as the host entry point runs it: all by this kernel
+    hs = HostSearch(galv, w, 1 | RES)
     for _ in range(2):
         res = {k: v.copy() for k, v in hs.run().items()}
         ref = oracle_search_many(orc, w, w.time_q, w.mem_q, w.trans_q, list(range(B)))
@@ -82,3 +98,51 @@ def test_probe_of_the_first_rows(orc, galv, twins):
         w.trans_q[1::2, twins[1]] = w.trans_q[1::2, twins[0]]
     for flags in (1, 0):
         check_batch(orc, galv, w, flags)
+
+
+@pytest.mark.parametrize("block", range(6))
+def test_against_reference_kernel_on_many_shapes(galv, block):
+    """Random shapes, cluster sizes, classes (or none), memory distributions and per-layer matrices against the
+    one-thread-per-cell kernel, which other tests tie to the oracle.  Two runs per shape on the same buffers."""
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    rng = np.random.default_rng(5200 + block)
+    ran = 0
+    for case in range(12):
+        S = int(rng.choice([1, 3, 8, 13, 16, 17, 24, 32, 40, 64, 100, 128]))
+        Lmax, M, B = int(rng.integers(1, 14)), int(rng.integers(31, 4000)), int(rng.choice([1, 2, 5, 16, 40, 130]))
+        kw = dict(ragged=bool(rng.integers(0, 2)), mem_lo=0, mem_hi=int(rng.choice([0, 5, M // 30 + 1, M // 4 + 1, M + 50, 3 * M])),
+                  time_hi=int(rng.choice([5, 10 ** 4, 10 ** 6])))
+        K = int(rng.choice([0, 1, 4, 8, 16]))
+        w = classed(71000 + 100 * block + case, B, Lmax, S, M, K, max(1, K - 1), **kw) if K else \
+            inputs.random_tables(71000 + 100 * block + case, B, Lmax, S, M, trans_hi=int(rng.choice([0, 9, 40000])), **kw)
+        if Lmax > 2 and rng.integers(0, 2):
+            w.mem_q[:, int(rng.integers(1, Lmax)), :] += M // 2                          # one heavy layer
+        per_layer = case % 4 == 3 and Lmax > 1
+        if per_layer:
+            w.trans_q = np.ascontiguousarray(np.repeat(w.trans_q[:, None], Lmax, 1))
+            w.trans_q[:, 1:] += rng.integers(0, 50, size=(B, Lmax - 1, S, S), dtype=np.int32)
+        size = int(rng.choice([0, 0, 1, 2, 3, 4, 6, 8, 11, 16]))
+        table = (gb.STORE_C_FULL, gb.STORE_C_FULL | gb.STORE_ARGMIN, 0, gb.STORE_C_FULL)[case % 4 if not per_layer else 0]
+        ref = SearchBuffers(galv, w, gb.STORE_C_FULL | gb.KERNEL_REFERENCE)
+        ref.dp_search(); ref.backtrack()
+        one = SearchBuffers(galv, w, table | RES | gb.CLUSTER_SIZE(size))
+        for _ in range(2):
+            one.C_last.fill_(-7)
+            if table:
+                one.C.fill_(-7)
+            one.dp_search(); one.backtrack()
+            torch.cuda.synchronize()
+            ran += not table & 2 and galv.galv_dp_search_path(one.shape, one.workspace) == 2
+            st = ref.status.cpu().numpy()
+            assert (one.status.cpu().numpy() == st).all() and torch.equal(one.opt_cost, ref.opt_cost), (block, case)
+            assert not table or torch.equal(one.plan, ref.plan), (block, case)
+            for i in np.flatnonzero((st & ~1) == 0) if table else ():
+                Li = int(w.L[i])
+                assert torch.equal(one.C[i, :Li], ref.C[i, :Li]), (block, case, int(i), S, Lmax, M, B, size)
+            ok = torch.from_numpy((st & ~1) == 0).to(one.C_last.device)
+            assert torch.equal(one.C_last[ok], ref.C_last[ok]), (block, case)
+        del ref, one
+        torch.cuda.empty_cache()
+    assert ran >= 10                                             # most of the shapes without an argmin table were searched by this kernel alone
