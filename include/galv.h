@@ -54,7 +54,8 @@ extern "C" {
 #define GALV_STATUS_INFEASIBLE 1    /* no plan fits the budget (not an error) */
 #define GALV_STATUS_BAD_INPUT 2     /* negative entry, L[i] out of 1..Lmax, bad descriptor */
 #define GALV_STATUS_OVERFLOW_RISK 4 /* a path sum could reach GALV_INF */
-#define GALV_STATUS_TIMEOUT 8       /* a bounded device-side wait ran out while this batch ran */
+#define GALV_STATUS_TIMEOUT 8       /* a bounded device-side wait ran out while this batch ran (resident kernel: while this
+                                       instance did) */
 
 /* shape.flags */
 #define GALV_STORE_C_FULL 1 /* keep every layer of C (needed to backtrack without A) */
@@ -79,9 +80,11 @@ extern "C" {
                                                    the cluster size of that kernel */
 #define GALV_KERNEL_RESIDENT 2097152 /* the resident kernel whenever the shape allows it (S <= 128), also where another one
                                         would be taken on its own; instances it has no room for go to the tiled kernels */
-#define GALV_DEBUG_WITHHOLD_LOAD 2048 /* test hook for the time-out path: one CTA never receives its first stage, every
-                                         bounded wait that depends on it runs out (about a second each), status gets
-                                         GALV_STATUS_TIMEOUT and the call's results are void; nothing faults or hangs */
+#define GALV_DEBUG_WITHHOLD_LOAD 2048 /* test hook for the time-out path, on the tiled kernels: one CTA never receives its
+                                     first stage; with GALV_KERNEL_RESIDENT, on that kernel: the first CTA of a cluster keeps
+                                     the halo of layer 0 to itself.  Every bounded wait that depends on it runs out (about a
+                                     second each), status gets GALV_STATUS_TIMEOUT and the call's results are void; nothing
+                                     faults or hangs */
 #define GALV_SKIP_INFEASIBLE 1024 /* tiles wholly below the previous layer's feasibility frontier (sum of the
                                      layers' smallest mem) read only +inf: write their +inf results without
                                      loading or relaxing anything.  Same tables, less work on tight budgets. */

@@ -1823,6 +1823,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
 {
     cudaError_t e;
     DpArgs a = args;
+    a.withhold = (sh->flags & GALV_DEBUG_WITHHOLD_LOAD) != 0;
     const int B = a.B, Lmax = a.Lmax, S = a.S;
     const int pk = ctx->prof_count % 64;
     if (ctx->profiling) cudaEventRecord(ctx->pev[2 * pk], st);
@@ -1941,7 +1942,6 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         }
     }
     DpArgs ap = a;
-    ap.withhold = (sh->flags & GALV_DEBUG_WITHHOLD_LOAD) != 0;
     ap.skip_dom = (planned.flags & GALV_SKIP_DOMINATED) != 0;
     ap.keyed = keyed_possible;
     if (!(sh->flags & GALV_SKIP_INFEASIBLE)) ap.front = nullptr;

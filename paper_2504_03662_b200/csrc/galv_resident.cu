@@ -57,6 +57,7 @@ struct RsArgs {
     int sorted;        // clusters take the instances longest first
     int second;        // only the instances earlier launches left alone
     int probed;        // done[] says which matrices are unstructured
+    int withhold;      // test hook: a cluster's first CTA keeps the halo of layer 0 to itself, so that the waits for it run out
     const int32_t* L;
     const int32_t* time_q;
     const int32_t* mem_q;
@@ -68,7 +69,7 @@ struct RsArgs {
     uint8_t* A;        // argmin table or NULL
     int32_t* C_last;
     int32_t* status;
-    int32_t* path;     // [4] device flags of the search: error, -, -, kernel that ran
+    int32_t* path;     // [4] device flags of the search; [3]: kernel that ran
     int32_t* done;     // [B] 1: this instance needs nothing more
 };
 
@@ -83,6 +84,8 @@ __device__ __forceinline__ int ld_cluster(uint32_t addr) {
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
+__device__ __forceinline__ void st_cluster(uint32_t addr, int v) { asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ void red_min_cluster(uint32_t addr, int v) { asm volatile("red.relaxed.cluster.shared::cluster.min.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 __device__ __forceinline__ int ld_cluster_u8(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
@@ -171,8 +174,9 @@ struct Ctx {
     uint32_t bars;             // address of the two mbarriers the halo's bytes are counted on (even, odd layers)
     uint32_t halo_bytes;       // bytes of halo that arrive a layer
     bool strict;               // some shift reaches beyond the halo: layers end with the full cluster barrier
-    int* late;                 // set when a bounded wait ran out
+    int* late;                 // [0] set when a bounded wait ran out; [1] the layer from whose halo on they do not go round any more
 };
+constexpr int kNever = 0x7fffffff;
 
 // End of a layer, by every warp of the CTA.  The state of layer l+1 is complete in this CTA; its last columns go to the
 // halo of the CTAs further up that hold them, one bulk copy (through the TMA unit) a row and CTA, the warps sharing the
@@ -181,15 +185,21 @@ struct Ctx {
 // The cluster barrier only keeps the buffers apart: an arrival says that this CTA has gathered from the older buffer
 // and received its halo, and it is waited for a layer later, before the copies that overwrite that buffer are issued.
 // With shifts beyond the halo other CTAs' state is read as well, and the barrier is waited for at once.
-constexpr int kWaitPolls = 1 << 20;                            // try_wait sleeps in hardware between polls: about a second
+//
+// A wait that runs out sets late[0], at which the CTA's other waits give up too.  If it is the service warp's, it also
+// writes its layer v into late[1] of every CTA (the smallest stays) before it arrives at the barrier of layer v.  All service
+// warps have waited for that barrier when they look at the word in layer v + 2: from there on no halo is sent or expected
+// anywhere in the cluster, and the layers run out with their barriers alone.  (Bytes of layer v + 2 would be counted on the
+// mbarrier whose phase of layer v is still open.)  Before anybody leaves, each CTA waits once more, with the same limit, for
+// what of layers v and v + 1 may still be under way to it.
 template <bool ARG>
-__device__ __forceinline__ void send_halo(const Ctx& c, int l, int warp, int lane)
+__device__ __forceinline__ void send_halo(const Ctx& c, int l, int warp, int lane, bool on = true)
 {
     cta_barrier();
     if (c.CL == 1) return;
     if (!c.strict) cluster_wait();
     const uint32_t bar = c.bars + 8u * (l & 1);
-    if (warp == c.NW) {
+    if (warp == c.NW && on) {
         const uint32_t gn = smem_addr(c.g0 + ((l + 1) & 1) * c.gints), an = ARG ? smem_addr(c.a0 + ((l + 1) & 1) * c.gints) : 0u;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // plain stores of the state, read next by bulk copies
         for (int d = c.rank + 1, low = c.W - c.H; d < c.CL && low < c.W; ++d, low += c.W) {
@@ -203,17 +213,35 @@ __device__ __forceinline__ void send_halo(const Ctx& c, int l, int warp, int lan
         }
     }
 }
-template <bool ARG>
-__device__ __forceinline__ void await_halo(const Ctx& c, int l, int warp, int lane)
+constexpr int kWaitPolls = 1 << 18;                            // try_wait sleeps in hardware between polls: one second (2^20: four)
+__device__ __forceinline__ bool halo_came(const Ctx& c, int l)
+{
+    const uint32_t bar = c.bars + 8u * (l & 1), parity = (uint32_t)(l >> 1) & 1u;
+    int polls = 0;
+    while (!mbar_try(bar, parity))
+        if (++polls > kWaitPolls || *(volatile int*)c.late) { *(volatile int*)c.late = 1; return false; }
+    return true;
+}
+__device__ __forceinline__ void await_halo(const Ctx& c, int l)
 {
     if (c.CL == 1) return;
-    const uint32_t bar = c.bars + 8u * (l & 1);
-    if (c.halo_bytes) {
-        if (warp == c.NW && lane == 0) mbar_expect(bar, c.halo_bytes);
-        const uint32_t parity = (uint32_t)(l >> 1) & 1u;
-        int polls = 0;
-        while (!mbar_try(bar, parity))
-            if (++polls > kWaitPolls || *(volatile int*)c.late) { *(volatile int*)c.late = 1; break; }
+    if (c.halo_bytes) halo_came(c, l);
+    if (c.strict) { cluster_arrive(); cluster_wait(); }
+    else cluster_arrive_relaxed();
+}
+// ... by the service warp
+__device__ __forceinline__ void await_halo_service(const Ctx& c, int l, int lane, bool on)
+{
+    if (c.CL == 1) return;
+    if (c.halo_bytes && on) {
+        if (lane == 0) mbar_expect(c.bars + 8u * (l & 1), c.halo_bytes);
+        if (!halo_came(c, l)) {
+            for (int d = 0; d < c.CL; ++d) {
+                st_cluster(smem_addr(c.late) + (uint32_t)c.cdelta[d], 1);
+                red_min_cluster(smem_addr(c.late + 1) + (uint32_t)c.cdelta[d], l);
+            }
+            asm volatile("fence.acq_rel.cluster;" ::: "memory");            // the arrivals below may order nothing
+        }
     }
     if (c.strict) { cluster_arrive(); cluster_wait(); }
     else cluster_arrive_relaxed();
@@ -706,7 +734,7 @@ __device__ __forceinline__ void run_layers(const Ctx& c, int warp, int lane)
             for (; g < g1; ++g) tile<KC, 1, PRUNE, STORE, ARG, STAGE, true>(c, l, g * 32, lane);
         }
         send_halo<ARG>(c, l, warp, lane);
-        await_halo<ARG>(c, l, warp, lane);
+        await_halo(c, l);
     }
     if (c.reach[c.slot[(c.Li - 1) & 3]] <= c.H) {
         for (int g = g0; g < g1; ++g) last_tile<STORE, ARG, STAGE, false>(c, c.Li - 1, g * 32, lane);
@@ -727,7 +755,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     __shared__ int s_cdelta[16], s_front[4], s_reach[4], s_slot[4], s_inst, s_K[2];
     __shared__ struct { long long sum; int tmax, bad, mmax; } s_part, s_all;
     __shared__ __align__(8) unsigned long long s_bar[2];
-    __shared__ int s_late;
+    __shared__ int s_late[2];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x, NW = (NT >> 5) - 1;
     const int CL = a.CL, rank = CL > 1 ? (int)cluster_rank() : 0, cid = blockIdx.x / CL;
@@ -744,7 +772,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     int32_t* const stage_rows = reinterpret_cast<int32_t*>(smem_raw) + a.stage_at;         // [2][S][W] rows on their way to the table
     uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * ((S + 3) & ~3));                           // [2][gints] argmin of the state
 
-    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = ARG ? 0 : 2; }
+    if (blockIdx.x == 0 && tid == 0) a.path[3] = ARG ? 0 : 2;
 
     // ---- which instance: clusters are dispatched in order, so the longest instances go first
     int i = cid;
@@ -798,7 +826,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     }
     if (tid == 0) { s_part.sum = 0; s_part.tmax = 0; s_part.bad = 0; s_part.mmax = 0; }
     if (tid == 0) {
-        s_late = 0;
+        s_late[0] = 0; s_late[1] = kNever;
         mbar_init(smem_addr(&s_bar[0])); mbar_init(smem_addr(&s_bar[1]));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1105,7 +1133,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     c.bars = smem_addr(&s_bar[0]);
     c.halo_bytes = (uint32_t)(Kc * min(H, rank * W)) * (ARG ? 5u : 4u);
     c.strict = strict;
-    c.late = &s_late;
+    c.late = s_late;
     if (CL > 1 && !c.strict) cluster_arrive();                  // nobody has read anything yet: the first copies may come
     if (warp == NW) {
         // ---------------------------------------------------------------- service warp
@@ -1131,13 +1159,14 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
                 if (lane == 0) bulk_wait_read();                // layer l - 1 has left its buffer, which layer l + 1 fills
                 __syncwarp();
             }
-            send_halo<ARG>(c, l, warp, lane);
+            const bool on = *(volatile int*)(c.late + 1) > l - 2;            // see send_halo
+            send_halo<ARG>(c, l, warp, lane, on && !(a.withhold && l == 0 && rank == 0));
             if (STAGE && lane == 0) {
                 if (CL == 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 tensor_store_3d(&map_c, c.stage + (l & 1) * S * W, rank * (W / 32), (i * Lmax + l) * S);
                 bulk_commit();
             }
-            await_halo<ARG>(c, l, warp, lane);
+            await_halo_service(c, l, lane, on);
         }
         if (STAGE) {
             if (lane == 0) bulk_wait_read();
@@ -1164,10 +1193,12 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     }
     if (CL > 1) {
         if (!c.strict) cluster_wait();
-        whole_barrier(CL);                                      // nobody's shared memory goes away while it is being read
-        if (rank == 0 && tid == 0 && s_late) a.path[0] = 1;
+        if (s_late[1] != kNever && c.halo_bytes && warp == 0)    // copies of these two layers may still land here
+            for (int l = s_late[1]; l <= s_late[1] + 1 && l + 1 < Li; ++l)
+                for (int polls = 0; polls < kWaitPolls && !mbar_try(c.bars + 8u * (l & 1), (uint32_t)(l >> 1) & 1u); ++polls) { }
+        whole_barrier(CL);                                      // nobody's shared memory goes away while it is being read or written
+        if (s_late[0] && tid == 0) atomicOr(reinterpret_cast<int*>(a.status + i), GALV_STATUS_TIMEOUT);
     }
-    if (s_late && tid == 0) atomicOr(reinterpret_cast<int*>(a.status + i), GALV_STATUS_TIMEOUT);
 }
 
 // Which matrices are worth the resident kernel's look: of kClassMax + 1 rows two are equal if there are at most kClassMax
@@ -1350,7 +1381,8 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
 
 int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
 {
-    if (sh->flags & (GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_DEBUG_WITHHOLD_LOAD | GALV_KERNEL_NO_CLUSTER)) return 0;
+    if (sh->flags & (GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_KERNEL_NO_CLUSTER)) return 0;
+    if ((sh->flags & GALV_DEBUG_WITHHOLD_LOAD) && !(sh->flags & GALV_KERNEL_RESIDENT)) return 0;
     if (sh->S > kMaxS || (long long)sh->S * sh->m_pitch >= (1ll << 29)) return 0;      // row offsets are 32-bit
     if (ctx->plan_valid && std::memcmp(&ctx->plan_shape, sh, sizeof(*sh)) == 0) {       // the shape of the last call
         plans[0] = ctx->plans[0]; plans[1] = ctx->plans[1];
@@ -1390,7 +1422,7 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
 {
     RsArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
-    a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second;
+    a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second; a.withhold = d.withhold;
     a.probed = !p.dense && d.S > kClassMax && !second;
     if (a.probed) probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.trans_q, d.trans_inst, d.done);
     a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept

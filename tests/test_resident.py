@@ -146,3 +146,26 @@ def test_against_reference_kernel_on_many_shapes(galv, block):
         del ref, one
         torch.cuda.empty_cache()
     assert ran >= 10                                             # most of the shapes without an argmin table were searched by this kernel alone
+
+
+# a halo within the neighbours' columns; shifts beyond the halo (every layer then ends with the full barrier); argmin states
+@pytest.mark.parametrize("S,M,n,mem_hi,flags", [(24, 1000, 4, 60, 1), (24, 1000, 4, 60, 2), (64, 2880, 16, 1500, 1), (24, 1000, 5, 700, 0)])
+def test_a_halo_that_never_comes(orc, galv, S, M, n, mem_hi, flags):
+    """The wait for a halo gives up: the kernel returns, the status says TIMEOUT, the plan step walks nothing, the context
+    keeps working."""
+    import time
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    w = inputs.random_tables(3, 3, 6, S, M, mem_lo=1, mem_hi=mem_hi)
+    flags |= RES | gb.CLUSTER_SIZE(n)
+    bad = SearchBuffers(galv, w, flags | gb.DEBUG_WITHHOLD_LOAD)
+    t0 = time.time()
+    bad.dp_search()
+    torch.cuda.synchronize()
+    assert time.time() - t0 < 60
+    assert (bad.status.cpu().numpy() == gb.STATUS_TIMEOUT).all()
+    bad.backtrack()
+    r = bad.results()
+    assert (r["status"] & gb.STATUS_TIMEOUT).all() and (r["opt_cost"] == 2 ** 30 - 1).all() and (r["plan"] == -1).all()
+    check_resident(orc, galv, w, flags)
