@@ -105,7 +105,7 @@ __device__ __forceinline__ void cluster_arrive() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
-// an arrival that orders nothing: a release would wait for the table stores in flight
+// an arrival that orders nothing
 __device__ __forceinline__ void cluster_arrive_relaxed() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
@@ -185,6 +185,9 @@ constexpr int kNever = 0x7fffffff;
 // The cluster barrier only keeps the buffers apart: an arrival says that this CTA has gathered from the older buffer
 // and received its halo, and it is waited for a layer later, before the copies that overwrite that buffer are issued.
 // With shifts beyond the halo other CTAs' state is read as well, and the barrier is waited for at once.
+// Of the arrivals only the service warp's is a release: the compute warps' reads of the older buffer come before its own by
+// the CTA's barrier at the start of the hand-over, and a release covers what its warp has so observed.  The compute warps'
+// arrivals order nothing: a release of theirs would wait for their table stores in flight.
 //
 // A wait that runs out sets late[0], at which the CTA's other waits give up too.  If it is the service warp's, it also
 // writes its layer v into late[1] of every CTA (the smallest stays) before it arrives at the barrier of layer v.  All service
@@ -240,11 +243,10 @@ __device__ __forceinline__ void await_halo_service(const Ctx& c, int l, int lane
                 st_cluster(smem_addr(c.late) + (uint32_t)c.cdelta[d], 1);
                 red_min_cluster(smem_addr(c.late + 1) + (uint32_t)c.cdelta[d], l);
             }
-            asm volatile("fence.acq_rel.cluster;" ::: "memory");            // the arrivals below may order nothing
         }
     }
-    if (c.strict) { cluster_arrive(); cluster_wait(); }
-    else cluster_arrive_relaxed();
+    cluster_arrive();
+    if (c.strict) cluster_wait();
 }
 
 // Records of a layer, one entry per strategy in class order, three arrays of S2 entries each (a slot of the ring):
