@@ -1705,6 +1705,32 @@ typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_
                                     const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                     CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// Dense int32 tensor map of any rank; the driver's encoder is looked up once a process (contexts on several host threads).
+static cudaError_t encode_tiled(CUtensorMap* map, int rank, void* base, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
+                                CUtensorMapL2promotion promotion)
+{
+    static const PFN_encodeTiled fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess) { (void)cudaGetLastError(); p = nullptr; }
+        else if (q != cudaDriverEntryPointSuccess) p = nullptr;
+        return reinterpret_cast<PFN_encodeTiled>(p);
+    }();
+    if (!fn) return cudaErrorNotSupported;
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_INT32, (cuuint32_t)rank, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          CU_TENSOR_MAP_SWIZZLE_NONE, promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+cudaError_t galv_encode_table_3d(CUtensorMap* map, void* base, size_t rows, int m_pitch, int box_rows, int box_groups)
+{
+    const cuuint64_t dims[3] = {32, (cuuint64_t)(m_pitch / 32), (cuuint64_t)rows};
+    const cuuint64_t strides[2] = {128, (cuuint64_t)m_pitch * 4};
+    const cuuint32_t box[3] = {32, (cuuint32_t)box_groups, (cuuint32_t)box_rows};
+    return encode_tiled(map, 3, base, dims, strides, box, CU_TENSOR_MAP_L2_PROMOTION_NONE);
+}
+
 WsLayout galv_ws_layout(const galv_shape* sh)
 {
     WsLayout w;
@@ -1786,22 +1812,10 @@ bool galv_dp_make_plan(const galv_ctx* ctx, const galv_shape* sh, DpPlan* pl)
 // Tensor map of a row-major int32 matrix [rows][cols] (row pitch = cols * 4 bytes) with a dense box.
 static cudaError_t encode_2d(CUtensorMap* map, void* base, size_t cols, size_t rows, int box_cols, int box_rows)
 {
-    static PFN_encodeTiled fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q);
-        if (e != cudaSuccess) return e;
-        if (q != cudaDriverEntryPointSuccess || !p) return cudaErrorNotSupported;
-        fn = reinterpret_cast<PFN_encodeTiled>(p);
-    }
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
     const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_INT32, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+    return encode_tiled(map, 2, base, dims, strides, box, CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
 cudaError_t galv_dp_configure(const galv_ctx* ctx)

@@ -1,6 +1,7 @@
 // Internal declarations shared by the translation units of libgalv.so.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
@@ -100,6 +101,9 @@ int galv_set_error(galv_ctx* ctx, int code, const char* text);
 // workspace carve-up (offsets in bytes, all 256-aligned)
 struct WsLayout { size_t order, done, nactive, scratch, err, minmem_l, ntiles, istart, tcount, front, tile_done, trans_p, roll, total; };
 WsLayout galv_ws_layout(const galv_shape* sh);
+
+// Tensor map of an int32 table [rows][m_pitch] seen as [rows][m_pitch / 32][32], box [box_rows][box_groups][32].
+cudaError_t galv_encode_table_3d(CUtensorMap* map, void* base, size_t rows, int m_pitch, int box_rows, int box_groups);
 
 // launches to make (0: the shape is left to the tiled kernels); the last one takes every instance when it is dense
 int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2]);

@@ -1231,31 +1231,6 @@ __global__ void __launch_bounds__(256) probe_kernel(int B, int S, const int32_t*
 
 // ---------------------------------------------------------------- host side
 
-typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                    const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                    CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// Tensor map of an int32 table [rows][m_pitch] seen as [rows][m_pitch / 32][32], box [box_rows][box_groups][32].
-cudaError_t encode_table_3d(CUtensorMap* map, void* base, size_t rows, int m_pitch, int box_rows, int box_groups)
-{
-    static PFN_encodeTiled fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q);
-        if (e != cudaSuccess) return e;
-        if (q != cudaDriverEntryPointSuccess || !p) return cudaErrorNotSupported;
-        fn = reinterpret_cast<PFN_encodeTiled>(p);
-    }
-    const cuuint64_t dims[3] = {32, (cuuint64_t)(m_pitch / 32), (cuuint64_t)rows};
-    const cuuint64_t strides[2] = {128, (cuuint64_t)m_pitch * 4};
-    const cuuint32_t box[3] = {32, (cuuint32_t)box_groups, (cuuint32_t)box_rows};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_INT32, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 typedef void (*RsKernel)(const RsArgs, const CUtensorMap, const CUtensorMap);
 RsKernel kernel_of(bool store, bool arg, bool stage)
 {
@@ -1438,8 +1413,8 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
     std::memset(&mc, 0, sizeof(mc));
     std::memset(&ml, 0, sizeof(ml));
     if (p.stage) {
-        cudaError_t e = encode_table_3d(&ml, d.C_last, (size_t)d.B * d.S, d.m_pitch, d.S, p.w / 32);
-        if (e == cudaSuccess) e = encode_table_3d(&mc, d.C, (size_t)d.B * d.Lmax * d.S, d.m_pitch, d.S, p.w / 32);
+        cudaError_t e = galv_encode_table_3d(&ml, d.C_last, (size_t)d.B * d.S, d.m_pitch, d.S, p.w / 32);
+        if (e == cudaSuccess) e = galv_encode_table_3d(&mc, d.C, (size_t)d.B * d.Lmax * d.S, d.m_pitch, d.S, p.w / 32);
         if (e != cudaSuccess) return e;
     }
     return launch_resident(kernel_of(a.C != nullptr, d.A != nullptr, p.stage), a, p, mc, ml, st, nullptr);
