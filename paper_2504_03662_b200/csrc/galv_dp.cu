@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
 // C[0][s][m] = time(0,s) if mem(0,s) <= m else INF; pad columns INF; A = 255.
 __device__ __forceinline__ void base_row(const DpArgs& a, int i, int s)
 {
-    if (a.status[i] != 0 || (a.done && a.done[i] == 1)) return;
+    if (a.status[i] != 0) return;
     const int tt = a.time_q[(size_t)i * a.Lmax * a.S + s];
     const int mm = a.mem_q[(size_t)i * a.Lmax * a.S + s];
     const size_t row = ((size_t)i * a.S + s) * a.m_pitch;
@@ -344,11 +344,11 @@ __device__ __forceinline__ void base_row(const DpArgs& a, int i, int s)
     }
 }
 __global__ void base_layer_kernel(DpArgs a) { base_row(a, blockIdx.z, blockIdx.y); }
-// After the resident kernel, which leaves few instances or none: a few blocks look after all rows.
+// After the resident kernel, which leaves few instances or none: a few blocks look after all rows of what the schedule holds.
 __global__ void base_layer_rest_kernel(DpArgs a)
 {
-    if (a.nactive[0] == 0) return;
-    for (int r = blockIdx.y; r < a.B * a.S; r += gridDim.y) base_row(a, r / a.S, r % a.S);
+    const long long rows = (long long)a.nactive[0] * a.S;
+    for (long long r = blockIdx.y; r < rows; r += gridDim.y) base_row(a, a.order[r / a.S], (int)(r % a.S));
 }
 
 // ---------------------------------------------------------------- reference layer kernel (one thread per cell)
@@ -1612,11 +1612,16 @@ __global__ void __launch_bounds__((NSG * NMS + (P16 ? (DOM ? 7 : 5) : 4)) * 32, 
 }
 
 // C_last[i] = layer L[i]-1 of instance i (from the full table, or from the rolling buffer that
-// layer was written to), 128 bits per thread.
-__global__ void copy_last_kernel(DpArgs a)
+// layer was written to), 128 bits per thread.  After the resident kernel: of the instances in the schedule.
+__global__ void copy_last_kernel(DpArgs a, int first)
 {
-    const int i = blockIdx.y;
-    if (a.status[i] != 0 || (a.done && a.done[i] == 1)) return;
+    int i = first + blockIdx.y;
+    if (a.done) {
+        if (i >= a.nactive[0]) return;
+        i = a.order[i];
+    } else if (a.status[i] != 0) {
+        return;
+    }
     const int Li = a.L[i];
     const size_t slice = (size_t)a.S * a.m_pitch;
     const int32_t* src = a.C ? a.C + ((size_t)i * a.Lmax + (Li - 1)) * slice : a.roll + ((size_t)((Li - 1) & 1) * a.B + i) * slice;
@@ -1736,7 +1741,6 @@ WsLayout galv_ws_layout(const galv_shape* sh)
     WsLayout w;
     size_t off = 0;
     w.order = off;   off = align256(off + (size_t)sh->B * 4);
-    w.done = off;    off = align256(off + (size_t)sh->B * 4);
     w.nactive = off; off = align256(off + (size_t)(sh->Lmax + 1) * 4);
     w.scratch = off; off = align256(off + (size_t)4 * (sh->Lmax + 2) * 4);    // two int32 arrays, one 64-bit array
     w.err = off;     off = align256(off + 32);                 // error flag, largest mem, largest trans, path chosen, keyed argmin
@@ -1745,6 +1749,7 @@ WsLayout galv_ws_layout(const galv_shape* sh)
     w.istart = off;   off = align256(off + (size_t)(sh->Lmax + 1) * 8);
     w.tcount = off;   off = align256(off + (size_t)sh->Lmax * ((sh->M + 128) / 128) * 4);
     w.front = off;    off = align256(off + (size_t)sh->B * sh->Lmax * 4);
+    w.done = off;                                              // who is finished is read before the tiles' counters are zeroed: same place
     w.tile_done = off; off = align256(off + (size_t)sh->B * ((sh->M + 128) / 128) * 4);   // per (instance, tile of >= 128 columns)
     w.trans_p = off;                                           // packed trans rows for the 16-bit path (S <= 64, S % 4 == 0)
     if (sh->S <= 64 && sh->S % 4 == 0 && !(sh->flags & (GALV_KERNEL_NO_PACKED | GALV_STORE_ARGMIN | GALV_KERNEL_PER_LAYER | GALV_KERNEL_REFERENCE)))
@@ -2014,16 +2019,9 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     }
     if (ctx->profiling) { cudaEventRecord(ctx->pev[2 * pk + 1], st); ++ctx->prof_count; }
     for (int b0 = 0; b0 < B; b0 += 65535) {                   // grid.y limit
-        DpArgs c = a;
-        const int nb = (B - b0 < 65535) ? B - b0 : 65535;
-        c.L += b0; c.status += b0;
-        if (c.done) c.done += b0;
-        if (c.C) c.C += (size_t)b0 * Lmax * S * a.m_pitch;
-        c.C_last += (size_t)b0 * S * a.m_pitch;
-        c.roll += (size_t)b0 * S * a.m_pitch;
         size_t per = ((size_t)S * a.m_pitch / 4 + 255) / 256;
         if (per > (a.done ? 8 : 64)) per = a.done ? 8 : 64;
-        copy_last_kernel<<<dim3((unsigned)per, nb), 256, 0, st>>>(c);
+        copy_last_kernel<<<dim3((unsigned)per, (unsigned)(B - b0 < 65535 ? B - b0 : 65535)), 256, 0, st>>>(a, b0);
     }
     finalize_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, a.err, a.status);
     return cudaGetLastError();

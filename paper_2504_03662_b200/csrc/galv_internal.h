@@ -90,7 +90,8 @@ struct DpArgs {
     int32_t* status;
     int32_t* lean_map;   // host entry point (nobody sees the table): [B][S] state row of each strategy where the resident kernel has left
                          // the states between the layers in C in place of its values; -1 where C holds the values.  Else NULL
-    int32_t* done;       // [B] 1: searched or flagged already, 2: an unstructured matrix, not searched; or NULL when the resident kernel was not launched
+    int32_t* done;       // [B] 1: searched or flagged already, 2: an unstructured matrix, not searched; or NULL when the resident kernel was not launched.
+                         // Lies over tile_done: read until the schedule is made
     int withhold;        // test hook: CTA 0 never loads its first chunk, so that the bounded waits run out
     int skip_dom;        // packed path: leave out row pairs that cannot win in any column of a warp group's tile
 };

@@ -52,6 +52,15 @@ def test_host_side_answers_without_a_device(lib):
     assert lib.galv_create(None, 0) == gb.ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("B,Lmax,S,M,flags", [(6372, 24, 32, 2000, 1 | 4096), (776, 24, 24, 2880, 1), (32704, 6, 8, 100, 1 | 4096),
+                                              (161, 12, 40, 500, 3)])
+def test_batches_that_just_fit_the_built_in_workspace(lib, B, Lmax, S, M, flags):
+    """The largest batch of a shape that galv_dp_search_static takes stays accepted (nothing per instance was added)."""
+    from paper_2504_03662_b200 import binding as gb
+    need = [lib.galv_dp_workspace_bytes(None, C.byref(gb.make_shape(b, Lmax, S, M, flags))) for b in (B, B + 64)]
+    assert need[0] <= gb.STATIC_WORKSPACE_BYTES < need[1]
+
+
 def test_struct_sizes_match_the_header():
     from paper_2504_03662_b200 import inputs, binding as gb
     assert C.sizeof(gb.galv_shape) == 24
