@@ -94,8 +94,9 @@ extern "C" {
                                     loop.  Same tables (argmin table included); the work then depends on the spread
                                     of the costs.  Honoured when S <= 64 and, in the 32-bit loop, a tile's S rows fit
                                     one stage; ignored elsewhere (GALV_KERNEL_REFERENCE among them).  Where the tiled
-                                    kernels run without an argmin table and without GALV_KERNEL_NO_CLUSTER they do so
-                                    unasked; the resident kernel always does. */
+                                    kernels run all layers in one launch, without an argmin table and without
+                                    GALV_KERNEL_NO_CLUSTER, they do so unasked when a quarter of the rows or more have a time
+                                    that far above their layer's best; the resident kernel always does. */
 
 typedef struct galv_ctx galv_ctx;
 

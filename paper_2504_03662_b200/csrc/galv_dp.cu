@@ -144,16 +144,19 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // One CTA per instance: entries >= 0, L in range, worst-case path sum below kInf.
 // tl: entries between the transition matrices of consecutive layers (0: one matrix per instance; S*S: matrix l
 // is paid between layers l-1 and l, matrix 0 unused).
+// dominated (or NULL): three times the rows whose time exceeds their layer's smallest by more than the largest transition
+// entry, less the other rows, over the valid instances.
 __global__ void validate_kernel(int B, int Lmax, int S, int M, long long tl, const int32_t* __restrict__ L,
                                 const int32_t* __restrict__ time_q, const int32_t* __restrict__ mem_q,
                                 const int32_t* __restrict__ trans_q, int32_t* __restrict__ status, const int32_t* __restrict__ done,
-                                int32_t* __restrict__ maxmem, int32_t* __restrict__ minmem_l, int32_t* __restrict__ front)
+                                int32_t* __restrict__ maxmem, int32_t* __restrict__ minmem_l, int32_t* __restrict__ front,
+                                long long* __restrict__ dominated)
 {
     const int i = blockIdx.x;
     if (done && done[i] == 1) return;                              // searched, or flagged, by the cluster kernel
     __shared__ long long s_sum;
-    __shared__ int s_tmax, s_bad, s_mmax;
-    if (threadIdx.x == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; s_mmax = 0; }
+    __shared__ int s_tmax, s_bad, s_mmax, s_dom;
+    if (threadIdx.x == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; s_mmax = 0; s_dom = 0; }
     __syncthreads();
     const int Li = L[i];
     if (Li < 1 || Li > Lmax) {
@@ -212,6 +215,19 @@ __global__ void validate_kernel(int B, int Lmax, int S, int M, long long tl, con
                 if (front) front[(size_t)i * Lmax + l] = mn;
             }
         }
+        if (dominated) {
+            int more = 0;
+            for (int l = threadIdx.x >> 5; l < Li; l += nwarps) {
+                int mn = 0x7fffffff;
+                for (int s = lane; s < S; s += 32) mn = min(mn, t[l * S + s]);
+                mn = __reduce_min_sync(0xffffffffu, mn);
+                for (int s = lane; s < S; s += 32) more += t[l * S + s] - mn > s_tmax ? 3 : -1;
+            }
+            more = __reduce_add_sync(0xffffffffu, more);
+            if (lane == 0) atomicAdd(&s_dom, more);
+            __syncthreads();
+            if (threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long*>(dominated), static_cast<unsigned long long>((long long)s_dom));
+        }
         if (front) {
             // feasibility frontier: no cell of layer l is finite below the sum of the layers' smallest mem
             __syncthreads();
@@ -268,7 +284,10 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
 {
     __shared__ long long warp_sums[32];
     // The packed 16-bit path needs every trans entry, and twice the largest plus one, to fit 16 bits.
-    if (threadIdx.x == 0) maxmem[2] = (p16_possible && maxmem[1] <= 32767) ? 1 : 0;
+    if (threadIdx.x == 0) {
+        maxmem[2] = (p16_possible && maxmem[1] <= 32767) ? 1 : 0;
+        maxmem[4] = *reinterpret_cast<const long long*>(maxmem + 5) >= 0;      // of the rows a quarter or more
+    }
     int32_t* hist = scratch;
     int32_t* fill = scratch + Lmax + 2;
     for (int i = threadIdx.x; i < B; i += blockDim.x)
@@ -551,6 +570,7 @@ __global__ void __launch_bounds__((NSG * NMS + (P16 ? (DOM ? 7 : 5) : 4)) * 32, 
 
     // Which of the two one-launch kernels runs is decided on the device (largest transition entry).
     if (MULTI && !KEY && (a.maxmem[2] != 0) != P16) return;
+    if (P16 && a.dom_auto && (a.maxmem[4] != 0) != DOM) return;
     // Argmin table: the keys-only kernel (one launch over all layers) runs when the transition entries are small
     // enough for keys; the launches per layer that follow it then have nothing left to do.
     if (KEY && a.maxmem[3] == 0) return;
@@ -1022,6 +1042,8 @@ __global__ void __launch_bounds__((NSG * NMS + (P16 ? (DOM ? 7 : 5) : 4)) * 32, 
     (void)arg;
     int n = 0, cst = 0;
     uint32_t cph = 0;
+    const bool leave_out = DOM && (!a.dom_auto || a.maxmem[4] != 0);     // dominated rows: asked for, or enough of them.  (The packed
+                                                           // loop has a launch for each: both in one kernel cost S = 48 5 and 9 %)
     // bounded wait until the store warp has read items 0 .. upto-1 out of the staging tile
     auto drained_wait = [&](int upto) -> bool {
         WaitClock wc;
@@ -1421,7 +1443,7 @@ __global__ void __launch_bounds__((NSG * NMS + (P16 ? (DOM ? 7 : 5) : 4)) * 32, 
             }
             if constexpr (KEY) {
             } else if (keyed_done) {
-            } else if constexpr (DOM && !P16) {
+            } else if (DOM && !P16 && leave_out) {
                 // Dominated rows left out (one chunk per item, S <= 64: the host takes this instantiation only then).
                 // A candidate more than the largest transition entry above its column's best cannot win or tie;
                 // a row that is such in every column of this group's tile is not relaxed.  Each warp scans its
@@ -1613,9 +1635,14 @@ __global__ void __launch_bounds__((NSG * NMS + (P16 ? (DOM ? 7 : 5) : 4)) * 32, 
 
 // C_last[i] = layer L[i]-1 of instance i (from the full table, or from the rolling buffer that
 // layer was written to), 128 bits per thread.  After the resident kernel: of the instances in the schedule.
+// Sets the TIMEOUT bit everywhere when a bounded wait ran out.
 __global__ void copy_last_kernel(DpArgs a, int first)
 {
     int i = first + blockIdx.y;
+    if (*a.err != 0) {                                             // the tables are void
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.status[i] |= GALV_STATUS_TIMEOUT;
+        return;
+    }
     if (a.done) {
         if (i >= a.nactive[0]) return;
         i = a.order[i];
@@ -1628,14 +1655,6 @@ __global__ void copy_last_kernel(DpArgs a, int first)
     const int4* s4 = reinterpret_cast<const int4*>(src);
     int4* d4 = reinterpret_cast<int4*>(a.C_last + (size_t)i * slice);
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < slice / 4; k += (size_t)gridDim.x * blockDim.x) d4[k] = s4[k];
-}
-
-// Sets the TIMEOUT bit everywhere when a bounded wait ran out.
-__global__ void finalize_kernel(int B, const int32_t* err, int32_t* status)
-{
-    if (*err == 0) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < B; i += gridDim.x * blockDim.x)
-        status[i] |= GALV_STATUS_TIMEOUT;
 }
 
 // maps == nullptr: only opt the instantiation into its dynamic shared memory.  Layers l_first..l_last-1;
@@ -1742,7 +1761,7 @@ WsLayout galv_ws_layout(const galv_shape* sh)
     size_t off = 0;
     w.order = off;   off = align256(off + (size_t)sh->B * 4);
     w.nactive = off; off = align256(off + (size_t)(sh->Lmax + 1) * 4);
-    w.scratch = off; off = align256(off + (size_t)4 * (sh->Lmax + 2) * 4);    // two int32 arrays, one 64-bit array
+    w.scratch = off; off = align256(off + (size_t)4 * (sh->Lmax + 2) * 4);    // two int32 arrays, one 64-bit array; zeroed together with
     w.err = off;     off = align256(off + 32);                 // error flag, largest mem, largest trans, path chosen, keyed argmin
     w.minmem_l = off; off = align256(off + (size_t)(sh->Lmax + 1) * 4);
     w.ntiles = off;   off = align256(off + (size_t)(sh->Lmax + 1) * 4);
@@ -1879,20 +1898,33 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
             (void)cudaGetLastError();                        // the clusters cannot be placed on this device right now: tiled kernels
         }
     }
-    e = cudaMemsetAsync(a.scratch, 0, (size_t)4 * (Lmax + 2) * 4, st);      // histogram, fill and work counters
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(a.err, 0, 32, st);                       // error flag, largest mem, largest trans, path, keyed
+    // histogram, fill and work counters, and behind them error flag, largest mem, largest trans, path, keyed, dominated rows
+    e = cudaMemsetAsync(a.scratch, 0, reinterpret_cast<char*>(a.err) + 32 - reinterpret_cast<char*>(a.scratch), st);
     if (e != cudaSuccess) return e;
     const bool reference = (sh->flags & GALV_KERNEL_REFERENCE) != 0;
-    // Matrices that come this far are unstructured.  Without an argmin table the rows that cannot win are left out unasked
-    // (GALV_KERNEL_NO_CLUSTER takes the tiled kernels as the other flags say): 1024 instances of 48 layers, S = 32, 2048
-    // columns 7.8 -> 4.6 ms, 300 of S = 64 7.7 -> 4.1; with one, the loop on keys does about as well without (1.69 / 1.73).
-    galv_shape planned = *sh;
-    if (!a.A && S <= 64 && !(sh->flags & (GALV_KERNEL_NO_CLUSTER | GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_DEBUG_WITHHOLD_LOAD)))
-        planned.flags |= GALV_SKIP_DOMINATED;
+    // Matrices that come this far are unstructured.  All layers in one launch without an argmin table, the kernel that can
+    // leave dominated rows out is taken unasked and does so where a quarter of the rows or more look it, in the packed loop
+    // beside the kernel that does not (GALV_KERNEL_NO_CLUSTER takes the tiled kernels as the other flags say).  What it gives
+    // depends on how many rows of a layer lie more than the largest transition entry above its best.  80 instances of 32
+    // layers and 2048 columns, rows kept / left out: S = 32 93 % 560 / 423 us, 53 % 560 / 479, 27 % 560 / 520, 19 % 560 / 540,
+    // 5 % 560 / 578, none 560 / 600; S = 48 94 % 961 / 686, 56 % 961 / 795, 29 % 961 / 932, 20 % 961 / 993, none 961 / 1200;
+    // packed loop, S = 48: 73 % 848 / 772, 40 % 848 / 860, 2 % 848 / 930; 60 of S = 64: 57 % 1162 / 875, 21 % 1162 / 1121,
+    // 5 % 1162 / 1280, none 1162 / 1376.
+    bool dom_auto = !reference && !a.A && Lmax > 2 && S <= 64 &&
+                    !(sh->flags & (GALV_KERNEL_NO_CLUSTER | GALV_KERNEL_PER_LAYER | GALV_SKIP_DOMINATED | GALV_DEBUG_WITHHOLD_LOAD));
     DpPlan pl;
     std::memset(&pl, 0, sizeof(pl));
-    if (!reference && !galv_dp_make_plan(ctx, &planned, &pl)) return cudaErrorInvalidConfiguration;
+    if (!reference && !galv_dp_make_plan(ctx, sh, &pl)) return cudaErrorInvalidConfiguration;
+    bool dom_32 = (sh->flags & GALV_SKIP_DOMINATED) != 0;    // also in the 32-bit loop
+    if (dom_auto) {
+        galv_shape with = *sh;                               // its items carry live-row words: fewer rows may fit a stage
+        with.flags |= GALV_SKIP_DOMINATED;
+        DpPlan pd;
+        std::memset(&pd, 0, sizeof(pd));
+        dom_32 = galv_dp_make_plan(ctx, &with, &pd) && pd.nkc == 1;
+        if (dom_32) pl = pd;
+        dom_auto = dom_32 || pl.p16;                         // the packed loop's stages are the same either way
+    }
     if (reference) { pl.tmb = 256; pl.ntiles_m = (a.M + 256) / 256; }
     e = cudaMemsetAsync(a.minmem_l, 0x7f, (size_t)(Lmax + 1) * 4, st);
     if (e != cudaSuccess) return e;
@@ -1906,7 +1938,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     const int will_p16 = persistent && pl.p16 && !(sh->flags & GALV_KERNEL_NO_PACKED);
     // one matrix per layer is a thousand words a thread for 128 threads (96 instances of 40 layers, S = 44: 50 us)
     validate_kernel<<<B, a.trans_layer || B <= 148 ? 512 : 128, 0, st>>>(B, Lmax, S, a.M, (long long)a.trans_layer, a.L, a.time_q, a.mem_q, a.trans_q, a.status, a.done, a.err + 1, a.minmem_l,
-                                       (sh->flags & GALV_SKIP_INFEASIBLE) ? a.front : nullptr);
+                                       (sh->flags & GALV_SKIP_INFEASIBLE) ? a.front : nullptr, dom_auto ? reinterpret_cast<long long*>(a.err + 6) : nullptr);
     schedule_kernel<<<1, 1024, 0, st>>>(B, Lmax, a.M, pl.tmb, pl.ntiles_m, pl.nsb, a.L, a.status, a.done, a.order, a.nactive, a.scratch,
                                          a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.A ? 0 : 2, a.err + 1);
     auto base_layer = [&]() {
@@ -1961,7 +1993,8 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         }
     }
     DpArgs ap = a;
-    ap.skip_dom = (planned.flags & GALV_SKIP_DOMINATED) != 0;
+    ap.skip_dom = dom_auto || (sh->flags & GALV_SKIP_DOMINATED) != 0;
+    ap.dom_auto = dom_auto;
     ap.keyed = keyed_possible;
     if (!(sh->flags & GALV_SKIP_INFEASIBLE)) ap.front = nullptr;
     ap.tile_done = nullptr;
@@ -1988,12 +2021,18 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         ap.tile_done = nullptr;
     }
     if (persistent) {
-        // packed kernel first where possible, then the 32-bit one: each returns at once unless it is the one chosen
+        // packed kernels first where possible, then the 32-bit one: each returns at once unless it is the one chosen
         e = will_p16 ? launch_tiled<false>(ap, pl, 1, Lmax, st, maps, true) : cudaSuccess;
+        if (e == cudaSuccess && will_p16 && dom_auto) {
+            DpArgs plain = ap;
+            plain.skip_dom = 0;
+            e = launch_tiled<false>(plain, pl, 1, Lmax, st, maps, true);
+        }
+        if (!dom_32) ap.skip_dom = ap.dom_auto = 0;
         if (e == cudaSuccess) e = launch_tiled<false>(ap, pl, 1, Lmax, st, maps);
         if (e == cudaErrorCooperativeLaunchTooLarge) {
             // the grid cannot be co-resident right now (SMs taken by another context): one launch per layer instead.
-            // If the packed kernel was accepted before the 32-bit one was refused it may have run every layer, and on
+            // If a packed kernel was accepted before the next one was refused it may have run every layer, and on
             // the rolling buffer that overwrote layer 0: write the base layer again behind it.
             (void)cudaGetLastError();
             ap.tile_done = nullptr;
@@ -2023,6 +2062,5 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         if (per > (a.done ? 8 : 64)) per = a.done ? 8 : 64;
         copy_last_kernel<<<dim3((unsigned)per, (unsigned)(B - b0 < 65535 ? B - b0 : 65535)), 256, 0, st>>>(a, b0);
     }
-    finalize_kernel<<<(B + 255) / 256, 256, 0, st>>>(B, a.err, a.status);
     return cudaGetLastError();
 }

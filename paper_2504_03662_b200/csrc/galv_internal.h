@@ -77,7 +77,8 @@ struct DpArgs {
     int32_t* err;        // device error flag
     int32_t* tile_done;  // [B][ntiles_m] finished items per (instance, tile); NULL when layers are separate launches
     int32_t* maxmem;     // largest mem over the valid instances (min(.., M+1)); [1] largest trans entry; [2] 1: packed 16-bit path;
-                         // [3] 1: trans_k holds shifted entries (keyed argmin loop)
+                         // [3] 1: trans_k holds shifted entries (keyed argmin loop); [4] 1: a quarter of the rows or more look dominated;
+                         // [5], [6]: 64-bit count behind that
     uint32_t* trans_p;   // packed pairs of trans rows for the 16-bit path: [B][(Lmax)][S/2][S], entry = T[2q][s] | T[2q+1][s] << 16
     int32_t* trans_k;    // argmin table with keys: copy of trans_q with every entry << 6 (same place in the workspace as trans_p;
                          // a plain copy when the entries are too large for keys: maxmem[3] says which)
@@ -93,7 +94,8 @@ struct DpArgs {
     int32_t* done;       // [B] 1: searched or flagged already, 2: an unstructured matrix, not searched; or NULL when the resident kernel was not launched.
                          // Lies over tile_done: read until the schedule is made
     int withhold;        // test hook: CTA 0 never loads its first chunk, so that the bounded waits run out
-    int skip_dom;        // packed path: leave out row pairs that cannot win in any column of a warp group's tile
+    int skip_dom;        // leave out rows (packed path: row pairs) that cannot win in any column of a warp group's tile
+    int dom_auto;        // ... where a quarter of the rows or more look it (maxmem[4])
 };
 
 // records `text` as the context's last error and returns `code`

@@ -648,6 +648,33 @@ def test_dominated_rows_left_out(orc, galv, S, M, trans_hi, time_hi):
                 assert (sb.argmin_table(i)[:Li] == r["A"]).all(), (flags, i)
 
 
+@pytest.mark.parametrize("S,trans_hi,flags", [(32, 900, 1), (32, 60000, 1), (48, 900, 0), (40, 60000, 0), (64, 900, 1), (64, 60000, 1), (13, 60000, 1)])
+def test_dominated_rows_left_out_unasked(galv, S, trans_hi, flags):
+    """Times that spread far beyond the transitions, far less, and a quarter of the rows: the share decides on the device
+    whether the rows are looked at (packed and 32-bit loop), the tables never differ."""
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    B, Lmax, M = 150, 18, 1100                               # more instances than the pushing cluster kernel takes at once
+    for spread in ("far", "near", "quarter"):
+        w = inputs.random_tables(8100 + S, B, Lmax, S, M, ragged=True, mem_lo=0, mem_hi=90, trans_hi=trans_hi, time_hi=1)
+        w.trans_q[:, 0, 1] = trans_hi
+        x = np.random.default_rng(S).integers(0, trans_hi, w.time_q.shape, np.int32)
+        w.time_q += x // 8 if spread == "near" else 4 * x
+        if spread == "quarter":
+            w.time_q[:, :, : 3 * S // 4] = 1 + x[:, :, : 3 * S // 4] // 8
+        ref = SearchBuffers(galv, w, gb.STORE_C_FULL | gb.KERNEL_REFERENCE)
+        ref.dp_search(); ref.backtrack()
+        one = SearchBuffers(galv, w, flags)
+        one.dp_search(); one.backtrack()
+        torch.cuda.synchronize()
+        if S > 16:                                           # up to 16 rows are classes whatever they hold
+            assert galv.galv_dp_search_path(one.shape, one.workspace) == int(S % 4 == 0 and trans_hi <= 32767)
+        assert torch.equal(one.status, ref.status) and torch.equal(one.opt_cost, ref.opt_cost) and torch.equal(one.C_last, ref.C_last)
+        for i in range(B) if flags else ():
+            assert torch.equal(one.C[i, :int(w.L[i])], ref.C[i, :int(w.L[i])]), (spread, i)
+
+
 def test_packed_path_with_costs_near_the_limit(orc, galv):
     """Path sums just below 2^30 (the validation bound), tiny transitions: the packed loop works on differences,
     so the size of the costs themselves must not matter; a column without any finite value stays +inf."""
