@@ -308,6 +308,19 @@ __device__ __forceinline__ void lds_row(uint32_t a, int (&g)[TM]) {
     if constexpr (J + 1 < TM) lds_row<TM, J + 1>(a, g);
 }
 
+// Where the cell lies that column `col` of this CTA reads at a shift of mem: the CTA that owns it and its column there.  The
+// 32 columns of a warp start in one CTA and end in it or in the next, so the division is the warp's.
+struct Owner { int at, delta; bool in; };
+__device__ __forceinline__ Owner owner_of(const Ctx& c, int col, int mem)
+{
+    const int first = c.rank * c.W + (col & ~31) - mem;        // may lie below column 0, by less than the cluster's columns
+    int o = (first + c.CL * c.W) / c.W - c.CL;
+    int at = first + (col & 31) - o * c.W;
+    if (at >= c.W) { at -= c.W; ++o; }
+    const bool in = o >= 0;
+    return {at, c.cdelta[in ? o : 0], in};
+}
+
 // G at the columns that column `col` of this CTA (and those 32, 64, ... after it) reads; ga: the state's address plus
 // 4 * col.  FAR: the layer has shifts beyond the halo, whose cells are read from the CTA that owns them.
 template <int TM, bool FAR>
@@ -317,14 +330,10 @@ __device__ __forceinline__ void gather(const Ctx& c, uint32_t ga, int x, int who
     if (!FAR || mem <= c.H) {
         lds_row<TM>(ga + (uint32_t)x, g);
     } else {
-        const uint32_t row = ga - 4u * (uint32_t)col + (uint32_t)x + (uint32_t)mem * 4u;
-#pragma unroll
-        for (int j = 0; j < TM; ++j) {
-            const int src = c.rank * c.W + col + 32 * j - mem;
-            const int o = src / c.W;
-            g[j] = kInf;
-            if (src >= 0 && col + 32 * j < c.W) g[j] = ld_cluster(row + (uint32_t)((src - o * c.W) * 4 + c.cdelta[o]));
-        }
+        static_assert(!FAR || TM == 1, "a run of 32 columns has two owners at most");
+        const Owner o = owner_of(c, col, mem);
+        g[0] = kInf;
+        if (o.in) g[0] = ld_cluster(ga - 4u * (uint32_t)col + (uint32_t)x + (uint32_t)mem * 4u + (uint32_t)(o.at * 4 + o.delta));
     }
 }
 // ... and their argmin entries; aa: the argmin state's address plus col
@@ -336,14 +345,9 @@ __device__ __forceinline__ void gather_arg(const Ctx& c, uint32_t aa, int x, int
 #pragma unroll
         for (int j = 0; j < TM; ++j) a[j] = lds_u8(aa + (uint32_t)(off + 32 * j));
     } else {
-        const uint32_t row = aa - (uint32_t)col + (uint32_t)(off + mem);
-#pragma unroll
-        for (int j = 0; j < TM; ++j) {
-            const int src = c.rank * c.W + col + 32 * j - mem;
-            const int o = src / c.W;
-            a[j] = 255;
-            if (src >= 0 && col + 32 * j < c.W) a[j] = ld_cluster_u8(row + (uint32_t)(src - o * c.W + c.cdelta[o]));
-        }
+        const Owner o = owner_of(c, col, mem);
+        a[0] = 255;
+        if (o.in) a[0] = ld_cluster_u8(aa - (uint32_t)col + (uint32_t)(off + mem) + (uint32_t)(o.at + o.delta));
     }
 }
 
@@ -591,7 +595,7 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
                 int4 t4[KC / 4];
 #pragma unroll
                 for (int q = 0; q < KC / 4; ++q) t4[q] = lds4(ta + (uint32_t)(k * kClassMax + 4 * q) * 4u);
-                constexpr int U = FAR ? 1 : TM > 4 && STORE ? 2 : 4;
+                constexpr int U = TM > 4 && STORE ? 2 : 4;
                 for (; e + U <= end; e += U) scan<U, TM, STORE, ARG, STAGE, FAR>(c, out, la + 8u * e, rowa + 4u * e, ga, aa, col, h, hs);
                 if (U == 4 && e < end) { scan<2, TM, STORE, ARG, STAGE, FAR>(c, out, la + 8u * e, rowa + 4u * e, ga, aa, col, h, hs); e += 2; }
 #pragma unroll
@@ -620,8 +624,7 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
 #pragma unroll
         for (int j = 0; j < TM; ++j) { thr[j] = kInf; dummy[j] = 255; }
         int s = 0;
-        if (!FAR)
-            for (; s + 4 <= c.S; s += 4) scan<4, TM, STORE, ARG, STAGE, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
+        for (; s + 4 <= c.S; s += 4) scan<4, TM, STORE, ARG, STAGE, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
         for (; s < c.S; ++s) scan<1, TM, STORE, ARG, STAGE, FAR>(c, out, ra + 8u * s, rowa + 4u * s, ga, aa, col, thr, dummy);
         // a candidate beyond the column's best plus the largest entry cannot win; a column without a finite value
         // keeps nothing alive
@@ -634,8 +637,7 @@ __device__ __forceinline__ void tile(const Ctx& c, int l, int colb, int lane)
             if (32 * b < c.S) {
                 const int n = min(32, c.S - 32 * b);
                 int q = 0;
-                if (!FAR)
-                    for (; q + 4 <= n; q += 4) live[b] |= alive<4, TM, FAR>(c, ra + 8u * (32 * b + q), rowa + 4u * (32 * b + q), ga, col, thr) << q;
+                for (; q + 4 <= n; q += 4) live[b] |= alive<4, TM, FAR>(c, ra + 8u * (32 * b + q), rowa + 4u * (32 * b + q), ga, col, thr) << q;
                 for (; q < n; ++q) live[b] |= alive<1, TM, FAR>(c, ra + 8u * (32 * b + q), rowa + 4u * (32 * b + q), ga, col, thr) << q;
             }
         }
@@ -713,8 +715,7 @@ __device__ __forceinline__ void last_tile(const Ctx& c, int l, int colb, int lan
         }
     };
     int e = 0;
-    if (!FAR)
-        for (; e + 4 <= c.n_all; e += 4) steps(std::integral_constant<int, 4>(), e);
+    for (; e + 4 <= c.n_all; e += 4) steps(std::integral_constant<int, 4>(), e);
     for (; e < c.n_all; ++e) steps(std::integral_constant<int, 1>(), e);
 }
 
@@ -1347,10 +1348,12 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
         t += cl == 1 ? 200.0 : (cl > 8 ? 1250.0 : 1100.0);
         const double share = (double)(sh->B < slots ? sh->B : slots) * cl / ctx->num_sms;      // several CTAs on an SM share its issue slots
         if (share > 1.0) t *= share;
+        // layers with shifts beyond the halo are gathered four strategies and one column group at a time, at about the
+        // latency of another CTA's memory
+        p.halo_fits = cl == 1 || (long long)rows * (w + halo) <= p.gints;
+        if (!p.halo_fits) t += S * width * 300.0;
         p.rounds = (sh->B + slots - 1) / slots;
         t *= p.rounds > 3 ? (double)sh->B / slots + 0.5 : p.rounds;          // ragged batches fill the last round
-        p.halo_fits = cl == 1 || (long long)rows * (w + halo) <= p.gints;
-        if (!p.halo_fits) t *= 4.0;                            // shifts beyond the halo take the slow way
         // Of two sizes that come out about the same the finer one: ragged batches, whose lengths the host does not know,
         // fill the SMs better with it (64 instances of 1 to 96 layers: 0.79 ms on clusters of 2, 0.51 on clusters of 4;
         // with 96 layers each 0.79 and 0.94).
