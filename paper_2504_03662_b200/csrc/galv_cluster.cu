@@ -56,7 +56,7 @@ struct ClArgs {
     int32_t* C_last;
     int32_t* status;
     int32_t* path;     // [4] device flags of the search: error, -, -, kernel that ran
-    const int32_t* done;   // [B] instances that need nothing more, or NULL
+    const int32_t* done;   // [B] instances that need nothing more, or NULL: written by the resident kernel, which may still be running
 };
 
 // 3-D view of a table for the tensor-map store: [rows of S strategies per (instance, layer)][m_pitch / 32][32].
@@ -178,13 +178,18 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
         i = s_inst;
     }
 
-    if (a.done && a.done[i] == 1) return;
+    // Behind the resident kernel this grid starts beside it.  It leaves a matrix none of whose first 17 rows are equal to this
+    // kernel, so such an instance is searched at once; the others' answer is waited for.  Nobody leaves before the resident
+    // kernel has ended: what comes next in the stream waits for this grid alone.
+    constexpr int kProbeRows = kResidentClassMax + 1;
+    auto resident_over = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
     // ---- validation (every CTA of the cluster comes to the same result: nobody is left waiting at a barrier)
     if (tid == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; }
     __syncthreads();
     const int Li = a.L[i];
     if (Li < 1 || Li > Lmax) {
         if (rank == 0 && tid == 0) a.status[i] = GALV_STATUS_BAD_INPUT;
+        resident_over();
         return;
     }
     const int32_t* const tq = a.time_q + (size_t)i * Lmax * S;
@@ -210,6 +215,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
             const int v = x[k];
             bad |= (v < 0);
             tmax = max(tmax, v);
+            if (a.done && k < kProbeRows * S) buf0[k] = v;       // (one matrix per instance where there is a resident kernel in front)
         }
         tmax = __reduce_max_sync(0xffffffffu, tmax);
         bad = __any_sync(0xffffffffu, bad != 0);
@@ -220,12 +226,26 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
         }
     }
     __syncthreads();
+    if (a.done) {
+        bool equal = S < kProbeRows;
+        for (int x = warp; x < kProbeRows * kProbeRows && !equal; x += NW + 1) {
+            const int p = x / kProbeRows, q = x - p * kProbeRows;
+            if (p >= q) continue;
+            bool diff = false;
+            for (int s = lane; s < S; s += 32) diff |= buf0[p * S + s] != buf0[q * S + s];
+            equal = !__any_sync(0xffffffffu, diff);
+        }
+        if (__syncthreads_or(equal)) {
+            resident_over();
+            if (*(volatile const int32_t*)(a.done + i) == 1) return;
+        }
+    }
     {
         int st = 0;
         if (s_bad) st = GALV_STATUS_BAD_INPUT;
         else if (s_sum + (long long)(Li - 1) * s_tmax >= (long long)kInf) st = GALV_STATUS_OVERFLOW_RISK;
         if (rank == 0 && tid == 0) a.status[i] = st;
-        if (st) return;                                        // flagged: tables left untouched
+        if (st) { resident_over(); return; }                   // flagged: tables left untouched
     }
 
     const int col_g0 = rank * W;                               // first budget column of this CTA
@@ -438,6 +458,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
         bulk_commit();
         bulk_wait_all();
     }
+    resident_over();
 }
 
 }  // namespace
@@ -455,13 +476,15 @@ cudaError_t launch_cluster(const ClArgs& a, const ClPlan& p, const CUtensorMap& 
     cfg.blockDim = dim3((unsigned)((p.nw + 1) * 32));
     cfg.dynamicSmemBytes = (size_t)p.smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)p.cl;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;        // behind the resident kernel: may start beside it
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = a.done ? 2 : 1;
     if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, cluster_search_kernel<TM>, &cfg);
     return cudaLaunchKernelEx(&cfg, cluster_search_kernel<TM>, a, mc, ml);
 }
@@ -563,6 +586,7 @@ bool galv_cluster_plan(const galv_ctx* ctx, const galv_shape* sh, ClPlan* out)
             best_time = t;
             found = true;
             p.sorted = sh->B > slots;                        // more clusters than fit at once: the longest instances first
+            p.est = t;
             *out = p;
         }
     }

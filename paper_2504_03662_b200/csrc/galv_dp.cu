@@ -1885,7 +1885,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         // 14 layers of an analytic model, S = 16: 62 against 73).  So do fewer than a thousand columns, a few warps' worth
         // of work a layer (5 instances of 52 layers, S = 22, 126 columns: 136 against 185).
         const bool pushing_alone = pushing_asked || (pushing && (Lmax <= 16 || a.M < 1024));
-        const int n = pushing_alone ? 0 : galv_resident_plan(ctx, &kept, rp);
+        const int n = pushing_alone ? 0 : galv_resident_plan(ctx, &kept, pushing ? &cp : nullptr, rp);
         int launched = 0;
         while (launched < n) {
             if (galv_resident_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now

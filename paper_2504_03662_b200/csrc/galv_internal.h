@@ -8,6 +8,8 @@
 
 #include "galv.h"
 
+constexpr int kResidentClassMax = 16;      // classes beyond which a matrix counts as unstructured in the resident kernel
+
 // How the resident kernel (one thread-block cluster per instance, the state between layers in shared memory) cuts an instance.
 struct RsPlan {
     int cl;        // CTAs per cluster
@@ -20,6 +22,8 @@ struct RsPlan {
     int halo_fits, rounds;
     int stage;     // a layer's rows are collected in shared memory and leave with one tensor store
     int stage_at;  // word offset of the collected rows
+    int follow;    // the pushing cluster kernel stands behind this launch: what it does better is left to it
+    int k_max;     // ... instances of more classes
 };
 
 struct galv_ctx {
@@ -108,8 +112,9 @@ WsLayout galv_ws_layout(const galv_shape* sh);
 // Tensor map of an int32 table [rows][m_pitch] seen as [rows][m_pitch / 32][32], box [box_rows][box_groups][32].
 cudaError_t galv_encode_table_3d(CUtensorMap* map, void* base, size_t rows, int m_pitch, int box_rows, int box_groups);
 
-// launches to make (0: the shape is left to the tiled kernels); the last one takes every instance when it is dense
-int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2]);
+// launches to make (0: the shape is left to the other kernels); the last one takes every instance when it is dense
+// pushing: the plan of the pushing cluster kernel, which takes what is left; NULL when it cannot run the shape
+int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, const struct ClPlan* pushing, RsPlan plans[2]);
 cudaError_t galv_resident_configure(galv_ctx* ctx);
 cudaError_t galv_resident_launch(const RsPlan& plan, int second, const struct DpArgs& a, cudaStream_t st);
 
@@ -126,6 +131,7 @@ struct ClPlan {
     int nw;        // warps per CTA
     int smem;      // dynamic shared memory bytes
     int sorted;    // clusters take the instances longest first
+    double est;    // estimated SM cycles per layer
 };
 bool galv_cluster_plan(const galv_ctx* ctx, const galv_shape* sh, ClPlan* plan);
 cudaError_t galv_cluster_configure(galv_ctx* ctx);

@@ -18,12 +18,12 @@
 //
 // The budget columns are split over the CTAs of the cluster: CTA r owns columns r*W .. r*W+W-1 and keeps their G in two
 // buffers (this layer's, the next one's), with a halo of H columns to their left: C is produced by GATHERING G at
-// m - mem(l,s), from this CTA's own shared memory as long as the shift stays within the halo.  Whoever computes a column
-// writes it to its own buffer and into the halo of the CTAs further up that hold it (distributed shared memory; a store
-// is fired and forgotten, while reading the cells from their owner instead puts a round trip on every gather's chain:
-// 8.4 us a layer on one instance of 24 strategies over 16 CTAs).  A layer ends with one cluster barrier (a block barrier
-// where the cluster is one CTA).  No spin-waits, no cooperative launch, no cluster multicast, no workspace but a word per
-// instance and the path flag; the tables go out as full 128-byte lines and are never read back.
+// m - mem(l,s), from this CTA's own shared memory as long as the shift stays within the halo, else from its owner's.  After
+// a layer the service warp sends each row's last columns to the CTAs further up as bulk copies counted on their mbarriers (a
+// store through the cluster window took 100 cycles a warp, reading the cells from their owner a round trip on every gather's
+// chain: 8.4 us a layer on one instance of 24 strategies over 16 CTAs).  Each CTA waits for its halo with a limit (GALV_STATUS_TIMEOUT);
+// the cluster barrier's arrival of one layer is waited for in the next.  No cooperative launch, no cluster multicast, no
+// workspace but a word per instance and the path flag; the tables go out as full 128-byte lines and are never read back.
 //
 // Validation is the kernel's own (same rules and status bits as everywhere).  An instance whose state does not fit this
 // launch's shared memory is left alone and marked in done[]; a second launch with larger clusters or the tiled kernels
@@ -45,7 +45,7 @@ constexpr int kMaxSortedB = 512;          // instances whose lengths fit the ran
 constexpr int kMaxS = 128;
 constexpr int kMaxWarps = 15;             // compute warps per CTA (with the service warp 512 threads: 128 registers each)
 constexpr int kStaticSmem = 5632;         // the kernel's static shared memory, rounded up
-constexpr int kClassMax = 16;             // classes beyond which the matrix counts as unstructured
+constexpr int kClassMax = kResidentClassMax;
 
 struct RsArgs {
     int B, Lmax, S, M, m_pitch;
@@ -57,6 +57,7 @@ struct RsArgs {
     int sorted;        // clusters take the instances longest first
     int second;        // only the instances earlier launches left alone
     int probed;        // done[] says which matrices are unstructured
+    int follow, k_max;             // see RsPlan
     int withhold;      // test hook: a cluster's first CTA keeps the halo of layer 0 to itself, so that the waits for it run out
     const int32_t* L;
     const int32_t* time_q;
@@ -180,8 +181,8 @@ struct Ctx {
 constexpr int kNever = 0x7fffffff;
 
 // End of a layer, by every warp of the CTA.  The state of layer l+1 is complete in this CTA; its last columns go to the
-// halo of the CTAs further up that hold them, one bulk copy (through the TMA unit) a row and CTA, the warps sharing the
-// rows: plain stores through the cluster window took about 100 cycles a warp store, 13 thousand a layer for 7 rows of
+// halo of the CTAs further up that hold them, one bulk copy (through the TMA unit) a row and CTA, issued by the
+// service warp: plain stores through the cluster window took about 100 cycles a warp store, 13 thousand a layer for 7 rows of
 // 608 columns.  Then the wait for this CTA's own halo.
 // The cluster barrier only keeps the buffers apart: an arrival says that this CTA has gathered from the older buffer
 // and received its halo, and it is waited for a layer later, before the copies that overwrite that buffer are issued.
@@ -786,6 +787,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * ((S + 3) & ~3));                           // [2][gints] argmin of the state
 
     if (blockIdx.x == 0 && tid == 0) a.path[3] = ARG ? 0 : 2;
+    if (a.follow) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");    // the pushing kernel may start beside this one
 
     // ---- which instance: clusters are dispatched in order, so the longest instances go first
     int i = cid;
@@ -893,29 +895,46 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     // ---- classes of equal rows and equal columns
     int K = S;                                                  // unstructured unless found otherwise
     if (staged) {
-        // the nearest earlier twin of every row (0 .. S-1) and column (S .. 2S-1), compared word by word, a warp each
-        auto twins = [&](auto words) {
+        // the nearest earlier twin of every row (0 .. S-1) and column (S .. 2S-1), compared word by word, a warp each.
+        // With the pushing kernel behind this one the first kClassMax + 1 rows first: two of them are equal if there are at
+        // most kClassMax classes.  It makes the same test and has started on the instance already if none are.
+        // (One copy of the loop: code that runs once is fetched from L2, and its length is what the start takes.)
+        auto twins = [&](auto words) -> bool {
             constexpr int N = decltype(words)::value;
-            for (int x = warp; x < 2 * S; x += NW + 1) {
-                const bool row = x < S;
-                const int me = row ? x : x - S, step = row ? TP : 1, word = row ? 1 : TP;      // from one row / column, or word, to the next
-                int w[N];
+            const int probe = a.follow && S > kClassMax ? kClassMax + 1 : 0;
+            int x = warp, found = 0;
+#pragma unroll 1
+            for (int to = probe; ; to = 2 * S) {
+#pragma unroll 1
+                for (; x < to; x += NW + 1) {
+                    const bool row = x < S;
+                    const int me = row ? x : x - S, step = row ? TP : 1, word = row ? 1 : TP;      // from one row / column, or word, to the next
+                    int w[N];
 #pragma unroll
-                for (int j = 0; j < N; ++j) w[j] = lane + 32 * j < S ? stage[me * step + (lane + 32 * j) * word] : 0;
-                int twin = me;
-                for (int o = me - 1; o >= 0; --o) {
-                    bool diff = false;
+                    for (int j = 0; j < N; ++j) w[j] = lane + 32 * j < S ? stage[me * step + (lane + 32 * j) * word] : 0;
+                    int twin = me;
+                    for (int o = me - 1; o >= 0; --o) {
+                        bool diff = false;
 #pragma unroll
-                    for (int j = 0; j < N; ++j)
-                        if (lane + 32 * j < S) diff |= stage[o * step + (lane + 32 * j) * word] != w[j];
-                    if (!__any_sync(0xffffffffu, diff)) { twin = o; break; }
+                        for (int j = 0; j < N; ++j)
+                            if (lane + 32 * j < S) diff |= stage[o * step + (lane + 32 * j) * word] != w[j];
+                        if (!__any_sync(0xffffffffu, diff)) { twin = o; break; }
+                    }
+                    if (lane == 0) s_twin[x] = twin;
+                    found |= twin != me;
                 }
-                if (lane == 0) s_twin[x] = twin;
+                if (to == 2 * S) return true;
+                if (to && !__syncthreads_or(found)) return false;
             }
         };
-        if (S <= 32) twins(std::integral_constant<int, 1>());
-        else if (S <= 64) twins(std::integral_constant<int, 2>());
-        else twins(std::integral_constant<int, kMaxS / 32>());
+        const bool some = S <= 32 ? twins(std::integral_constant<int, 1>()) :
+                          S <= 64 ? twins(std::integral_constant<int, 2>()) : twins(std::integral_constant<int, kMaxS / 32>());
+        if (!some) {
+            if (rank == 0 && tid == 0) a.done[i] = 0;
+            if (warp == NW) cp_async_wait<0>();                  // nothing may land in shared memory that is no longer ours
+            if (CL > 1) cluster_wait();
+            return;
+        }
         __syncthreads();
         // a class is the twins that lead back to the same first; classes are numbered in the order of their firsts, and
         // the strategies put into the order of their rows' classes: one warp for the rows, one for the columns
@@ -1014,12 +1033,13 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     __syncthreads();                                            // s_all, classes; the staged matrix is no longer read
     if (s_all.bad) st = GALV_STATUS_BAD_INPUT;
     else if (s_all.sum + (long long)(Li - 1) * s_all.tmax >= (long long)kInf) st = GALV_STATUS_OVERFLOW_RISK;
-    const bool run = st == 0 && (classes || dense);
-    if (rank == 0 && tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run; }
+    const bool run = st == 0 && (classes || dense) && !(a.follow && K > a.k_max);
 
     // The halo: columns left of this CTA's own that its gathers reach, as many as the largest shift asks for or as fit;
     // a multiple of 32.  Below column 0 it holds +inf.
     const int H = max(0, min((s_all.mmax + 31) & ~31, (gints / Kc - W) & ~31)), P = W + H;
+
+    if (rank == 0 && tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run; }
 
     const int n_all = classes ? s_first[Kr] : S;
     const bool strict = s_all.mmax > H;                         // some shift reaches beyond the halo
@@ -1369,7 +1389,7 @@ bool best_plan(const galv_ctx* ctx, const galv_shape* sh, int rows, bool dense, 
 
 }  // namespace
 
-int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
+int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, const ClPlan* pushing, RsPlan plans[2])
 {
     if (sh->flags & (GALV_KERNEL_REFERENCE | GALV_KERNEL_PER_LAYER | GALV_KERNEL_NO_CLUSTER)) return 0;
     if ((sh->flags & GALV_DEBUG_WITHHOLD_LOAD) && !(sh->flags & GALV_KERNEL_RESIDENT)) return 0;
@@ -1389,9 +1409,25 @@ int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, RsPlan plans[2])
     bool d = (sh->S <= 32 || arg || forced) && best_plan(ctx, sh, sh->S, true, &plans[1], &td);
     if (d && !forced) d = plans[1].halo_fits && plans[1].rounds == 1;
     const bool c = !(sh->flags & GALV_TRANS_PER_LAYER) && sh->S > 8 && best_plan(ctx, sh, sh->S < 9 ? sh->S : 9, false, &plans[0], &tc);
+    // Where the pushing kernel's clusters find room beside this one's, a state of S rows has to be worth it: about 260 cycles a
+    // layer, strategy and column group (40 layers, 2880 columns, one instance, pushing / dense: S = 20 142 / 162 us,
+    // S = 32 172 / 201).  Up to 16 strategies are classes whatever the matrix: k_max sees to those.  Without that room it would
+    // start behind this kernel and cost structured batches 5 us (12 of S = 24: 99 / 106).
+    if (d && !forced && c && pushing && sh->B * (plans[0].cl + pushing->cl) <= ctx->num_sms) {
+        const int g = plans[1].w / 32, width = (g + plans[1].nw - 1) / plans[1].nw;
+        d = sh->S > kClassMax && 1600.0 + 260.0 * sh->S * width <= 0.9 * pushing->est;
+    }
     // a launch that takes every instance spares the ones after it, which find nothing to do (20 us, 40 thousand cycles)
     if (d && (!c || forced || td * sh->Lmax <= tc * sh->Lmax * 1.05 + 40000.0)) { plans[0] = plans[1]; n = 1; }
     else if (c) n = d ? 2 : 1;
+    if (c && n == 1 && !plans[0].dense && pushing) {
+        // The pushing kernel's time does not depend on classes; here one costs about 400 cycles a layer and column group.
+        // 40 layers, 2880 columns, one instance, pushing / 8 / 12 / 16 classes: S = 16 115 / 101 / 140 / 169 us,
+        // S = 24 152 / 133 / 146 / 179, S = 48 268 / 162 / 196 / 237; 30 instances, pushing / 16: S = 16 187 / 257.
+        const double width = plans[0].w / 32.0 / plans[0].nw, k = (0.9 * pushing->est - 1600.0 - 30.0 * (sh->S - 16)) / (400.0 * width);
+        plans[0].follow = 1;
+        plans[0].k_max = k < 8.0 ? 8 : k > kClassMax ? kClassMax : (int)k;
+    }
     ctx->plan_shape = *sh; ctx->plans[0] = plans[0]; ctx->plans[1] = plans[1]; ctx->plan_launches = n; ctx->plan_valid = 1;
     return n;
 }
@@ -1413,7 +1449,8 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
     RsArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
     a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second; a.withhold = d.withhold;
-    a.probed = !p.dense && d.S > kClassMax && !second;
+    a.follow = p.follow; a.k_max = p.k_max;
+    a.probed = !p.dense && d.S > kClassMax && !second && !p.follow;
     if (a.probed) probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.trans_q, d.trans_inst, d.done);
     a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;

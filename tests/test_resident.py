@@ -169,3 +169,69 @@ def test_a_halo_that_never_comes(orc, galv, S, M, n, mem_hi, flags):
     r = bad.results()
     assert (r["status"] & gb.STATUS_TIMEOUT).all() and (r["opt_cost"] == 2 ** 30 - 1).all() and (r["plan"] == -1).all()
     check_resident(orc, galv, w, flags)
+
+
+# S <= 16: classes whatever the matrix holds; 24, 40: unstructured ones are told by their first rows; 130 columns a CTA with
+# shifts over many CTAs and beyond the halo
+@pytest.mark.parametrize("S,M,mem_hi", [(12, 1100, 90), (16, 1100, 90), (24, 1500, 1500), (40, 1500, 700), (48, 1500, 1500)])
+def test_two_cluster_kernels_beside_one_another(orc, galv, S, M, mem_hi):
+    """Small batches: the pushing kernel starts beside the resident one, searches what that one leaves to it (no equal rows,
+    many classes, long halos) and nothing else.  The same buffers again and again without a pause, the matrices changing."""
+    import torch
+    from paper_2504_03662_b200.search import SearchBuffers
+    w = classed(300 + S, 5, 18, S, M, 4, 4, ragged=True, mem_lo=0, mem_hi=mem_hi)
+    other = classed(301 + S, 5, 18, S, M, 4, 4, ragged=True, mem_lo=0, mem_hi=60)
+    rng = np.random.default_rng(S)
+    w.trans_q[1] = rng.integers(0, 3000, (S, S), np.int32)
+    w.trans_q[2] = rng.integers(0, 2000, (12, 12), np.int32)[np.arange(S) % 12][:, np.arange(S) % 12]
+    w.mem_q[3] //= 20                                            # short shifts
+    w.time_q[4, 0, 0] = -1
+    other.trans_q[[0, 3]] = rng.integers(0, 3000, (2, S, S), np.int32)
+    for flags in (1, 0):
+        sets = []
+        for x in (w, other):
+            sb, res = check_batch(orc, galv, x, flags, idx=[0, 1, 2, 3])
+            assert galv.galv_dp_search_path(sb.shape, sb.workspace) == 2
+            sets.append((sb, {k: getattr(sb, k).clone() for k in ("opt_cost", "plan", "status", "C_last")}))
+        assert sets[0][1]["status"][4] == 2
+        one = SearchBuffers(galv, w, flags)
+        got = []
+        for _ in range(10):
+            for sb, _r in sets:
+                for k in ("time_q", "mem_q", "trans_q", "L"):
+                    getattr(one, k).copy_(getattr(sb, k))
+                one.dp_search(); one.backtrack()
+                got.append({k: getattr(one, k).clone() for k in ("opt_cost", "plan", "status", "C_last")})
+        torch.cuda.synchronize()
+        for n, g in enumerate(got):
+            ref = sets[n % 2][1]
+            ok = ref["status"] & ~1 == 0
+            for k in ("opt_cost", "plan", "status"):
+                assert torch.equal(g[k], ref[k]), (n, k)
+            assert torch.equal(g["C_last"][ok], ref["C_last"][ok]), n
+
+
+def test_both_cluster_kernels_in_a_graph(galv):
+    """The launch that may start early is captured as such: replays with changing matrices equal plain calls."""
+    import torch
+    from paper_2504_03662_b200.search import SearchBuffers
+    w = classed(77, 3, 18, 40, 1500, 4, 4, mem_lo=0, mem_hi=200)
+    plain, one = SearchBuffers(galv, w, 1), SearchBuffers(galv, w, 1)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        one.dp_search(); one.backtrack()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            one.dp_search(); one.backtrack()
+    rng = np.random.default_rng(3)
+    for k in range(6):
+        x = w.trans_q if k % 2 else rng.integers(0, 3000, w.trans_q.shape, np.int32)
+        for sb in (plain, one):
+            sb.trans_q.copy_(torch.from_numpy(np.ascontiguousarray(x)))
+        torch.cuda.synchronize()
+        plain.dp_search(); plain.backtrack()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(plain.C, one.C) and torch.equal(plain.plan, one.plan) and torch.equal(plain.opt_cost, one.opt_cost), k
+    del g
