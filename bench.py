@@ -247,13 +247,18 @@ def cost_model_scaled(torch, galv, hbm_gbs, barrier, copies=8192):
 
 
 def launches_per_step(w, cluster: bool = False) -> int:
-    if cluster:                                   # the cost model's kernel, the resident kernel for the whole search, backtrack
-        return (1 if w.has_model else 0) + 1 + 1
-    # the cost model's kernel, validate + schedule + base layer, ONE cooperative launch over all layers,
-    # copy-last + finalize, backtrack; where the shape allows the packed 16-bit path, the kernel that packs
-    # the trans rows and the launch of the other inner-loop variant (it returns at once) come on top
+    # the tiled kernels: validate + schedule + base layer, ONE cooperative launch over all layers, copy-last; where the shape
+    # allows the packed 16-bit path, the kernel that packs the trans rows and the launches of the two packed variants come on
+    # top (those not chosen return at once)
     packable = w.S <= 64 and w.S % 4 == 0
-    return (1 if w.has_model else 0) + 3 + 1 + 2 + 1 + (2 if packable else 0)
+    tiled = 3 + 1 + 1 + (3 if packable else 0)
+    if cluster and w.S <= 32:                     # the resident kernel for the whole search
+        search = 1
+    elif cluster:                                 # ... and, where it has no room for an unstructured matrix, who would take one:
+        search = 2 if w.B <= 16 and w.M < 4096 else 2 + tiled      # the pushing kernel, or a probe in front and the tiled kernels
+    else:
+        search = 2 + tiled                        # the probe and the resident kernel turn the batch away
+    return (1 if w.has_model else 0) + search + 1               # the cost model's kernel, the search, backtrack
 
 
 def bench_workload(torch, galv, w, steps, warmup, barrier, flags=1):
@@ -426,7 +431,7 @@ def main():
                      "traffic_unit": "bytes per launch (ncu dram read+write per layer x layers)",
                      "algorithmic_bytes_per_launch": 2 * 4 * w.B * w.S * w.m_pitch * (w.Lmax - 1),
                      "algorithmic_ops_per_launch": relax_per_launch,
-                     "kernel": ("cluster_search_kernel (one thread-block cluster per instance, all layers in one launch)" if r["cluster"] else
+                     "kernel": ("a cluster kernel (one thread-block cluster per instance, all layers in one launch)" if r["cluster"] else
                                 "layer_tiled_kernel (one cooperative launch over all layers"
                                 + (", packed 16-bit variant)" if r["packed"] else ")")),
                      "launch_ms": r["layer_loop_ms"], "launch_ms_min": r["layer_loop_ms_min"],
@@ -451,7 +456,7 @@ def main():
                                  "algorithmic_ops_per_launch": None,
                                  "inner_loop": "one add and one class minimum a cell, 32-bit",
                                  "relaxations_stood_for_of_alu_peak": achieved / ALU_PEAK_GOPS,
-                                 "kernel": "resident_kernel (one thread-block cluster per instance, the state between layers in shared memory)",
+                                 "kernel": "resident_kernel (one thread-block cluster per instance, the state between layers in shared memory; short stacks: cluster_search_kernel)",
                                  "peak_source": "measured copy bandwidth" if peaks else "fallback copy bandwidth"})
         del line["roofline"]["frac_of_32bit_peak"]
         achieved = line["roofline"]["achieved"]

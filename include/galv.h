@@ -69,7 +69,9 @@ extern "C" {
                                       one launch and every transition entry <= 32767; same results) */
 #define GALV_KERNEL_NO_CLUSTER 16384 /* the tiled kernels only: neither the resident kernel (one thread-block cluster per
                                         instance, the state between layers kept in shared memory: one row per distinct
-                                        column of the transition matrix) nor the pushing cluster kernel (small batches,
+                                        column of the transition matrix; taken on its own from 9 strategies on, S <= 128,
+                                        where that state fits, but for stacks of up to 16 layers or fewer than 1024
+                                        columns that the other one can take) nor the pushing cluster kernel (small batches,
                                         the table slice kept in shared memory).  Same results */
 #define GALV_KERNEL_CLUSTER 32768 /* the pushing cluster kernel whenever the shape allows it (S <= 128, no argmin table),
                                      also for batches that need several rounds of clusters (at most 512 instances then);
