@@ -112,6 +112,7 @@ int galv_create(galv_ctx** out, int device_ordinal)
     e = galv_dp_configure(ctx);
     if (e == cudaSuccess) e = galv_cluster_configure(ctx);
     if (e == cudaSuccess) e = galv_resident_configure(ctx);
+    if (e == cudaSuccess) e = galv_solo_configure(ctx);
     for (auto& ev : ctx->pev)
         if (e == cudaSuccess) e = cudaEventCreate(&ev);
     if (cur >= 0 && cur != device_ordinal) cudaSetDevice(cur);

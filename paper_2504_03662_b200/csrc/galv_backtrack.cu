@@ -101,12 +101,17 @@ __device__ __forceinline__ long long walk_states(int Li, int S, int m_pitch, con
 {
     const int lane = threadIdx.x;
     long long used = 0;
+    // The solo kernel's states are a row of bases and rows of differences' words, two rows to a word if 16 bits do.
+    const int form = row_of[0] & (kStateHalf | kStateWord);
     int mnext[NJ], tnext[NJ];                                  // rows of layer l-1
     int crow[NJ], rows = 0;                                    // state row of each of this lane's strategies, rows a layer
+    int half[NJ];                                              // ... where its bits begin in the row's words
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
-        crow[j] = k < S ? row_of[k] : 0;
+        crow[j] = k < S ? row_of[k] & 0xffff : 0;
+        half[j] = form == kStateHalf ? 16 * (crow[j] & 1) : 0;
+        if (form) crow[j] = 1 + (form == kStateHalf ? crow[j] >> 1 : crow[j]);
         rows = max(rows, crow[j] + 1);
         mnext[j] = k < S && Li > 1 ? mq[(Li - 2) * S + k] : 0;
         tnext[j] = k < S && Li > 1 ? tq[(Li - 2) * S + k] : 0;
@@ -135,7 +140,20 @@ __device__ __forceinline__ long long walk_states(int Li, int S, int m_pitch, con
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
             const int k = lane + 32 * j, src = m - mm - mnext[j];
-            const int g = k < S && src >= 0 ? (l > 1 ? prev[(size_t)crow[j] * m_pitch + src] : 0) : kInf;
+            int g = kInf;
+            if (k < S && src >= 0) {
+                g = 0;
+                if (l > 1) {
+                    const int word = prev[(size_t)crow[j] * m_pitch + src];
+                    g = word;
+                    if (form) {
+                        const int base = prev[src];
+                        g = (int)((uint32_t)word >> half[j]);
+                        if (form == kStateHalf) g &= 0xffff;
+                        g = base < kInf ? base + g : kInf;     // where nothing is finite the words are not there
+                    }
+                }
+            }
             cv[j] = g < kInf ? g + tnext[j] : kInf;
             tv[j] = k < S ? (STAGED ? s_trans[k * S + s] : T[k * S + s]) : 0;
         }

@@ -56,7 +56,8 @@ struct ClArgs {
     int32_t* C_last;
     int32_t* status;
     int32_t* path;     // [4] device flags of the search: error, -, -, kernel that ran
-    const int32_t* done;   // [B] instances that need nothing more, or NULL: written by the resident kernel, which may still be running
+    const int32_t* done;   // [B] instances that need nothing more, or NULL: written by the kernel before this one, which may still be running
+    int wait_done;         // ... and may take any instance: it is waited for first
 };
 
 // 3-D view of a table for the tensor-map store: [rows of S strategies per (instance, layer)][m_pitch / 32][32].
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
     }
     __syncthreads();
     if (a.done) {
-        bool equal = S < kProbeRows;
+        bool equal = S < kProbeRows || a.wait_done;
         for (int x = warp; x < kProbeRows * kProbeRows && !equal; x += NW + 1) {
             const int p = x / kProbeRows, q = x - p * kProbeRows;
             if (p >= q) continue;
@@ -620,7 +621,7 @@ cudaError_t galv_cluster_launch(galv_ctx* ctx, const galv_shape* sh, const ClPla
     a.CL = p.cl; a.W = p.w; a.G = p.g; a.NSG = p.nsg; a.SP8 = p.sp8; a.nct = p.nct; a.units = p.units; a.sorted = p.sorted;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
-    a.C = d.C; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done;
+    a.C = d.C; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done; a.wait_done = d.wait_done;
     (void)sh;
     CUtensorMap mc, ml;
     std::memset(&mc, 0, sizeof(mc));

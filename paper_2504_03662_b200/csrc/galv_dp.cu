@@ -284,6 +284,8 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
 {
     __shared__ long long warp_sums[32];
     // The packed 16-bit path needs every trans entry, and twice the largest plus one, to fit 16 bits.
+    const int path_so_far = maxmem[2];                 // of the kernel in front, if it has taken every instance
+    __syncthreads();
     if (threadIdx.x == 0) {
         maxmem[2] = (p16_possible && maxmem[1] <= 32767) ? 1 : 0;
         maxmem[4] = *reinterpret_cast<const long long*>(maxmem + 5) >= 0;      // of the rows a quarter or more
@@ -305,7 +307,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
     __syncthreads();
     if (done && !s_any) {                              // every instance is finished: an empty schedule
         for (int l = threadIdx.x; l <= Lmax; l += blockDim.x) { nactive[l] = 0; istart[l] = 0; }
-        if (threadIdx.x == 0) maxmem[2] = path_done;
+        if (threadIdx.x == 0) maxmem[2] = path_done >= 0 ? path_done : path_so_far;
         return;
     }
     {
@@ -1865,6 +1867,11 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     const int B = a.B, Lmax = a.Lmax, S = a.S;
     const int pk = ctx->prof_count % 64;
     if (ctx->profiling) cudaEventRecord(ctx->pev[2 * pk], st);
+    bool cleared = false, solo = false;
+    auto clear = [&]() {     // histogram, fill and work counters, and behind them error flag, largest mem, largest trans, path, keyed, dominated rows
+        cleared = true;
+        return cudaMemsetAsync(a.scratch, 0, reinterpret_cast<char*>(a.err) + 32 - reinterpret_cast<char*>(a.scratch), st);
+    };
     {
         // The state between layers kept in shared memory wherever it fits.  What these launches leave alone is known on
         // the device only: it goes to the pushing cluster kernel (small batches) or to the tiled kernels, which find
@@ -1877,30 +1884,44 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         galv_shape kept = *sh;
         if (a.lean_map) kept.flags &= ~GALV_STORE_C_FULL;
         ClPlan cp;
+        SoPlan sp;
         const bool resident_asked = (sh->flags & GALV_KERNEL_RESIDENT) != 0;
         const bool pushing_asked = !resident_asked && ((sh->flags & GALV_KERNEL_CLUSTER) != 0 || ((sh->flags >> 16) & 31) != 0);
+        solo = !resident_asked && !pushing_asked && galv_solo_plan(ctx, &kept, a.lean_map != nullptr, &sp);
         const bool pushing = !resident_asked && galv_cluster_plan(ctx, sh, &cp);
+        a.wait_done = 0;
+        int first = 0;
+        if (solo) {
+            // What this launch has no room for is known on the device only.
+            const bool probed = !sp.dense && !pushing;
+            if (probed) galv_probe_matrices(a, st);
+            // what the tiled kernels start from is cleared first: it lies around the word that says which kernel ran
+            if (!sp.certain && !pushing && (e = clear()) != cudaSuccess) return e;
+            if ((e = galv_solo_launch(sp, a, pushing, probed, st)) != cudaSuccess) return e;
+            if (sp.certain) return finished();
+            a.wait_done = sp.dense;
+            first = 1;
+        }
         // A short stack is over before the resident kernel has looked at its matrix: up to 16 layers the pushing cluster
         // kernel alone, where it can (3 instances of 6 layers, S = 7: 21 us against 33; 10 layers, S = 18: 47 against 55;
         // 14 layers of an analytic model, S = 16: 62 against 73).  So do fewer than a thousand columns, a few warps' worth
         // of work a layer (5 instances of 52 layers, S = 22, 126 columns: 136 against 185).
-        const bool pushing_alone = pushing_asked || (pushing && (Lmax <= 16 || a.M < 1024));
-        const int n = pushing_alone ? 0 : galv_resident_plan(ctx, &kept, pushing ? &cp : nullptr, rp);
+        const bool pushing_alone = pushing_asked || (pushing && (solo || Lmax <= 16 || a.M < 1024));
+        int n = pushing_alone ? 0 : galv_resident_plan(ctx, &kept, pushing ? &cp : nullptr, rp);
+        if (n && solo && sp.classes && !rp[0].dense) { rp[0] = rp[1]; --n; }       // nothing with classes is left
         int launched = 0;
         while (launched < n) {
-            if (galv_resident_launch(rp[launched], launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now
+            if (galv_resident_launch(rp[launched], first + launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now
             ++launched;
         }
         if (launched && launched == n && rp[n - 1].dense) return finished();
-        if (!launched) a.done = nullptr;
+        if (!launched && !first) a.done = nullptr;
         if (pushing) {
             if (galv_cluster_launch(ctx, sh, cp, a, st) == cudaSuccess) return finished();
             (void)cudaGetLastError();                        // the clusters cannot be placed on this device right now: tiled kernels
         }
     }
-    // histogram, fill and work counters, and behind them error flag, largest mem, largest trans, path, keyed, dominated rows
-    e = cudaMemsetAsync(a.scratch, 0, reinterpret_cast<char*>(a.err) + 32 - reinterpret_cast<char*>(a.scratch), st);
-    if (e != cudaSuccess) return e;
+    if (!cleared && (e = clear()) != cudaSuccess) return e;
     const bool reference = (sh->flags & GALV_KERNEL_REFERENCE) != 0;
     // Matrices that come this far are unstructured.  All layers in one launch without an argmin table, the kernel that can
     // leave dominated rows out is taken unasked and does so where a quarter of the rows or more look it, in the packed loop
@@ -1940,7 +1961,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     validate_kernel<<<B, a.trans_layer || B <= 148 ? 512 : 128, 0, st>>>(B, Lmax, S, a.M, (long long)a.trans_layer, a.L, a.time_q, a.mem_q, a.trans_q, a.status, a.done, a.err + 1, a.minmem_l,
                                        (sh->flags & GALV_SKIP_INFEASIBLE) ? a.front : nullptr, dom_auto ? reinterpret_cast<long long*>(a.err + 6) : nullptr);
     schedule_kernel<<<1, 1024, 0, st>>>(B, Lmax, a.M, pl.tmb, pl.ntiles_m, pl.nsb, a.L, a.status, a.done, a.order, a.nactive, a.scratch,
-                                         a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.A ? 0 : 2, a.err + 1);
+                                         a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.A ? 0 : solo ? -1 : 2, a.err + 1);
     auto base_layer = [&]() {
         int gx = (a.m_pitch + 255) / 256;
         if (gx > 8) gx = 8;

@@ -8,6 +8,7 @@
 
 #include "galv.h"
 
+constexpr int kStateHalf = 1 << 16, kStateWord = 1 << 17;      // DpArgs::lean_map: states of bases and 16-bit (two rows a word) or 32-bit differences
 constexpr int kResidentClassMax = 16;      // classes beyond which a matrix counts as unstructured in the resident kernel
 
 // How the resident kernel (one thread-block cluster per instance, the state between layers in shared memory) cuts an instance.
@@ -24,6 +25,20 @@ struct RsPlan {
     int stage_at;  // word offset of the collected rows
     int follow;    // the pushing cluster kernel stands behind this launch: what it does better is left to it
     int k_max;     // ... instances of more classes
+};
+
+// How the solo kernel (an instance's state on one SM) cuts a batch.
+struct SoPlan {
+    int nw;        // compute warps per CTA
+    int mats;      // words of the transition matrices in shared memory
+    int smem;      // dynamic shared memory bytes
+    int room;      // ... of which for the state
+    int sorted;    // CTA c takes the c-th longest instance
+    int dense;     // unstructured matrices fit, with transition entries up to 65535 at least
+    int certain;   // every instance can run
+    int classes;   // every matrix of up to 9 classes of equal columns can
+    int rounds;    // more instances than SMs
+    int packed;    // packed relaxations are allowed
 };
 
 struct galv_ctx {
@@ -94,10 +109,12 @@ struct DpArgs {
     int32_t* tcount;     // [Lmax][ntiles_m] layers 1..l whose items include tile t
     int32_t* status;
     int32_t* lean_map;   // host entry point (nobody sees the table): [B][S] state row of each strategy where the resident kernel has left
-                         // the states between the layers in C in place of its values; -1 where C holds the values.  Else NULL
+                         // the states between the layers in C in place of its values (with kStateHalf or kStateWord added: the solo
+                         // kernel); -1 where C holds the values.  Else NULL
     int32_t* done;       // [B] 1: searched or flagged already, 2: an unstructured matrix, not searched; or NULL when the resident kernel was not launched.
                          // Lies over tile_done: read until the schedule is made
     int withhold;        // test hook: CTA 0 never loads its first chunk, so that the bounded waits run out
+    int wait_done;       // done[] is to be waited for before anything is searched: the launch before this one may take any instance
     int skip_dom;        // leave out rows (packed path: row pairs) that cannot win in any column of a warp group's tile
     int dom_auto;        // ... where a quarter of the rows or more look it (maxmem[4])
 };
@@ -111,6 +128,14 @@ WsLayout galv_ws_layout(const galv_shape* sh);
 
 // Tensor map of an int32 table [rows][m_pitch] seen as [rows][m_pitch / 32][32], box [box_rows][box_groups][32].
 cudaError_t galv_encode_table_3d(CUtensorMap* map, void* base, size_t rows, int m_pitch, int box_rows, int box_groups);
+
+// whether it can take the shape, which has no table to write; states: they are kept in its place
+bool galv_solo_plan(const galv_ctx* ctx, const galv_shape* sh, bool states, SoPlan* plan);
+cudaError_t galv_solo_configure(galv_ctx* ctx);
+// follow: the next kernel of the stream may start beside this one; probed: done[] = 2 where a matrix is unstructured
+cudaError_t galv_solo_launch(const SoPlan& plan, const struct DpArgs& a, int follow, int probed, cudaStream_t st);
+// done[i] = 2 where no two of the first rows of a matrix are equal, else 0
+void galv_probe_matrices(const struct DpArgs& a, cudaStream_t st);
 
 // launches to make (0: the shape is left to the other kernels); the last one takes every instance when it is dense
 // pushing: the plan of the pushing cluster kernel, which takes what is left; NULL when it cannot run the shape

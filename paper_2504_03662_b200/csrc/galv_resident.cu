@@ -786,7 +786,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     int32_t* const stage_rows = reinterpret_cast<int32_t*>(smem_raw) + a.stage_at;         // [2][S][W] rows on their way to the table
     uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * ((S + 3) & ~3));                           // [2][gints] argmin of the state
 
-    if (blockIdx.x == 0 && tid == 0) a.path[3] = ARG ? 0 : 2;
+    if (blockIdx.x == 0 && tid == 0 && !a.second) a.path[3] = ARG ? 0 : 2;
     if (a.follow) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");    // the pushing kernel may start beside this one
 
     // ---- which instance: clusters are dispatched in order, so the longest instances go first
@@ -1444,6 +1444,8 @@ cudaError_t galv_resident_configure(galv_ctx* ctx)
     return cudaSuccess;
 }
 
+void galv_probe_matrices(const DpArgs& d, cudaStream_t st) { probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.trans_q, d.trans_inst, d.done); }
+
 cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, cudaStream_t st)
 {
     RsArgs a;
@@ -1451,7 +1453,7 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
     a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second; a.withhold = d.withhold;
     a.follow = p.follow; a.k_max = p.k_max;
     a.probed = !p.dense && d.S > kClassMax && !second && !p.follow;
-    if (a.probed) probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.trans_q, d.trans_inst, d.done);
+    if (a.probed) galv_probe_matrices(d, st);
     a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;

@@ -1,0 +1,125 @@
+"""The kernel that keeps an instance's state on one SM: every table, optimum and plan against the one-thread-per-cell kernel,
+which other tests tie to the CPU oracle, and against the oracle itself.  Whole numbers: exact.
+"""
+import numpy as np
+import pytest
+
+from paper_2504_03662_b200 import inputs
+from tests.test_gpu_parity import INF, check_batch, galv, oracle_search_many  # noqa: F401  (galv is a fixture)
+from tests.test_resident import classed
+
+pytestmark = pytest.mark.gpu
+
+
+def against_reference(galv, w, flags):
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    ref = SearchBuffers(galv, w, flags | gb.KERNEL_REFERENCE)
+    ref.dp_search(); ref.backtrack()
+    one = SearchBuffers(galv, w, flags)
+    for t in (one.C, one.A, one.C_last):
+        if t is not None:
+            t.fill_(77)
+    for _ in range(2):
+        one.dp_search(); one.backtrack()
+        torch.cuda.synchronize()
+        assert torch.equal(one.status, ref.status)
+        assert torch.equal(one.opt_cost, ref.opt_cost)
+        assert torch.equal(one.plan, ref.plan) and torch.equal(one.mem_used, ref.mem_used)
+        ok = [i for i in range(w.B) if int(ref.status[i]) in (0, 1)]
+        for i in ok:
+            Li = int(w.L[i])
+            assert torch.equal(one.C_last[i], ref.C_last[i]), i
+            if ref.C is not None:
+                assert torch.equal(one.C[i, :Li], ref.C[i, :Li]), i
+                assert Li == w.Lmax or bool((one.C[i, Li:] == 77).all())          # layers that are not there are not touched
+            if ref.A is not None:
+                assert torch.equal(one.A[i, :Li], ref.A[i, :Li]), i
+    return one
+
+
+# S and classes at the edges of the accumulator widths (8 / 16 / 32 / 64 rows), of a warp's lanes and of the boxes of collected rows
+@pytest.mark.parametrize("S,rows,cols", [(1, 1, 1), (5, 1, 1), (7, 0, 0), (8, 0, 0), (9, 0, 0), (16, 0, 0), (17, 0, 0), (24, 4, 4), (24, 5, 9), (31, 0, 0),
+                                         (32, 0, 0), (33, 8, 7), (33, 0, 0), (44, 0, 0), (64, 9, 16), (64, 16, 9), (64, 0, 0), (65, 3, 3), (128, 8, 8)])
+@pytest.mark.parametrize("flags", [1, 0, 3, 2])
+def test_rows_of_the_state(galv, S, rows, cols, flags):
+    M = 700
+    kw = dict(ragged=True, mem_lo=0, mem_hi=M // 5, time_hi=4000)
+    w = classed(300 + S + rows, 6, 7, S, M, rows, cols, **kw) if rows else inputs.random_tables(300 + S, 6, 7, S, M, **kw)
+    w.mem_q[1, 2, : S // 2] = M + 3                              # rows that never fit
+    w.time_q[2, 1, :] = 9                                        # ties: the lowest strategy must win
+    w.time_q[4, :, :] = 3
+    w.mem_q[3, 0, :] = M // 2                                    # the lower half of every later column is +inf
+    w.L[5] = 1
+    against_reference(galv, w, flags)
+
+
+# columns: less than a group, one more than a group, a step of tiles and one more, several steps; largest shifts from none to the budget
+@pytest.mark.parametrize("M,mem_hi", [(0, 0), (5, 2), (31, 9), (32, 32), (607, 40), (608, 700), (2880, 300), (3040, 3040), (8191, 700)])
+@pytest.mark.parametrize("S,K", [(24, 4), (12, 0), (20, 0)])
+def test_columns_and_shifts(galv, M, mem_hi, S, K):
+    kw = dict(ragged=True, mem_lo=0, mem_hi=mem_hi, time_hi=10 ** 6)
+    for B in (1, 3):
+        w = classed(M + 40, B, 5, S, M, K, K, **kw) if K else inputs.random_tables(M + 41, B, 5, S, M, **kw)
+        w.mem_q[0, min(1, w.Lmax - 1), 0] = M
+        for flags in (1, 0, 2):
+            against_reference(galv, w, flags)
+
+
+# largest transition entry: differences of 16 and of 32 bits, packed relaxations or not, keys of the argmin
+@pytest.mark.parametrize("top", [0, 1, 32767, 32768, 65535, 65536, (1 << 23) - 1, 1 << 23])
+@pytest.mark.parametrize("S,K", [(24, 6), (16, 0), (40, 0), (64, 0)])
+def test_largest_transition_entry(galv, top, S, K):
+    for time_hi in (50, 60_000_000):
+        w = inputs.random_tables(S + top % 97, 4, 6, S, 900, ragged=True, mem_lo=0, mem_hi=150, time_hi=time_hi, trans_hi=top)
+        if K:
+            rng = np.random.default_rng(S)
+            for i in range(w.B):
+                w.trans_q[i] = rng.integers(0, top + 1, (K, K), np.int32)[rng.integers(0, K, S)][:, rng.integers(0, K, S)]
+        w.trans_q[:, 0, S - 1] = top
+        for flags in (1, 2):
+            against_reference(galv, w, flags)
+
+
+@pytest.mark.parametrize("block", range(6))
+def test_against_reference_kernel_on_many_shapes(galv, block):
+    rng = np.random.default_rng(7700 + block)
+    for case in range(14):
+        S = int(rng.choice([1, 3, 8, 13, 16, 17, 24, 32, 40, 64, 100, 128]))
+        Lmax, M, B = int(rng.integers(1, 14)), int(rng.integers(0, 4000)), int(rng.choice([1, 2, 5, 16, 40, 130, 200]))
+        kw = dict(ragged=bool(rng.integers(0, 2)), mem_lo=0, mem_hi=int(rng.choice([0, 5, M // 30 + 1, M // 4 + 1, M + 50, 3 * M + 1])),
+                  time_hi=int(rng.choice([5, 10 ** 4, 10 ** 6])))
+        K = int(rng.choice([0, 1, 4, 8, 16]))
+        w = classed(91000 + 100 * block + case, B, Lmax, S, M, K, max(1, K - 1), **kw) if K else \
+            inputs.random_tables(91000 + 100 * block + case, B, Lmax, S, M, trans_hi=int(rng.choice([0, 9, 40000, 200000])), **kw)
+        if Lmax > 2 and rng.integers(0, 2):
+            w.time_q[:, 2] = w.time_q[:, 1]; w.mem_q[:, 2] = w.mem_q[:, 1]         # layers with the same rows share their records
+        if rng.integers(0, 4) == 0 and B * Lmax * S * S < 4_000_000:
+            w.trans_q = np.ascontiguousarray(rng.integers(0, 3000, (B, Lmax, S, S), np.int32))
+        against_reference(galv, w, int(rng.choice([1, 0, 2, 3])))
+
+
+@pytest.mark.parametrize("S,K,top", [(64, 7, 2000), (24, 4, 50000), (40, 0, 900), (30, 0, 60000), (12, 0, 90000), (48, 8, 300000), (2, 0, 9), (1, 0, 9)])
+def test_host_plans_from_states(galv, S, K, top):
+    """The host entry point, whose table nobody sees: states of 16- and 32-bit differences, odd numbers of rows, +inf regions."""
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import HostSearch, SearchBuffers
+    for M, B in ((1100, 5), (95, 3)):
+        w = inputs.random_tables(17 + S, B, 20, S, M, ragged=True, mem_lo=0, mem_hi=max(1, M // 12), trans_hi=top, time_hi=4 * top)
+        if K:
+            rng = np.random.default_rng(S)
+            for i in range(B):
+                w.trans_q[i] = rng.integers(0, top + 1, (K, K), np.int32)[rng.integers(0, K, S)][:, rng.integers(0, K, S)]
+        w.mem_q[1, 3, : S // 2] = M + 3
+        w.mem_q[2, 0, :] = M // 2
+        w.time_q[0, ::2] = 5                                     # ties: the lowest strategy must win
+        ref = SearchBuffers(galv, w, gb.STORE_C_FULL | gb.KERNEL_REFERENCE)
+        ref.dp_search(); ref.backtrack()
+        want = ref.results()
+        hs = HostSearch(galv, w, gb.STORE_C_FULL)
+        for _ in range(2):
+            res = hs.run()
+            for k in ("status", "opt_cost", "plan", "mem_used"):
+                assert (res[k] == want[k]).all(), (k, M)
