@@ -82,6 +82,9 @@ extern "C" {
                                                    the cluster size of that kernel */
 #define GALV_KERNEL_RESIDENT 2097152 /* the resident kernel whenever the shape allows it (S <= 128), also where another one
                                         would be taken on its own; instances it has no room for go to the tiled kernels */
+#define GALV_KERNEL_SOLO 4194304 /* where no table is written (neither GALV_STORE_C_FULL nor GALV_STORE_ARGMIN; the host entry point, whose table
+                                    nobody sees): the solo kernel, an instance's state on one SM, whenever that fits; otherwise it
+                                    is taken on its own where instances are many or stacks long */
 #define GALV_DEBUG_WITHHOLD_LOAD 2048 /* test hook for the time-out path, on the tiled kernels: one CTA never receives its
                                      first stage; with GALV_KERNEL_RESIDENT, on that kernel: the first CTA of a cluster keeps
                                      the halo of layer 0 to itself.  Every bounded wait that depends on it runs out (about a
@@ -204,9 +207,11 @@ int galv_dp_search(galv_ctx* ctx, const galv_shape* shape, const int32_t* L,
 /*
  * Which kernel the most recent galv_dp_search on `workspace` ran: *packed = 1 for the tiled kernel
  * with the packed 16-bit inner loop (two relaxations per instruction; see GALV_KERNEL_NO_PACKED),
- * 0 for the tiled kernel with the 32-bit one, 2 for the cluster kernels (one thread-block cluster per instance: the
+ * 0 for the tiled kernel with the 32-bit one, 2 for the kernels that keep an instance on chip (one thread-block cluster per instance: the
  * resident one, the pushing one, or the first and what it left alone the second; see GALV_KERNEL_CLUSTER,
- * GALV_KERNEL_RESIDENT).  Where the tiled kernels took some of the batch, theirs.  With an argmin table always 0: the
+ * GALV_KERNEL_RESIDENT).  Where the tiled kernels took some of the batch, theirs.
+ * The solo kernel (GALV_KERNEL_SOLO) counts as 2; for unstructured matrices of more instances than SMs, which take several
+ * rounds, as 1 or 0: whether it relaxes them packed in 16 bits or in 32.  With an argmin table always 0: the
  * arithmetic is 32-bit in the tiled kernels and in the resident one, and this word does not say which of them ran.  Part
  * of the choice is made on the device; this call waits for `stream` and reads the answer back (host pointer).
  */

@@ -20,7 +20,7 @@ STORE_C_FULL, STORE_ARGMIN, KERNEL_REFERENCE, KERNEL_PER_LAYER, SKIP_INFEASIBLE 
 SKIP_DOMINATED = 8192
 DEBUG_WITHHOLD_LOAD = 2048
 KERNEL_NO_PACKED = 4096
-KERNEL_NO_CLUSTER, KERNEL_CLUSTER, KERNEL_RESIDENT = 16384, 32768, 1 << 21
+KERNEL_NO_CLUSTER, KERNEL_CLUSTER, KERNEL_RESIDENT, KERNEL_SOLO = 16384, 32768, 1 << 21, 1 << 22
 PATH_TILED_32, PATH_TILED_PACKED, PATH_CLUSTER = 0, 1, 2
 
 

@@ -1887,8 +1887,21 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         SoPlan sp;
         const bool resident_asked = (sh->flags & GALV_KERNEL_RESIDENT) != 0;
         const bool pushing_asked = !resident_asked && ((sh->flags & GALV_KERNEL_CLUSTER) != 0 || ((sh->flags >> 16) & 31) != 0);
-        solo = !resident_asked && !pushing_asked && galv_solo_plan(ctx, &kept, a.lean_map != nullptr, &sp);
         const bool pushing = !resident_asked && galv_cluster_plan(ctx, sh, &cp);
+        // A short stack is over before the resident or the solo kernel has looked at its matrix: up to 16 layers the pushing cluster
+        // kernel alone, where it can (3 instances of 6 layers, S = 7: 21 us against 33; 10 layers, S = 18: 47 against 55;
+        // 14 layers of an analytic model, S = 16: 62 against 73).  So do fewer than a thousand columns, a few warps' worth
+        // of work a layer (5 instances of 52 layers, S = 22, 126 columns: 136 against 185).
+        const bool solo_asked = (sh->flags & GALV_KERNEL_SOLO) != 0, brief = !solo_asked && pushing && (Lmax <= 16 || a.M < 1024);
+        // The solo kernel's start is longer than the resident one's, and of an SM an instance is a part of the chip where there are few:
+        // resident / solo us, optima of analytic models: 2 instances of 148 layers, 2880 columns 401 / 258; 9 of 116, 8192 columns 329 / 274;
+        // 31 of 89, 2880 columns 220 / 170; 198 of 6, 8192 columns 195 / 159; but 25 of 25, 8192 columns 136 / 174, 26 of 19, 2880 columns
+        // 97 / 110, and 3 of 54 measured layers, S = 21, 5727 columns 189 / 201.  Where it writes its states for the host entry
+        // point's walk one SM's store port is short as well: 128 of 160, 8192 columns 3525 / 2190, 197 of 14 463 / 401, but 41 of 73,
+        // 2880 columns 336 / 472, 19 of 135, 2406 columns 719 / 1704.
+        const bool many = B > ctx->num_sms || solo_asked;
+        const bool worth = a.lean_map ? (many || (B >= 96 && Lmax >= 32)) : many || (Lmax >= 32 && (B > 4 || a.M <= 5000));
+        solo = !resident_asked && !pushing_asked && !brief && worth && galv_solo_plan(ctx, &kept, a.lean_map != nullptr, &sp);
         a.wait_done = 0;
         int first = 0;
         if (solo) {
@@ -1902,11 +1915,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
             a.wait_done = sp.dense;
             first = 1;
         }
-        // A short stack is over before the resident kernel has looked at its matrix: up to 16 layers the pushing cluster
-        // kernel alone, where it can (3 instances of 6 layers, S = 7: 21 us against 33; 10 layers, S = 18: 47 against 55;
-        // 14 layers of an analytic model, S = 16: 62 against 73).  So do fewer than a thousand columns, a few warps' worth
-        // of work a layer (5 instances of 52 layers, S = 22, 126 columns: 136 against 185).
-        const bool pushing_alone = pushing_asked || (pushing && (solo || Lmax <= 16 || a.M < 1024));
+        const bool pushing_alone = pushing_asked || (pushing && (solo || brief));
         int n = pushing_alone ? 0 : galv_resident_plan(ctx, &kept, pushing ? &cp : nullptr, rp);
         if (n && solo && sp.classes && !rp[0].dense) { rp[0] = rp[1]; --n; }       // nothing with classes is left
         int launched = 0;
