@@ -93,7 +93,7 @@ __device__ __forceinline__ long long walk_table(int Li, int S, int m_pitch, cons
 // its time on top of its state row at the column its memory leaves, so rows are fetched two layers ahead.  (A walk of its own:
 // the choice inside one loop stood between a candidate's load and its transition entry's, a round trip each, and cost the
 // table's walk a fifth: 48 layers of S = 40 20.7 -> 28.9 us.)  s_trans: the transition matrix, or NULL.
-template <int NJ, bool STAGED>
+template <int NJ, bool STAGED, int FORM>
 __device__ __forceinline__ long long walk_states(int Li, int S, int m_pitch, const int32_t* __restrict__ tq, const int32_t* __restrict__ mq,
                                                  const int32_t* __restrict__ T0, long long trans_layer, const int32_t* __restrict__ C,
                                                  const int32_t* __restrict__ row_of, const int32_t* s_trans, int (&mrow)[NJ], int (&trow)[NJ],
@@ -101,8 +101,7 @@ __device__ __forceinline__ long long walk_states(int Li, int S, int m_pitch, con
 {
     const int lane = threadIdx.x;
     long long used = 0;
-    // The solo kernel's states are a row of bases and rows of differences' words, two rows to a word if 16 bits do.
-    const int form = row_of[0] & (kStateHalf | kStateWord);
+    // FORM: the solo kernel's states are a row of bases and rows of differences' words, two rows to a word if 16 bits do.
     int mnext[NJ], tnext[NJ];                                  // rows of layer l-1
     int crow[NJ], rows = 0;                                    // state row of each of this lane's strategies, rows a layer
     int half[NJ];                                              // ... where its bits begin in the row's words
@@ -110,8 +109,8 @@ __device__ __forceinline__ long long walk_states(int Li, int S, int m_pitch, con
     for (int j = 0; j < NJ; ++j) {
         const int k = lane + 32 * j;
         crow[j] = k < S ? row_of[k] & 0xffff : 0;
-        half[j] = form == kStateHalf ? 16 * (crow[j] & 1) : 0;
-        if (form) crow[j] = 1 + (form == kStateHalf ? crow[j] >> 1 : crow[j]);
+        half[j] = FORM == kStateHalf ? 16 * (crow[j] & 1) : 0;
+        if (FORM) crow[j] = 1 + (FORM == kStateHalf ? crow[j] >> 1 : crow[j]);
         rows = max(rows, crow[j] + 1);
         mnext[j] = k < S && Li > 1 ? mq[(Li - 2) * S + k] : 0;
         tnext[j] = k < S && Li > 1 ? tq[(Li - 2) * S + k] : 0;
@@ -140,19 +139,14 @@ __device__ __forceinline__ long long walk_states(int Li, int S, int m_pitch, con
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
             const int k = lane + 32 * j, src = m - mm - mnext[j];
-            int g = kInf;
-            if (k < S && src >= 0) {
-                g = 0;
-                if (l > 1) {
-                    const int word = prev[(size_t)crow[j] * m_pitch + src];
-                    g = word;
-                    if (form) {
-                        const int base = prev[src];
-                        g = (int)((uint32_t)word >> half[j]);
-                        if (form == kStateHalf) g &= 0xffff;
-                        g = base < kInf ? base + g : kInf;     // where nothing is finite the words are not there
-                    }
-                }
+            int g;
+            if (FORM == 0) {
+                g = k < S && src >= 0 ? (l > 1 ? prev[(size_t)crow[j] * m_pitch + src] : 0) : kInf;
+            } else {
+                const bool in = k < S && src >= 0;
+                const int base = in ? (l > 1 ? prev[src] : 0) : kInf;
+                const uint32_t word = in && l > 1 ? (uint32_t)prev[(size_t)crow[j] * m_pitch + src] : 0u;
+                g = base < kInf ? base + (int)(FORM == kStateHalf ? (word >> half[j]) & 0xffffu : word) : kInf;     // where nothing is finite the words are not there
             }
             cv[j] = g < kInf ? g + tnext[j] : kInf;
             tv[j] = k < S ? (STAGED ? s_trans[k * S + s] : T[k * S + s]) : 0;
@@ -254,10 +248,13 @@ __global__ void backtrack_kernel(int B, int Lmax, int S, int M, int m_pitch, lon
     const int32_t* Ci = SRC == kArgmin ? nullptr : C + (size_t)i * Lmax * slice;
     bool bad = false;
     long long used;
-    if (SRC == kStates && lean_map[(size_t)i * S] >= 0)
-        used = walk_states<NJ, STAGED>(Li, S, m_pitch, tq, mq, T0, trans_layer, Ci, lean_map + (size_t)i * S, s_trans, mrow, trow, s, bud, opt, pl, &bad);
+    const int form = SRC == kStates ? lean_map[(size_t)i * S] : -1;
+#define GALV_WALK_STATES(FORM) walk_states<NJ, STAGED, FORM>(Li, S, m_pitch, tq, mq, T0, trans_layer, Ci, lean_map + (size_t)i * S, s_trans, mrow, trow, s, bud, opt, pl, &bad)
+    if (SRC == kStates && form >= 0)
+        used = form & kStateHalf ? GALV_WALK_STATES(kStateHalf) : form & kStateWord ? GALV_WALK_STATES(kStateWord) : GALV_WALK_STATES(0);
     else
         used = walk_table<NJ, SRC == kArgmin>(Li, S, m_pitch, tq, mq, T0, trans_layer, Ci, SRC == kArgmin ? A + (size_t)i * Lmax * slice : nullptr, mrow, trow, s, bud, opt, pl, &bad);
+#undef GALV_WALK_STATES
     if (bad && lane == 0) status[i] = st0 | GALV_STATUS_BAD_INPUT;
     if (lane == 0 && mem_used) mem_used[i] = (int32_t)used;
 }
