@@ -115,3 +115,33 @@ def test_large_batch_takes_two_kernels_and_small_batch_one(orc, galv):
         st = sb.status.cpu().numpy()
         assert st[B - 3] == 2 and st[B // 2] == 2 and (st != 0).sum() == 2
         assert (sb.trans_q[B - 3].cpu().numpy() == -1).all() and (sb.trans_q[B // 2].cpu().numpy() == -1).all()
+
+
+@pytest.mark.parametrize("pattern,Lmax,S", [("uniform", 1, 8), ("alternate", 37, 48), ("distinct", 60, 48), (13, 40, 84), ("distinct", 5, 4)])
+def test_large_batch_of_one_stack(orc, galv, pattern, Lmax, S):
+    """Several instances a round: as many kinds as fit one, more than fit (60 of 48 strategies), one instance a round and eight,
+    lengths on both sides of a bad layer and out of range, bad instances, an odd number of instances left over."""
+    strat = inputs.strategy_table((1, 2, 4, 8, 16, 32, 64), (0, 2, 3), (0, 1), (0, 1))[:S]
+    B = 1037
+    w = stack(200 + Lmax, B, Lmax, strat, pattern, ragged=True)
+    w.inst["bw_tp"][[3, 500, B - 1]] = (-1.0, 0.0, float("inf"))
+    if Lmax > 9:
+        w.layers["h"][0, Lmax - 3] = float("nan")              # flags the instances that are that long
+    w.L[7], w.L[8], w.L[9] = 0, Lmax + 1, -5                   # nothing is written
+    import torch
+    from paper_2504_03662_b200.search import SearchBuffers
+    sb = SearchBuffers(galv, w, 0)
+    for t in (sb.time_q, sb.mem_q, sb.trans_q):
+        t.fill_(-7)
+    sb.eval_costs()
+    torch.cuda.synchronize()
+    tq, mq, xq, st = (t.cpu().numpy() for t in (sb.time_q, sb.mem_q, sb.trans_q, sb.status))
+    for i in list(range(0, 40)) + list(range(480, 520)) + list(range(B - 30, B)):
+        Li = int(w.L[i])
+        if not 1 <= Li <= Lmax:
+            assert st[i] == 2 and (tq[i] == -7).all() and (mq[i] == -7).all() and (xq[i] == -7).all(), i
+            continue
+        _, _, rtq, rmq, rxq = orc.eval_costs(w.layers[0], w.strat, w.inst[i], Li)
+        assert st[i] == orc.descriptor_status(w.layers[0], w.strat, w.inst[i], Li), i
+        assert (tq[i, :Li] == rtq).all() and (mq[i, :Li] == rmq).all() and (xq[i] == rxq).all(), i
+        assert (tq[i, Li:] == -7).all() and (mq[i, Li:] == -7).all(), i
