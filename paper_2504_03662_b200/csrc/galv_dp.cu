@@ -1906,7 +1906,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         int first = 0;
         if (solo) {
             // What this launch has no room for is known on the device only.
-            const bool probed = !sp.dense && !pushing;
+            const bool probed = !sp.dense && !pushing && galv_probe_applies(a);
             if (probed) galv_probe_matrices(a, st);
             // what the tiled kernels start from is cleared first: it lies around the word that says which kernel ran
             if (!sp.certain && !pushing && (e = clear()) != cudaSuccess) return e;

@@ -134,7 +134,8 @@ bool galv_solo_plan(const galv_ctx* ctx, const galv_shape* sh, bool states, SoPl
 cudaError_t galv_solo_configure(galv_ctx* ctx);
 // follow: the next kernel of the stream may start beside this one; probed: done[] = 2 where a matrix is unstructured
 cudaError_t galv_solo_launch(const SoPlan& plan, const struct DpArgs& a, int follow, int probed, cudaStream_t st);
-// done[i] = 2 where no two of the first rows of a matrix are equal, else 0
+// done[i] = 2 where no two of the first rows of a matrix are equal, else 0; for the strategies that galv_probe_applies to
+bool galv_probe_applies(const struct DpArgs& a);
 void galv_probe_matrices(const struct DpArgs& a, cudaStream_t st);
 
 // launches to make (0: the shape is left to the other kernels); the last one takes every instance when it is dense

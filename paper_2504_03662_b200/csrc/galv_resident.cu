@@ -1235,13 +1235,14 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
 }
 
 // Which matrices are worth the resident kernel's look: of kClassMax + 1 rows two are equal if there are at most kClassMax
-// classes.  done[i] = 2: no two of the first rows are.  A kernel of a few hundred instructions, as it is latency alone: the
+// classes.  done[i] = 2: no two of the first rows are.  Not for matrices of fewer rows: those always have few enough classes
+// (and the rows it reads are not there).  A kernel of a few hundred instructions, as it is latency alone: the
 // same look inside the resident kernel cost a batch it turns away 15 us, most of them spent on fetching its code.
 __global__ void __launch_bounds__(256) probe_kernel(int B, int S, const int32_t* __restrict__ trans_q, long long trans_inst, int32_t* __restrict__ done)
 {
-    constexpr int R = kClassMax + 1;
-    __shared__ int32_t rows[R * kMaxS];
+    __shared__ int32_t rows[(kClassMax + 1) * kMaxS];
     __shared__ int s_pair;
+    const int R = min(kClassMax + 1, S);                        // a matrix has S rows
     const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int32_t* const T = trans_q + (size_t)i * trans_inst;
     if (tid == 0) s_pair = 0;
@@ -1444,6 +1445,8 @@ cudaError_t galv_resident_configure(galv_ctx* ctx)
     return cudaSuccess;
 }
 
+bool galv_probe_applies(const DpArgs& d) { return d.S > kClassMax && d.S <= kMaxS; }
+
 void galv_probe_matrices(const DpArgs& d, cudaStream_t st) { probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.trans_q, d.trans_inst, d.done); }
 
 cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, cudaStream_t st)
@@ -1452,7 +1455,7 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
     a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second; a.withhold = d.withhold;
     a.follow = p.follow; a.k_max = p.k_max;
-    a.probed = !p.dense && d.S > kClassMax && !second && !p.follow;
+    a.probed = !p.dense && galv_probe_applies(d) && !second && !p.follow;
     if (a.probed) galv_probe_matrices(d, st);
     a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;

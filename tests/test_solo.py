@@ -123,3 +123,28 @@ def test_host_plans_from_states(galv, S, K, top):
             res = hs.run()
             for k in ("status", "opt_cost", "plan", "mem_used"):
                 assert (res[k] == want[k]).all(), (k, M)
+
+
+@pytest.mark.parametrize("S,M", [(11, 8191), (12, 8191), (13, 7400), (14, 7400), (15, 6500), (16, 6500), (16, 8191)])
+def test_what_lies_behind_the_matrices(galv, S, M):
+    """Too many columns for an unstructured state of 32-bit rows, fewer rows than a look at the first 17 would read: what follows
+    the last matrix is not looked at, and whatever it holds the results are the same."""
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    B = 160                                                      # more instances than SMs
+    w = inputs.random_tables(500 + S, B, 3, S, M, ragged=True, mem_lo=0, mem_hi=M // 3, trans_hi=900)
+    ref = SearchBuffers(galv, w, gb.STORE_C_FULL | gb.KERNEL_REFERENCE)
+    ref.dp_search(); ref.backtrack()
+    ref.C = None
+    for flags in (0, gb.KERNEL_SOLO):
+        for behind in ("rows of it", "others"):
+            one = SearchBuffers(galv, w, flags)
+            n = one.trans_q.numel()
+            room = torch.full((n + 17 * S,), 7, dtype=torch.int32, device=one.dev)
+            room[:n] = one.trans_q.flatten()
+            room[n:] = one.trans_q[-1, 0].repeat(17) if behind == "rows of it" else torch.arange(-17 * S, 0, dtype=torch.int32, device=one.dev)
+            one.trans_q = room[:n].view(B, S, S)
+            one.dp_search(); one.backtrack()
+            torch.cuda.synchronize()
+            assert torch.equal(one.status, ref.status) and torch.equal(one.opt_cost, ref.opt_cost) and torch.equal(one.C_last, ref.C_last), (flags, behind)
