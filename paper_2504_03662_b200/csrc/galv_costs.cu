@@ -353,13 +353,14 @@ __global__ void __launch_bounds__(kThreads) cost_kernel(int Lmax, int S, int KC,
 // 160 layers, 64 strategies: 229 us in two kernels, 175 here (0.8 GB written: 4.6 TB/s).  Other large batches (a stack each, doubles
 // asked for, strategies not a multiple of four) take the two kernels.
 constexpr int kBulkRoom = 2048;    // (layer kind, strategy) pairs a round
+struct BulkShared { int ndist, ncls, sbad, lbad, ok[8], len[8]; };
 __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax, int S, const int32_t* __restrict__ L, const galv_layer_desc* __restrict__ layers,
                                                                 const galv_strategy_desc* __restrict__ strat, const galv_inst_params* __restrict__ inst,
                                                                 int32_t* __restrict__ time_q, int32_t* __restrict__ mem_q, int32_t* __restrict__ trans_q,
                                                                 int32_t* __restrict__ status)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_ndist, s_ncls, s_sbad, s_lbad, s_ok[8], s_len[8];
+    __shared__ BulkShared sh;
     const int tid = threadIdx.x;
     int32_t* const tabq = reinterpret_cast<int32_t*>(smem_raw);
     int32_t* const tabm = tabq + kBulkRoom;
@@ -369,10 +370,10 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
     int* const list = slot + Lmax;
     int* const cls = list + Lmax;                              // transition class of each strategy
     int* const rep = cls + S;
-    if (tid == 0) { s_ndist = 0; s_ncls = 0; s_sbad = 0; s_lbad = Lmax; }
+    if (tid == 0) { sh.ndist = 0; sh.ncls = 0; sh.sbad = 0; sh.lbad = Lmax; }
     __syncthreads();
     for (int l = tid; l < Lmax; l += kThreads) {
-        if (!layer_ok(layers[l])) atomicMin(&s_lbad, l);       // flags the instances that have this layer
+        if (!layer_ok(layers[l])) atomicMin(&sh.lbad, l);       // flags the instances that have this layer
         int parent = l;
         for (int d = 1; d <= kWindow && d <= l; ++d)
             if (same_bytes(layers + l, layers + l - d)) { parent = l - d; break; }
@@ -380,19 +381,19 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
     }
     for (int s = tid; s < S; s += kThreads) {
         const galv_strategy_desc me = strat[s];
-        if (!strat_ok(me)) atomicOr(&s_sbad, 1);
+        if (!strat_ok(me)) atomicOr(&sh.sbad, 1);
         int first = s;
         for (int o = 0; o < s; ++o) {
             const galv_strategy_desc ot = strat[o];
             if (ot.tp == me.tp && ot.sp == me.sp && __double_as_longlong(ot.batch_div) == __double_as_longlong(me.batch_div)) { first = o; break; }
         }
         cls[s] = -first - 1;
-        if (first == s) rep[atomicAdd(&s_ncls, 1)] = s;
+        if (first == s) rep[atomicAdd(&sh.ncls, 1)] = s;
     }
     __syncthreads();
     for (int l = tid; l < Lmax; l += kThreads)
-        if (root[l] == l) { const int p = atomicAdd(&s_ndist, 1); list[p] = l; slot[l] = p; }
-    for (int k = tid; k < s_ncls; k += kThreads) cls[rep[k]] = k;
+        if (root[l] == l) { const int p = atomicAdd(&sh.ndist, 1); list[p] = l; slot[l] = p; }
+    for (int k = tid; k < sh.ncls; k += kThreads) cls[rep[k]] = k;
     for (int span = 1; span < Lmax; span <<= 1) {
         __syncthreads();
         volatile int* const vr = root;
@@ -403,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
         if (cls[s] < 0) cls[s] = cls[-cls[s] - 1];
     for (int l = tid; l < Lmax; l += kThreads) root[l] = slot[root[l]];
     __syncthreads();
-    const int ndist = s_ndist, nn = s_ncls * s_ncls, kc = min(ndist, kBulkRoom / S);
+    const int ndist = sh.ndist, nn = sh.ncls * sh.ncls, kc = min(ndist, kBulkRoom / S);
     // instances a round: as many as the threads evaluate at once and the tables hold
     const int g = max(1, min(min(8, kThreads / (kc * S)), S * S / nn));
     const int S4 = S >> 2, rows = kThreads / S4, c = tid % S4, r0 = tid / S4;
@@ -411,9 +412,9 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
         const int m = min(g, B - i0);
         if (tid < m) {
             const int Li = L[i0 + tid], in_range = Li >= 1 && Li <= Lmax;
-            const int ok = in_range && !s_sbad && s_lbad >= Li && inst_ok(inst[i0 + tid]);
-            s_len[tid] = in_range ? Li : 0;                    // out of range: nothing is written
-            s_ok[tid] = ok;
+            const int ok = in_range && !sh.sbad && sh.lbad >= Li && inst_ok(inst[i0 + tid]);
+            sh.len[tid] = in_range ? Li : 0;                    // out of range: nothing is written
+            sh.ok[tid] = ok;
             status[i0 + tid] = ok ? 0 : GALV_STATUS_BAD_INPUT;
         }
         __syncthreads();
@@ -421,7 +422,7 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
             const int kn = min(kc, ndist - k0), per = kn * S;
             for (int e = tid; e < m * per; e += kThreads) {
                 const int n = e / per, r = e - n * per, k = r / S, s = r - k * S;
-                if (!s_ok[n]) continue;
+                if (!sh.ok[n]) continue;
                 const galv_inst_params in = inst[i0 + n];
                 double t, b;
                 cost_of(layers[list[k0 + k]], strat[s], in, &t, &b);
@@ -430,8 +431,8 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
             }
             if (k0 == 0)
                 for (int e = tid; e < m * nn; e += kThreads) {
-                    const int n = e / nn, r = e - n * nn, ka = r / s_ncls, kb = r - ka * s_ncls;
-                    if (!s_ok[n]) continue;
+                    const int n = e / nn, r = e - n * nn, ka = r / sh.ncls, kb = r - ka * sh.ncls;
+                    if (!sh.ok[n]) continue;
                     const galv_inst_params in = inst[i0 + n];
                     const galv_strategy_desc sa = strat[rep[ka]], sc = strat[rep[kb]];
                     const double bq = in.b / sc.batch_div;
@@ -442,8 +443,8 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
             __syncthreads();
             for (int n = 0; n < m; ++n) {
                 const size_t base = (size_t)(i0 + n) * Lmax * S;
-                const bool ok = s_ok[n] != 0;
-                const int Li = s_len[n];
+                const bool ok = sh.ok[n] != 0;
+                const int Li = sh.len[n];
                 if (r0 < rows)
                     for (int l = r0; l < Li; l += rows) {
                         const int k = root[l] - k0;
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
                         for (int a = r0; a < S; a += rows) {
                             int4 v = make_int4(-1, -1, -1, -1);
                             if (ok) {
-                                const int32_t* row = pairs + n * nn + cls[a] * s_ncls;
+                                const int32_t* row = pairs + n * nn + cls[a] * sh.ncls;
                                 v = make_int4(row[k4[0]], row[k4[1]], row[k4[2]], row[k4[3]]);
                             }
                             reinterpret_cast<int4*>(out + (size_t)a * S)[c] = v;
@@ -594,7 +595,7 @@ cudaError_t galv_costs_launch(const galv_shape* sh, const int32_t* L, const galv
         smem = fixed + (size_t)kc * per_kind + 16;
     }
     const size_t bulk = ((size_t)2 * kBulkRoom + (size_t)S * S + 3 * (size_t)Lmax + 2 * (size_t)S) * 4;
-    if (sh->B > 1024 && layer_stride_B == 0 && !want_d && S % 4 == 0 && bulk <= 48 * 1024) {      // four CTAs an SM
+    if (sh->B > 1024 && layer_stride_B == 0 && !want_d && S % 4 == 0 && bulk + sizeof(BulkShared) <= 48 * 1024) {      // four CTAs an SM, and no opt-in beyond 48 KB
         int dev = 0, sms = 148;
         if (cudaGetDevice(&dev) == cudaSuccess) (void)cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cost_bulk_kernel<<<4 * sms, kThreads, bulk, st>>>(sh->B, Lmax, S, L, layers, strat, inst, time_q, mem_q, trans_q, status);

@@ -117,10 +117,12 @@ def test_large_batch_takes_two_kernels_and_small_batch_one(orc, galv):
         assert (sb.trans_q[B - 3].cpu().numpy() == -1).all() and (sb.trans_q[B // 2].cpu().numpy() == -1).all()
 
 
-@pytest.mark.parametrize("pattern,Lmax,S", [("uniform", 1, 8), ("alternate", 37, 48), ("distinct", 60, 48), (13, 40, 84), ("distinct", 5, 4)])
+@pytest.mark.parametrize("pattern,Lmax,S", [("uniform", 1, 8), ("alternate", 37, 48), ("distinct", 60, 48), (13, 40, 84), ("distinct", 5, 4),
+                                            ("alternate", 316, 84), ("alternate", 319, 84), ("alternate", 322, 84), (13, 323, 84)])
 def test_large_batch_of_one_stack(orc, galv, pattern, Lmax, S):
     """Several instances a round: as many kinds as fit one, more than fit (60 of 48 strategies), one instance a round and eight,
-    lengths on both sides of a bad layer and out of range, bad instances, an odd number of instances left over."""
+    lengths on both sides of a bad layer and out of range, bad instances, an odd number of instances left over; stacks around the
+    length at which the kernel's shared memory, its static part with it, no longer fits 48 KB."""
     strat = inputs.strategy_table((1, 2, 4, 8, 16, 32, 64), (0, 2, 3), (0, 1), (0, 1))[:S]
     B = 1037
     w = stack(200 + Lmax, B, Lmax, strat, pattern, ragged=True)
