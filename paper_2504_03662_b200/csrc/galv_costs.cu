@@ -550,6 +550,9 @@ __global__ void cost_direct_kernel(int B, int Lmax, int S, const int32_t* __rest
 
 }  // namespace
 
+// Dynamic shared memory a kernel may have without opting in: 48 KB less its static part (at most 48 bytes in these).
+constexpr size_t kPlainSmem = 48 * 1024 - 64;
+
 cudaError_t galv_costs_launch(const galv_shape* sh, const int32_t* L, const galv_layer_desc* layers,
                               int64_t layer_stride_B, const galv_strategy_desc* strat,
                               const galv_inst_params* inst, double* time_s, double* mem_bytes,
@@ -576,7 +579,7 @@ cudaError_t galv_costs_launch(const galv_shape* sh, const int32_t* L, const galv
         if (blocks > 148 * 16) blocks = 148 * 16;
         cost_direct_kernel<<<(int)blocks, 256, 0, st>>>(sh->B, Lmax, S, L, layers, (long long)layer_stride_B, strat, inst, status, time_s, mem_bytes,
                                                         time_q, mem_q);
-        if (tsmem > 48 * 1024) {                                   // long stacks or many strategies only; per device, so asked every time
+        if (tsmem > kPlainSmem) {                                   // long stacks or many strategies only; per device, so asked every time
             cudaError_t e = cudaFuncSetAttribute(trans_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem);
             if (e != cudaSuccess) return e;
         }
@@ -602,13 +605,13 @@ cudaError_t galv_costs_launch(const galv_shape* sh, const int32_t* L, const galv
         return cudaGetLastError();
     }
     if (sh->B > 1024) {
-        if (smem > 48 * 1024) {                                   // long stacks or many strategies only; per device, so asked every time
+        if (smem > kPlainSmem) {                                   // long stacks or many strategies only; per device, so asked every time
             cudaError_t e = cudaFuncSetAttribute(cost_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
         cost_kernel<<<sh->B, kThreads, smem, st>>>(Lmax, S, kc, L, layers, (long long)layer_stride_B, strat, inst, time_s, mem_bytes, time_q,
                                                    mem_q, trans_q, status);
-        if (tsmem > 48 * 1024) {                                   // long stacks or many strategies only; per device, so asked every time
+        if (tsmem > kPlainSmem) {                                   // long stacks or many strategies only; per device, so asked every time
             cudaError_t e = cudaFuncSetAttribute(trans_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsmem);
             if (e != cudaSuccess) return e;
         }
@@ -616,7 +619,7 @@ cudaError_t galv_costs_launch(const galv_shape* sh, const int32_t* L, const galv
         return cudaGetLastError();
     }
     if (tsmem > smem) smem = tsmem;                                   // one launch, two roles: the larger of their needs
-    if (smem > 48 * 1024) {                                   // long stacks or many strategies only; per device, so asked every time
+    if (smem > kPlainSmem) {                                   // long stacks or many strategies only; per device, so asked every time
         cudaError_t e = cudaFuncSetAttribute(cost_trans_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }

@@ -117,6 +117,23 @@ def test_large_batch_takes_two_kernels_and_small_batch_one(orc, galv):
         assert (sb.trans_q[B - 3].cpu().numpy() == -1).all() and (sb.trans_q[B // 2].cpu().numpy() == -1).all()
 
 
+@pytest.mark.parametrize("B", [2, 1025])
+@pytest.mark.parametrize("Lmax", [4084, 4085, 4087, 4088, 4089])
+def test_stacks_around_48_kb_of_index_arrays(orc, galv, B, Lmax):
+    """12 bytes a layer: the lengths at which the kernels need the larger shared memory, counted with their static part."""
+    strat = inputs.strategy_table((1, 2, 4, 8), (0, 3), (0,), (0,))[:8]
+    w = stack(7, B, Lmax, strat, "alternate")
+    w.inst["time_unit_ns"] = 1e6
+    w.L[1:] = 3
+    from paper_2504_03662_b200.search import SearchBuffers
+    sb = SearchBuffers(galv, w, 0)
+    sb.eval_costs()
+    for i in (0, 1, B - 1):
+        Li = int(w.L[i])
+        _, _, tq, mq, xq = orc.eval_costs(w.layers[0], w.strat, w.inst[i], Li)
+        assert (sb.time_q[i, :Li].cpu().numpy() == tq).all() and (sb.mem_q[i, :Li].cpu().numpy() == mq).all() and (sb.trans_q[i].cpu().numpy() == xq).all()
+
+
 @pytest.mark.parametrize("pattern,Lmax,S", [("uniform", 1, 8), ("alternate", 37, 48), ("distinct", 60, 48), (13, 40, 84), ("distinct", 5, 4),
                                             ("alternate", 316, 84), ("alternate", 319, 84), ("alternate", 322, 84), (13, 323, 84)])
 def test_large_batch_of_one_stack(orc, galv, pattern, Lmax, S):
