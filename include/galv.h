@@ -84,7 +84,8 @@ extern "C" {
                                         would be taken on its own; instances it has no room for go to the tiled kernels */
 #define GALV_KERNEL_SOLO 4194304 /* where no table is written (neither GALV_STORE_C_FULL nor GALV_STORE_ARGMIN; the host entry point, whose table
                                     nobody sees): the solo kernel, an instance's state on one SM, whenever that fits; otherwise it
-                                    is taken on its own where instances are many or stacks long */
+                                    is taken on its own where the estimates for the shape and a look at some instances' tables say that
+                                    the batch costs less there */
 #define GALV_DEBUG_WITHHOLD_LOAD 2048 /* test hook for the time-out path, on the tiled kernels: one CTA never receives its
                                      first stage; with GALV_KERNEL_RESIDENT, on that kernel: the first CTA of a cluster keeps
                                      the halo of layer 0 to itself.  Every bounded wait that depends on it runs out (about a

@@ -57,7 +57,8 @@ struct ClArgs {
     int32_t* status;
     int32_t* path;     // [4] device flags of the search: error, -, -, kernel that ran
     const int32_t* done;   // [B] instances that need nothing more, or NULL: written by the kernel before this one, which may still be running
-    int wait_done;         // ... and may take any instance: it is waited for first
+    int after_solo;        // done[] = 3: by a kernel that had ended before the one in front was launched
+    int beside;            // launched so as to start beside the kernel in front
 };
 
 // 3-D view of a table for the tensor-map store: [rows of S strategies per (instance, layer)][m_pitch / 32][32].
@@ -185,6 +186,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
     constexpr int kProbeRows = kResidentClassMax + 1;
     auto resident_over = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
     // ---- validation (every CTA of the cluster comes to the same result: nobody is left waiting at a barrier)
+    if (a.after_solo && a.done[i] == 3) { resident_over(); return; }      // (nobody writes this value any more)
     if (tid == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; }
     __syncthreads();
     const int Li = a.L[i];
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
             const int v = x[k];
             bad |= (v < 0);
             tmax = max(tmax, v);
-            if (a.done && k < kProbeRows * S) buf0[k] = v;       // (one matrix per instance where there is a resident kernel in front)
+            if (a.done && k < kProbeRows * S) buf0[k] = v;       // (with a matrix per layer there is no resident kernel in front, and nothing to wait for)
         }
         tmax = __reduce_max_sync(0xffffffffu, tmax);
         bad = __any_sync(0xffffffffu, bad != 0);
@@ -228,7 +230,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
     }
     __syncthreads();
     if (a.done) {
-        bool equal = S < kProbeRows || a.wait_done;
+        bool equal = S < kProbeRows;
         for (int x = warp; x < kProbeRows * kProbeRows && !equal; x += NW + 1) {
             const int p = x / kProbeRows, q = x - p * kProbeRows;
             if (p >= q) continue;
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
         }
         if (__syncthreads_or(equal)) {
             resident_over();
-            if (*(volatile const int32_t*)(a.done + i) == 1) return;
+            if (*(volatile const int32_t*)(a.done + i) & 1) return;
         }
     }
     {
@@ -485,7 +487,7 @@ cudaError_t launch_cluster(const ClArgs& a, const ClPlan& p, const CUtensorMap& 
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;        // behind the resident kernel: may start beside it
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = a.done ? 2 : 1;
+    cfg.numAttrs = a.done && a.beside ? 2 : 1;
     if (max_clusters) return cudaOccupancyMaxActiveClusters(max_clusters, cluster_search_kernel<TM>, &cfg);
     return cudaLaunchKernelEx(&cfg, cluster_search_kernel<TM>, a, mc, ml);
 }
@@ -621,7 +623,7 @@ cudaError_t galv_cluster_launch(galv_ctx* ctx, const galv_shape* sh, const ClPla
     a.CL = p.cl; a.W = p.w; a.G = p.g; a.NSG = p.nsg; a.SP8 = p.sp8; a.nct = p.nct; a.units = p.units; a.sorted = p.sorted;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
-    a.C = d.C; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done; a.wait_done = d.wait_done;
+    a.C = d.C; a.C_last = d.C_last; a.status = d.status; a.path = d.err; a.done = d.done; a.after_solo = d.done && d.after_solo; a.beside = d.beside;
     (void)sh;
     CUtensorMap mc, ml;
     std::memset(&mc, 0, sizeof(mc));

@@ -153,7 +153,7 @@ __global__ void validate_kernel(int B, int Lmax, int S, int M, long long tl, con
                                 long long* __restrict__ dominated)
 {
     const int i = blockIdx.x;
-    if (done && done[i] == 1) return;                              // searched, or flagged, by the cluster kernel
+    if (done && (done[i] & 1)) return;                             // searched, or flagged, by the kernels in front
     __shared__ long long s_sum;
     __shared__ int s_tmax, s_bad, s_mmax, s_dom;
     if (threadIdx.x == 0) { s_sum = 0; s_tmax = 0; s_bad = 0; s_mmax = 0; s_dom = 0; }
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
     int32_t* hist = scratch;
     int32_t* fill = scratch + Lmax + 2;
     for (int i = threadIdx.x; i < B; i += blockDim.x)
-        if (status[i] == 0 && !(done && done[i] == 1)) atomicAdd(&hist[L[i]], 1);
+        if (status[i] == 0 && !(done && (done[i] & 1))) atomicAdd(&hist[L[i]], 1);
     for (int l = threadIdx.x; l <= Lmax; l += blockDim.x) {
         int nt = 1;
         if (l < Lmax && minmem_l[l] <= M) nt = min(ntiles_m, (M - minmem_l[l]) / tmb + 1);
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(1024) schedule_kernel(int B, int Lmax, int M, 
     }
     __syncthreads();
     for (int i = threadIdx.x; i < B; i += blockDim.x)
-        if (status[i] == 0 && !(done && done[i] == 1)) {
+        if (status[i] == 0 && !(done && (done[i] & 1))) {
             const int Li = L[i];
             order[nactive[Li] + atomicAdd(&fill[Li], 1)] = i;   // instances longer than Li come first
         }
@@ -1893,31 +1893,21 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         // 14 layers of an analytic model, S = 16: 62 against 73).  So do fewer than a thousand columns, a few warps' worth
         // of work a layer (5 instances of 52 layers, S = 22, 126 columns: 136 against 185).
         const bool solo_asked = (sh->flags & GALV_KERNEL_SOLO) != 0, brief = !solo_asked && pushing && (Lmax <= 16 || a.M < 1024);
-        // The solo kernel's start is longer than the resident one's, and of an SM an instance is a part of the chip where there are few:
-        // resident / solo us, optima of analytic models: 2 instances of 148 layers, 2880 columns 401 / 258; 9 of 116, 8192 columns 329 / 274;
-        // 31 of 89, 2880 columns 220 / 170; 198 of 6, 8192 columns 195 / 159; but 25 of 25, 8192 columns 136 / 174, 26 of 19, 2880 columns
-        // 97 / 110, and 3 of 54 measured layers, S = 21, 5727 columns 189 / 201.  Where it writes its states for the host entry
-        // point's walk one SM's store port is short as well: 128 of 160, 8192 columns 3525 / 2190, 197 of 14 463 / 401, but 41 of 73,
-        // 2880 columns 336 / 472, 19 of 135, 2406 columns 719 / 1704.
-        const bool many = B > ctx->num_sms || solo_asked;
-        const bool worth = a.lean_map ? (many || (B >= 96 && Lmax >= 32)) : many || (Lmax >= 32 && (B > 4 || a.M <= 5000));
-        solo = !resident_asked && !pushing_asked && !brief && worth && galv_solo_plan(ctx, &kept, a.lean_map != nullptr, &sp);
-        a.wait_done = 0;
+        const bool pushing_alone = pushing_asked || brief;
+        const int n = pushing_alone ? 0 : galv_resident_plan(ctx, &kept, pushing ? &cp : nullptr, rp);
+        // The solo kernel goes first where the batch may be worth it; whether it is, and what there is no room for, is known on the
+        // device only, and the others stand behind it.
+        solo = !resident_asked && !pushing_alone && galv_solo_plan(ctx, &kept, a.lean_map != nullptr, &sp) &&
+               (solo_asked || galv_solo_worth(ctx, &kept, a.lean_map != nullptr, n, rp, pushing ? &cp : nullptr, &sp));
+        a.after_solo = solo;
         int first = 0;
         if (solo) {
-            // What this launch has no room for is known on the device only.
-            const bool probed = !sp.dense && !pushing && galv_probe_applies(a);
-            if (probed) galv_probe_matrices(a, st);
             // what the tiled kernels start from is cleared first: it lies around the word that says which kernel ran
-            if (!sp.certain && !pushing && (e = clear()) != cudaSuccess) return e;
-            if ((e = galv_solo_launch(sp, a, pushing, probed, st)) != cudaSuccess) return e;
+            if (!sp.certain && (e = clear()) != cudaSuccess) return e;
+            if ((e = galv_solo_launch(sp, a, st)) != cudaSuccess) return e;
             if (sp.certain) return finished();
-            a.wait_done = sp.dense;
             first = 1;
         }
-        const bool pushing_alone = pushing_asked || (pushing && (solo || brief));
-        int n = pushing_alone ? 0 : galv_resident_plan(ctx, &kept, pushing ? &cp : nullptr, rp);
-        if (n && solo && sp.classes && !rp[0].dense) { rp[0] = rp[1]; --n; }       // nothing with classes is left
         int launched = 0;
         while (launched < n) {
             if (galv_resident_launch(rp[launched], first + launched, a, st) != cudaSuccess) { (void)cudaGetLastError(); break; }   // cannot be placed on this device right now
@@ -1925,6 +1915,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
         }
         if (launched && launched == n && rp[n - 1].dense) return finished();
         if (!launched && !first) a.done = nullptr;
+        a.beside = launched > 0;
         if (pushing) {
             if (galv_cluster_launch(ctx, sh, cp, a, st) == cudaSuccess) return finished();
             (void)cudaGetLastError();                        // the clusters cannot be placed on this device right now: tiled kernels

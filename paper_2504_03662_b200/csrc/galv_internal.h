@@ -25,6 +25,18 @@ struct RsPlan {
     int stage_at;  // word offset of the collected rows
     int follow;    // the pushing cluster kernel stands behind this launch: what it does better is left to it
     int k_max;     // ... instances of more classes
+    double est;    // estimated SM cycles per layer, all rounds of clusters
+};
+
+// What a layer of a batch costs in the other kernels, in SM cycles for each round of instances on the solo kernel.
+struct SoOther {
+    float resident;       // matrices of few classes, by the resident kernel's plan
+    int gints, w;         // ... its room and columns (w = 0: it does not take them)
+    float past_halo;      // ... for each strategy, where shifts pass the halo
+    float tiled;          // the tiled kernels, for a cycle of a column group
+    int packed;           // ... their packed loop is possible
+    float most;           // the pushing kernel, or the resident one for any matrix
+    float start;          // of the solo kernel's own start, for a layer
 };
 
 // How the solo kernel (an instance's state on one SM) cuts a batch.
@@ -35,10 +47,11 @@ struct SoPlan {
     int room;      // ... of which for the state
     int sorted;    // CTA c takes the c-th longest instance
     int dense;     // unstructured matrices fit, with transition entries up to 65535 at least
-    int certain;   // every instance can run
-    int classes;   // every matrix of up to 9 classes of equal columns can
+    int certain;   // every instance can run, and is worth it
     int rounds;    // more instances than SMs
     int packed;    // packed relaxations are allowed
+    int guessed;   // instances that are looked at to see whether the batch is worth it; 0: it is
+    SoOther other;
 };
 
 struct galv_ctx {
@@ -88,7 +101,7 @@ struct DpArgs {
     uint8_t* A;          // argmin table or NULL
     int32_t* C_last;
     int32_t* roll;       // [2][B][S][m_pitch] when C == NULL
-    int32_t* order;      // [B]   valid instances, longest first
+    int32_t* order;      // [B]   valid instances, longest first; before that, what the solo kernel would cost some of them
     int32_t* nactive;    // [Lmax+1] instances with L > l
     int32_t* scratch;    // [2*(Lmax+2)] histogram / fill counters, then the work counters below (zeroed together)
     unsigned long long* work;  // [Lmax+2] next item to hand out: [0] when all layers are one launch, else [l]
@@ -111,10 +124,12 @@ struct DpArgs {
     int32_t* lean_map;   // host entry point (nobody sees the table): [B][S] state row of each strategy where the resident kernel has left
                          // the states between the layers in C in place of its values (with kStateHalf or kStateWord added: the solo
                          // kernel); -1 where C holds the values.  Else NULL
-    int32_t* done;       // [B] 1: searched or flagged already, 2: an unstructured matrix, not searched; or NULL when the resident kernel was not launched.
+    int32_t* done;       // [B] 1: searched or flagged already, 3: by a kernel that has ended, 2: an unstructured matrix, not searched; or NULL when
+                         // neither the resident nor the solo kernel was launched.
                          // Lies over tile_done: read until the schedule is made
     int withhold;        // test hook: CTA 0 never loads its first chunk, so that the bounded waits run out
-    int wait_done;       // done[] is to be waited for before anything is searched: the launch before this one may take any instance
+    int after_solo;      // the solo kernel has run: done[] = 3 are its own
+    int beside;          // the pushing kernel may start beside the kernel in front, the resident one
     int skip_dom;        // leave out rows (packed path: row pairs) that cannot win in any column of a warp group's tile
     int dom_auto;        // ... where a quarter of the rows or more look it (maxmem[4])
 };
@@ -132,9 +147,10 @@ cudaError_t galv_encode_table_3d(CUtensorMap* map, void* base, size_t rows, int 
 // whether it can take the shape, which has no table to write; states: they are kept in its place
 bool galv_solo_plan(const galv_ctx* ctx, const galv_shape* sh, bool states, SoPlan* plan);
 cudaError_t galv_solo_configure(galv_ctx* ctx);
-// follow: the next kernel of the stream may start beside this one; probed: done[] = 2 where a matrix is unstructured
-cudaError_t galv_solo_launch(const SoPlan& plan, const struct DpArgs& a, int follow, int probed, cudaStream_t st);
-// done[i] = 2 where no two of the first rows of a matrix are equal, else 0; for the strategies that galv_probe_applies to
+// whether a batch of some matrices can be worth it, given what the others' plans cost; n: of the resident kernel's launches; pushing: NULL when it cannot run the shape
+bool galv_solo_worth(const galv_ctx* ctx, const galv_shape* sh, bool states, int n, const RsPlan resident[2], const struct ClPlan* pushing, SoPlan* plan);
+cudaError_t galv_solo_launch(const SoPlan& plan, const struct DpArgs& a, cudaStream_t st);
+// done[i] = 2 where no two of the first rows of a matrix are equal, else 0, but for those the solo kernel has finished; for the strategies that galv_probe_applies to
 bool galv_probe_applies(const struct DpArgs& a);
 void galv_probe_matrices(const struct DpArgs& a, cudaStream_t st);
 

@@ -811,7 +811,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     }
     // finished before, or (no room here for an unstructured matrix) found to be one by the probe: nobody in the cluster
     // writes the word before all have read it
-    if ((a.second && a.done[i] == 1) || (a.probed && a.done[i] == 2)) return;
+    if ((a.second && (a.done[i] & 1)) || (a.probed && a.done[i] == 2)) return;
     const int Li = a.L[i];
     if (Li < 1 || Li > Lmax) {
         if (rank == 0 && tid == 0) { a.status[i] = GALV_STATUS_BAD_INPUT; a.done[i] = 1; }
@@ -1238,12 +1238,13 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
 // classes.  done[i] = 2: no two of the first rows are.  Not for matrices of fewer rows: those always have few enough classes
 // (and the rows it reads are not there).  A kernel of a few hundred instructions, as it is latency alone: the
 // same look inside the resident kernel cost a batch it turns away 15 us, most of them spent on fetching its code.
-__global__ void __launch_bounds__(256) probe_kernel(int B, int S, const int32_t* __restrict__ trans_q, long long trans_inst, int32_t* __restrict__ done)
+__global__ void __launch_bounds__(256) probe_kernel(int B, int S, int after_solo, const int32_t* __restrict__ trans_q, long long trans_inst, int32_t* __restrict__ done)
 {
     __shared__ int32_t rows[(kClassMax + 1) * kMaxS];
     __shared__ int s_pair;
     const int R = min(kClassMax + 1, S);                        // a matrix has S rows
     const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    if (after_solo && done[i] == 3) return;
     const int32_t* const T = trans_q + (size_t)i * trans_inst;
     if (tid == 0) s_pair = 0;
     for (int k = tid; k < R * S; k += 256) rows[k] = T[k];
@@ -1418,6 +1419,7 @@ int galv_resident_plan(galv_ctx* ctx, const galv_shape* sh, const ClPlan* pushin
         const int g = plans[1].w / 32, width = (g + plans[1].nw - 1) / plans[1].nw;
         d = sh->S > kClassMax && 1600.0 + 260.0 * sh->S * width <= 0.9 * pushing->est;
     }
+    plans[0].est = tc; plans[1].est = td;
     // a launch that takes every instance spares the ones after it, which find nothing to do (20 us, 40 thousand cycles)
     if (d && (!c || forced || td * sh->Lmax <= tc * sh->Lmax * 1.05 + 40000.0)) { plans[0] = plans[1]; n = 1; }
     else if (c) n = d ? 2 : 1;
@@ -1447,7 +1449,7 @@ cudaError_t galv_resident_configure(galv_ctx* ctx)
 
 bool galv_probe_applies(const DpArgs& d) { return d.S > kClassMax && d.S <= kMaxS; }
 
-void galv_probe_matrices(const DpArgs& d, cudaStream_t st) { probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.trans_q, d.trans_inst, d.done); }
+void galv_probe_matrices(const DpArgs& d, cudaStream_t st) { probe_kernel<<<d.B, 256, 0, st>>>(d.B, d.S, d.after_solo, d.trans_q, d.trans_inst, d.done); }
 
 cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, cudaStream_t st)
 {
@@ -1455,7 +1457,7 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
     a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second; a.withhold = d.withhold;
     a.follow = p.follow; a.k_max = p.k_max;
-    a.probed = !p.dense && galv_probe_applies(d) && !second && !p.follow;
+    a.probed = !p.dense && galv_probe_applies(d) && second == d.after_solo && !p.follow;       // the first launch of this kernel
     if (a.probed) galv_probe_matrices(d, st);
     a.SP = p.dense ? (d.S + 3) & ~3 : 0;                       // rows are read as int4, 32 entries at a time: what lies beyond a row is never kept
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;

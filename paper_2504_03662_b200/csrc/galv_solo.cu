@@ -21,6 +21,11 @@
 // Taken where no table is written: optima, and the states that the host entry point's walk wants.  128 instances of 160 layers, 64
 // strategies, 8192 columns, optima: 2976 us in the resident kernel, 1165 here; host entry point 3525 / 2069.  A step of tiles takes 2300
 // cycles, latencies of its test, its walk and its writes in turn; one with the edge of the feasible region in it 5000.
+//
+// How many strategies pass depends on the tables: with times that lie close together, or transitions as large as the times, most of
+// them do, and the kernels that relax every row of a register tile are several times as fast (40 instances of 40 layers, S = 64 of 4
+// classes, 4000 columns, transitions up to a tenth / half / twice the median time: 480 / 975 / 1387 us here, 400 in the resident
+// kernel).  So a batch is searched here only where a guess of that number (guess_kernel) says that it costs less.
 
 #include <cstring>
 #include <type_traits>
@@ -46,9 +51,10 @@ struct SoArgs {
     int mats;          // words of the transition matrices in shared memory
     int sorted;        // CTA c takes the c-th longest instance
     int dense;         // unstructured matrices are searched here (else left to the kernels behind)
-    int follow;        // the next kernel may start beside this one
     int rounds;        // more instances than SMs
     int packed;        // packed relaxations are allowed
+    int guessed;       // entries of `guess`; 0: every instance that fits is searched
+    const int32_t* guess;
     const int32_t* L;
     const int32_t* time_q;
     const int32_t* mem_q;
@@ -59,8 +65,7 @@ struct SoArgs {
     int32_t* map;      // [B][S] with `states`: state row of each strategy, kStateHalf or kStateWord added
     int32_t* status;
     int32_t* path;     // [4] device flags of the search; [3]: kernel that ran
-    int32_t* done;     // [B] 1: this instance needs nothing more; 2 on entry: unstructured
-    int probed;        // done[] says which matrices are unstructured
+    int32_t* done;     // [B] 3: this instance needs nothing more, 0: it does
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
@@ -530,6 +535,222 @@ __device__ __forceinline__ void run(const Ctx& c, int warp, int lane)
     else run_layers<KC, 1, F>(c, warp, lane);
 }
 
+// What a step of tiles costs here, in SM cycles: by how many strategies pass the test at a column group, and how many are listed.
+// Fitted on B200 to 400 shapes of analytic and of measured tables: unstructured matrices to 10 %, classes, whose tiles of several
+// groups go by their worst one, to 30 % for the most part.  states: they are written too.
+__host__ __device__ inline float step_cycles(int KC, bool word, bool states, float alive, float listed)
+{
+    if (listed > 64.0f) alive += listed - 64.0f;               // beyond the 64th of a list all of them pass
+    const float t = KC == 8    ? 1000.0f + 110.0f * listed + 1100.0f * alive
+                    : KC == 16 ? 600.0f + 60.0f * listed + 1300.0f * alive
+                    : KC == 32 ? 2000.0f + 640.0f * alive
+                               : 2400.0f + 1700.0f * alive;
+    return t * (word ? 1.25f : 1.0f) + (states ? 2500.0f : 0.0f);
+}
+
+// What a layer costs a column group and an SM in the tiled kernels, which take unstructured matrices of large batches (to 12 %): the
+// packed loop, and the 32-bit one with dominated rows left out.
+__host__ __device__ inline float tiled_cycles(int S, bool packed, float alive)
+{
+    return packed ? 82.0f + 16.05f * S + 0.13f * S * S : 34.0f + 10.76f * S + 0.197f * S * S + 0.33f * alive * S;
+}
+// The resident kernel against its plan's estimate: stacks of layers that repeat (0.8 to 2.0 of it), of layers that all differ (1.6 to
+// 3.5: a warp prepares each one's records), and what a strategy and column group of a warp adds where shifts pass the halo (40 to 230).
+constexpr float kResidentRepeats = 1.2f, kResidentDiffers = 1.7f, kResidentPastHalo = 60.0f;
+
+// Whether a batch is worth the solo kernel: what it would cost there over what it costs elsewhere, in units of 1 / kGuessUnit,
+// for up to kGuessed of its instances; -1: an instance that is not searched at all.
+//
+// What it costs hangs on how many strategies pass the test at a column group, which is guessed from a few layers' rows.  Where C
+// falls by `slope` a column a strategy weighs time + slope * mem, and passes if that is within the largest transition entry of the
+// layer's best; and there a layer of the best plan takes the mem of that best one.  So slopes from 0 (the budget is no bound)
+// upwards, each with the layers and columns that lie between its mem and the next one's: within a quarter of what passes, on all
+// tables tried (independent times and memories, less memory for more time, analytic models).
+//
+// One answer for the batch, as a mixed one pays for both kernels in turn (100 instances of 40 layers, S = 24 of 3000 columns, some of
+// them taken: 1044 us against 542 and 575).  A kernel of its own, as the solo kernel's start is 20 thousand cycles, most of them
+// spent on fetching its code: a batch that is turned away pays 15 to 20 us.  Taken where the guess leaves a tenth.
+// Without / with it, us: 2 instances of 96 layers of an analytic model, S = 60 of 2880 columns 2470 / 325 (resident kernel 307); 31 of
+// 90, S = 20 of 8192 1885 / 804; 200 of 40, S = 64 of 4 classes, transitions twice the layer times 2700 / 1160; 16 of 48 measured layers,
+// S = 32 of 2048 457 / 235; taken: 200 of 40, S = 64 of 9 classes 2195 before it / 439; 300 of 30 measured, S = 24 of 3000 1529 / 830.
+constexpr int kGuessed = 32, kGuessUnit = 1024, kGuessTaken = 920, kGuessMost = 1 << 20, kGuessThreads = 512, kGuessLayers = 8, kSlopes = 6;
+struct GuessArgs {
+    int B, Lmax, S, M, n;
+    int nw, groups, dense, states;
+    SoOther other;
+    const int32_t* L;
+    const int32_t* time_q;
+    const int32_t* mem_q;
+    const int32_t* trans_q;
+    long long trans_inst, trans_layer;
+    int32_t* guess;
+};
+__global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
+{
+    constexpr int NW = kGuessThreads / 32, kRows = 4;          // rows of the matrix a warp looks at together
+    __shared__ uint32_t s_row[kMaxS + kRows * NW], s_col[kMaxS];
+    __shared__ int s_kind[kMaxS];
+    __shared__ int4 s_at[kGuessLayers][kMaxS];                 // mem, time, kind of the strategy
+    __shared__ float2 s_point[kGuessLayers][kMaxS];            // time, mem; +inf where it does not fit or another one of its kind is as good
+    __shared__ float s_time[NW], s_mem[NW];
+    __shared__ int s_tmax, s_kinds[2], s_listed, s_mmax, s_pass[kSlopes], s_used[kSlopes];
+    __shared__ uint32_t s_rows[kGuessLayers];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, S = a.S, M = a.M;
+    const int i = a.n > 1 ? (int)((long long)blockIdx.x * (a.B - 1) / (a.n - 1)) : 0;
+    const int Li = a.L[i];
+    if (Li < 1 || Li > a.Lmax) {
+        if (tid == 0) a.guess[blockIdx.x] = -1;
+        return;
+    }
+    const int32_t* const T = a.trans_q + (size_t)i * a.trans_inst;
+    const int layers = min(Li, kGuessLayers);
+    auto layer_of = [&](int q) { return layers > 1 ? (int)((long long)q * (Li - 1) / (layers - 1)) : 0; };
+    if (tid < S) s_col[tid] = 0;
+    if (tid < kSlopes) { s_pass[tid] = 0; s_used[tid] = 0; }
+    if (tid < kGuessLayers) s_rows[tid] = 0;
+    if (tid == 0) { s_tmax = 0; s_kinds[0] = 0; s_kinds[1] = 0; s_listed = 0; s_mmax = 0; }
+    __syncthreads();
+    {
+        float time = 0.0f, mem = 0.0f;
+        for (int x = tid; x < layers * S; x += kGuessThreads) {
+            const int q = x / S, s = x - q * S;
+            const size_t at = ((size_t)i * a.Lmax + layer_of(q)) * S + s;
+            const int4 me = make_int4(a.mem_q[at], a.time_q[at], s, 0);
+            s_at[q][s] = me;
+            atomicAdd(&s_rows[q], ((uint32_t)me.x * 0x85EBCA6Bu + (uint32_t)me.y) * ((uint32_t)s * 0x9E3779B2u + 0x7F4A7C15u));
+            time += (float)me.y; mem += (float)min(me.x, M);
+        }
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1) { time += __shfl_xor_sync(0xffffffffu, time, o); mem += __shfl_xor_sync(0xffffffffu, mem, o); }
+        if (lane == 0) { s_time[warp] = time; s_mem[warp] = mem; }
+    }
+    // ---- the matrix: sums over the words of its rows and columns, which tell the classes, and its largest entry.  Of matrices per
+    // layer, whose rows are all kinds of their own, a few rows each.
+    {
+        int tmax = 0;
+        if (!a.trans_layer) {
+#pragma unroll 1
+            for (int r0 = warp; r0 < S; r0 += kRows * NW) {
+                uint32_t row[kRows] = {};
+#pragma unroll 1
+                for (int s = lane; s < S; s += 32) {
+                    int v[kRows];
+                    uint32_t col = 0;
+#pragma unroll
+                    for (int u = 0; u < kRows; ++u) v[u] = r0 + u * NW < S ? T[(r0 + u * NW) * S + s] : 0;
+#pragma unroll
+                    for (int u = 0; u < kRows; ++u) {
+                        tmax = max(tmax, v[u]);
+                        row[u] += (uint32_t)v[u] * ((uint32_t)s * 0x9E3779B2u + 0x7F4A7C15u);
+                        col += (uint32_t)v[u] * ((uint32_t)(r0 + u * NW) * 0x9E3779B2u + 0x7F4A7C15u);
+                    }
+                    atomicAdd(&s_col[s], col);
+                }
+#pragma unroll
+                for (int u = 0; u < kRows; ++u) {
+                    row[u] = __reduce_add_sync(0xffffffffu, row[u]);
+                    if (lane == 0) s_row[r0 + u * NW] = row[u];
+                }
+            }
+        } else if (warp < layers && layer_of(warp) > 0) {
+            const int32_t* const Tl = T + (size_t)layer_of(warp) * a.trans_layer;
+#pragma unroll 4
+            for (int k = lane; k < min(S, 8) * S; k += 32) tmax = max(tmax, Tl[k]);
+        }
+        tmax = __reduce_max_sync(0xffffffffu, tmax);
+        if (lane == 0) atomicMax(&s_tmax, tmax);
+    }
+    __syncthreads();
+    if (!a.trans_layer && tid < S) {                            // the first strategy of the same row, of the same column, of both
+        const uint32_t hr = s_row[tid], hc = s_col[tid];
+        int row = tid, col = tid, both = tid;
+#pragma unroll 4
+        for (int o = tid - 1; o >= 0; --o) {
+            const bool r = s_row[o] == hr, c = s_col[o] == hc;
+            if (r) row = o;
+            if (c) col = o;
+            if (r && c) both = o;
+        }
+        s_kind[tid] = both;
+        if (row == tid) atomicAdd(&s_kinds[0], 1);
+        if (col == tid) atomicAdd(&s_kinds[1], 1);
+    }
+    __syncthreads();
+    const bool classes = !a.trans_layer && max(s_kinds[0], s_kinds[1]) <= kClassMax;
+    const int Kr = classes ? s_kinds[0] : S, Kc = classes ? s_kinds[1] : S;
+    for (int x = tid; x < layers * S; x += kGuessThreads) {
+        const int q = x / S, s = x - q * S;
+        const int4 me = s_at[q][s];
+        bool in = me.x <= M;
+        if (classes && in) {
+            const int kind = s_kind[s];
+#pragma unroll 4
+            for (int o = 0; o < S; ++o) {
+                const int4 ot = s_at[q][o];
+                in &= !(s_kind[o] == kind && ot.x <= me.x && ot.y <= me.y && (o < s || ot.y < me.y));
+            }
+        }
+        s_point[q][s] = in ? make_float2((float)me.y, (float)me.x) : make_float2(__uint_as_float(0x7f800000u), 0.0f);
+        if (in) { atomicAdd(&s_listed, 1); atomicMax(&s_mmax, me.x); }
+    }
+    __syncthreads();
+    // ---- a layer and a slope a warp
+    float scale = 0.0f, over = 0.0f;                           // the slope at which time and memory weigh the same
+#pragma unroll 1
+    for (int q = 0; q < NW; ++q) { scale += s_time[q]; over += s_mem[q]; }
+    scale /= fmaxf(over, 1.0f);
+#pragma unroll 1
+    for (int x = warp; x < layers * kSlopes; x += NW) {
+        const int q = x / kSlopes, k = x - q * kSlopes;
+        const float slope = k == 0 ? 0.0f : scale * (float)(1 << 2 * k) * 0.0078125f;       // 0, 1/32, 1/8, .. 8 times
+        const uint32_t none = 0x7f800000u;                     // +inf as bits: sorts behind every weight
+        uint32_t best = none, used = 0x7fffffffu;
+        int pass = 0;
+#pragma unroll 1
+        for (int s = lane; s < S; s += 32) best = min(best, __float_as_uint(__fmaf_rn(slope, s_point[q][s].y, s_point[q][s].x)));
+        best = __reduce_min_sync(0xffffffffu, best);
+        const float limit = __uint_as_float(best) + (float)s_tmax + 32.0f * slope;
+#pragma unroll 1
+        for (int s = lane; s < S; s += 32) {
+            const float2 p = s_point[q][s];
+            const float v = __fmaf_rn(slope, p.y, p.x);
+            pass += __float_as_uint(v) != none && v <= limit;
+            if (__float_as_uint(v) == best) used = min(used, (uint32_t)p.y);
+        }
+        pass = __reduce_add_sync(0xffffffffu, pass);
+        used = __reduce_min_sync(0xffffffffu, used);
+        if (lane == 0 && best != none) { atomicAdd(&s_pass[k], pass); atomicAdd(&s_used[k], (int)used); }
+    }
+    __syncthreads();
+    if (tid != 0) return;
+    // ---- layers and columns below the line column = layer * mem, slope by slope
+    const float cols = (float)(M + 1), deep = (float)Li, all = cols * deep, per = 1.0f / (float)layers;
+    float left = all, sum = 0.0f, before = 0.0f;
+#pragma unroll 1
+    for (int k = 0; k < kSlopes; ++k) {
+        const float mem = (float)s_used[k] * per, pass = (float)s_pass[k] * per;
+        const float below = fminf(left, mem * deep <= cols ? 0.5f * mem * deep * deep : all - 0.5f * cols * cols / mem);
+        sum += (left - below) * (k == 0 ? pass : 0.5f * (pass + before));
+        left = below; before = pass;
+    }
+    const float alive = sum / all, listed = (float)s_listed * per;
+    const int KC = Kc <= 8 && Kr <= 16 ? 8 : Kc <= 16 ? 16 : Kc <= 32 ? 32 : 64, step = a.nw * max_tile(KC);
+    const float cost = (float)((a.groups + step - 1) / step) * step_cycles(KC, s_tmax > 65535, a.states, alive, listed) + a.other.start;
+    float other;
+    if (classes && a.other.w && Kc * a.other.w <= a.other.gints) {
+        bool repeats = layers < kGuessLayers;
+        for (int q = 1; q < layers; ++q)
+            for (int o = 0; o < q; ++o) repeats |= s_rows[o] == s_rows[q];
+        other = a.other.resident * (repeats ? kResidentRepeats : kResidentDiffers);
+        if (s_mmax > ((a.other.gints / Kc - a.other.w) & ~31)) other += a.other.past_halo * listed;
+    } else {
+        other = a.other.tiled * tiled_cycles(S, a.other.packed && s_tmax <= 32767, alive);
+    }
+    other = fminf(other, a.other.most);
+    const bool fits = classes || a.dense;
+    a.guess[blockIdx.x] = fits && cost < other * (float)(kGuessMost / kGuessUnit) ? (int)(cost / other * (float)kGuessUnit) : kGuessMost;
+}
+
 __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -551,8 +772,16 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
     int32_t* const tsm = raw + 8 * S4;
     unsigned char* const state = reinterpret_cast<unsigned char*>(tsm + a.mats);
 
+    if (a.guessed) {                                            // the batch as a whole, the same in every CTA
+        int ratio = 0, asked = 0;
+        if (lane < a.guessed) { ratio = a.guess[lane]; asked = ratio >= 0; ratio = max(ratio, 0); }
+        if (__reduce_add_sync(0xffffffffu, ratio) > kGuessTaken * __reduce_add_sync(0xffffffffu, asked)) {
+            if (tid == 0) a.done[blockIdx.x] = 0;
+            if (blockIdx.x == 0 && tid == 0) a.path[3] = 2;
+            return;
+        }
+    }
     if (blockIdx.x == 0 && tid == 0) a.path[3] = 2;
-    if (a.follow) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // ---- which instance: CTAs are dispatched in order, so the longest instances go first
     int i = blockIdx.x;
@@ -576,10 +805,9 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
         i = s_inst;
     }
     const int G = Mp / 32;
-    if (a.probed && a.done[i] == 2) return;                     // found to be unstructured, which this launch has no room for
     const int Li = a.L[i];
     if (Li < 1 || Li > Lmax) {
-        if (tid == 0) { a.status[i] = GALV_STATUS_BAD_INPUT; a.done[i] = 1; }
+        if (tid == 0) { a.status[i] = GALV_STATUS_BAD_INPUT; a.done[i] = 3; }
         return;
     }
     const int32_t* const tq = a.time_q + (size_t)i * Lmax * S;
@@ -740,7 +968,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
     const int per_warp = max_tile(KC), steps = (G + NW * per_warp - 1) / (NW * per_warp), per_step = (G + steps - 1) / steps;
     const bool run_it = st == 0 && (classes || (a.dense && S <= kDenseMax)) && base_bytes + d_bytes <= a.room && steps * NW <= kMaxTiles &&
                         (!a.states || 1 + words <= S);          // the place of a table row each
-    if (tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run_it; }
+    if (tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run_it ? 3 : 0; }
     if (blockIdx.x == 0 && tid == 0 && run_it && a.rounds && !classes) a.path[3] = form == kPacked;
     if (!run_it) {
         if (warp == NW) cp_async_wait<0>();                     // nothing may land in shared memory that is no longer ours
@@ -958,7 +1186,6 @@ bool galv_solo_plan(const galv_ctx* ctx, const galv_shape* sh, bool states, SoPl
         p->certain = need == 0 && !states;
         p->smem = need == 0 ? (int)(fixed + room) : room_max;
         p->room = (int)((p->smem - fixed) & ~15ll);
-        p->classes = !states && state_bytes(sh, rows[3], 4, sh->M) <= p->room;
         p->rounds = sh->B > ctx->num_sms;
         p->packed = !(sh->flags & GALV_KERNEL_NO_PACKED);
         p->sorted = sh->B > ctx->num_sms && sh->B <= kMaxSorted;
@@ -967,16 +1194,76 @@ bool galv_solo_plan(const galv_ctx* ctx, const galv_shape* sh, bool states, SoPl
     return false;
 }
 
+// Whether the look at the tables is worth its launch: not for shapes that every batch is better off elsewhere with (most batches of a
+// few instances, whose layers take the other kernels a few thousand cycles), nor for batches that are short everywhere.
+bool galv_solo_worth(const galv_ctx* ctx, const galv_shape* sh, bool states, int n, const RsPlan resident[2], const ClPlan* pushing, SoPlan* p)
+{
+    const int S = sh->S, G = sh->m_pitch / 32;
+    const float rounds = (float)((sh->B + ctx->num_sms - 1) / ctx->num_sms), none = 1e30f;
+    SoOther& o = p->other;
+    o.start = 10000.0f / (float)sh->Lmax;                      // twenty thousand cycles, of which the others have half
+    o.packed = S <= 64 && S % 4 == 0 && !(sh->flags & GALV_KERNEL_NO_PACKED);
+    o.tiled = 0.95f * (float)G * (float)sh->B / (float)ctx->num_sms / rounds;
+    o.most = pushing ? 0.9f * (float)pushing->est / rounds : none;
+    if (n && resident[n - 1].dense && 1.5f * (float)resident[n - 1].est / rounds < o.most) o.most = 1.5f * (float)resident[n - 1].est / rounds;
+    if (n && !resident[0].dense) {
+        const RsPlan& r = resident[0];
+        const int g = r.w / 32;
+        o.resident = (float)r.est / rounds; o.gints = r.gints; o.w = r.w;
+        o.past_halo = kResidentPastHalo * (float)((g + r.nw - 1) / r.nw * r.rounds) / rounds;
+    }
+    auto layer = [&](int KC, bool word, float alive, float listed) {
+        const int step = p->nw * max_tile(KC);
+        return (float)((G + step - 1) / step) * step_cycles(KC, word, states, alive, listed) + o.start;
+    };
+    // No batch of this shape is worth it: few strategies pass, and elsewhere it goes as badly as it can.
+    const int KC = S <= 8 ? 8 : S <= 16 ? 16 : S <= 32 ? 32 : 64;
+    const float taken = (float)kGuessTaken / kGuessUnit, few = 0.7f;
+    auto at_most = [&](float a) { return a < o.most ? a : o.most; };
+    const float tiled = at_most(o.tiled * (tiled_cycles(S, false, (float)S) > tiled_cycles(S, true, 0.0f) ? tiled_cycles(S, false, (float)S) : tiled_cycles(S, true, 0.0f)));
+    const float classes = o.w ? at_most(o.resident * kResidentDiffers + o.past_halo * (float)S) : tiled;
+    p->dense = p->dense && layer(KC, false, few, KC <= 16 ? 0.5f * S : (float)S) <= taken * tiled;
+    const bool some = layer(8, false, few, (float)S / 3.0f) <= taken * classes;
+    if (!p->dense && !some) return false;
+    // The look at the batch, 15 us where it is turned away, has to be small beside it: at most 300 us elsewhere, or 100 at best, are
+    // not worth it.
+    const float lowest = o.packed && tiled_cycles(S, true, 0.0f) < tiled_cycles(S, false, 0.0f) ? tiled_cycles(S, true, 0.0f) : tiled_cycles(S, false, 0.0f);
+    const float least_tiled = at_most(o.tiled * lowest), least_classes = o.w ? at_most(o.resident * kResidentRepeats) : least_tiled;
+    const float batch = rounds * (float)sh->Lmax;
+    if ((p->dense && (!some || tiled > classes) ? tiled : classes) * batch < 600e3f) return false;
+    if ((some && (!p->dense || least_classes < least_tiled) ? least_classes : least_tiled) * batch < 200e3f) return false;
+    p->guessed = sh->B < kGuessed ? sh->B : kGuessed;
+    // Every batch of this shape is, whatever it holds.
+    const float least = least_classes < least_tiled ? least_classes : least_tiled;
+    bool all = p->certain && p->dense;
+    for (int k = 8; k <= KC; k <<= 1) all = all && layer(k, true, (float)S, (float)S) <= taken * least;
+    p->certain = all;
+    if (all) p->guessed = 0;
+    return true;
+}
+
 cudaError_t galv_solo_configure(galv_ctx* ctx)
 {
     return cudaFuncSetAttribute(solo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin - kStaticSmem);
 }
 
-cudaError_t galv_solo_launch(const SoPlan& p, const DpArgs& d, int follow, int probed, cudaStream_t st)
+cudaError_t galv_solo_launch(const SoPlan& p, const DpArgs& d, cudaStream_t st)
 {
+    if (p.guessed) {
+        GuessArgs g;
+        g.B = d.B; g.Lmax = d.Lmax; g.S = d.S; g.M = d.M; g.n = p.guessed;
+        g.nw = p.nw; g.groups = d.m_pitch / 32; g.dense = p.dense; g.states = d.lean_map != nullptr;
+        g.other = p.other;
+        g.L = d.L; g.time_q = d.time_q; g.mem_q = d.mem_q; g.trans_q = d.trans_q; g.trans_inst = d.trans_inst; g.trans_layer = d.trans_layer;
+        g.guess = d.order;
+        guess_kernel<<<p.guessed, kGuessThreads, 0, st>>>(g);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     SoArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
-    a.NW = p.nw; a.room = p.room; a.mats = p.mats; a.sorted = p.sorted; a.dense = p.dense; a.follow = follow; a.probed = probed;
+    a.NW = p.nw; a.room = p.room; a.mats = p.mats; a.sorted = p.sorted; a.dense = p.dense;
+    a.guessed = p.guessed; a.guess = d.order;
     a.rounds = p.rounds; a.packed = p.packed;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;

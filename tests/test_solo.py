@@ -148,3 +148,42 @@ def test_what_lies_behind_the_matrices(galv, S, M):
             one.dp_search(); one.backtrack()
             torch.cuda.synchronize()
             assert torch.equal(one.status, ref.status) and torch.equal(one.opt_cost, ref.opt_cost) and torch.equal(one.C_last, ref.C_last), (flags, behind)
+
+
+def milliseconds(sb):
+    import torch
+    sb.dp_search()
+    best = 1e9
+    for _ in range(5):
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record()
+        sb.dp_search()
+        t1.record()
+        torch.cuda.synchronize()
+        best = min(best, t0.elapsed_time(t1))
+    return best
+
+
+# (instances, layers, strategies, budget, classes or 0, largest transition entry over the median time, by the kernel that suits it)
+@pytest.mark.parametrize("B,Lmax,S,M,K,share,kernel", [(6, 40, 64, 4000, 8, 2.0, "KERNEL_RESIDENT"), (40, 48, 64, 4000, 7, 1.0, "KERNEL_RESIDENT"),
+                                                       (200, 40, 64, 4000, 4, 2.0, "KERNEL_RESIDENT"), (6, 48, 48, 1500, 0, 0.03, "KERNEL_CLUSTER"),
+                                                       (200, 24, 16, 2880, 0, 1.0, "KERNEL_NO_CLUSTER")])
+def test_batches_that_nothing_can_be_ruled_out_in(galv, B, Lmax, S, M, K, share, kernel):
+    """Without a flag a batch that most strategies matter in goes where all of them are relaxed fast: on the solo kernel these
+    take 2.2 to 5 times as long.  Twice as long as the kernel that suits them leaves room for the look and for the clock."""
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    rng = np.random.default_rng(S + B)
+    w = inputs.random_tables(800 + B, B, Lmax, S, M, mem_lo=M // (6 * Lmax), mem_hi=3 * M // Lmax)
+    w.time_q[:] = np.sort(np.rint(5e5 * np.exp(0.5 * rng.standard_normal(w.time_q.shape))).astype(np.int32), axis=2)
+    w.mem_q[:] = -np.sort(-w.mem_q, axis=2)                      # less memory costs time
+    top = int(5e5 * share) + 1
+    w.trans_q[:] = rng.integers(0, top, w.trans_q.shape, np.int32)
+    if K:
+        for i in range(B):
+            w.trans_q[i] = rng.integers(0, top, (K, K), np.int32)[rng.integers(0, K, S)][:, rng.integers(0, K, S)]
+    plain, suited = SearchBuffers(galv, w, 0), SearchBuffers(galv, w, getattr(gb, kernel))
+    assert milliseconds(plain) < 2 * milliseconds(suited)
+    plain.backtrack(); suited.backtrack()
+    import torch
+    assert torch.equal(plain.status, suited.status) and torch.equal(plain.opt_cost, suited.opt_cost) and torch.equal(plain.C_last, suited.C_last)
