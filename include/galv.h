@@ -208,11 +208,10 @@ int galv_dp_search(galv_ctx* ctx, const galv_shape* shape, const int32_t* L,
 /*
  * Which kernel the most recent galv_dp_search on `workspace` ran: *packed = 1 for the tiled kernel
  * with the packed 16-bit inner loop (two relaxations per instruction; see GALV_KERNEL_NO_PACKED),
- * 0 for the tiled kernel with the 32-bit one, 2 for the kernels that keep an instance on chip (one thread-block cluster per instance: the
+ * 0 for the tiled kernel with the 32-bit one, 2 for the cluster kernels (one thread-block cluster per instance: the
  * resident one, the pushing one, or the first and what it left alone the second; see GALV_KERNEL_CLUSTER,
- * GALV_KERNEL_RESIDENT).  Where the tiled kernels took some of the batch, theirs.
- * The solo kernel (GALV_KERNEL_SOLO) counts as 2; for unstructured matrices of more instances than SMs, which take several
- * rounds, as 1 or 0: whether it relaxes them packed in 16 bits or in 32.  With an argmin table always 0: the
+ * GALV_KERNEL_RESIDENT), 3 for the solo kernel (GALV_KERNEL_SOLO).  Where the tiled kernels took some of the batch, theirs;
+ * 3 only where the solo kernel took every instance that could be searched.  With an argmin table always 0: the
  * arithmetic is 32-bit in the tiled kernels and in the resident one, and this word does not say which of them ran.  Part
  * of the choice is made on the device; this call waits for `stream` and reads the answer back (host pointer).
  */

@@ -21,7 +21,7 @@ SKIP_DOMINATED = 8192
 DEBUG_WITHHOLD_LOAD = 2048
 KERNEL_NO_PACKED = 4096
 KERNEL_NO_CLUSTER, KERNEL_CLUSTER, KERNEL_RESIDENT, KERNEL_SOLO = 16384, 32768, 1 << 21, 1 << 22
-PATH_TILED_32, PATH_TILED_PACKED, PATH_CLUSTER = 0, 1, 2
+PATH_TILED_32, PATH_TILED_PACKED, PATH_CLUSTER, PATH_SOLO = 0, 1, 2, 3
 
 
 def CLUSTER_SIZE(n: int) -> int:
@@ -221,7 +221,7 @@ class Galv:
 
     def galv_dp_search_path(self, shape, workspace) -> int:
         """Kernel of the most recent search on this workspace: 1 tiled kernel with the packed 16-bit inner loop
-        (truthy, as before), 0 tiled kernel with the 32-bit loop, 2 cluster kernel."""
+        (truthy, as before), 0 tiled kernel with the 32-bit loop, 2 cluster kernels, 3 solo kernel."""
         out = C.c_int32()
         self._check(self.lib.galv_dp_search_path(self.h, C.byref(shape), _ptr(workspace), C.byref(out), _stream()))
         return int(out.value)

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
     int32_t* const dump = fillmax + 4;                                                     // [32 * TM] where stores of skipped strategies go
     int* const cdelta = dump + 32 * TM;                                                    // [16] cluster-window address of CTA d minus this CTA's own shared address
 
-    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; a.path[3] = 2; }      // no error flag to raise; the cluster kernel ran
+    if (blockIdx.x == 0 && tid == 0) { a.path[0] = 0; if (!a.after_solo) a.path[3] = kPathCluster; }      // no error flag to raise; the cluster kernel ran
 
     // ---- which instance: clusters are dispatched in order, so the longest instances go first
     int i = cid;
@@ -462,6 +462,7 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
         bulk_wait_all();
     }
     resident_over();
+    if (a.after_solo && rank == 0 && tid == 0) a.path[3] = kPathCluster;
 }
 
 }  // namespace

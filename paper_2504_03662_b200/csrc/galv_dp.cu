@@ -1961,7 +1961,7 @@ cudaError_t galv_dp_launch(galv_ctx* ctx, const galv_shape* sh, const DpArgs& ar
     validate_kernel<<<B, a.trans_layer || B <= 148 ? 512 : 128, 0, st>>>(B, Lmax, S, a.M, (long long)a.trans_layer, a.L, a.time_q, a.mem_q, a.trans_q, a.status, a.done, a.err + 1, a.minmem_l,
                                        (sh->flags & GALV_SKIP_INFEASIBLE) ? a.front : nullptr, dom_auto ? reinterpret_cast<long long*>(a.err + 6) : nullptr);
     schedule_kernel<<<1, 1024, 0, st>>>(B, Lmax, a.M, pl.tmb, pl.ntiles_m, pl.nsb, a.L, a.status, a.done, a.order, a.nactive, a.scratch,
-                                         a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.A ? 0 : solo ? -1 : 2, a.err + 1);
+                                         a.minmem_l, a.ntiles, a.istart, a.tcount, will_p16, a.A ? 0 : solo ? -1 : kPathCluster, a.err + 1);
     auto base_layer = [&]() {
         int gx = (a.m_pitch + 255) / 256;
         if (gx > 8) gx = 8;

@@ -9,6 +9,7 @@
 #include "galv.h"
 
 constexpr int kStateHalf = 1 << 16, kStateWord = 1 << 17;      // DpArgs::lean_map: states of bases and 16-bit (two rows a word) or 32-bit differences
+constexpr int kPathCluster = 2, kPathSolo = 3;                // what galv_dp_search_path says beside the tiled kernels' 1 (packed) and 0
 constexpr int kResidentClassMax = 16;      // classes beyond which a matrix counts as unstructured in the resident kernel
 
 // How the resident kernel (one thread-block cluster per instance, the state between layers in shared memory) cuts an instance.
@@ -48,7 +49,6 @@ struct SoPlan {
     int sorted;    // CTA c takes the c-th longest instance
     int dense;     // unstructured matrices fit, with transition entries up to 65535 at least
     int certain;   // every instance can run, and is worth it
-    int rounds;    // more instances than SMs
     int packed;    // packed relaxations are allowed
     int guessed;   // instances that are looked at to see whether the batch is worth it; 0: it is
     SoOther other;
@@ -128,7 +128,7 @@ struct DpArgs {
                          // neither the resident nor the solo kernel was launched.
                          // Lies over tile_done: read until the schedule is made
     int withhold;        // test hook: CTA 0 never loads its first chunk, so that the bounded waits run out
-    int after_solo;      // the solo kernel has run: done[] = 3 are its own
+    int after_solo;      // the solo kernel has run: done[] = 3 are its own, and the word that says which kernel ran until another one searches something
     int beside;          // the pushing kernel may start beside the kernel in front, the resident one
     int skip_dom;        // leave out rows (packed path: row pairs) that cannot win in any column of a warp group's tile
     int dom_auto;        // ... where a quarter of the rows or more look it (maxmem[4])

@@ -51,7 +51,6 @@ struct SoArgs {
     int mats;          // words of the transition matrices in shared memory
     int sorted;        // CTA c takes the c-th longest instance
     int dense;         // unstructured matrices are searched here (else left to the kernels behind)
-    int rounds;        // more instances than SMs
     int packed;        // packed relaxations are allowed
     int guessed;       // entries of `guess`; 0: every instance that fits is searched
     const int32_t* guess;
@@ -572,7 +571,7 @@ constexpr float kResidentRepeats = 1.2f, kResidentDiffers = 1.7f, kResidentPastH
 // spent on fetching its code: a batch that is turned away pays 15 to 20 us.  Taken where the guess leaves a tenth.
 // Without / with it, us: 2 instances of 96 layers of an analytic model, S = 60 of 2880 columns 2470 / 325 (resident kernel 307); 31 of
 // 90, S = 20 of 8192 1885 / 804; 200 of 40, S = 64 of 4 classes, transitions twice the layer times 2700 / 1160; 16 of 48 measured layers,
-// S = 32 of 2048 457 / 235; taken: 200 of 40, S = 64 of 9 classes 2195 before it / 439; 300 of 30 measured, S = 24 of 3000 1529 / 830.
+// S = 32 of 2048 457 / 235; taken: 200 of 40, S = 64 of 7 classes 2195 before it / 439; 300 of 30 measured, S = 24 of 3000 1529 / 830.
 constexpr int kGuessed = 32, kGuessUnit = 1024, kGuessTaken = 920, kGuessMost = 1 << 20, kGuessThreads = 512, kGuessLayers = 8, kSlopes = 6;
 struct GuessArgs {
     int B, Lmax, S, M, n;
@@ -777,11 +776,11 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
         if (lane < a.guessed) { ratio = a.guess[lane]; asked = ratio >= 0; ratio = max(ratio, 0); }
         if (__reduce_add_sync(0xffffffffu, ratio) > kGuessTaken * __reduce_add_sync(0xffffffffu, asked)) {
             if (tid == 0) a.done[blockIdx.x] = 0;
-            if (blockIdx.x == 0 && tid == 0) a.path[3] = 2;
+            if (blockIdx.x == 0 && tid == 0) a.path[3] = kPathCluster;
             return;
         }
     }
-    if (blockIdx.x == 0 && tid == 0) a.path[3] = 2;
+    if (blockIdx.x == 0 && tid == 0) a.path[3] = kPathSolo;
 
     // ---- which instance: CTAs are dispatched in order, so the longest instances go first
     int i = blockIdx.x;
@@ -962,14 +961,13 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
                              : s_all.sum + (long long)(Li - 1) * s_all.tmax >= (long long)kInf ? GALV_STATUS_OVERFLOW_RISK : 0;
     // ---- the state: guard columns of +inf below column 0, as many as the largest shift; rows lie one behind the other, so what
     // a shift finds below its own row's column 0 is a difference of another column, or a zero before the first row
-    const int form = s_all.tmax > 65535 ? kWord : a.packed && s_all.tmax <= 32767 && (S % 4 == 0 || classes) ? kPacked : kHalf;
+    const int form = s_all.tmax > 65535 ? kWord : a.packed && s_all.tmax <= 32767 ? kPacked : kHalf;
     const int H = (s_all.mmax + 31) & ~31, words = form == kWord ? Kc : (Kc + 1) >> 1;      // words of a column's differences
     const long long base_bytes = 4ll * (H + Mp), d_bytes = 4ll * (H + (long long)words * Mp);
     const int per_warp = max_tile(KC), steps = (G + NW * per_warp - 1) / (NW * per_warp), per_step = (G + steps - 1) / steps;
     const bool run_it = st == 0 && (classes || (a.dense && S <= kDenseMax)) && base_bytes + d_bytes <= a.room && steps * NW <= kMaxTiles &&
                         (!a.states || 1 + words <= S);          // the place of a table row each
     if (tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run_it ? 3 : 0; }
-    if (blockIdx.x == 0 && tid == 0 && run_it && a.rounds && !classes) a.path[3] = form == kPacked;
     if (!run_it) {
         if (warp == NW) cp_async_wait<0>();                     // nothing may land in shared memory that is no longer ours
         return;
@@ -1186,7 +1184,6 @@ bool galv_solo_plan(const galv_ctx* ctx, const galv_shape* sh, bool states, SoPl
         p->certain = need == 0 && !states;
         p->smem = need == 0 ? (int)(fixed + room) : room_max;
         p->room = (int)((p->smem - fixed) & ~15ll);
-        p->rounds = sh->B > ctx->num_sms;
         p->packed = !(sh->flags & GALV_KERNEL_NO_PACKED);
         p->sorted = sh->B > ctx->num_sms && sh->B <= kMaxSorted;
         return true;
@@ -1264,7 +1261,7 @@ cudaError_t galv_solo_launch(const SoPlan& p, const DpArgs& d, cudaStream_t st)
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
     a.NW = p.nw; a.room = p.room; a.mats = p.mats; a.sorted = p.sorted; a.dense = p.dense;
     a.guessed = p.guessed; a.guess = d.order;
-    a.rounds = p.rounds; a.packed = p.packed;
+    a.packed = p.packed;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
     a.C_last = d.C_last; a.states = d.lean_map ? reinterpret_cast<uint32_t*>(d.C) : nullptr; a.map = d.lean_map;

@@ -133,21 +133,25 @@ def test_what_lies_behind_the_matrices(galv, S, M):
     from paper_2504_03662_b200 import binding as gb
     from paper_2504_03662_b200.search import SearchBuffers
     B = 160                                                      # more instances than SMs
-    w = inputs.random_tables(500 + S, B, 3, S, M, ragged=True, mem_lo=0, mem_hi=M // 3, trans_hi=900)
-    ref = SearchBuffers(galv, w, gb.STORE_C_FULL | gb.KERNEL_REFERENCE)
-    ref.dp_search(); ref.backtrack()
-    ref.C = None
-    for flags in (0, gb.KERNEL_SOLO):
-        for behind in ("rows of it", "others"):
-            one = SearchBuffers(galv, w, flags)
-            n = one.trans_q.numel()
-            room = torch.full((n + 17 * S,), 7, dtype=torch.int32, device=one.dev)
-            room[:n] = one.trans_q.flatten()
-            room[n:] = one.trans_q[-1, 0].repeat(17) if behind == "rows of it" else torch.arange(-17 * S, 0, dtype=torch.int32, device=one.dev)
-            one.trans_q = room[:n].view(B, S, S)
-            one.dp_search(); one.backtrack()
-            torch.cuda.synchronize()
-            assert torch.equal(one.status, ref.status) and torch.equal(one.opt_cost, ref.opt_cost) and torch.equal(one.C_last, ref.C_last), (flags, behind)
+    for cols in (S, 4):                                          # no two rows alike; with few kinds of columns the state fits all the same
+        w = inputs.random_tables(500 + S, B, 3, S, M, ragged=True, mem_lo=0, mem_hi=M // 3, trans_hi=900)
+        if cols < S:
+            w.trans_q[:] = np.ascontiguousarray(w.trans_q[:, :, np.random.default_rng(S).integers(0, cols, S)])
+        ref = SearchBuffers(galv, w, gb.STORE_C_FULL | gb.KERNEL_REFERENCE)
+        ref.dp_search(); ref.backtrack()
+        ref.C = None
+        for flags in (0, gb.KERNEL_SOLO):
+            for behind in ("rows of it", "others"):
+                one = SearchBuffers(galv, w, flags)
+                n = one.trans_q.numel()
+                room = torch.full((n + 17 * S,), 7, dtype=torch.int32, device=one.dev)
+                room[:n] = one.trans_q.flatten()
+                room[n:] = one.trans_q[-1, 0].repeat(17) if behind == "rows of it" else torch.arange(-17 * S, 0, dtype=torch.int32, device=one.dev)
+                one.trans_q = room[:n].view(B, S, S)
+                one.dp_search(); one.backtrack()
+                torch.cuda.synchronize()
+                assert torch.equal(one.status, ref.status) and torch.equal(one.opt_cost, ref.opt_cost) and torch.equal(one.C_last, ref.C_last), (flags, behind)
+                assert not flags or cols == S or galv.galv_dp_search_path(one.shape, one.workspace) == gb.PATH_SOLO
 
 
 def milliseconds(sb):
@@ -187,3 +191,45 @@ def test_batches_that_nothing_can_be_ruled_out_in(galv, B, Lmax, S, M, K, share,
     plain.backtrack(); suited.backtrack()
     import torch
     assert torch.equal(plain.status, suited.status) and torch.equal(plain.opt_cost, suited.opt_cost) and torch.equal(plain.C_last, suited.C_last)
+
+
+def path_of(galv, w, flags):
+    import torch
+    from paper_2504_03662_b200.search import SearchBuffers
+    sb = SearchBuffers(galv, w, flags)
+    sb.dp_search()
+    torch.cuda.synchronize()
+    return galv.galv_dp_search_path(sb.shape, sb.workspace)
+
+
+def test_path_word(galv):
+    """What galv_dp_search_path says is what ran: the solo kernel alone (structured and unstructured matrices, also more instances
+    than SMs), or who took the instances it has no room for, or the batches it is not worth its while for."""
+    from paper_2504_03662_b200 import binding as gb
+    kw = dict(mem_lo=0, mem_hi=90)
+    for B in (5, 160):
+        for S in (24, 30):
+            for w in (inputs.random_tables(50 + S, B, 6, S, 900, trans_hi=900, **kw), inputs.random_tables(50 + S, B, 6, S, 900, trans_hi=90000, **kw),
+                      classed(50 + S, B, 6, S, 900, 4, 5, **kw)):
+                assert path_of(galv, w, gb.KERNEL_SOLO) == gb.PATH_SOLO, (B, S)
+    w = classed(60, 5, 6, 100, 900, 4, 5, **kw)
+    assert path_of(galv, w, gb.KERNEL_SOLO) == gb.PATH_SOLO
+    w.trans_q[2] = np.random.default_rng(1).integers(0, 3000, (100, 100), np.int32)      # no room for 100 rows
+    assert path_of(galv, w, gb.KERNEL_SOLO) == gb.PATH_CLUSTER
+    big = classed(61, 160, 4, 64, 2500, 4, 5, **kw)
+    assert path_of(galv, big, gb.KERNEL_SOLO) == gb.PATH_SOLO
+    for top, want in ((3000, gb.PATH_TILED_PACKED), (40000, gb.PATH_TILED_32)):          # ... nor for 64 of 2500 columns
+        big.trans_q[7] = np.random.default_rng(1).integers(0, top + 1, (64, 64), np.int32)
+        big.trans_q[7, 0, 1] = top
+        assert path_of(galv, big, gb.KERNEL_SOLO) == want
+    # without a flag: times far apart, and times that lie close together
+    for S, K in ((24, 0), (64, 7)):
+        w = classed(63, 300, 30, S, 3000, K, K, mem_lo=16, mem_hi=300) if K else inputs.random_tables(63, 300, 30, S, 3000, mem_lo=16, mem_hi=300, trans_hi=2000)
+        w.time_q[:] = np.rint(5e5 * np.exp(0.5 * np.random.default_rng(S).standard_normal(w.time_q.shape))).astype(np.int32)
+        assert path_of(galv, w, 0) == gb.PATH_SOLO
+        w.time_q[:] = 500000 + w.time_q // 1000
+        assert path_of(galv, w, 0) == (gb.PATH_CLUSTER if K else gb.PATH_TILED_PACKED)
+    # with another kernel asked for, or a table to write, the word is that kernel's
+    w = classed(62, 5, 40, 24, 900, 4, 5, **kw)
+    assert path_of(galv, w, gb.KERNEL_RESIDENT) == gb.PATH_CLUSTER and path_of(galv, w, gb.KERNEL_CLUSTER) == gb.PATH_CLUSTER
+    assert path_of(galv, w, gb.KERNEL_NO_CLUSTER) == gb.PATH_TILED_PACKED and path_of(galv, w, gb.STORE_C_FULL | gb.KERNEL_SOLO) == gb.PATH_CLUSTER
