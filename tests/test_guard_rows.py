@@ -61,9 +61,9 @@ def guarded_buffers(galv, w, flags):
     return sb, guards
 
 
-NC, CLU, RES = 16384, 32768, 1 << 21        # tiled kernels only / the pushing, the resident cluster kernel wherever the shape allows
+NC, CLU, RES, SOLO = 16384, 32768, 1 << 21, 1 << 22        # tiled kernels only / the pushing, the resident cluster kernel, the solo kernel wherever the shape allows
 MODES = [1 | NC, 3, 2, NC, 1 | 512, 1 | 1024 | 8192 | NC, 1 | 4096 | NC, 2 | 8192, 1 | 256, 1 | CLU, CLU, 1 | CLU | (2 << 16), 1 | CLU | (16 << 16),
-         1 | RES, RES, 3 | RES, 1 | RES | (2 << 16)]
+         1 | RES, RES, 3 | RES, 1 | RES | (2 << 16), SOLO]
 
 
 @pytest.mark.parametrize("flags", MODES)

@@ -1,58 +1,62 @@
-"""The kernel that keeps an instance's state on one SM: every table, optimum and plan against the one-thread-per-cell kernel,
-which other tests tie to the CPU oracle, and against the oracle itself.  Whole numbers: exact.
+"""The kernel that keeps an instance's state on one SM: the last layer's table and the optimum against the one-thread-per-cell
+kernel, which other tests tie to the CPU oracle.  Whole numbers: exact.  It writes no table and walks no plan; the host entry
+point's plans come from its states.
 """
 import numpy as np
 import pytest
 
 from paper_2504_03662_b200 import inputs
-from tests.test_gpu_parity import INF, check_batch, galv, oracle_search_many  # noqa: F401  (galv is a fixture)
+from tests.test_gpu_parity import galv  # noqa: F401  (a fixture)
 from tests.test_resident import classed
 
 pytestmark = pytest.mark.gpu
 
 
-def against_reference(galv, w, flags):
-    import torch
+def reference(galv, w):
     from paper_2504_03662_b200 import binding as gb
     from paper_2504_03662_b200.search import SearchBuffers
-    ref = SearchBuffers(galv, w, flags | gb.KERNEL_REFERENCE)
+    ref = SearchBuffers(galv, w, gb.KERNEL_REFERENCE)
     ref.dp_search(); ref.backtrack()
-    one = SearchBuffers(galv, w, flags | (0 if flags & (gb.STORE_C_FULL | gb.STORE_ARGMIN) else gb.KERNEL_SOLO))
-    for t in (one.C, one.A, one.C_last):
-        if t is not None:
-            t.fill_(77)
+    return ref
+
+
+def same(one, ref, what=""):
+    import torch
+    torch.cuda.synchronize()
+    assert torch.equal(one.status, ref.status) and torch.equal(one.opt_cost, ref.opt_cost), what
+    ok = (ref.status & ~1) == 0                                  # tables of flagged instances are left untouched
+    assert torch.equal(one.C_last[ok], ref.C_last[ok]), what
+    assert bool((one.C_last[~ok] == 77).all()), what
+
+
+def against_reference(galv, w, path=True):
+    """On the solo kernel.  path: it must take every instance; else whether it did is returned."""
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    ref = reference(galv, w)
+    one = SearchBuffers(galv, w, gb.KERNEL_SOLO)
     for _ in range(2):
+        one.C_last.fill_(77)
         one.dp_search(); one.backtrack()
-        torch.cuda.synchronize()
-        assert torch.equal(one.status, ref.status)
-        assert torch.equal(one.opt_cost, ref.opt_cost)
-        assert torch.equal(one.plan, ref.plan) and torch.equal(one.mem_used, ref.mem_used)
-        ok = [i for i in range(w.B) if int(ref.status[i]) in (0, 1)]
-        for i in ok:
-            Li = int(w.L[i])
-            assert torch.equal(one.C_last[i], ref.C_last[i]), i
-            if ref.C is not None:
-                assert torch.equal(one.C[i, :Li], ref.C[i, :Li]), i
-                assert Li == w.Lmax or bool((one.C[i, Li:] == 77).all())          # layers that are not there are not touched
-            if ref.A is not None:
-                assert torch.equal(one.A[i, :Li], ref.A[i, :Li]), i
-    return one
+        same(one, ref)
+    ran = galv.galv_dp_search_path(one.shape, one.workspace) == gb.PATH_SOLO
+    assert ran or not path
+    return ran
 
 
-# S and classes at the edges of the accumulator widths (8 / 16 / 32 / 64 rows), of a warp's lanes and of the boxes of collected rows
-@pytest.mark.parametrize("S,rows,cols", [(1, 1, 1), (5, 1, 1), (7, 0, 0), (8, 0, 0), (9, 0, 0), (16, 0, 0), (17, 0, 0), (24, 4, 4), (24, 5, 9), (31, 0, 0),
+# S and classes at the edges of the accumulator widths (8 / 16 / 32 / 64 rows) and of a warp's lanes, odd numbers of packed rows
+@pytest.mark.parametrize("S,rows,cols", [(1, 1, 1), (5, 1, 1), (7, 0, 0), (8, 0, 0), (9, 0, 0), (16, 0, 0), (17, 0, 0), (24, 4, 4), (24, 5, 9), (30, 0, 0), (31, 0, 0),
                                          (32, 0, 0), (33, 8, 7), (33, 0, 0), (44, 0, 0), (64, 9, 16), (64, 16, 9), (64, 0, 0), (65, 3, 3), (128, 8, 8)])
-@pytest.mark.parametrize("flags", [0])
-def test_rows_of_the_state(galv, S, rows, cols, flags):
+def test_rows_of_the_state(galv, S, rows, cols):
     M = 700
     kw = dict(ragged=True, mem_lo=0, mem_hi=M // 5, time_hi=4000)
     w = classed(300 + S + rows, 6, 7, S, M, rows, cols, **kw) if rows else inputs.random_tables(300 + S, 6, 7, S, M, **kw)
     w.mem_q[1, 2, : S // 2] = M + 3                              # rows that never fit
-    w.time_q[2, 1, :] = 9                                        # ties: the lowest strategy must win
+    w.time_q[2, 1, :] = 9                                        # ties
     w.time_q[4, :, :] = 3
     w.mem_q[3, 0, :] = M // 2                                    # the lower half of every later column is +inf
     w.L[5] = 1
-    against_reference(galv, w, flags)
+    against_reference(galv, w)
 
 
 # columns: less than a group, one more than a group, a step of tiles and one more, several steps; largest shifts from none to the budget
@@ -63,13 +67,12 @@ def test_columns_and_shifts(galv, M, mem_hi, S, K):
     for B in (1, 3):
         w = classed(M + 40, B, 5, S, M, K, K, **kw) if K else inputs.random_tables(M + 41, B, 5, S, M, **kw)
         w.mem_q[0, min(1, w.Lmax - 1), 0] = M
-        for flags in (0,):
-            against_reference(galv, w, flags)
+        against_reference(galv, w, path=bool(K) or M <= 2880)    # a budget's worth of guard columns, or 8192 columns, beside 12 rows: no room
 
 
-# largest transition entry: differences of 16 and of 32 bits, packed relaxations or not, keys of the argmin
+# largest transition entry: differences of 16 and of 32 bits, packed relaxations or not
 @pytest.mark.parametrize("top", [0, 1, 32767, 32768, 65535, 65536, (1 << 23) - 1, 1 << 23])
-@pytest.mark.parametrize("S,K", [(24, 6), (16, 0), (40, 0), (64, 0)])
+@pytest.mark.parametrize("S,K", [(24, 6), (16, 0), (40, 0), (30, 0), (64, 0)])
 def test_largest_transition_entry(galv, top, S, K):
     for time_hi in (50, 60_000_000):
         w = inputs.random_tables(S + top % 97, 4, 6, S, 900, ragged=True, mem_lo=0, mem_hi=150, time_hi=time_hi, trans_hi=top)
@@ -78,16 +81,16 @@ def test_largest_transition_entry(galv, top, S, K):
             for i in range(w.B):
                 w.trans_q[i] = rng.integers(0, top + 1, (K, K), np.int32)[rng.integers(0, K, S)][:, rng.integers(0, K, S)]
         w.trans_q[:, 0, S - 1] = top
-        for flags in (0,):
-            against_reference(galv, w, flags)
+        against_reference(galv, w, path=S < 64 or top <= 65535)  # 64 rows of 32-bit differences: no room
 
 
 @pytest.mark.parametrize("block", range(6))
 def test_against_reference_kernel_on_many_shapes(galv, block):
     rng = np.random.default_rng(7700 + block)
+    ran = 0
     for case in range(14):
         S = int(rng.choice([1, 3, 8, 13, 16, 17, 24, 32, 40, 64, 100, 128]))
-        Lmax, M, B = int(rng.integers(1, 14)), int(rng.integers(0, 4000)), int(rng.choice([1, 2, 5, 16, 40, 130, 200]))
+        Lmax, M, B = int(rng.choice([1, 2, 5, 9, 13, 40])), int(rng.integers(0, 4000)), int(rng.choice([1, 2, 5, 16, 40, 130, 200]))
         kw = dict(ragged=bool(rng.integers(0, 2)), mem_lo=0, mem_hi=int(rng.choice([0, 5, M // 30 + 1, M // 4 + 1, M + 50, 3 * M + 1])),
                   time_hi=int(rng.choice([5, 10 ** 4, 10 ** 6])))
         K = int(rng.choice([0, 1, 4, 8, 16]))
@@ -97,7 +100,8 @@ def test_against_reference_kernel_on_many_shapes(galv, block):
             w.time_q[:, 2] = w.time_q[:, 1]; w.mem_q[:, 2] = w.mem_q[:, 1]         # layers with the same rows share their records
         if rng.integers(0, 4) == 0 and B * Lmax * S * S < 4_000_000:
             w.trans_q = np.ascontiguousarray(rng.integers(0, 3000, (B, Lmax, S, S), np.int32))
-        against_reference(galv, w, 0)
+        ran += against_reference(galv, w, path=False)
+    assert ran >= 7                                              # most of the shapes were searched by this kernel alone
 
 
 @pytest.mark.parametrize("S,K,top", [(64, 7, 2000), (24, 4, 50000), (40, 0, 900), (30, 0, 60000), (12, 0, 90000), (48, 8, 300000), (2, 0, 9), (1, 0, 9)])
@@ -233,3 +237,137 @@ def test_path_word(galv):
     w = classed(62, 5, 40, 24, 900, 4, 5, **kw)
     assert path_of(galv, w, gb.KERNEL_RESIDENT) == gb.PATH_CLUSTER and path_of(galv, w, gb.KERNEL_CLUSTER) == gb.PATH_CLUSTER
     assert path_of(galv, w, gb.KERNEL_NO_CLUSTER) == gb.PATH_TILED_PACKED and path_of(galv, w, gb.STORE_C_FULL | gb.KERNEL_SOLO) == gb.PATH_CLUSTER
+
+
+@pytest.mark.parametrize("S,M,B,Lmax,path", [(40, 1500, 9, 20, "PATH_SOLO"),        # everything fits
+                                             (100, 1100, 9, 20, "PATH_CLUSTER"),   # unstructured ones do not: the pushing kernel beside the resident one
+                                             (32, 3600, 12, 20, "PATH_CLUSTER"),   # ... the resident one, which has room for them
+                                             (64, 2500, 160, 6, "PATH_TILED_PACKED"), (72, 2500, 160, 6, "PATH_TILED_32")])    # ... the tiled ones
+def test_one_batch_for_several_kernels(galv, S, M, B, Lmax, path):
+    """Structured, unstructured and flagged instances in one batch; the solo kernel takes what fits, the kernels behind the rest
+    and nothing else.  The same buffers again and again without a pause, the matrices changing places."""
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    rng = np.random.default_rng(S)
+    sets = []
+    for k in range(2):
+        w = classed(40 + S + k, B, Lmax, S, M, 5, 6, ragged=True, mem_lo=0, mem_hi=M // 20)
+        for i in range(k, B, 3):
+            w.trans_q[i] = rng.integers(0, 3000, (S, S), np.int32)
+        w.time_q[2, 0, 0] = -1
+        w.L[4], w.L[5] = 0, Lmax + 1
+        w.L[0] = w.L[1] = w.L[7] = Lmax
+        ref = reference(galv, w)
+        assert ref.status.cpu().numpy()[[2, 4, 5]].tolist() == [2, 2, 2]
+        sets.append((w, ref))
+    one = SearchBuffers(galv, sets[0][0], gb.KERNEL_SOLO)
+    got = []
+    for n in range(8):
+        w, ref = sets[n % 2]
+        for name in ("time_q", "mem_q", "trans_q", "L"):
+            getattr(one, name).copy_(getattr(ref, name))
+        one.C_last.fill_(77)
+        one.dp_search(); one.backtrack()
+        got.append([t.clone() for t in (one.status, one.opt_cost, one.C_last)])
+    torch.cuda.synchronize()
+    assert galv.galv_dp_search_path(one.shape, one.workspace) == getattr(gb, path)
+    for n, (status, opt, last) in enumerate(got):
+        one.status, one.opt_cost, one.C_last = status, opt, last
+        same(one, sets[n % 2][1], n)
+
+
+def spread(w, seed, near=False):
+    """Measured layer times: half a millisecond, half of it a standard deviation, or all of them within a thousandth."""
+    w.time_q[:] = np.rint(5e5 * np.exp(0.5 * np.random.default_rng(seed).standard_normal(w.time_q.shape))).astype(np.int32)
+    if near:
+        w.time_q[:] = 500000 + w.time_q // 1000
+    return w
+
+
+@pytest.mark.parametrize("S,K,B,Lmax,M", [(24, 0, 300, 30, 3000), (64, 7, 160, 40, 4000), (64, 5, 600, 24, 2880), (12, 0, 200, 40, 3000)])
+def test_unasked(galv, S, K, B, Lmax, M):
+    """Without a flag, more instances than SMs (600: more than are sorted by length), stacks of 24 to 40 layers: batches whose times
+    are far apart are taken, batches whose times lie close together are not, flagged instances or not; the results are the same."""
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    for near in (False, True):
+        kw = dict(ragged=B == 600, mem_lo=M // (6 * Lmax), mem_hi=3 * M // Lmax)
+        w = spread(classed(S, B, Lmax, S, M, K, K, **kw) if K else inputs.random_tables(S, B, Lmax, S, M, trans_hi=2000, **kw), S, near)
+        w.mem_q[1, 2, :] = M + 1                                 # nothing fits
+        w.L[0], w.L[B - 1] = 0, Lmax + 1
+        w.time_q[B // 2, 0, 0] = -1
+        one = SearchBuffers(galv, w, 0)
+        one.C_last.fill_(77)
+        one.dp_search(); one.backtrack()
+        same(one, reference(galv, w), near)
+        assert (galv.galv_dp_search_path(one.shape, one.workspace) == gb.PATH_SOLO) == (not near), near
+
+
+def test_host_plans_unasked(galv):
+    """The host entry point without a flag, where it takes the solo kernel's states, and where it does not."""
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import HostSearch, SearchBuffers
+    for B, Lmax, near in ((130, 60, False), (130, 60, True), (200, 14, False)):
+        w = spread(classed(B, B, Lmax, 32, 8000, 6, 7, ragged=True, mem_lo=8000 // (6 * Lmax), mem_hi=24000 // Lmax), B, near)
+        w.L[3] = 0
+        ref = SearchBuffers(galv, w, gb.STORE_ARGMIN | gb.KERNEL_NO_CLUSTER)
+        ref.dp_search(); ref.backtrack()
+        want = ref.results()
+        del ref
+        hs = HostSearch(galv, w, gb.STORE_C_FULL)
+        res = hs.run()
+        for k in ("status", "opt_cost", "plan", "mem_used"):
+            assert (res[k] == want[k]).all(), (k, B, near)
+
+
+@pytest.mark.parametrize("flags", ["KERNEL_SOLO", None])
+def test_in_a_graph(galv, flags):
+    """Captured with what stands behind it: replays with changing matrices and times equal plain calls, whoever takes them."""
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    f = getattr(gb, flags) if flags else 0
+    w = spread(classed(77, 200, 24, 40, 2000, 4, 4, mem_lo=14, mem_hi=250), 3)
+    plain, one = SearchBuffers(galv, w, f), SearchBuffers(galv, w, f)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        one.dp_search(); one.backtrack()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            one.dp_search(); one.backtrack()
+    rng = np.random.default_rng(3)
+    near, far = (torch.from_numpy(spread(w, 3, n).time_q.copy()) for n in (True, False))
+    paths = set()
+    for k in range(6):
+        x = torch.from_numpy(np.ascontiguousarray(w.trans_q if k % 2 else rng.integers(0, 3000, w.trans_q.shape, np.int32)))
+        for sb in (plain, one):
+            sb.trans_q.copy_(x)
+            sb.time_q.copy_(near if k // 2 == 1 else far)
+        torch.cuda.synchronize()
+        plain.dp_search(); plain.backtrack()
+        g.replay()
+        torch.cuda.synchronize()
+        path = galv.galv_dp_search_path(one.shape, one.workspace)
+        assert path == galv.galv_dp_search_path(plain.shape, plain.workspace)
+        paths.add(path)
+        assert torch.equal(plain.C_last, one.C_last) and torch.equal(plain.opt_cost, one.opt_cost) and torch.equal(plain.status, one.status), k
+    assert gb.PATH_SOLO in paths and len(paths) > 1 - bool(flags)
+    del g
+
+
+def test_in_the_library_s_own_scratch(galv):
+    """galv_dp_search_static: no table, so the scratch has to hold two layers whichever kernel runs; flagged instances among them."""
+    import torch
+    from paper_2504_03662_b200 import binding as gb
+    from paper_2504_03662_b200.search import SearchBuffers
+    for seed in (1, 2):
+        w = classed(seed, 7, 12, 9, 900, 4, 4, ragged=True, mem_lo=0, mem_hi=80)
+        w.time_q[seed, 0, 0] = -3
+        one = SearchBuffers(galv, w, gb.KERNEL_SOLO)
+        one.workspace = None
+        one.C_last.fill_(77)
+        galv.galv_dp_search_static(one.shape, one.L, one.time_q, one.mem_q, one.trans_q, one.C, one.A, one.C_last, one.status)
+        one.backtrack()
+        same(one, reference(galv, w), seed)
