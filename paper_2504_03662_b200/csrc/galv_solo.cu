@@ -588,8 +588,8 @@ __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
 {
     constexpr int NW = kGuessThreads / 32, kRows = 4;          // rows of the matrix a warp looks at together
     __shared__ uint32_t s_row[kMaxS + kRows * NW], s_col[kMaxS];
-    __shared__ int s_kind[kMaxS];
-    __shared__ int4 s_at[kGuessLayers][kMaxS];                 // mem, time, kind of the strategy
+    __shared__ int s_next[kMaxS];                              // the next strategy of the same row and column, round and round
+    __shared__ int2 s_at[kGuessLayers][kMaxS];                 // mem, time
     __shared__ float2 s_point[kGuessLayers][kMaxS];            // time, mem; +inf where it does not fit or another one of its kind is as good
     __shared__ float s_time[NW], s_mem[NW];
     __shared__ int s_tmax, s_kinds[2], s_listed, s_mmax, s_pass[kSlopes], s_used[kSlopes];
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
         for (int x = tid; x < layers * S; x += kGuessThreads) {
             const int q = x / S, s = x - q * S;
             const size_t at = ((size_t)i * a.Lmax + layer_of(q)) * S + s;
-            const int4 me = make_int4(a.mem_q[at], a.time_q[at], s, 0);
+            const int2 me = make_int2(a.mem_q[at], a.time_q[at]);
             s_at[q][s] = me;
             atomicAdd(&s_rows[q], ((uint32_t)me.x * 0x85EBCA6Bu + (uint32_t)me.y) * ((uint32_t)s * 0x9E3779B2u + 0x7F4A7C15u));
             time += (float)me.y; mem += (float)min(me.x, M);
@@ -660,35 +660,33 @@ __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
         if (lane == 0) atomicMax(&s_tmax, tmax);
     }
     __syncthreads();
-    if (!a.trans_layer && tid < S) {                            // the first strategy of the same row, of the same column, of both
+    if (!a.trans_layer && tid < S) {                            // the first ones of their rows and of their columns, and who shares both
         const uint32_t hr = s_row[tid], hc = s_col[tid];
-        int row = tid, col = tid, both = tid;
+        int row = 0, col = 0, both = tid, next = -1;
 #pragma unroll 4
-        for (int o = tid - 1; o >= 0; --o) {
+        for (int o = S - 1; o >= 0; --o) {
             const bool r = s_row[o] == hr, c = s_col[o] == hc;
-            if (r) row = o;
-            if (c) col = o;
-            if (r && c) both = o;
+            row += r && o < tid;
+            col += c && o < tid;
+            if (r && c) { both = o; if (o > tid) next = o; }
         }
-        s_kind[tid] = both;
-        if (row == tid) atomicAdd(&s_kinds[0], 1);
-        if (col == tid) atomicAdd(&s_kinds[1], 1);
+        s_next[tid] = next < 0 ? both : next;
+        if (row == 0) atomicAdd(&s_kinds[0], 1);
+        if (col == 0) atomicAdd(&s_kinds[1], 1);
     }
     __syncthreads();
     const bool classes = !a.trans_layer && max(s_kinds[0], s_kinds[1]) <= kClassMax;
     const int Kr = classes ? s_kinds[0] : S, Kc = classes ? s_kinds[1] : S;
     for (int x = tid; x < layers * S; x += kGuessThreads) {
         const int q = x / S, s = x - q * S;
-        const int4 me = s_at[q][s];
+        const int2 me = s_at[q][s];
         bool in = me.x <= M;
-        if (classes && in) {
-            const int kind = s_kind[s];
-#pragma unroll 4
-            for (int o = 0; o < S; ++o) {
-                const int4 ot = s_at[q][o];
-                in &= !(s_kind[o] == kind && ot.x <= me.x && ot.y <= me.y && (o < s || ot.y < me.y));
+        if (classes)
+#pragma unroll 1
+            for (int o = s_next[s]; in && o != s; o = s_next[o]) {
+                const int2 ot = s_at[q][o];
+                in = ot.x > me.x || ot.y > me.y || (o > s && ot.y == me.y);
             }
-        }
         s_point[q][s] = in ? make_float2((float)me.y, (float)me.x) : make_float2(__uint_as_float(0x7f800000u), 0.0f);
         if (in) { atomicAdd(&s_listed, 1); atomicMax(&s_mmax, me.x); }
     }
