@@ -257,7 +257,7 @@ int galv_dp_search_path(galv_ctx* ctx, const galv_shape* sh, const void* workspa
     cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
     if (e == cudaSuccess) e = cudaMemcpy(flags, static_cast<const char*>(workspace) + w.err, sizeof(flags), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(ctx, "galv_dp_search_path", e);
-    *packed = flags[3];
+    *packed = (flags[3] & kPathRest) ? kPathCluster : flags[3];
     return GALV_OK;
 }
 

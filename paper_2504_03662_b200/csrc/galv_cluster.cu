@@ -462,7 +462,6 @@ __global__ void __launch_bounds__(416, 1) cluster_search_kernel(const ClArgs a, 
         bulk_wait_all();
     }
     resident_over();
-    if (a.after_solo && rank == 0 && tid == 0) a.path[3] = kPathCluster;
 }
 
 }  // namespace

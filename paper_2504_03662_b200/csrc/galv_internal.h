@@ -9,7 +9,9 @@
 #include "galv.h"
 
 constexpr int kStateHalf = 1 << 16, kStateWord = 1 << 17;      // DpArgs::lean_map: states of bases and 16-bit (two rows a word) or 32-bit differences
-constexpr int kPathCluster = 2, kPathSolo = 3;                // what galv_dp_search_path says beside the tiled kernels' 1 (packed) and 0
+// Which kernel ran: 1 the tiled kernels' packed loop, 0 their 32-bit one, these two, and with kPathRest the solo kernel has left something to
+// the cluster kernels behind it (the tiled ones write their own).
+constexpr int kPathCluster = 2, kPathSolo = 3, kPathRest = 4;
 constexpr int kResidentClassMax = 16;      // classes beyond which a matrix counts as unstructured in the resident kernel
 
 // How the resident kernel (one thread-block cluster per instance, the state between layers in shared memory) cuts an instance.
@@ -29,7 +31,7 @@ struct RsPlan {
     double est;    // estimated SM cycles per layer, all rounds of clusters
 };
 
-// What a layer of a batch costs in the other kernels, in SM cycles for each round of instances on the solo kernel.
+// What a layer of a batch costs in the other kernels, in SM cycles, and what the solo kernel's own multiplies with.
 struct SoOther {
     float resident;       // matrices of few classes, by the resident kernel's plan
     int gints, w;         // ... its room and columns (w = 0: it does not take them)
@@ -37,7 +39,9 @@ struct SoOther {
     float tiled;          // the tiled kernels, for a cycle of a column group
     int packed;           // ... their packed loop is possible
     float most;           // the pushing kernel, or the resident one for any matrix
-    float start;          // of the solo kernel's own start, for a layer
+    float rounds;         // of instances on the solo kernel
+    float start;          // its own start, once
+    int one_round, other_one_round;        // all instances run at once, here, in the resident kernel
 };
 
 // How the solo kernel (an instance's state on one SM) cuts a batch.
@@ -128,7 +132,7 @@ struct DpArgs {
                          // neither the resident nor the solo kernel was launched.
                          // Lies over tile_done: read until the schedule is made
     int withhold;        // test hook: CTA 0 never loads its first chunk, so that the bounded waits run out
-    int after_solo;      // the solo kernel has run: done[] = 3 are its own, and the word that says which kernel ran until another one searches something
+    int after_solo;      // the solo kernel has run: done[] = 3 are its own
     int beside;          // the pushing kernel may start beside the kernel in front, the resident one
     int skip_dom;        // leave out rows (packed path: row pairs) that cannot win in any column of a warp group's tile
     int dom_auto;        // ... where a quarter of the rows or more look it (maxmem[4])

@@ -56,7 +56,6 @@ struct RsArgs {
     int SP;            // row pitch of the full transition matrix in shared memory; 0: no room for unstructured matrices
     int sorted;        // clusters take the instances longest first
     int second;        // only the instances earlier launches left alone
-    int after_solo;    // the solo kernel's among them: the path flag is that one's until this kernel searches something
     int probed;        // done[] says which matrices are unstructured
     int follow, k_max;             // see RsPlan
     int withhold;      // test hook: a cluster's first CTA keeps the halo of layer 0 to itself, so that the waits for it run out
@@ -787,7 +786,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     int32_t* const stage_rows = reinterpret_cast<int32_t*>(smem_raw) + a.stage_at;         // [2][S][W] rows on their way to the table
     uint8_t* const a0 = reinterpret_cast<uint8_t*>(raw + 8 * ((S + 3) & ~3));                           // [2][gints] argmin of the state
 
-    if (blockIdx.x == 0 && tid == 0 && !a.after_solo) a.path[3] = ARG ? 0 : kPathCluster;
+    if (blockIdx.x == 0 && tid == 0 && !a.second) a.path[3] = ARG ? 0 : kPathCluster;
     if (a.follow) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");    // the pushing kernel may start beside this one
 
     // ---- which instance: clusters are dispatched in order, so the longest instances go first
@@ -1040,10 +1039,7 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
     // a multiple of 32.  Below column 0 it holds +inf.
     const int H = max(0, min((s_all.mmax + 31) & ~31, (gints / Kc - W) & ~31)), P = W + H;
 
-    if (rank == 0 && tid == 0) {
-        a.status[i] = st; a.done[i] = st != 0 || run;
-        if (run && a.after_solo) a.path[3] = kPathCluster;
-    }
+    if (rank == 0 && tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run; }
 
     const int n_all = classes ? s_first[Kr] : S;
     const bool strict = s_all.mmax > H;                         // some shift reaches beyond the halo
@@ -1459,7 +1455,7 @@ cudaError_t galv_resident_launch(const RsPlan& p, int second, const DpArgs& d, c
 {
     RsArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
-    a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second; a.after_solo = d.after_solo; a.withhold = d.withhold;
+    a.CL = p.cl; a.W = p.w; a.gints = p.gints; a.sorted = p.sorted; a.second = second; a.withhold = d.withhold;
     a.follow = p.follow; a.k_max = p.k_max;
     a.probed = !p.dense && galv_probe_applies(d) && second == d.after_solo && !p.follow;       // the first launch of this kernel
     if (a.probed) galv_probe_matrices(d, st);

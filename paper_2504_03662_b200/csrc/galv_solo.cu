@@ -52,8 +52,10 @@ struct SoArgs {
     int sorted;        // CTA c takes the c-th longest instance
     int dense;         // unstructured matrices are searched here (else left to the kernels behind)
     int packed;        // packed relaxations are allowed
+    int certain;       // nothing is left to the kernels behind
     int guessed;       // entries of `guess`; 0: every instance that fits is searched
-    const int32_t* guess;
+    int one_round, other_one_round;        // see SoOther
+    const float2* guess;
     const int32_t* L;
     const int32_t* time_q;
     const int32_t* mem_q;
@@ -534,17 +536,20 @@ __device__ __forceinline__ void run(const Ctx& c, int warp, int lane)
     else run_layers<KC, 1, F>(c, warp, lane);
 }
 
-// What a step of tiles costs here, in SM cycles: by how many strategies pass the test at a column group, and how many are listed.
-// Fitted on B200 to 400 shapes of analytic and of measured tables: unstructured matrices to 10 %, classes, whose tiles of several
-// groups go by their worst one, to 30 % for the most part.  states: they are written too.
-__host__ __device__ inline float step_cycles(int KC, bool word, bool states, float alive, float listed)
+// What a step of tiles costs here, in SM cycles: by how many strategies are listed, how many of them pass the test at a column group,
+// and the share of tiles that are shared out group by group (and how many pass there).  Fitted on B200 to 460 shapes of analytic and
+// of measured tables: tiles of one group to 15 %, of several groups to 25 % for the most part, below 700 columns to a factor of two.
+// fill: the share of a step's column groups that there are.  states: they are written too.
+struct Passing { float listed, alive, shared, shared_alive; };
+__host__ __device__ inline float step_cycles(int KC, bool word, bool states, const Passing& p, float fill)
 {
-    if (listed > 64.0f) alive += listed - 64.0f;               // beyond the 64th of a list all of them pass
-    const float t = KC == 8    ? 1000.0f + 110.0f * listed + 1100.0f * alive
-                    : KC == 16 ? 600.0f + 60.0f * listed + 1300.0f * alive
-                    : KC == 32 ? 2000.0f + 640.0f * alive
-                               : 2400.0f + 1700.0f * alive;
-    return t * (word ? 1.25f : 1.0f) + (states ? 2500.0f : 0.0f);
+    const float past = p.listed > 64.0f ? p.listed - 64.0f : 0.0f, alive = p.alive + past;      // beyond the 64th of a list all of them pass
+    const float shared_alive = p.shared_alive + past * p.shared;
+    const float t = KC == 8    ? 1950.0f + 24.0f * p.listed + 210.0f * alive + (5600.0f * p.shared + 1320.0f * shared_alive) * fill
+                    : KC == 16 ? 2280.0f + 26.0f * p.listed + 3000.0f * p.shared + 550.0f * shared_alive + 100.0f * alive
+                    : KC == 32 ? 430.0f + 51.0f * p.listed + 640.0f * alive
+                               : 2480.0f + 32.0f * p.listed + 1055.0f * alive;
+    return t * (word ? 1.9f : 1.0f) + (states ? 2500.0f : 0.0f);
 }
 
 // What a layer costs a column group and an SM in the tiled kernels, which take unstructured matrices of large batches (to 12 %): the
@@ -557,8 +562,8 @@ __host__ __device__ inline float tiled_cycles(int S, bool packed, float alive)
 // 3.5: a warp prepares each one's records), and what a strategy and column group of a warp adds where shifts pass the halo (40 to 230).
 constexpr float kResidentRepeats = 1.2f, kResidentDiffers = 1.7f, kResidentPastHalo = 60.0f;
 
-// Whether a batch is worth the solo kernel: what it would cost there over what it costs elsewhere, in units of 1 / kGuessUnit,
-// for up to kGuessed of its instances; -1: an instance that is not searched at all.
+// Whether a batch is worth the solo kernel: the SM cycles it would take there, and elsewhere, if all its instances were like one, for up
+// to kGuessed of them; -1: an instance that is not searched at all.
 //
 // What it costs hangs on how many strategies pass the test at a column group, which is guessed from a few layers' rows.  Where C
 // falls by `slope` a column a strategy weighs time + slope * mem, and passes if that is within the largest transition entry of the
@@ -569,20 +574,22 @@ constexpr float kResidentRepeats = 1.2f, kResidentDiffers = 1.7f, kResidentPastH
 // One answer for the batch, as a mixed one pays for both kernels in turn (100 instances of 40 layers, S = 24 of 3000 columns, some of
 // them taken: 1044 us against 542 and 575).  A kernel of its own, as the solo kernel's start is 20 thousand cycles, most of them
 // spent on fetching its code: a batch that is turned away pays 15 to 20 us.  Taken where the guess leaves a tenth.
-// Without / with it, us: 2 instances of 96 layers of an analytic model, S = 60 of 2880 columns 2470 / 325 (resident kernel 307); 31 of
-// 90, S = 20 of 8192 1885 / 804; 200 of 40, S = 64 of 4 classes, transitions twice the layer times 2700 / 1160; 16 of 48 measured layers,
-// S = 32 of 2048 457 / 235; taken: 200 of 40, S = 64 of 7 classes 2195 before it / 439; 300 of 30 measured, S = 24 of 3000 1529 / 830.
-constexpr int kGuessed = 32, kGuessUnit = 1024, kGuessTaken = 920, kGuessMost = 1 << 20, kGuessThreads = 512, kGuessLayers = 8, kSlopes = 6;
+// Other kernels / solo kernel / with this rule, us: 64 instances of 60 layers of an analytic model, S = 32 of 2880 columns 278 / 482 / 295;
+// 200 of 40, S = 64 of 4 classes and 4000 columns, transitions twice the layer times 1143 / 2700 / 1165; 200 of 40 of an analytic model,
+// S = 64 of 2880 columns 2195 / 421 / 436; 300 of 30 measured, S = 24 of 3000 1529 / 799 / 825; host entry point, 130 of 60, S = 32 of 8192
+// 4563 / 2159 / 2176.
+constexpr int kGuessed = 32, kGuessThreads = 512, kGuessLayers = 8, kSlopes = 6;
+constexpr float kGuessTaken = 0.9f, kGuessNoRoom = 1e30f;
 struct GuessArgs {
     int B, Lmax, S, M, n;
-    int nw, groups, dense, states;
+    int nw, groups, dense, states, room;
     SoOther other;
     const int32_t* L;
     const int32_t* time_q;
     const int32_t* mem_q;
     const int32_t* trans_q;
     long long trans_inst, trans_layer;
-    int32_t* guess;
+    float2* guess;
 };
 __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
 {
@@ -592,20 +599,20 @@ __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
     __shared__ int2 s_at[kGuessLayers][kMaxS];                 // mem, time
     __shared__ float2 s_point[kGuessLayers][kMaxS];            // time, mem; +inf where it does not fit or another one of its kind is as good
     __shared__ float s_time[NW], s_mem[NW];
-    __shared__ int s_tmax, s_kinds[2], s_listed, s_mmax, s_pass[kSlopes], s_used[kSlopes];
+    __shared__ int s_tmax, s_kinds[2], s_listed, s_mmax, s_pass[kSlopes], s_used[kSlopes], s_shared[kSlopes], s_shared_pass[kSlopes];
     __shared__ uint32_t s_rows[kGuessLayers];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, S = a.S, M = a.M;
     const int i = a.n > 1 ? (int)((long long)blockIdx.x * (a.B - 1) / (a.n - 1)) : 0;
     const int Li = a.L[i];
     if (Li < 1 || Li > a.Lmax) {
-        if (tid == 0) a.guess[blockIdx.x] = -1;
+        if (tid == 0) a.guess[blockIdx.x] = make_float2(-1.0f, -1.0f);
         return;
     }
     const int32_t* const T = a.trans_q + (size_t)i * a.trans_inst;
     const int layers = min(Li, kGuessLayers);
     auto layer_of = [&](int q) { return layers > 1 ? (int)((long long)q * (Li - 1) / (layers - 1)) : 0; };
     if (tid < S) s_col[tid] = 0;
-    if (tid < kSlopes) { s_pass[tid] = 0; s_used[tid] = 0; }
+    if (tid < kSlopes) { s_pass[tid] = 0; s_used[tid] = 0; s_shared[tid] = 0; s_shared_pass[tid] = 0; }
     if (tid < kGuessLayers) s_rows[tid] = 0;
     if (tid == 0) { s_tmax = 0; s_kinds[0] = 0; s_kinds[1] = 0; s_listed = 0; s_mmax = 0; }
     __syncthreads();
@@ -677,6 +684,7 @@ __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
     __syncthreads();
     const bool classes = !a.trans_layer && max(s_kinds[0], s_kinds[1]) <= kClassMax;
     const int Kr = classes ? s_kinds[0] : S, Kc = classes ? s_kinds[1] : S;
+    const int KC = Kc <= 8 && Kr <= 16 ? 8 : Kc <= 16 ? 16 : Kc <= 32 ? 32 : 64;
     for (int x = tid; x < layers * S; x += kGuessThreads) {
         const int q = x / S, s = x - q * S;
         const int2 me = s_at[q][s];
@@ -702,50 +710,61 @@ __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
         const float slope = k == 0 ? 0.0f : scale * (float)(1 << 2 * k) * 0.0078125f;       // 0, 1/32, 1/8, .. 8 times
         const uint32_t none = 0x7f800000u;                     // +inf as bits: sorts behind every weight
         uint32_t best = none, used = 0x7fffffffu;
-        int pass = 0;
+        int pass = 0, tile = 0;
 #pragma unroll 1
         for (int s = lane; s < S; s += 32) best = min(best, __float_as_uint(__fmaf_rn(slope, s_point[q][s].y, s_point[q][s].x)));
         best = __reduce_min_sync(0xffffffffu, best);
-        const float limit = __uint_as_float(best) + (float)s_tmax + 32.0f * slope;
+        const float limit = __uint_as_float(best) + (float)s_tmax + 32.0f * slope, tile_limit = limit + 32.0f * (float)(max_tile(KC) - 1) * slope;
 #pragma unroll 1
         for (int s = lane; s < S; s += 32) {
             const float2 p = s_point[q][s];
             const float v = __fmaf_rn(slope, p.y, p.x);
             pass += __float_as_uint(v) != none && v <= limit;
+            tile += __float_as_uint(v) != none && v <= tile_limit;
             if (__float_as_uint(v) == best) used = min(used, (uint32_t)p.y);
         }
         pass = __reduce_add_sync(0xffffffffu, pass);
+        tile = __reduce_add_sync(0xffffffffu, tile);
         used = __reduce_min_sync(0xffffffffu, used);
-        if (lane == 0 && best != none) { atomicAdd(&s_pass[k], pass); atomicAdd(&s_used[k], (int)used); }
+        if (lane == 0 && best != none) {
+            atomicAdd(&s_pass[k], pass); atomicAdd(&s_used[k], (int)used);
+            if (tile > 4) { atomicAdd(&s_shared[k], 1); atomicAdd(&s_shared_pass[k], pass); }      // see tile
+        }
     }
     __syncthreads();
     if (tid != 0) return;
     // ---- layers and columns below the line column = layer * mem, slope by slope
     const float cols = (float)(M + 1), deep = (float)Li, all = cols * deep, per = 1.0f / (float)layers;
-    float left = all, sum = 0.0f, before = 0.0f;
+    Passing sum{(float)s_listed * per, 0.0f, 0.0f, 0.0f};
+    float left = all;
 #pragma unroll 1
     for (int k = 0; k < kSlopes; ++k) {
-        const float mem = (float)s_used[k] * per, pass = (float)s_pass[k] * per;
+        const float mem = (float)s_used[k] * per;
         const float below = fminf(left, mem * deep <= cols ? 0.5f * mem * deep * deep : all - 0.5f * cols * cols / mem);
-        sum += (left - below) * (k == 0 ? pass : 0.5f * (pass + before));
-        left = below; before = pass;
+        const float weight = (left - below) / all * per * (k == 0 ? 1.0f : 0.5f);
+        const int b = max(k - 1, 0), both = k > 0;             // between a slope and the one before it: half of each
+        sum.alive += weight * (float)(s_pass[k] + both * s_pass[b]);
+        sum.shared += weight * (float)(s_shared[k] + both * s_shared[b]);
+        sum.shared_alive += weight * (float)(s_shared_pass[k] + both * s_shared_pass[b]);
+        left = below;
     }
-    const float alive = sum / all, listed = (float)s_listed * per;
-    const int KC = Kc <= 8 && Kr <= 16 ? 8 : Kc <= 16 ? 16 : Kc <= 32 ? 32 : 64, step = a.nw * max_tile(KC);
-    const float cost = (float)((a.groups + step - 1) / step) * step_cycles(KC, s_tmax > 65535, a.states, alive, listed) + a.other.start;
+    const int step = a.nw * max_tile(KC), steps = (a.groups + step - 1) / step;
+    const float cost = a.other.rounds * (float)steps * step_cycles(KC, s_tmax > 65535, a.states, sum, (float)a.groups / (float)(steps * step));
     float other;
     if (classes && a.other.w && Kc * a.other.w <= a.other.gints) {
         bool repeats = layers < kGuessLayers;
         for (int q = 1; q < layers; ++q)
             for (int o = 0; o < q; ++o) repeats |= s_rows[o] == s_rows[q];
         other = a.other.resident * (repeats ? kResidentRepeats : kResidentDiffers);
-        if (s_mmax > ((a.other.gints / Kc - a.other.w) & ~31)) other += a.other.past_halo * listed;
+        if (s_mmax > ((a.other.gints / Kc - a.other.w) & ~31)) other += a.other.past_halo * sum.listed;
     } else {
-        other = a.other.tiled * tiled_cycles(S, a.other.packed && s_tmax <= 32767, alive);
+        other = a.other.tiled * tiled_cycles(S, a.other.packed && s_tmax <= 32767, sum.alive);
     }
     other = fminf(other, a.other.most);
-    const bool fits = classes || a.dense;
-    a.guess[blockIdx.x] = fits && cost < other * (float)(kGuessMost / kGuessUnit) ? (int)(cost / other * (float)kGuessUnit) : kGuessMost;
+    // as the solo kernel sees it, but for the largest shift, which is the sampled layers'
+    const long long H = (s_mmax + 31) & ~31, words = s_tmax > 65535 ? Kc : (Kc + 1) >> 1, Mp = 32 * a.groups;
+    const bool fits = (classes || a.dense) && 4 * (H + Mp) + 4 * (H + words * Mp) <= a.room && (!a.states || 1 + words <= S);
+    a.guess[blockIdx.x] = make_float2(fits ? cost * deep + a.other.start : kGuessNoRoom, other * deep);
 }
 
 __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoArgs a)
@@ -769,16 +788,29 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
     int32_t* const tsm = raw + 8 * S4;
     unsigned char* const state = reinterpret_cast<unsigned char*>(tsm + a.mats);
 
-    if (a.guessed) {                                            // the batch as a whole, the same in every CTA
-        int ratio = 0, asked = 0;
-        if (lane < a.guessed) { ratio = a.guess[lane]; asked = ratio >= 0; ratio = max(ratio, 0); }
-        if (__reduce_add_sync(0xffffffffu, ratio) > kGuessTaken * __reduce_add_sync(0xffffffffu, asked)) {
+    if (a.guessed) {
+        // The batch as a whole, the same in every CTA.  Where a round holds all instances the longest one counts, else their sum;
+        // what there is no room for here goes elsewhere afterwards.
+        float2 mine = make_float2(-1.0f, 0.0f);
+        if (lane < a.guessed) mine = a.guess[lane];
+        const bool any = mine.x >= 0.0f, fits = mine.x < kGuessNoRoom;
+        const float none = 0.0f, here = any && fits ? mine.x : none, after = any && !fits ? mine.y : none, other = any ? mine.y : none;
+        auto all = [](float v, bool most) {
+            for (int o = 16; o > 0; o >>= 1) { const float w = __shfl_xor_sync(0xffffffffu, v, o); v = most ? fmaxf(v, w) : v + w; }
+            return v;
+        };
+        const float n = (float)__popc(__ballot_sync(0xffffffffu, any));
+        const float cost = a.one_round ? n * all(here, true) : all(here, false), elsewhere = a.other_one_round ? n * all(other, true) : all(other, false);
+        if (cost + (a.other_one_round ? n * all(after, true) : all(after, false)) > kGuessTaken * elsewhere) {
             if (tid == 0) a.done[blockIdx.x] = 0;
-            if (blockIdx.x == 0 && tid == 0) a.path[3] = kPathCluster;
+            if (blockIdx.x == 0 && tid == 0) a.path[3] = kPathSolo | kPathRest;
             return;
         }
     }
-    if (blockIdx.x == 0 && tid == 0) a.path[3] = kPathSolo;
+    if (blockIdx.x == 0 && tid == 0) {
+        if (a.certain) a.path[3] = kPathSolo;
+        else atomicOr(a.path + 3, kPathSolo);                    // cleared before
+    }
 
     // ---- which instance: CTAs are dispatched in order, so the longest instances go first
     int i = blockIdx.x;
@@ -965,7 +997,10 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
     const int per_warp = max_tile(KC), steps = (G + NW * per_warp - 1) / (NW * per_warp), per_step = (G + steps - 1) / steps;
     const bool run_it = st == 0 && (classes || (a.dense && S <= kDenseMax)) && base_bytes + d_bytes <= a.room && steps * NW <= kMaxTiles &&
                         (!a.states || 1 + words <= S);          // the place of a table row each
-    if (tid == 0) { a.status[i] = st; a.done[i] = st != 0 || run_it ? 3 : 0; }
+    if (tid == 0) {
+        a.status[i] = st; a.done[i] = st != 0 || run_it ? 3 : 0;
+        if (st == 0 && !run_it) atomicOr(a.path + 3, kPathRest);
+    }
     if (!run_it) {
         if (warp == NW) cp_async_wait<0>();                     // nothing may land in shared memory that is no longer ours
         return;
@@ -1189,49 +1224,57 @@ bool galv_solo_plan(const galv_ctx* ctx, const galv_shape* sh, bool states, SoPl
     return false;
 }
 
-// Whether the look at the tables is worth its launch: not for shapes that every batch is better off elsewhere with (most batches of a
-// few instances, whose layers take the other kernels a few thousand cycles), nor for batches that are short everywhere.
+// Whether the look at the tables is worth its launch: not for shapes that every batch is better off elsewhere with, not for a few
+// instances (whose layers take clusters a few thousand cycles; and the look's answers want two words an instance), of a few hundred
+// columns (step_cycles), nor for batches that are short everywhere.
 bool galv_solo_worth(const galv_ctx* ctx, const galv_shape* sh, bool states, int n, const RsPlan resident[2], const ClPlan* pushing, SoPlan* p)
 {
     const int S = sh->S, G = sh->m_pitch / 32;
-    const float rounds = (float)((sh->B + ctx->num_sms - 1) / ctx->num_sms), none = 1e30f;
+    if (sh->B < 2 * kGuessed || sh->M < 1000) return false;
     SoOther& o = p->other;
-    o.start = 10000.0f / (float)sh->Lmax;                      // twenty thousand cycles, of which the others have half
+    // CTAs an SM holds: four warps of 128 registers a scheduler, and its shared memory
+    int per_sm = 16 / (p->nw + 1);
+    if (per_sm > (ctx->smem_optin + 1024) / (p->smem + kStaticSmem + 1024)) per_sm = (ctx->smem_optin + 1024) / (p->smem + kStaticSmem + 1024);
+    const int slots = ctx->num_sms * (per_sm > 1 ? per_sm : 1), rounds = (sh->B + slots - 1) / slots;
+    o.rounds = rounds == 1 ? 1.0f : (float)sh->B / (float)slots + 0.5f;
+    o.one_round = rounds == 1;
+    o.start = 30000.0f;                                        // the look's launch, and half of this kernel's start, the half that the others do not have
     o.packed = S <= 64 && S % 4 == 0 && !(sh->flags & GALV_KERNEL_NO_PACKED);
-    o.tiled = 0.95f * (float)G * (float)sh->B / (float)ctx->num_sms / rounds;
-    o.most = pushing ? 0.9f * (float)pushing->est / rounds : none;
-    if (n && resident[n - 1].dense && 1.5f * (float)resident[n - 1].est / rounds < o.most) o.most = 1.5f * (float)resident[n - 1].est / rounds;
+    // a tile costs about the same whatever part of it there are columns for
+    const int nsg = S < 64 ? (S + 7) / 8 : 8, tile = 16 / nsg * 4, tiles = (sh->M / 32 + tile) / tile * tile;
+    o.tiled = 0.9f * (float)(tiles > G ? tiles : G) * (float)sh->B / (float)ctx->num_sms;
+    o.most = pushing ? 0.9f * (float)pushing->est : 1e30f;
+    if (n && resident[n - 1].dense && 1.5f * (float)resident[n - 1].est < o.most) o.most = 1.5f * (float)resident[n - 1].est;
     if (n && !resident[0].dense) {
         const RsPlan& r = resident[0];
         const int g = r.w / 32;
-        o.resident = (float)r.est / rounds; o.gints = r.gints; o.w = r.w;
-        o.past_halo = kResidentPastHalo * (float)((g + r.nw - 1) / r.nw * r.rounds) / rounds;
+        o.resident = (float)r.est; o.gints = r.gints; o.w = r.w;
+        o.past_halo = kResidentPastHalo * (float)((g + r.nw - 1) / r.nw * r.rounds);
+        o.other_one_round = r.rounds == 1;
     }
-    auto layer = [&](int KC, bool word, float alive, float listed) {
+    auto layer = [&](int KC, bool word, const Passing& pass) {
         const int step = p->nw * max_tile(KC);
-        return (float)((G + step - 1) / step) * step_cycles(KC, word, states, alive, listed) + o.start;
+        return o.rounds * (float)((G + step - 1) / step) * step_cycles(KC, word, states, pass, 1.0f) + o.start / (float)sh->Lmax;
     };
     // No batch of this shape is worth it: few strategies pass, and elsewhere it goes as badly as it can.
     const int KC = S <= 8 ? 8 : S <= 16 ? 16 : S <= 32 ? 32 : 64;
-    const float taken = (float)kGuessTaken / kGuessUnit, few = 0.7f;
+    const float s1 = (float)S, few = 0.7f;
     auto at_most = [&](float a) { return a < o.most ? a : o.most; };
     const float tiled = at_most(o.tiled * (tiled_cycles(S, false, (float)S) > tiled_cycles(S, true, 0.0f) ? tiled_cycles(S, false, (float)S) : tiled_cycles(S, true, 0.0f)));
     const float classes = o.w ? at_most(o.resident * kResidentDiffers + o.past_halo * (float)S) : tiled;
-    p->dense = p->dense && layer(KC, false, few, KC <= 16 ? 0.5f * S : (float)S) <= taken * tiled;
-    const bool some = layer(8, false, few, (float)S / 3.0f) <= taken * classes;
+    p->dense = p->dense && layer(KC, false, Passing{s1, few, 0.0f, 0.0f}) <= kGuessTaken * tiled;
+    const bool some = layer(8, false, Passing{s1 / 3.0f, few, 0.0f, 0.0f}) <= kGuessTaken * classes;
     if (!p->dense && !some) return false;
-    // The look at the batch, 15 us where it is turned away, has to be small beside it: at most 300 us elsewhere, or 100 at best, are
-    // not worth it.
+    // The look at the batch, 15 to 20 us where it is turned away, has to be small beside it.
     const float lowest = o.packed && tiled_cycles(S, true, 0.0f) < tiled_cycles(S, false, 0.0f) ? tiled_cycles(S, true, 0.0f) : tiled_cycles(S, false, 0.0f);
     const float least_tiled = at_most(o.tiled * lowest), least_classes = o.w ? at_most(o.resident * kResidentRepeats) : least_tiled;
-    const float batch = rounds * (float)sh->Lmax;
-    if ((p->dense && (!some || tiled > classes) ? tiled : classes) * batch < 600e3f) return false;
-    if ((some && (!p->dense || least_classes < least_tiled) ? least_classes : least_tiled) * batch < 200e3f) return false;
-    p->guessed = sh->B < kGuessed ? sh->B : kGuessed;
+    if ((p->dense && (!some || tiled > classes) ? tiled : classes) * (float)sh->Lmax < 800e3f) return false;
+    if ((some && (!p->dense || least_classes < least_tiled) ? least_classes : least_tiled) * (float)sh->Lmax < 300e3f) return false;
+    p->guessed = kGuessed;
     // Every batch of this shape is, whatever it holds.
     const float least = least_classes < least_tiled ? least_classes : least_tiled;
     bool all = p->certain && p->dense;
-    for (int k = 8; k <= KC; k <<= 1) all = all && layer(k, true, (float)S, (float)S) <= taken * least;
+    for (int k = 8; k <= KC; k <<= 1) all = all && layer(k, true, Passing{s1, s1, 1.0f, s1}) <= kGuessTaken * least;
     p->certain = all;
     if (all) p->guessed = 0;
     return true;
@@ -1247,10 +1290,10 @@ cudaError_t galv_solo_launch(const SoPlan& p, const DpArgs& d, cudaStream_t st)
     if (p.guessed) {
         GuessArgs g;
         g.B = d.B; g.Lmax = d.Lmax; g.S = d.S; g.M = d.M; g.n = p.guessed;
-        g.nw = p.nw; g.groups = d.m_pitch / 32; g.dense = p.dense; g.states = d.lean_map != nullptr;
+        g.nw = p.nw; g.groups = d.m_pitch / 32; g.dense = p.dense; g.states = d.lean_map != nullptr; g.room = p.room;
         g.other = p.other;
         g.L = d.L; g.time_q = d.time_q; g.mem_q = d.mem_q; g.trans_q = d.trans_q; g.trans_inst = d.trans_inst; g.trans_layer = d.trans_layer;
-        g.guess = d.order;
+        g.guess = reinterpret_cast<float2*>(d.order);
         guess_kernel<<<p.guessed, kGuessThreads, 0, st>>>(g);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -1258,8 +1301,8 @@ cudaError_t galv_solo_launch(const SoPlan& p, const DpArgs& d, cudaStream_t st)
     SoArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
     a.NW = p.nw; a.room = p.room; a.mats = p.mats; a.sorted = p.sorted; a.dense = p.dense;
-    a.guessed = p.guessed; a.guess = d.order;
-    a.packed = p.packed;
+    a.guessed = p.guessed; a.guess = reinterpret_cast<const float2*>(d.order); a.one_round = p.other.one_round; a.other_one_round = p.other.other_one_round;
+    a.packed = p.packed; a.certain = p.certain;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
     a.C_last = d.C_last; a.states = d.lean_map ? reinterpret_cast<uint32_t*>(d.C) : nullptr; a.map = d.lean_map;
