@@ -53,8 +53,7 @@ struct SoArgs {
     int dense;         // unstructured matrices are searched here (else left to the kernels behind)
     int packed;        // packed relaxations are allowed
     int certain;       // nothing is left to the kernels behind
-    int guessed;       // entries of `guess`; 0: every instance that fits is searched
-    int one_round, other_one_round;        // see SoOther
+    int guessed;       // `guess` holds the verdict on the batch; 0: every instance that fits is searched
     const float2* guess;
     const int32_t* L;
     const int32_t* time_q;
@@ -579,7 +578,7 @@ constexpr float kResidentRepeats = 1.2f, kResidentDiffers = 1.7f, kResidentPastH
 // S = 64 of 2880 columns 2195 / 421 / 436; 300 of 30 measured, S = 24 of 3000 1529 / 799 / 825; host entry point, 130 of 60, S = 32 of 8192
 // 4563 / 2159 / 2176.
 constexpr int kGuessed = 32, kGuessThreads = 512, kGuessLayers = 8, kSlopes = 6;
-constexpr float kGuessTaken = 0.9f, kGuessNoRoom = 1e30f;
+constexpr float kGuessTaken = 0.9f, kGuessNoRoom = 1e30f, kGuessAway = -4.0f;
 struct GuessArgs {
     int B, Lmax, S, M, n;
     int nw, groups, dense, states, room;
@@ -590,7 +589,27 @@ struct GuessArgs {
     const int32_t* trans_q;
     long long trans_inst, trans_layer;
     float2* guess;
+    int32_t* ticket;               // 0 before and afterwards
 };
+
+// What the looks at the instances come to, by one warp.  Where a round holds all instances the longest one counts, else their sum;
+// what there is no room for goes elsewhere afterwards.
+__device__ __forceinline__ bool turned_away(const float2* guess, int n, bool one_round, bool other_one_round)
+{
+    const int lane = threadIdx.x & 31;
+    float2 mine = make_float2(-1.0f, 0.0f);
+    if (lane < n) mine = __ldcg(guess + lane);
+    const bool any = mine.x >= 0.0f, fits = mine.x < kGuessNoRoom;
+    const float here = any && fits ? mine.x : 0.0f, after = any && !fits ? mine.y : 0.0f, other = any ? mine.y : 0.0f;
+    auto all = [](float v, bool most) {
+        for (int o = 16; o > 0; o >>= 1) { const float w = __shfl_xor_sync(0xffffffffu, v, o); v = most ? fmaxf(v, w) : v + w; }
+        return v;
+    };
+    const float count = (float)__popc(__ballot_sync(0xffffffffu, any));
+    const float cost = one_round ? count * all(here, true) : all(here, false), elsewhere = other_one_round ? count * all(other, true) : all(other, false);
+    return cost + (other_one_round ? count * all(after, true) : all(after, false)) > kGuessTaken * elsewhere;
+}
+
 __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
 {
     constexpr int NW = kGuessThreads / 32, kRows = 4;          // rows of the matrix a warp looks at together
@@ -601,13 +620,23 @@ __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
     __shared__ float s_time[NW], s_mem[NW];
     __shared__ int s_tmax, s_kinds[2], s_listed, s_mmax, s_pass[kSlopes], s_used[kSlopes], s_shared[kSlopes], s_shared_pass[kSlopes];
     __shared__ uint32_t s_rows[kGuessLayers];
+    __shared__ bool s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, S = a.S, M = a.M;
     const int i = a.n > 1 ? (int)((long long)blockIdx.x * (a.B - 1) / (a.n - 1)) : 0;
     const int Li = a.L[i];
-    if (Li < 1 || Li > a.Lmax) {
-        if (tid == 0) a.guess[blockIdx.x] = make_float2(-1.0f, -1.0f);
-        return;
-    }
+    auto finish = [&](float2 mine) {                           // thread 0's; the CTA that comes last says what they all come to
+        if (tid == 0) {
+            a.guess[blockIdx.x] = mine;
+            __threadfence();
+            s_last = atomicAdd(a.ticket, 1) == a.n - 1;
+        }
+        __syncthreads();
+        if (!s_last || warp != 0) return;
+        __threadfence();
+        const bool away = turned_away(a.guess, a.n, a.other.one_round, a.other.other_one_round);
+        if (lane == 0) { if (away) a.guess[0].x = kGuessAway; *a.ticket = 0; }
+    };
+    if (Li < 1 || Li > a.Lmax) { finish(make_float2(-1.0f, 0.0f)); return; }
     const int32_t* const T = a.trans_q + (size_t)i * a.trans_inst;
     const int layers = min(Li, kGuessLayers);
     auto layer_of = [&](int q) { return layers > 1 ? (int)((long long)q * (Li - 1) / (layers - 1)) : 0; };
@@ -732,39 +761,43 @@ __global__ void __launch_bounds__(kGuessThreads) guess_kernel(const GuessArgs a)
         }
     }
     __syncthreads();
-    if (tid != 0) return;
     // ---- layers and columns below the line column = layer * mem, slope by slope
-    const float cols = (float)(M + 1), deep = (float)Li, all = cols * deep, per = 1.0f / (float)layers;
-    Passing sum{(float)s_listed * per, 0.0f, 0.0f, 0.0f};
-    float left = all;
+    float2 mine = make_float2(-1.0f, 0.0f);
+    if (tid == 0) {
+        const float cols = (float)(M + 1), deep = (float)Li, all = cols * deep, per = 1.0f / (float)layers;
+        Passing sum{(float)s_listed * per, 0.0f, 0.0f, 0.0f};
+        float left = all;
 #pragma unroll 1
-    for (int k = 0; k < kSlopes; ++k) {
-        const float mem = (float)s_used[k] * per;
-        const float below = fminf(left, mem * deep <= cols ? 0.5f * mem * deep * deep : all - 0.5f * cols * cols / mem);
-        const float weight = (left - below) / all * per * (k == 0 ? 1.0f : 0.5f);
-        const int b = max(k - 1, 0), both = k > 0;             // between a slope and the one before it: half of each
-        sum.alive += weight * (float)(s_pass[k] + both * s_pass[b]);
-        sum.shared += weight * (float)(s_shared[k] + both * s_shared[b]);
-        sum.shared_alive += weight * (float)(s_shared_pass[k] + both * s_shared_pass[b]);
-        left = below;
+        for (int k = 0; k < kSlopes; ++k) {
+            const float mem = (float)s_used[k] * per;
+            const float below = fminf(left, mem * deep <= cols ? 0.5f * mem * deep * deep : all - 0.5f * cols * cols / mem);
+            const float weight = (left - below) / all * per * (k == 0 ? 1.0f : 0.5f);
+            const int b = max(k - 1, 0), both = k > 0;             // between a slope and the one before it: half of each
+            sum.alive += weight * (float)(s_pass[k] + both * s_pass[b]);
+            sum.shared += weight * (float)(s_shared[k] + both * s_shared[b]);
+            sum.shared_alive += weight * (float)(s_shared_pass[k] + both * s_shared_pass[b]);
+            left = below;
+        }
+        const int step = a.nw * max_tile(KC), steps = (a.groups + step - 1) / step;
+        const float cost = a.other.rounds * (float)steps * step_cycles(KC, s_tmax > 65535, a.states, sum, (float)a.groups / (float)(steps * step));
+        float other;
+        if (classes && a.other.w && Kc * a.other.w <= a.other.gints) {
+            bool repeats = layers < kGuessLayers;
+            for (int q = 1; q < layers; ++q)
+                for (int o = 0; o < q; ++o) repeats |= s_rows[o] == s_rows[q];
+            other = a.other.resident * (repeats ? kResidentRepeats : kResidentDiffers);
+            if (s_mmax > ((a.other.gints / Kc - a.other.w) & ~31)) other += a.other.past_halo * sum.listed;
+        } else {
+            other = a.other.tiled * tiled_cycles(S, a.other.packed && s_tmax <= 32767, sum.alive);
+        }
+        other = fminf(other, a.other.most);
+        // as the solo kernel sees it, but for the largest shift, which is the sampled layers'
+        const long long H = (s_mmax + 31) & ~31, words = s_tmax > 65535 ? Kc : (Kc + 1) >> 1, Mp = 32 * a.groups;
+        const bool fits = (classes || a.dense) && 4 * (H + Mp) + 4 * (H + words * Mp) <= a.room && (!a.states || 1 + words <= S);
+        mine = make_float2(fits ? cost * deep + a.other.start : kGuessNoRoom, other * deep);
     }
-    const int step = a.nw * max_tile(KC), steps = (a.groups + step - 1) / step;
-    const float cost = a.other.rounds * (float)steps * step_cycles(KC, s_tmax > 65535, a.states, sum, (float)a.groups / (float)(steps * step));
-    float other;
-    if (classes && a.other.w && Kc * a.other.w <= a.other.gints) {
-        bool repeats = layers < kGuessLayers;
-        for (int q = 1; q < layers; ++q)
-            for (int o = 0; o < q; ++o) repeats |= s_rows[o] == s_rows[q];
-        other = a.other.resident * (repeats ? kResidentRepeats : kResidentDiffers);
-        if (s_mmax > ((a.other.gints / Kc - a.other.w) & ~31)) other += a.other.past_halo * sum.listed;
-    } else {
-        other = a.other.tiled * tiled_cycles(S, a.other.packed && s_tmax <= 32767, sum.alive);
-    }
-    other = fminf(other, a.other.most);
-    // as the solo kernel sees it, but for the largest shift, which is the sampled layers'
-    const long long H = (s_mmax + 31) & ~31, words = s_tmax > 65535 ? Kc : (Kc + 1) >> 1, Mp = 32 * a.groups;
-    const bool fits = (classes || a.dense) && 4 * (H + Mp) + 4 * (H + words * Mp) <= a.room && (!a.states || 1 + words <= S);
-    a.guess[blockIdx.x] = make_float2(fits ? cost * deep + a.other.start : kGuessNoRoom, other * deep);
+    __syncwarp();
+    finish(mine);
 }
 
 __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoArgs a)
@@ -788,24 +821,10 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
     int32_t* const tsm = raw + 8 * S4;
     unsigned char* const state = reinterpret_cast<unsigned char*>(tsm + a.mats);
 
-    if (a.guessed) {
-        // The batch as a whole, the same in every CTA.  Where a round holds all instances the longest one counts, else their sum;
-        // what there is no room for here goes elsewhere afterwards.
-        float2 mine = make_float2(-1.0f, 0.0f);
-        if (lane < a.guessed) mine = a.guess[lane];
-        const bool any = mine.x >= 0.0f, fits = mine.x < kGuessNoRoom;
-        const float none = 0.0f, here = any && fits ? mine.x : none, after = any && !fits ? mine.y : none, other = any ? mine.y : none;
-        auto all = [](float v, bool most) {
-            for (int o = 16; o > 0; o >>= 1) { const float w = __shfl_xor_sync(0xffffffffu, v, o); v = most ? fmaxf(v, w) : v + w; }
-            return v;
-        };
-        const float n = (float)__popc(__ballot_sync(0xffffffffu, any));
-        const float cost = a.one_round ? n * all(here, true) : all(here, false), elsewhere = a.other_one_round ? n * all(other, true) : all(other, false);
-        if (cost + (a.other_one_round ? n * all(after, true) : all(after, false)) > kGuessTaken * elsewhere) {
-            if (tid == 0) a.done[blockIdx.x] = 0;
-            if (blockIdx.x == 0 && tid == 0) a.path[3] = kPathSolo | kPathRest;
-            return;
-        }
+    if (a.guessed && a.guess[0].x < kGuessAway * 0.5f) {
+        if (tid == 0) a.done[blockIdx.x] = 0;
+        if (blockIdx.x == 0 && tid == 0) a.path[3] = kPathSolo | kPathRest;
+        return;
     }
     if (blockIdx.x == 0 && tid == 0) {
         if (a.certain) a.path[3] = kPathSolo;
@@ -1293,7 +1312,7 @@ cudaError_t galv_solo_launch(const SoPlan& p, const DpArgs& d, cudaStream_t st)
         g.nw = p.nw; g.groups = d.m_pitch / 32; g.dense = p.dense; g.states = d.lean_map != nullptr; g.room = p.room;
         g.other = p.other;
         g.L = d.L; g.time_q = d.time_q; g.mem_q = d.mem_q; g.trans_q = d.trans_q; g.trans_inst = d.trans_inst; g.trans_layer = d.trans_layer;
-        g.guess = reinterpret_cast<float2*>(d.order);
+        g.guess = reinterpret_cast<float2*>(d.order); g.ticket = reinterpret_cast<int32_t*>(d.work);
         guess_kernel<<<p.guessed, kGuessThreads, 0, st>>>(g);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -1301,7 +1320,7 @@ cudaError_t galv_solo_launch(const SoPlan& p, const DpArgs& d, cudaStream_t st)
     SoArgs a;
     a.B = d.B; a.Lmax = d.Lmax; a.S = d.S; a.M = d.M; a.m_pitch = d.m_pitch;
     a.NW = p.nw; a.room = p.room; a.mats = p.mats; a.sorted = p.sorted; a.dense = p.dense;
-    a.guessed = p.guessed; a.guess = reinterpret_cast<const float2*>(d.order); a.one_round = p.other.one_round; a.other_one_round = p.other.other_one_round;
+    a.guessed = p.guessed; a.guess = reinterpret_cast<const float2*>(d.order);
     a.packed = p.packed; a.certain = p.certain;
     a.L = d.L; a.time_q = d.time_q; a.mem_q = d.mem_q; a.trans_q = d.trans_q;
     a.trans_inst = d.trans_inst; a.trans_layer = d.trans_layer;
