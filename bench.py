@@ -277,7 +277,7 @@ def bench_workload(torch, galv, w, steps, warmup, barrier, flags=1):
     res = sb.results()
     out = {"seconds": t, "ms_per_step": t / steps * 1e3, "cells_per_s": w.cells * steps / t,
            "relax_per_s": w.relaxations * steps / t, "searches_per_s": w.B * steps / t,
-           "layer_kernel_ms_avg": layer_ms / max(1, w.Lmax - 1), "layer_loop_ms": layer_ms, "packed": packed, "cluster": cluster,
+           "layer_kernel_ms_avg": layer_ms / max(1, w.Lmax - 1), "layer_loop_ms": layer_ms, "packed": packed, "cluster": cluster, "path": path,
            "ms_median": statistics.median(step_ms), "ms_best": step_ms[0], "layer_loop_ms_min": layer_min, "layer_loop_ms_max": layer_max, "layer_loop_launches_timed": layer_n,
            "feasible": int((res["status"] == 0).sum()), "opt_cost_sum": int(res["opt_cost"][res["status"] == 0].sum())}
     return sb, out
@@ -534,15 +534,18 @@ def main():
                                         "peak": ALU_PEAK_GOPS}
             del sb3
             torch.cuda.empty_cache()
-        # Cost-only search: no table kept, two layers roll in the workspace (optimum per instance, no plan).
-        # All the relaxations are done; the tables' HBM footprint is 2 layers instead of Lmax.
+        # Cost-only search: no table kept, optimum per instance, no plan.  The tiled kernels do all the relaxations and roll two layers
+        # in the workspace; the cluster kernels and the solo kernel keep the state on chip and write the last layer alone, the solo
+        # kernel without most of the relaxations: no fraction of the ALU peak for those.
         sbc, rc = bench_workload(torch, galv, w, max(5, args.steps // 2), 3, barrier, flags=0)
         line["cost_only"] = {"ms_per_step": rc["ms_per_step"], "cells_per_s": rc["cells_per_s"],
                              "searches_per_s": rc["searches_per_s"], "opt_cost_sum": rc["opt_cost_sum"],
-                             "alu_frac": w.relaxations / (rc["layer_loop_ms"] * 1e-3) / 1e9 / (ALU_PEAK_GOPS * (2 if rc["packed"] else 1)),
+                             "kernel": ("tiled 32-bit", "tiled packed", "cluster", "solo")[rc["path"]],
+                             "alu_frac": (w.relaxations / (rc["layer_loop_ms"] * 1e-3) / 1e9 / (ALU_PEAK_GOPS * (2 if rc["packed"] else 1))
+                                          if rc["path"] in (gb.PATH_TILED_32, gb.PATH_TILED_PACKED) else None),
                              "packed": rc["packed"],
-                             "table_bytes": 2 * 4 * w.B * w.S * sbc.shape.m_pitch,
-                             "note": "optimum per instance without a plan; same relaxations, two-layer rolling buffer"}
+                             "table_bytes": (2 if rc["path"] in (gb.PATH_TILED_32, gb.PATH_TILED_PACKED) else 1) * 4 * w.B * w.S * sbc.shape.m_pitch,
+                             "note": "optimum per instance without a plan; table_bytes: what the kernel writes layers to"}
         del sbc
         torch.cuda.empty_cache()
         others = {}

@@ -351,7 +351,8 @@ __global__ void __launch_bounds__(kThreads) cost_kernel(int Lmax, int S, int KC,
 // round of evaluations, a barrier and one run of stores, their transition matrices with them.  An instance a CTA spent two thirds of
 // its time on the index arrays and the chain of divisions, with four CTAs an SM to hide them (62 registers).  8192 instances of
 // 160 layers, 64 strategies: 229 us in two kernels, 175 here (0.8 GB written: 4.6 TB/s).  Other large batches (a stack each, doubles
-// asked for, strategies not a multiple of four) take the two kernels.
+// asked for, strategies not a multiple of four, index arrays beyond 48 KB) take the two kernels.  Held to 64 registers for the four
+// CTAs: 24 bytes of spill stores, 48 of loads.
 constexpr int kBulkRoom = 2048;    // (layer kind, strategy) pairs a round
 struct BulkShared { int ndist, ncls, sbad, lbad, ok[8], len[8]; };
 __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax, int S, const int32_t* __restrict__ L, const galv_layer_desc* __restrict__ layers,
@@ -478,7 +479,8 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
 
 // The whole cost model in one launch, for batches small enough that a launch counts: the first CTAs write the
 // transition matrices (they run longest and check the descriptors for themselves), the others evaluate one
-// instance's layers each.  Bandwidth-sized batches take the two kernels one after the other (2 % faster there).
+// instance's layers each.  Larger batches take the bulk kernel where one stack is all there is, else the two kernels one after the
+// other (2 % faster there).
 __global__ void __launch_bounds__(kThreads) cost_trans_kernel(int B, int Lmax, int S, int KC, const int32_t* __restrict__ L,
                                                               const galv_layer_desc* __restrict__ layers, long long layer_stride_B,
                                                               const galv_strategy_desc* __restrict__ strat,

@@ -15,11 +15,12 @@
 //  - C does not rise with m.  So a strategy's value at a tile's last column bounds it from below all over the tile, its value
 //    at the first column from above: two cells a strategy say that it can neither win nor tie anywhere in the tile, nor come
 //    within a transition entry of what wins.  A lane looks at a strategy, a warp at 32 of them; one or two of 64 pass on the
-//    analytic models (tiles of 160 columns), three of 32 on measured tables (tiles of 32), and only those are relaxed.
+//    analytic models (tiles of 160 columns), three of 32 on measured tables whose transitions are a tenth of the times (tiles of 32),
+//    and only those are relaxed.
 //    Where they are of one row class k, G is base + T[k][.]: rows that hold T[k][.] already are left as they are.
 //
 // Taken where no table is written: optima, and the states that the host entry point's walk wants.  128 instances of 160 layers, 64
-// strategies, 8192 columns, optima: 2976 us in the resident kernel, 1165 here; host entry point 3525 / 2069.  A step of tiles takes 2300
+// strategies, 8192 columns, optima: 2976 us in the resident kernel, 1171 here; host entry point 3525 / 2078.  A step of tiles takes 2300
 // cycles, latencies of its test, its walk and its writes in turn; one with the edge of the feasible region in it 5000.
 //
 // How many strategies pass depends on the tables: with times that lie close together, or transitions as large as the times, most of
@@ -1050,9 +1051,8 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) solo_kernel(const SoA
     __syncthreads();                                            // the staged matrix is no longer read
 
     // ---- records of a layer, by one warp: int4 (where the strategy's differences and bases are read, in bytes from the first guard
-    // column on; time; row class | strategy << 8); time = +inf where mem exceeds the budget.  Two lists: all strategies in the
-    // table's order (their last word: where the argmin entries are read), and those that can matter in the order of their row
-    // classes: one whose row and column class has a member that needs no more memory and no more time (and is the lower one
+    // column on; time; row class); time = +inf where mem exceeds the budget.  Two lists: all strategies in the
+    // table's order, for the last layer's values, and those that can matter in the order of their row classes: one whose row and column class has a member that needs no more memory and no more time (and is the lower one
     // where both are equal) never does, as C does not rise with the budget.  ZeRO stages and checkpointing mostly differ in
     // memory alone: about half drop out.
     auto prepare = [&](int l, int from) -> int {                // returns the new frontier
