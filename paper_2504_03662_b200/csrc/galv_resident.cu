@@ -1240,11 +1240,15 @@ __global__ void __launch_bounds__((kMaxWarps + 1) * 32, 1) resident_kernel(const
 // same look inside the resident kernel cost a batch it turns away 15 us, most of them spent on fetching its code.
 __global__ void __launch_bounds__(256) probe_kernel(int B, int S, int after_solo, const int32_t* __restrict__ trans_q, long long trans_inst, int32_t* __restrict__ done)
 {
-    __shared__ int32_t rows[(kClassMax + 1) * kMaxS];
+    constexpr int R = kClassMax + 1;
+    __shared__ int32_t rows[R * kMaxS];
     __shared__ int s_pair;
-    const int R = min(kClassMax + 1, S);                        // a matrix has S rows
     const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     if (after_solo && done[i] == 3) return;
+    if (S < R) {                                                // a matrix has S rows
+        if (tid == 0) done[i] = 0;
+        return;
+    }
     const int32_t* const T = trans_q + (size_t)i * trans_inst;
     if (tid == 0) s_pair = 0;
     for (int k = tid; k < R * S; k += 256) rows[k] = T[k];
