@@ -350,11 +350,170 @@ __global__ void __launch_bounds__(kThreads) cost_kernel(int Lmax, int S, int KC,
 // tests, the layers' twins, the strategies' transition classes) is found once a CTA, and several instances at a time go through one
 // round of evaluations, a barrier and one run of stores, their transition matrices with them.  An instance a CTA spent two thirds of
 // its time on the index arrays and the chain of divisions, with four CTAs an SM to hide them (62 registers).  8192 instances of
-// 160 layers, 64 strategies: 229 us in two kernels, 175 here (0.8 GB written: 4.6 TB/s).  Other large batches (a stack each, doubles
-// asked for, strategies not a multiple of four, index arrays beyond 48 KB) take the two kernels.  Held to 64 registers for the four
-// CTAs: 24 bytes of spill stores, 48 of loads.
+// 160 layers, 64 strategies: 229 us in two kernels, 169 here (0.8 GB written: 4.8 TB/s).  Stacks of 64 kinds and more stay 5 to 15 %
+// faster in the two kernels (8192 of 160 kinds, 48 strategies: 1820 us, 1998 here; ragged ones 999, 1155), but how many there are is
+// known on the device only.  Other large batches (a stack each, doubles asked for, strategies not a multiple of four, index arrays
+// beyond 48 KB) take the two kernels.  Held to 64 registers for the four CTAs; its two loops are functions of their own, each with the
+// registers to itself (as one body it spilled: 175 us).
 constexpr int kBulkRoom = 2048;    // (layer kind, strategy) pairs a round
 struct BulkShared { int ndist, ncls, sbad, lbad, ok[8], len[8]; };
+
+struct BulkTables {                // in dynamic shared memory
+    int32_t *tabq, *tabm, *pairs;                              // pairs: [S * S]
+    int *kind, *slot, *list;                                   // [Lmax] a layer's nearest twin, later its kind; a first layer's kind; a kind's first layer
+    int *cls, *rep;                                            // [S] a strategy's transition class; a class's first strategy
+    __device__ __forceinline__ BulkTables(unsigned char* smem_raw, int S, int Lmax)
+        : tabq(reinterpret_cast<int32_t*>(smem_raw)), tabm(tabq + kBulkRoom), pairs(tabm + kBulkRoom), kind(reinterpret_cast<int*>(pairs + S * S)),
+          slot(kind + Lmax), list(slot + Lmax), cls(list + Lmax), rep(cls + S) {}
+};
+
+// The instances one at a time, where the kinds of one keep the threads busy (in several rounds where their costs pass the room).  Kinds
+// that only longer instances have are left out, and a flagged instance is written in one go: 4096 instances of 160 kinds, lengths
+// 1 to 160, 48 strategies: 589 us (1083 with every kind evaluated for each); flagged ones, 64 strategies: 86 us (279 with a pass over
+// the layers for each round of kinds, as valid ones have it).
+__device__ __noinline__ void bulk_by_one(const BulkShared& sh, unsigned char* smem_raw, int B, int Lmax, int S, const int32_t* __restrict__ L,
+                                         const galv_layer_desc* __restrict__ layers, const galv_strategy_desc* __restrict__ strat,
+                                         const galv_inst_params* __restrict__ inst, int32_t* __restrict__ time_q, int32_t* __restrict__ mem_q,
+                                         int32_t* __restrict__ trans_q, int32_t* __restrict__ status)
+{
+    const BulkTables tb(smem_raw, S, Lmax);
+    const int tid = threadIdx.x, ndist = sh.ndist, ncls = sh.ncls, nn = ncls * ncls, kc = min(ndist, kBulkRoom / S);
+    const int S4 = S >> 2, rows = kThreads / S4, c = tid % S4, r0 = tid / S4;
+    for (int i = blockIdx.x; i < B; i += gridDim.x) {
+        const int Li = L[i];
+        if (Li < 1 || Li > Lmax) {                             // nothing is written
+            if (tid == 0) status[i] = GALV_STATUS_BAD_INPUT;
+            continue;
+        }
+        const galv_inst_params in = inst[i];
+        const bool ok = !sh.sbad && sh.lbad >= Li && inst_ok(in);
+        if (tid == 0) status[i] = ok ? 0 : GALV_STATUS_BAD_INPUT;
+        const size_t base = (size_t)i * Lmax * S;
+        int4* const tq = reinterpret_cast<int4*>(time_q + base);
+        int4* const mq = reinterpret_cast<int4*>(mem_q + base);
+        int4* const xq = reinterpret_cast<int4*>(trans_q + (size_t)i * S * S);
+        if (!ok) {                                             // its tables say so to the search's validation as well
+            const int4 bad = make_int4(-1, -1, -1, -1);
+            for (int e = tid; e < Li * S4; e += kThreads) { tq[e] = bad; mq[e] = bad; }
+            for (int e = tid; e < S * S4; e += kThreads) xq[e] = bad;
+            continue;
+        }
+        for (int k0 = 0; k0 < ndist; k0 += kc) {
+            const int kn = min(kc, ndist - k0);
+            for (int e = tid; e < kn * S; e += kThreads) {
+                const int k = e / S, s = e - k * S, l = tb.list[k0 + k];
+                if (l >= Li) continue;
+                double t, b;
+                cost_of(layers[l], strat[s], in, &t, &b);
+                tb.tabq[e] = quant_time(t, in.time_unit_ns);
+                tb.tabm[e] = quant_mem(b, in.bin_bytes);
+            }
+            if (k0 == 0)
+                for (int e = tid; e < nn; e += kThreads) {
+                    const int ka = e / ncls, kb = e - ka * ncls;
+                    const galv_strategy_desc sa = strat[tb.rep[ka]], sc = strat[tb.rep[kb]];
+                    const double bq = in.b / sc.batch_div;
+                    const double bytes = bq * layers[0].seq * layers[0].h * in.bytes_per_elem;
+                    const double t = pair_factor(sa, sc) * bytes / in.bw_tp;
+                    tb.pairs[e] = quant_time(t, in.time_unit_ns);
+                }
+            __syncthreads();
+            if (r0 < rows) {
+                for (int l = r0; l < Li; l += rows) {
+                    const int k = tb.kind[l] - k0;
+                    if (k < 0 || k >= kn) continue;
+                    tq[l * S4 + c] = reinterpret_cast<const int4*>(tb.tabq + k * S)[c];
+                    mq[l * S4 + c] = reinterpret_cast<const int4*>(tb.tabm + k * S)[c];
+                }
+                if (k0 == 0) {
+                    const int k4[4] = {tb.cls[4 * c], tb.cls[4 * c + 1], tb.cls[4 * c + 2], tb.cls[4 * c + 3]};
+                    for (int f = r0; f < S; f += rows) {
+                        const int32_t* row = tb.pairs + tb.cls[f] * ncls;
+                        xq[f * S4 + c] = make_int4(row[k4[0]], row[k4[1]], row[k4[2]], row[k4[3]]);
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// Several instances a round: all their kinds fit one.
+__device__ __noinline__ void bulk_rounds(BulkShared& sh, unsigned char* smem_raw, int g, int B, int Lmax, int S, const int32_t* __restrict__ L,
+                                         const galv_layer_desc* __restrict__ layers, const galv_strategy_desc* __restrict__ strat,
+                                         const galv_inst_params* __restrict__ inst, int32_t* __restrict__ time_q, int32_t* __restrict__ mem_q,
+                                         int32_t* __restrict__ trans_q, int32_t* __restrict__ status)
+{
+    const BulkTables tb(smem_raw, S, Lmax);
+    int32_t *const tabq = tb.tabq, *const tabm = tb.tabm, *const pairs = tb.pairs;
+    int *const root = tb.kind, *const list = tb.list, *const cls = tb.cls, *const rep = tb.rep;
+    const int tid = threadIdx.x, ndist = sh.ndist, nn = sh.ncls * sh.ncls;
+    const int S4 = S >> 2, rows = kThreads / S4, c = tid % S4, r0 = tid / S4;
+    for (int i0 = blockIdx.x * g; i0 < B; i0 += gridDim.x * g) {
+        const int m = min(g, B - i0);
+        if (tid < m) {
+            const int Li = L[i0 + tid], in_range = Li >= 1 && Li <= Lmax;
+            const int ok = in_range && !sh.sbad && sh.lbad >= Li && inst_ok(inst[i0 + tid]);
+            sh.len[tid] = in_range ? Li : 0;                    // out of range: nothing is written
+            sh.ok[tid] = ok ? Li : 0;
+            status[i0 + tid] = ok ? 0 : GALV_STATUS_BAD_INPUT;
+        }
+        __syncthreads();
+        const int per = ndist * S;
+        for (int e = tid; e < m * per; e += kThreads) {
+            const int n = e / per, r = e - n * per, k = r / S, s = r - k * S;
+            const int l = list[k];
+            if (l >= sh.ok[n]) continue;
+            const galv_inst_params in = inst[i0 + n];
+            double t, b;
+            cost_of(layers[l], strat[s], in, &t, &b);
+            tabq[e] = quant_time(t, in.time_unit_ns);
+            tabm[e] = quant_mem(b, in.bin_bytes);
+        }
+        for (int e = tid; e < m * nn; e += kThreads) {
+            const int n = e / nn, r = e - n * nn, ka = r / sh.ncls, kb = r - ka * sh.ncls;
+            if (!sh.ok[n]) continue;
+            const galv_inst_params in = inst[i0 + n];
+            const galv_strategy_desc sa = strat[rep[ka]], sc = strat[rep[kb]];
+            const double bq = in.b / sc.batch_div;
+            const double bytes = bq * layers[0].seq * layers[0].h * in.bytes_per_elem;
+            const double t = pair_factor(sa, sc) * bytes / in.bw_tp;
+            pairs[e] = quant_time(t, in.time_unit_ns);
+        }
+        __syncthreads();
+        for (int n = 0; n < m; ++n) {
+            const size_t base = (size_t)(i0 + n) * Lmax * S;
+            const bool ok = sh.ok[n] != 0;
+            const int Li = sh.len[n];
+            if (r0 < rows)
+                for (int l = r0; l < Li; l += rows) {
+                    const int k = root[l];
+                    int4 tv = make_int4(-1, -1, -1, -1), mv = tv;      // flagged: its tables say so to the search's validation as well
+                    if (ok) {
+                        tv = reinterpret_cast<const int4*>(tabq + n * per + k * S)[c];
+                        mv = reinterpret_cast<const int4*>(tabm + n * per + k * S)[c];
+                    }
+                    reinterpret_cast<int4*>(time_q + base + (size_t)l * S)[c] = tv;
+                    reinterpret_cast<int4*>(mem_q + base + (size_t)l * S)[c] = mv;
+                }
+            if (Li > 0) {
+                int32_t* const out = trans_q + (size_t)(i0 + n) * S * S;
+                const int k4[4] = {cls[4 * c], cls[4 * c + 1], cls[4 * c + 2], cls[4 * c + 3]};
+                if (r0 < rows)
+                    for (int a = r0; a < S; a += rows) {
+                        int4 v = make_int4(-1, -1, -1, -1);
+                        if (ok) {
+                            const int32_t* row = pairs + n * nn + cls[a] * sh.ncls;
+                            v = make_int4(row[k4[0]], row[k4[1]], row[k4[2]], row[k4[3]]);
+                        }
+                        reinterpret_cast<int4*>(out + (size_t)a * S)[c] = v;
+                    }
+            }
+        }
+        __syncthreads();
+    }
+}
+
 __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax, int S, const int32_t* __restrict__ L, const galv_layer_desc* __restrict__ layers,
                                                                 const galv_strategy_desc* __restrict__ strat, const galv_inst_params* __restrict__ inst,
                                                                 int32_t* __restrict__ time_q, int32_t* __restrict__ mem_q, int32_t* __restrict__ trans_q,
@@ -363,14 +522,8 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ BulkShared sh;
     const int tid = threadIdx.x;
-    int32_t* const tabq = reinterpret_cast<int32_t*>(smem_raw);
-    int32_t* const tabm = tabq + kBulkRoom;
-    int32_t* const pairs = tabm + kBulkRoom;                   // [S * S]
-    int* const root = reinterpret_cast<int*>(pairs + S * S);
-    int* const slot = root + Lmax;
-    int* const list = slot + Lmax;
-    int* const cls = list + Lmax;                              // transition class of each strategy
-    int* const rep = cls + S;
+    const BulkTables tb(smem_raw, S, Lmax);
+    int *const root = tb.kind, *const slot = tb.slot, *const list = tb.list, *const cls = tb.cls, *const rep = tb.rep;
     if (tid == 0) { sh.ndist = 0; sh.ncls = 0; sh.sbad = 0; sh.lbad = Lmax; }
     __syncthreads();
     for (int l = tid; l < Lmax; l += kThreads) {
@@ -408,73 +561,10 @@ __global__ void __launch_bounds__(kThreads, 4) cost_bulk_kernel(int B, int Lmax,
     const int ndist = sh.ndist, nn = sh.ncls * sh.ncls, kc = min(ndist, kBulkRoom / S);
     // instances a round: as many as the threads evaluate at once and the tables hold
     const int g = max(1, min(min(8, kThreads / (kc * S)), S * S / nn));
-    const int S4 = S >> 2, rows = kThreads / S4, c = tid % S4, r0 = tid / S4;
-    for (int i0 = blockIdx.x * g; i0 < B; i0 += gridDim.x * g) {
-        const int m = min(g, B - i0);
-        if (tid < m) {
-            const int Li = L[i0 + tid], in_range = Li >= 1 && Li <= Lmax;
-            const int ok = in_range && !sh.sbad && sh.lbad >= Li && inst_ok(inst[i0 + tid]);
-            sh.len[tid] = in_range ? Li : 0;                    // out of range: nothing is written
-            sh.ok[tid] = ok;
-            status[i0 + tid] = ok ? 0 : GALV_STATUS_BAD_INPUT;
-        }
-        __syncthreads();
-        for (int k0 = 0; k0 < ndist; k0 += kc) {
-            const int kn = min(kc, ndist - k0), per = kn * S;
-            for (int e = tid; e < m * per; e += kThreads) {
-                const int n = e / per, r = e - n * per, k = r / S, s = r - k * S;
-                if (!sh.ok[n]) continue;
-                const galv_inst_params in = inst[i0 + n];
-                double t, b;
-                cost_of(layers[list[k0 + k]], strat[s], in, &t, &b);
-                tabq[e] = quant_time(t, in.time_unit_ns);
-                tabm[e] = quant_mem(b, in.bin_bytes);
-            }
-            if (k0 == 0)
-                for (int e = tid; e < m * nn; e += kThreads) {
-                    const int n = e / nn, r = e - n * nn, ka = r / sh.ncls, kb = r - ka * sh.ncls;
-                    if (!sh.ok[n]) continue;
-                    const galv_inst_params in = inst[i0 + n];
-                    const galv_strategy_desc sa = strat[rep[ka]], sc = strat[rep[kb]];
-                    const double bq = in.b / sc.batch_div;
-                    const double bytes = bq * layers[0].seq * layers[0].h * in.bytes_per_elem;
-                    const double t = pair_factor(sa, sc) * bytes / in.bw_tp;
-                    pairs[e] = quant_time(t, in.time_unit_ns);
-                }
-            __syncthreads();
-            for (int n = 0; n < m; ++n) {
-                const size_t base = (size_t)(i0 + n) * Lmax * S;
-                const bool ok = sh.ok[n] != 0;
-                const int Li = sh.len[n];
-                if (r0 < rows)
-                    for (int l = r0; l < Li; l += rows) {
-                        const int k = root[l] - k0;
-                        if (ok && (k < 0 || k >= kn)) continue;
-                        int4 tv = make_int4(-1, -1, -1, -1), mv = tv;      // flagged: its tables say so to the search's validation as well
-                        if (ok) {
-                            tv = reinterpret_cast<const int4*>(tabq + n * per + k * S)[c];
-                            mv = reinterpret_cast<const int4*>(tabm + n * per + k * S)[c];
-                        }
-                        reinterpret_cast<int4*>(time_q + base + (size_t)l * S)[c] = tv;
-                        reinterpret_cast<int4*>(mem_q + base + (size_t)l * S)[c] = mv;
-                    }
-                if (k0 == 0 && Li > 0) {
-                    int32_t* const out = trans_q + (size_t)(i0 + n) * S * S;
-                    const int k4[4] = {cls[4 * c], cls[4 * c + 1], cls[4 * c + 2], cls[4 * c + 3]};
-                    if (r0 < rows)
-                        for (int a = r0; a < S; a += rows) {
-                            int4 v = make_int4(-1, -1, -1, -1);
-                            if (ok) {
-                                const int32_t* row = pairs + n * nn + cls[a] * sh.ncls;
-                                v = make_int4(row[k4[0]], row[k4[1]], row[k4[2]], row[k4[3]]);
-                            }
-                            reinterpret_cast<int4*>(out + (size_t)a * S)[c] = v;
-                        }
-                }
-            }
-            __syncthreads();
-        }
-    }
+    if (g == 1)
+        bulk_by_one(sh, smem_raw, B, Lmax, S, L, layers, strat, inst, time_q, mem_q, trans_q, status);
+    else
+        bulk_rounds(sh, smem_raw, g, B, Lmax, S, L, layers, strat, inst, time_q, mem_q, trans_q, status);
 }
 
 // The whole cost model in one launch, for batches small enough that a launch counts: the first CTAs write the

@@ -164,3 +164,31 @@ def test_large_batch_of_one_stack(orc, galv, pattern, Lmax, S):
         assert st[i] == orc.descriptor_status(w.layers[0], w.strat, w.inst[i], Li), i
         assert (tq[i, :Li] == rtq).all() and (mq[i, :Li] == rmq).all() and (xq[i] == rxq).all(), i
         assert (tq[i, Li:] == -7).all() and (mq[i, Li:] == -7).all(), i
+
+
+def test_flagged_instances_are_not_evaluated_kind_by_kind(galv):
+    """A stack of 300 kinds, every instance flagged: its tables are written once, not in eight rounds.  Valid ones take an
+    order of magnitude longer, so half is a wide line."""
+    import torch
+    from paper_2504_03662_b200.search import SearchBuffers
+    strat = inputs.strategy_table((1, 2, 4, 8, 16, 32, 64), (0, 2, 3), (0, 1), (0, 1))[:48]
+    us = []
+    for bw in (None, -1.0):
+        w = stack(11, 2048, 300, strat, "distinct")
+        w.L[:] = 300
+        if bw is not None:
+            w.inst["bw_tp"] = bw
+        sb = SearchBuffers(galv, w, 0)
+        for _ in range(3):
+            sb.eval_costs()
+        best = float("inf")
+        for _ in range(5):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            sb.eval_costs()
+            end.record()
+            end.synchronize()
+            best = min(best, start.elapsed_time(end))
+        us.append(best * 1e3)
+        assert (sb.status.cpu().numpy() == (0 if bw is None else 2)).all()
+    assert us[1] < 0.5 * us[0], us
