@@ -167,8 +167,8 @@ def test_large_batch_of_one_stack(orc, galv, pattern, Lmax, S):
 
 
 def test_flagged_instances_are_not_evaluated_kind_by_kind(galv):
-    """A stack of 300 kinds, every instance flagged: its tables are written once, not in eight rounds.  Valid ones take an
-    order of magnitude longer, so half is a wide line."""
+    """A stack of 300 kinds, every instance flagged: its tables are written once, in 0.07 of the time that valid ones take; with
+    a pass over the layers for each of the eight rounds of kinds it was 0.28."""
     import torch
     from paper_2504_03662_b200.search import SearchBuffers
     strat = inputs.strategy_table((1, 2, 4, 8, 16, 32, 64), (0, 2, 3), (0, 1), (0, 1))[:48]
@@ -191,4 +191,4 @@ def test_flagged_instances_are_not_evaluated_kind_by_kind(galv):
             best = min(best, start.elapsed_time(end))
         us.append(best * 1e3)
         assert (sb.status.cpu().numpy() == (0 if bw is None else 2)).all()
-    assert us[1] < 0.5 * us[0], us
+    assert us[1] < 0.15 * us[0], us
